@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/kvq.h"
+#include "kvq_device.cuh"
 #include "kvq_internal.h"
 
 namespace kvq {
@@ -625,6 +626,8 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
 static __global__ void kvq_calibrate_finish_kernel(float *lambda, int D)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_trigger();
+    grid_wait();
     if (c < D) {
         const float a = lambda[c];
         lambda[c] = a > 0.0f ? 1.0f / a : 1.0f;
@@ -655,9 +658,8 @@ kvq_status_t kvq_calibrate_lambda(kvq_plan_t *plan, const void *x, kvq_dtype_t d
             return KVQ_ERR_CUDA;
         }
     }
-    kvq_calibrate_finish_kernel<<<(plan->D + 127) / 128, 128, 0, stream>>>(lambda_out, plan->D);
-    count_launch();
-    if (cudaGetLastError() != cudaSuccess) return KVQ_ERR_CUDA;
+    if (launch_kernel(kvq_calibrate_finish_kernel, (unsigned)((plan->D + 127) / 128), 128, 0, stream, 1, reinterpret_cast<float *>(lambda_out), plan->D) != cudaSuccess)
+        return KVQ_ERR_CUDA;
     return KVQ_OK;
 }
 

@@ -339,6 +339,7 @@ __global__ void __launch_bounds__(WARPS * 32) kvq_encode_fft_kernel(const __grid
     float4 *stash = reinterpret_cast<float4 *>(wb + S::IN_BYTES + S::OUT_BYTES);
     float *lam_cache = reinterpret_cast<float *>(wb + S::IN_BYTES + S::OUT_BYTES + S::STASH_BYTES);
     const uint32_t bar0 = smem_u32(smem + warp * 16), bar1 = bar0 + 8;
+    grid_wait();
 
     if (lane == 0) {
         mbar_init(bar0, 32);
@@ -409,6 +410,7 @@ __global__ void __launch_bounds__(WARPS * 32) kvq_encode_fft_kernel(const __grid
             todo &= ~mine;
         }
     }
+    grid_trigger();
     bulk_wait_all();
 }
 
@@ -426,6 +428,7 @@ __global__ void __launch_bounds__(WARPS * 32) kvq_decode_fft_kernel(const __grid
     float4 *stash = reinterpret_cast<float4 *>(wb + S::IN_BYTES + S::OUT_BYTES);
     float *lam_cache = reinterpret_cast<float *>(wb + S::IN_BYTES + S::OUT_BYTES + S::STASH_BYTES);
     const uint32_t bar0 = smem_u32(smem + warp * 16), bar1 = bar0 + 8;
+    grid_wait();
 
     if (lane == 0) {
         mbar_init(bar0, 32);
@@ -536,6 +539,7 @@ __global__ void __launch_bounds__(WARPS * 32) kvq_decode_fft_kernel(const __grid
             todo &= ~mine;
         }
     }
+    grid_trigger();
     bulk_wait_all();
 }
 
@@ -564,9 +568,7 @@ static cudaError_t launch_persistent(Kern kern, int warps, size_t smem, int64_t 
     const int64_t want = (tiles + warps - 1) / warps;
     const int64_t cap = (int64_t)(*cached_blocks_per_sm) * (*cached_sms);
     const int grid = (int)(want < cap ? want : cap);
-    kern<<<grid, warps * 32, smem, stream>>>(prm);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kern, (unsigned)grid, (unsigned)(warps * 32), smem, stream, 1, prm);
 }
 
 // GRP == 0 stands for one group over the whole vector (GRP = D).

@@ -161,7 +161,7 @@ __device__ __forceinline__ void matvec(const float *__restrict__ table, float4 (
 // One batch of kV vectors.  t: the first pass of this warp's table rows, requested by the caller.
 template <int D, bool BF16, bool FLUSH>
 __device__ __forceinline__ void encode_batch(const MatvecParams &prm, const RowMap &out_map, float4 (&t)[Geo<D>::CH][Geo<D>::P], float *xs,
-                                             float *red, int warp, int lane, int64_t batch)
+                                             float *red, int warp, int lane, int64_t batch, bool last)
 {
     using Gm = Geo<D>;
     constexpr int P = Gm::P;
@@ -185,6 +185,7 @@ __device__ __forceinline__ void encode_batch(const MatvecParams &prm, const RowM
         xs[v * D + 2 * j] = f.x, xs[v * D + 2 * j + 1] = f.y;
     }
     __syncthreads();
+    if (last) grid_trigger();   // nothing but the tables is read from here on
 
     float z[P][4];
     matvec<D>(prm.table, t, xs, red, warp, lane, z);
@@ -291,15 +292,16 @@ __global__ void __launch_bounds__(kWarps * 32) kvq_encode_matvec_kernel(const __
     // ---- everything that does not depend on the vectors is requested first, so that one round trip covers it all
     float4 t[Gm::CH][Gm::P];
     load_rows<D>(prm.table, warp, lane, 0, t);
+    grid_wait();
     RowMap out_map;
     if (!resolve_out_map(prm, out_map)) return;   // uniform over the grid: no barrier is left waiting
     if constexpr (Gm::kLoops) {
         const int64_t n_batches = (prm.N + kV - 1) / kV;
 #pragma unroll 1
         for (int64_t batch = blockIdx.x; batch < n_batches; batch += gridDim.x)
-            encode_batch<D, BF16, FLUSH>(prm, out_map, t, xs, red, warp, lane, batch);
+            encode_batch<D, BF16, FLUSH>(prm, out_map, t, xs, red, warp, lane, batch, batch + gridDim.x >= n_batches);
     } else {
-        encode_batch<D, BF16, FLUSH>(prm, out_map, t, xs, red, warp, lane, blockIdx.x);
+        encode_batch<D, BF16, FLUSH>(prm, out_map, t, xs, red, warp, lane, blockIdx.x, true);
     }
 }
 
@@ -308,7 +310,7 @@ __global__ void __launch_bounds__(kWarps * 32) kvq_encode_matvec_kernel(const __
 // ------------------------------------------------------------------------------------------------
 template <int D, bool BF16>
 __device__ __forceinline__ void decode_batch(const MatvecParams &prm, float4 (&t)[Geo<D>::CH][Geo<D>::P], float *zs, float *red, int warp,
-                                             int lane, int64_t batch)
+                                             int lane, int64_t batch, bool last)
 {
     using Gm = Geo<D>;
     constexpr int P = Gm::P;
@@ -344,6 +346,7 @@ __device__ __forceinline__ void decode_batch(const MatvecParams &prm, float4 (&t
         *reinterpret_cast<float4 *>(zs + v * D + 4 * i) = o;
     }
     __syncthreads();
+    if (last) grid_trigger();   // nothing but the table is read from here on
 
     float y[P][4];
     matvec<D>(prm.table, t, zs, red, warp, lane, y);
@@ -368,12 +371,14 @@ __global__ void __launch_bounds__(kWarps * 32) kvq_decode_matvec_kernel(const __
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float4 t[Gm::CH][Gm::P];
     load_rows<D>(prm.table, warp, lane, 0, t);   // in flight while the codes are fetched and dequantised
+    grid_wait();
     if constexpr (Gm::kLoops) {   // as in the encode kernel
         const int64_t n_batches = (prm.N + kV - 1) / kV;
 #pragma unroll 1
-        for (int64_t batch = blockIdx.x; batch < n_batches; batch += gridDim.x) decode_batch<D, BF16>(prm, t, zs, red, warp, lane, batch);
+        for (int64_t batch = blockIdx.x; batch < n_batches; batch += gridDim.x)
+            decode_batch<D, BF16>(prm, t, zs, red, warp, lane, batch, batch + gridDim.x >= n_batches);
     } else {
-        decode_batch<D, BF16>(prm, t, zs, red, warp, lane, blockIdx.x);
+        decode_batch<D, BF16>(prm, t, zs, red, warp, lane, blockIdx.x, true);
     }
 }
 
@@ -398,9 +403,7 @@ cudaError_t launch(const MatvecParams &prm, cudaStream_t stream)
     if (batches > 0x7FFFFFFF) return cudaErrorInvalidValue;
     // one resident wave of CTAs that loop over batches where the kernel does; else a CTA per batch
     const int ctas = (int)(Geo<D>::kLoops && batches > slots.sms[dev] ? slots.sms[dev] : batches);
-    kern<<<ctas, kWarps * 32, Geo<D>::kSmemBytes, stream>>>(prm);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kern, (unsigned)ctas, kWarps * 32, Geo<D>::kSmemBytes, stream, 1, prm);
 }
 
 template <int MODE>

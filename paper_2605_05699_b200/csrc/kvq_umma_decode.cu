@@ -327,6 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (n_my > 0 && warp >= 2) {
         FirstRows<D, BF16OUT, BITS, R2> rows;
         rows.load(prm.g.b0, (warp - 2) * (C::kBRows / 16), lane);
+        grid_wait();
         if (warp < 10 && ((warp - 2) >> 2) < n_my) {   // dequant group g's first tile is tile_begin + g
             const TileCursor first(tile_begin + ((warp - 2) >> 2), tps);
             const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
@@ -353,6 +354,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
     } else {
+        grid_wait();
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
@@ -690,6 +692,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) bulk_wait_all();
     }
 
+    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -765,9 +768,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const ui
 
     const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
-    kvq_decode_umma_kernel<D, BF16OUT, BITS, R2><<<grid, kThreads, C::kSmemBytes, stream>>>(prm, maps);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 }  // namespace

@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * kD; };
 
+    grid_wait();
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
@@ -484,6 +485,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) bulk_wait_all();
     }
 
+    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -554,9 +556,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cud
 
     const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
-    kvq_decode_umma_d256_kernel<BF16OUT, BITS><<<grid, kThreads, C::kSmemBytes, stream>>>(prm, maps);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kvq_decode_umma_d256_kernel<BF16OUT, BITS>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 }  // namespace

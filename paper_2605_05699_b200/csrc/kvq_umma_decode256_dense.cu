@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     fence_proxy_async();
     tc_fence_before();
+    grid_wait();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
@@ -424,6 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) bulk_wait_all();
     }
 
+    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -490,9 +492,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream)
 
     const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int64_t pairs = tiles < sms / 2 ? tiles : sms / 2;
-    kvq_decode_umma_d256_dense_kernel<BF16OUT><<<(int)(2 * pairs), kThreads, C::kSmemBytes, stream>>>(prm, maps);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kvq_decode_umma_d256_dense_kernel<BF16OUT>, (unsigned)(2 * pairs), kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 }  // namespace

@@ -168,7 +168,7 @@ struct FirstRows {
     static constexpr int kRows = D / 16, kPasses = (D / 4 + 31) / 32;
     float4 m[kRows][kPasses];
     float lam_c[kRows];
-    __device__ __forceinline__ void load(const float *__restrict__ e0, const float *__restrict__ lam, int c0, int lane)
+    __device__ __forceinline__ void load_table(const float *__restrict__ e0, int c0, int lane)
     {
 #pragma unroll
         for (int k = 0; k < kRows; ++k) {
@@ -177,8 +177,12 @@ struct FirstRows {
                 const int i = lane + 32 * p;
                 m[k][p] = i < D / 4 ? __ldg(reinterpret_cast<const float4 *>(e0 + (size_t)(c0 + k) * D) + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
-            lam_c[k] = lam ? __ldg(lam + c0 + k) : 1.0f;
         }
+    }
+    __device__ __forceinline__ void load_lambda(const float *__restrict__ lam, int c0)
+    {
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) lam_c[k] = lam ? __ldg(lam + c0 + k) : 1.0f;
     }
     __device__ __forceinline__ void build(unsigned char *sB, float lift, int c0, int lane) const
     {
@@ -266,7 +270,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         first_seg = tile_begin / tps;
         const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : first_seg) * D;
         FirstRows<D, BF16, CALIB || WIDE> rows;
-        rows.load(prm.e0, lam, (warp - 2) * (D / 16), lane);
+        rows.load_table(prm.e0, (warp - 2) * (D / 16), lane);
+        grid_wait();
+        rows.load_lambda(lam, (warp - 2) * (D / 16));
         first_lift = lift_of<D>(lam, prm.table_max, lane);
         fence_proxy_async();
         tc_fence_before();
@@ -277,6 +283,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
     } else {
+        grid_wait();
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
@@ -548,6 +555,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
 
+    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -614,9 +622,7 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
 
     const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
-    kvq_encode_umma_kernel<D, BF16, CALIB, PERVEC, WIDE><<<grid, kThreads, C::kSmemBytes, stream>>>(prm, tm_x);
-    count_launch();
-    return cudaGetLastError();
+    return launch_kernel(kvq_encode_umma_kernel<D, BF16, CALIB, PERVEC, WIDE>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, tm_x);
 }
 
 }  // namespace

@@ -228,6 +228,7 @@ __device__ __forceinline__ void encode_d256_body(const UmmaEncode256Params &prm,
         mbar_init_fence();
     }
     if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
+    grid_wait();
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
@@ -518,6 +519,7 @@ __device__ __forceinline__ void encode_d256_body(const UmmaEncode256Params &prm,
         }
     }
 
+    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -620,14 +622,10 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     if constexpr (PERVEC) {
         const int fit = slots.blocks_per_sm[dev];   // clusters resident at once
         if (pairs > fit) pairs = fit;
-        cfg.gridDim = dim3((unsigned)(2 * pairs), 1, 1);
-        e = cudaLaunchKernelEx(&cfg, kern, prm, tm_x);
-        count_launch();
-        return e != cudaSuccess ? e : cudaGetLastError();
     }
-    kern<<<(int)(2 * pairs), kThreads, C::kSmemBytes, stream>>>(prm, tm_x);
-    count_launch();
-    return cudaGetLastError();
+    // the CTAs of a pair read the same tiles, the second one out of L2: they are to start together (212,992 bf16 vectors, 52 lambda
+    // rows: 65.5 us so, 67.2 us when they come up as the SMs of the kernel before fall free)
+    return launch_kernel<false>(kern, (unsigned)(2 * pairs), kThreads, C::kSmemBytes, stream, PERVEC ? 2 : 1, prm, tm_x);
 }
 
 }  // namespace

@@ -92,3 +92,56 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_service_returns():
     ora = ko.encode(wl.raw_bits(x), ko.F16, sg, lam.numpy(), G, want_v=True)
     parity.check_encode(packed.cpu().numpy(), wl.raw_bits(scales), ora, G, "encode after a reported time-out", min_agree=0.9995)
     plan.close()
+
+
+@pytest.mark.parametrize("D,dtype,group,nbits", [(64, "bf16", 32, 4), (96, "f16", 32, 4), (128, "f16", 32, 4), (128, "bf16", 128, 8),
+                                                 (160, "bf16", 32, 4), (256, "bf16", 32, 4), (256, "f16", 256, 4), (256, "bf16", 32, 8)])
+def test_a_call_queued_behind_another_sees_all_that_it_wrote(D, dtype, group, nbits):
+    """A grid may come up while its predecessor runs out: chains encode -> decode -> encode of the decoded rows -> append -> decode,
+    queued without a wait on one buffer set, on a side stream and as a replayed graph, against the same calls one by one."""
+    N, S = 3 * 128 * 148 + 77, 37
+    plan = kb.Plan(D, group, 5, bits=nbits)
+    dt = wl.torch_dtype(dtype)
+    kb.kvq_plan_prepare(plan.handle, dt)
+    xs = [wl.make_vectors(N, D, dtype, "gaussian", 6 + i, device="cuda") for i in range(2)]
+    new = wl.make_vectors(S, D, dtype, "gaussian", 9, device="cuda")
+    lam = wl.make_lambda(3, D, 8).cuda()
+    rpl, T = -(-N // 3), N // S
+
+    def buffers():
+        return [torch.zeros(N, D * nbits // 8, dtype=torch.uint8, device="cuda"),
+                torch.zeros(N, D // group, dtype=torch.float16, device="cuda"), torch.zeros(N, D, dtype=dt, device="cuda")]
+
+    def chain(b, wait):
+        packed, scales, out = b
+        for x in xs:
+            for src in (x, out):
+                kb.kvq_encode(plan.handle, src, lam, packed, scales, rpl)
+                wait()
+                kb.kvq_append(plan.handle, new, lam, packed[:S * T].view(S, T, -1), scales[:S * T].view(S, T, -1), T - 1, 13)
+                wait()
+                kb.kvq_decode(plan.handle, packed, scales, lam, out, rpl)
+                wait()
+
+    want = buffers()
+    chain(want, torch.cuda.synchronize)
+    side = torch.cuda.Stream()
+    for _ in range(4):
+        got = buffers()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            chain(got, lambda: None)
+        torch.cuda.current_stream().wait_stream(side)
+        assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(got, want))
+    got = buffers()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain(got, lambda: None)
+    for _ in range(3):
+        for b in got:
+            b.zero_()
+        graph.replay()
+        assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(got, want))
+    del graph
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    plan.close()
