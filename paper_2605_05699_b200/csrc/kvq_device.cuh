@@ -166,6 +166,12 @@ __device__ __forceinline__ void bulk_store(void *dst_gmem, uint32_t src_smem, ui
                  : "memory");
 }
 
+// asks for a contiguous run to be brought into L2; bytes % 16 == 0, address 16-byte aligned
+__device__ __forceinline__ void prefetch_l2(const void *src_gmem, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src_gmem), "r"(bytes) : "memory");
+}
+
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 
 // Waits until the shared-memory sources of all this thread's bulk stores have been read.
@@ -215,7 +221,7 @@ struct TileCursor {
 };
 
 // The contiguous share of a call's tiles that one CTA (or one CTA pair) of a persistent kernel takes: lambda segments of rpl
-// rows are cut into tiles of 128 rows (a segment's last tile may be short), n_seg * tps tiles in all, `parts` shares.
+// rows are cut into tiles of 128 rows (256 where a CTA pair works on one tile) (a segment's last tile may be short), n_seg * tps tiles in all, `parts` shares.
 // Contiguous, so that the B operand of a lambda row is rebuilt as rarely as possible.  A share that crosses into another
 // lambda row pays a rebuild of B, about one tile's time, so with several rows and at least eight tiles per share the shares
 // are equal in COST, each segment counting one unit more than its tiles (a share that would begin inside that unit begins
@@ -224,9 +230,9 @@ struct TileShare {
     int64_t tps;     // tiles per segment
     int64_t begin;   // first tile of this share
     int n;           // tiles in this share
-    __device__ __forceinline__ TileShare(int64_t n_seg, int64_t rpl, unsigned part, unsigned parts)
+    __device__ __forceinline__ TileShare(int64_t n_seg, int64_t rpl, unsigned part, unsigned parts, int tile_rows = 128)
     {
-        tps = (rpl + 127) / 128;
+        tps = (rpl + tile_rows - 1) / tile_rows;
         const int64_t n_tiles = n_seg * tps;
         const int64_t R = (n_seg > 1 && n_tiles >= 8 * (int64_t)parts) ? 1 : 0;   // cost units of a rebuild
         const int64_t C = tps + R, total = n_seg * C;

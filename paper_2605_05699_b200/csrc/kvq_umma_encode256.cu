@@ -1,127 +1,90 @@
 // Warp-specialised tcgen05 DFT-as-GEMM encode kernel of libkvq (sm_100a) for D = 256, fp16 or bf16 input.
 //
 // Same contraction and the same split of W into 16-bit terms as kvq_umma_encode.cu (v = lambda (.) M (s (.) x),
-// Sec. 3.1 Eq. 1-2, Sec. 5.1 item 1; W 2^k = W1 + W2, a third term for bf16 in the calibration pass), with the two changes
-// that D = 256 forces:
+// Sec. 3.1 Eq. 1-2, Sec. 5.1 item 1; W 2^k = W1 + W2, a third term for bf16 in the calibration pass).  The split B operand
+// (2 or 3 x 128 KB) does not fit one CTA's shared memory, so a PAIR of CTAs (a cluster of two) works on one tile of 256 vectors
+// (128 on short calls) with cta_group::2 instructions: each CTA holds its own half of the vectors and one half of B's rows
+// (channels), the leader's one thread issues MMAs of N = 256 over both, and each CTA's tensor memory receives all 256 channels
+// of its own vectors.
 //
-//   * the split B operand (2 or 3 x 128 KB) does not fit one CTA's shared memory, so CTAs work in pairs on the
-//     same tiles and each computes one half of the channels (four groups): B is [128 channels, K = 256] per
-//     term and CTA.  The two CTAs of a pair share nothing and never wait for each other; the x tile is read
-//     twice (the second read hits L2).
-//   * what shared memory is left holds little more than one x tile next to B, so x moves through a ring
-//     of K blocks (64 columns x 128 rows, 16 KB): the mma thread issues the K steps of a block for every term
-//     as soon as the block has landed and releases it with a commit of its own.
+// What bounds it: 32 MMAs of 128 cycles per tile (2.1 us per 128 vectors and SM at 1965 MHz; the bytes take 1.9), and, back to
+// back, the board's power limit.  The form before this one gave each CTA 128 channels of the same 128 vectors: every x block was
+// fetched by both CTAs, the ring beside B held less than the latency of its loads, and both split terms were added up in the
+// epilogue.  Before -> now, back to back: 212,992 bf16 vectors under 52 lambda rows 62.4 -> 58.6 us, 1,064,960 under one
+// 287 -> 266, one scale per vector 73.8 -> 64.0, calibration of 200,000 fp16 vectors 65.0 -> 51.9, 9000 vectors 10.3 -> 9.5.
+// Between 38,000 and 60,000 vectors, where a pair's three or four tall tiles take the place of five to seven, 5 to 9 % slower.
 //
-// Roles as in kvq_umma_encode.cu: producer (TMA), one mma thread, two epilogue sets of eight warps on
-// alternate tiles (thread = (row, two groups)).  With two terms they are stacked along N as there (one MMA of
-// N = 256 per K-step and CTA, two accumulator stages of 256 columns, the epilogue adds the halves); the three-term
-// calibration form keeps four stages of 128 columns.  Byte codes (fp16 input) are a run-time switch of the epilogue.
-// Every wait is bounded.
+//   warp 0        producer   (both CTAs) one TMA tensor load per K block of 64 columns into a ring of blocks; the
+//                            loads of both CTAs complete on the leader's barrier
+//   warp 1        mma        (leader) per tile every K step of the small term first, then of the large one: the small sums are
+//                            then added up before anything large is in the accumulator, so that each rounding of the fp32
+//                            accumulator is counted once per K step of the large term alone.  A block is released
+//                            in the second pass.  (Three terms: block by block, all terms; the ring holds two blocks.)
+//   warps 2-17    epilogue   (both CTAs) all sixteen warps on every tile, thread = (row, two of the row's eight groups, or one)
+//
+// Byte codes (fp16 input) are a run-time switch of the epilogue.  Every wait is bounded.
 #include "kvq_internal.h"
+#include "kvq_quantize.cuh"
 #include "kvq_umma.cuh"
 
 namespace kvq {
 
 namespace {
 
-constexpr int kTile = 128;                 // vectors per tile = MMA M
 constexpr int kGroup = 32;
 constexpr int kThreads = 576;              // producer, mma, 16 epilogue warps
 constexpr int kEpiWarps = 16;
-constexpr int kBlockBytes = kTile * 128;   // one K block of the x tile: 128 rows x 128 B
-constexpr int kCtrlBytes = 256;
+constexpr int kCtrlBytes = 512;
 constexpr int kSmemLimit = 232448;         // 227 KB of dynamic shared memory per CTA
 constexpr uint32_t kTmemCols = 512;
 
-
 constexpr int kD = 256;
 constexpr int kG = kD / kGroup;            // 8 scales per row
-constexpr int kHalfN = 128;                // channels per CTA = MMA N
+constexpr int kHalfN = 128;                // channels whose B rows a CTA holds
 constexpr int kKBlocks = kD / 64;          // 4 K blocks per tile
-constexpr int kBTermBytes = kKBlocks * kHalfN * 128;   // one split term of B: 128 rows x K = 256, 64 KB
-constexpr int kMaxRing = 6;
+constexpr int kBBlock = kHalfN * 128;      // one K block of one term of B: 128 rows x 128 B
+constexpr int kBTerm = kKBlocks * kBBlock; // one split term of B: 128 rows x K = 256, 64 KB
+constexpr int kMaxRing = 12;
+constexpr int kMaxAcc = 4;
+constexpr int64_t kShortTiles = 74;        // tiles of 128 vectors up to which a tile has 64 vectors per CTA: one per pair of SMs
 
 // CALIB: the calibration pass keeps a third bf16 term (it runs once; its result is compared at 1e-6 of the vector norm)
-// PERVEC: one scale per vector.  A row's 256 channels sit in two CTAs, so the pair runs as a thread-block cluster and
-// the four half-row maxima of a row (two warps in each CTA) meet in both CTAs' shared memory.
-template <bool BF16, bool CALIB = false, bool PERVEC = false>
+// PERVEC: one scale per vector: the four threads of a row trade their maxima through shared memory
+// ROWS: vectors per CTA and tile; a pair's tile has twice as many = MMA M.  128, or 64 where a call has no more than one tile of
+// 128 vectors per pair: its MMAs cost 1.3 us per tile instead of 2.1 and twice as many SMs take part (9000 vectors: 11.1 -> 9.5 us;
+// on long calls they are the dearer ones, 62 -> 71 us at 212,992 vectors).
+template <bool BF16, bool CALIB = false, bool PERVEC = false, int ROWS = 128>
 struct Cfg {
+    static_assert(ROWS == 64 || ROWS == 128, "tile heights");
+    static constexpr int kBlockBytes = ROWS * 128;   // one K block of a CTA's x: ROWS x 128 B
+    // tensor memory of an accumulator.  128 vectors: a lane per vector, 256 columns.  64: lanes 0-63 hold the vectors' channels
+    // 0-127, lanes 64-127 the rest, 128 columns.
+    static constexpr uint32_t kAccCols = 2 * ROWS;
+    static constexpr int kAccStages = 512 / (int)kAccCols;
+    static constexpr int kThreadGroups = ROWS / 64;  // groups of 32 channels per epilogue thread
     static constexpr int kSplit = (BF16 && CALIB) ? 3 : 2;
-    static constexpr int kBBytes = kSplit * kBTermBytes;
-    // Two terms: STACKED along N, rows [0, 128) of a K block the first term's, rows [128, 256) the second's, so that one
-    // MMA of N = 256 computes x W_hi into accumulator columns [0, 128) and x W_lo into [128, 256); the epilogue adds the
-    // two.  An MMA of M 128, N 128, K 16 costs about 120 cycles here, one of N = 256 about 176 (measured, operands in
-    // shared memory): the per-instruction overhead is paid once for both terms and x is read once instead of twice.
-    static constexpr bool kStack = kSplit == 2;
-    static constexpr int kNmma = kStack ? 2 * kHalfN : kHalfN;
-    static constexpr int kBBlock = kNmma * 128;                          // one K block of B: kNmma rows x 128 B
-    static constexpr int kBTerm = kStack ? kHalfN * 128 : kBTermBytes;   // from one term's row c to the next term's
-    static constexpr uint32_t kAccStride = kNmma;                        // tensor-memory columns per accumulator
-    static constexpr int kAccStages = 512 / kNmma;                       // 2 (stacked) or 4
-    static constexpr int kMaxBytes = PERVEC ? 2 * 2 * 4 * kTile * (int)sizeof(float) : 0;   // [tile parity][set][party][row]
+    static constexpr int kBBytes = kSplit * kBTerm;
+    static constexpr int kParties = kG / kThreadGroups;   // threads that share a row
+    static constexpr int kMaxBytes = PERVEC ? 2 * kParties * ROWS * (int)sizeof(float) : 0;   // one scale per vector: [tile parity][party][row]
     static constexpr int kRoom = (kSmemLimit - 1024 - kCtrlBytes - kMaxBytes - kBBytes) / kBlockBytes;
-    static constexpr int kRing = kRoom < kMaxRing ? kRoom : kMaxRing;   // K blocks of x in flight: 6 (2 next to a three-term B)
+    static constexpr int kWant = 6 * 128 / ROWS;
+    static constexpr int kRing = kRoom < kWant ? kRoom : kWant;   // K blocks of x in flight: 6 (12 short ones), one less with kMaxBytes, 2 beside three terms
     static_assert(kRing >= 2, "no room for the x ring");
+    static constexpr bool kSmallFirst = kRing > kKBlocks;   // a whole tile stays in the ring for two passes over it
     static constexpr int kSmemBytes = kBBytes + kRing * kBlockBytes + kCtrlBytes + kMaxBytes + 1024;
-    static constexpr uint32_t kIdesc = umma_idesc_m128(kNmma, BF16);
+    static constexpr uint32_t kIdesc = umma_idesc(2 * ROWS, kD, BF16);
 };
 
+// Barriers that count arrivals of both CTAs (in_full, acc_empty, b_first, b_ready) are used in the leader's copy only.
 struct Ctrl {
     uint64_t in_full[kMaxRing], in_empty[kMaxRing];
-    uint64_t acc_full[4], acc_empty[4];
+    uint64_t acc_full[kMaxAcc], acc_empty[kMaxAcc];
     uint64_t b_first, b_ready;
-    uint64_t quad[2][4];        // one scale per vector: the four warps (two per CTA of the pair) that share 32 rows of a set
+    uint64_t swap[4];           // one scale per vector: the warps that share 32 rows
     uint32_t tmem_base;
     volatile uint32_t abort;
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
-
-// ---- thread-block cluster of two CTAs: the partner's shared memory and barriers (one scale per vector only)
-__device__ __forceinline__ uint32_t cluster_map(uint32_t smem_addr, uint32_t cta_rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(cta_rank));
-    return r;
-}
-__device__ __forceinline__ void cluster_st_f32(uint32_t cluster_addr, float v)
-{
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void cluster_mbar_arrive(uint32_t cluster_addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// wait_or_abort with cluster-scope acquire: the values the partner CTA stored before its arrive are visible afterwards
-__device__ __forceinline__ bool wait_cluster_or_abort(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
-                                                      uint32_t reason)
-{
-    for (uint32_t it = 0; it < (1u << 22); ++it) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if (it > 32) {
-            if (*abort_flag) return false;
-            __nanosleep(32);
-        }
-    }
-    *abort_flag = 1u;
-    atomicOr(status, reason);
-    return false;
-}
 
 // 2^k for a lambda row: the power of two that brings max_c lambda_c max|table entry| (sqrt(2 / D) without a rotation) into [2^13, 2^14), so that
 // the first split term of W 2^k stays below fp16's maximum and the later ones above its subnormals.
@@ -145,41 +108,53 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
     return __uint_as_float((uint32_t)(127 + 13 - e) << 23);
 }
 
-// Rows [c0, c1) of every split term of this CTA's half of the B operand (channel 128 half + c), by one warp: a lane
-// reads four table entries per pass (coalesced rows), scales them by lambda_c 2^k, peels off 16-bit terms and
-// writes 8 bytes of each term's swizzled row.
+// Eight rows from c0 on of every split term of this CTA's half of the B operand (channel 128 half + c), by one warp: a lane
+// requests four table entries per pass and row, all at once (load), scales them by lambda_c 2^k, peels off 16-bit terms and
+// writes 8 bytes of each term's swizzled row (store).
+constexpr int kBuildRows = 8;
 template <bool BF16, bool CALIB>
-__device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__restrict__ e0, const float *__restrict__ lam, float lift,
-                                             int half, int c0, int c1, int lane)
-{
-    using C = Cfg<BF16, CALIB>;
-#pragma unroll 2   // (eight rows in flight were tried: slower, 60.3 against 55.9 us at 212,992 vectors and 52 lambda rows)
-    for (int c = c0; c < c1; ++c) {
-        const int cg = half * kHalfN + c;
-        const float f = lam ? __ldg(lam + cg) * lift : lift;
+struct BuildRows {
+    float4 m[kBuildRows][2];
+    __device__ __forceinline__ void load(const float *__restrict__ e0, int half, int c0, int lane)
+    {
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const int i = lane + 32 * p;
-            const float4 m = __ldg(reinterpret_cast<const float4 *>(e0 + (size_t)cg * kD) + i);
-            float w[4] = {m.x * f, m.y * f, m.z * f, m.w * f};
-            const int ch = i >> 1;   // 16-byte chunk of the K-major row: K block ch / 8, chunk ch % 8
-            const uint32_t off = (uint32_t)((ch >> 3) * C::kBBlock + c * 128 + (((ch & 7) ^ (c & 7)) << 4) + ((i & 1) ? 8 : 0));
+        for (int k = 0; k < kBuildRows; ++k)
 #pragma unroll
-            for (int t = 0; t < C::kSplit; ++t) {
-                const uint32_t lo = narrow2<BF16>(w[0], w[1]), hi = narrow2<BF16>(w[2], w[3]);
-                *reinterpret_cast<uint2 *>(sB + t * C::kBTerm + off) = make_uint2(lo, hi);
-                if (t + 1 < C::kSplit) {   // what the 16-bit term left behind (exact in fp32)
-                    const float2 a = widen2<BF16>(lo), b = widen2<BF16>(hi);
-                    w[0] -= a.x, w[1] -= a.y, w[2] -= b.x, w[3] -= b.y;
+            for (int p = 0; p < 2; ++p) m[k][p] = __ldg(reinterpret_cast<const float4 *>(e0 + (size_t)(half * kHalfN + c0 + k) * kD) + lane + 32 * p);
+    }
+    __device__ __forceinline__ void store(unsigned char *sB, const float *__restrict__ lam, float lift, int half, int c0, int lane) const
+    {
+        using C = Cfg<BF16, CALIB>;
+        float f[kBuildRows];
+#pragma unroll
+        for (int k = 0; k < kBuildRows; ++k) f[k] = lam ? __ldg(lam + half * kHalfN + c0 + k) * lift : lift;
+#pragma unroll
+        for (int k = 0; k < kBuildRows; ++k) {
+            const int c = c0 + k;
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const int i = lane + 32 * p;
+                float w[4] = {m[k][p].x * f[k], m[k][p].y * f[k], m[k][p].z * f[k], m[k][p].w * f[k]};
+                const int ch = i >> 1;   // 16-byte chunk of the K-major row: K block ch / 8, chunk ch % 8
+                const uint32_t off = (uint32_t)((ch >> 3) * kBBlock + c * 128 + (((ch & 7) ^ (c & 7)) << 4) + ((i & 1) ? 8 : 0));
+#pragma unroll
+                for (int t = 0; t < C::kSplit; ++t) {
+                    const uint32_t lo = narrow2<BF16>(w[0], w[1]), hi = narrow2<BF16>(w[2], w[3]);
+                    *reinterpret_cast<uint2 *>(sB + t * kBTerm + off) = make_uint2(lo, hi);
+                    if (t + 1 < C::kSplit) {   // what the 16-bit term left behind (exact in fp32)
+                        const float2 a = widen2<BF16>(lo), b = widen2<BF16>(hi);
+                        w[0] -= a.x, w[1] -= a.y, w[2] -= b.x, w[3] -= b.y;
+                    }
                 }
             }
         }
     }
-}
+};
 
 }  // namespace
 
 struct UmmaEncode256Params {
+    const unsigned char *x;   // [N, D] 16-bit: for prefetches, the loads go through the tensor map
     const float *lambda;   // [n_lambda, D] fp32
     const float *e0;       // plan table [D, D] fp32: e0[c][n] = M[c][n] s_n
     unsigned char *packed; // [*, D/2] bytes out
@@ -195,20 +170,21 @@ struct UmmaEncode256Params {
     int bits;                   // 4: nibble pairs; 8 (fp16 input): one two's-complement byte per code, scale = absmax / 127
 };
 
-template <bool BF16, bool CALIB, bool PERVEC>
-__device__ __forceinline__ void encode_d256_body(const UmmaEncode256Params &prm, const CUtensorMap &tm_x)
+template <bool BF16, bool CALIB, bool PERVEC, int ROWS>
+__global__ void __launch_bounds__(kThreads, 1)
+    kvq_encode_umma_d256_kernel(const __grid_constant__ UmmaEncode256Params prm, const __grid_constant__ CUtensorMap tm_x)
 {
-    using C = Cfg<BF16, CALIB, PERVEC>;
-    constexpr int kRing = C::kRing;
+    using C = Cfg<BF16, CALIB, PERVEC, ROWS>;
+    constexpr int kRing = C::kRing, kAccStages = C::kAccStages, kBlockBytes = C::kBlockBytes;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    unsigned char *sB = smem;                                   // kSplit terms
+    unsigned char *sB = smem;                                   // [term][K block][128 rows][128 B]
     unsigned char *sIn = sB + C::kBBytes;                       // ring of K blocks of x
     Ctrl *ctrl = reinterpret_cast<Ctrl *>(sIn + kRing * kBlockBytes);
-    float *rowmax = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(ctrl) + kCtrlBytes);   // PERVEC: [parity][set][party][row]
+    float *rowmax = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(ctrl) + kCtrlBytes);   // PERVEC: [parity][party][row]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int half = blockIdx.x & 1;            // which 128 channels this CTA computes
+    const int rank = (int)cluster_rank();       // which ROWS vectors of a tile, and which 128 rows of B, this CTA holds
     const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
     if (threadIdx.x == 0) {
@@ -216,62 +192,77 @@ __device__ __forceinline__ void encode_d256_body(const UmmaEncode256Params &prm,
             mbar_init(smem_u32(&ctrl->in_full[s]), 1);
             mbar_init(smem_u32(&ctrl->in_empty[s]), 1);
         }
-        for (int s = 0; s < C::kAccStages; ++s) {
+        for (int s = 0; s < kAccStages; ++s) {
             mbar_init(smem_u32(&ctrl->acc_full[s]), 1);
-            mbar_init(smem_u32(&ctrl->acc_empty[s]), kEpiWarps / 2);
+            mbar_init(smem_u32(&ctrl->acc_empty[s]), 2 * kEpiWarps);
         }
-        mbar_init(smem_u32(&ctrl->b_first), kEpiWarps);       // first B: all epilogue warps build it
-        mbar_init(smem_u32(&ctrl->b_ready), kEpiWarps / 2);   // later rebuilds: the set that owns the tile
-        for (int s = 0; s < 2; ++s)
-            for (int qq = 0; qq < 4; ++qq) mbar_init(smem_u32(&ctrl->quad[s][qq]), 4);
+        mbar_init(smem_u32(&ctrl->b_first), 2 * kEpiWarps);   // first B: all epilogue warps of both CTAs build it
+        mbar_init(smem_u32(&ctrl->b_ready), 2 * kEpiWarps);   // later rebuilds
+        for (int qq = 0; qq < 4; ++qq) mbar_init(smem_u32(&ctrl->swap[qq]), C::kParties);
         ctrl->abort = 0u;
         mbar_init_fence();
     }
-    if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
-    grid_wait();
-    fence_proxy_async();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if constexpr (PERVEC) cluster_sync_all();   // the partner's barriers exist before anyone arrives on them
+    if (warp == 0) tmem_alloc_pair(smem_u32(&ctrl->tmem_base), kTmemCols);
+
+    // ---- tiles: lambda segments of rpl rows, cut into tiles of 2 ROWS rows; a contiguous range per CTA pair
+    const int64_t N = prm.N, rpl = prm.rpl;
+    const TileShare share(prm.n_seg, rpl, (unsigned)pair, (unsigned)n_pairs, 2 * ROWS);
+    const int64_t tps = share.tps, tile_begin = share.begin;
+    const int n_my = share.n;
+
+    // ---- B for the pair's first lambda row: eight rows per epilogue warp, requested before the set-up barrier
+    float first_lift = 1.0f;
+    if (n_my > 0 && warp >= 2) {
+        const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : tile_begin / tps) * kD;
+        BuildRows<BF16, CALIB> rows;
+        rows.load(prm.e0, rank, (warp - 2) * 8, lane);
+        grid_wait();
+        first_lift = lift_of<kD>(lam, prm.table_max, lane);
+        tc_fence_before();
+        cluster_sync_all();   // both CTAs' barriers exist and both have their tensor memory
+        tc_fence_after();
+        rows.store(sB, lam, first_lift, rank, (warp - 2) * 8, lane);
+        fence_proxy_async();   // B is read by the tensor core through the async proxy
+        __syncwarp();
+        if (lane == 0) cluster_mbar_arrive(cluster_map(smem_u32(&ctrl->b_first), 0));
+    } else {
+        grid_wait();
+        tc_fence_before();
+        cluster_sync_all();
+        tc_fence_after();
+    }
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile uint32_t *abort_flag = &ctrl->abort;
     uint32_t *status = prm.status;
 
-    // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range per CTA pair
-    const int64_t N = prm.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, (unsigned)pair, (unsigned)n_pairs);
-    const int64_t tps = share.tps, tile_begin = share.begin;
-    const int n_my = share.n;
-
     if (warp == 0) {
         // =========================== producer ===========================
         if (lane == 0) {
-            int issued = 0;
             bool ok = true;
-            TileCursor cur(tile_begin, tps);
-            for (int j = 0; j < n_my && ok; ++j, cur.advance(1)) {
-                const int64_t row0 = cur.seg * rpl + cur.row_in_segment();
+            TileCursor cur(tile_begin, tps), ahead(tile_begin, tps);
+            ahead.advance(1);
+            for (int j = 0; j < n_my && ok; ++j, cur.advance(1), ahead.advance(1)) {
+                const int64_t row0 = cur.seg * rpl + cur.tin * (2 * ROWS) + rank * ROWS;   // may lie past the end: zeros
+                // The next tile's rows are one contiguous run: asked for as such, they come out of DRAM page by page, and the K block
+                // loads, 128 bytes of each row at a time, find them in L2 (1,064,960 bf16 vectors: 278 -> 269 us; two tiles ahead: 273).
+                if (j + 1 < n_my) {
+                    const int64_t next = ahead.seg * rpl + ahead.tin * (2 * ROWS) + rank * ROWS;
+                    const int64_t n = N - next < ROWS ? N - next : ROWS;
+                    if (n > 0) prefetch_l2(prm.x + next * (2 * kD), (uint32_t)n * (2 * kD));
+                }
 #pragma unroll
                 for (int kb = 0; kb < kKBlocks; ++kb) {
                     const int u = kKBlocks * j + kb, s = u % kRing;
                     ok = wait_or_abort(smem_u32(&ctrl->in_empty[s]), ((uint32_t)(u / kRing) & 1u) ^ 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT);
                     if (!ok) break;
-                    const uint32_t bar = smem_u32(&ctrl->in_full[s]);
-                    mbar_arrive_expect_tx(bar, kBlockBytes);
-                    tma_load_2d(smem_u32(sIn + s * kBlockBytes), &tm_x, 64 * kb, (int)row0, bar);
-                    issued = u + 1;
+                    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctrl->in_full[s]), 2 * kBlockBytes);   // this CTA's block and the partner's
+                    tma_load_2d_pair(smem_u32(sIn + s * kBlockBytes), &tm_x, 64 * kb, (int)row0, cluster_map(smem_u32(&ctrl->in_full[s]), 0));
                 }
-            }
-            if (!ok) {
-                // give this thread's own copies in flight a bounded chance to land before the CTA goes away
-                for (int u = issued > kRing ? issued - kRing : 0; u < issued; ++u)
-                    (void)mbar_wait_bounded(smem_u32(&ctrl->in_full[u % kRing]), (uint32_t)(u / kRing) & 1u, 1u << 16);
             }
         }
     } else if (warp == 1) {
-        // =========================== mma issuer ===========================
-        if (lane == 0) {
+        // =========================== mma issuer (leader) ===========================
+        if (rank == 0 && lane == 0) {
             // Descriptors differ only in their 14-bit start-address field (bytes >> 4): one base per operand, one add per MMA.
             const uint64_t b_desc = smem_desc_sw128(smem_u32(sB));
             const uint64_t a_desc = smem_desc_sw128(smem_u32(sIn));
@@ -281,108 +272,89 @@ __device__ __forceinline__ void encode_d256_body(const UmmaEncode256Params &prm,
             bool ok = true;
             TileCursor cur(tile_begin, tps);
             for (int j = 0; j < n_my && ok; ++j, cur.advance(1)) {
-                const int sc = j % C::kAccStages;
-                if (j == 0) {   // all epilogue warps build the first B while the first x blocks are in flight
-                    if (!wait_or_abort(smem_u32(&ctrl->b_first), 0u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
-                } else if (cur.first_of_segment()) {   // an epilogue set rebuilds B for this lambda row
-                    if (!wait_or_abort(smem_u32(&ctrl->b_ready), builds & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
+                const int sc = j % kAccStages;
+                if (j == 0) {   // the epilogue warps build the first B while the first x blocks are in flight
+                    if (!wait_cluster_or_abort(smem_u32(&ctrl->b_first), 0u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
+                } else if (!CALIB && prm.n_lambda > 1 && cur.first_of_segment()) {   // the epilogue warps rebuild B for this lambda row
+                    if (!wait_cluster_or_abort(smem_u32(&ctrl->b_ready), builds & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
                     ++builds;
                 }
-                if (!wait_or_abort(smem_u32(&ctrl->acc_empty[sc]), ((uint32_t)(j / C::kAccStages) & 1u) ^ 1u, abort_flag, status,
-                                   KVQ_DEV_SLOT_TIMEOUT))
+                if (!wait_cluster_or_abort(smem_u32(&ctrl->acc_empty[sc]), ((uint32_t)(j / kAccStages) & 1u) ^ 1u, abort_flag, status,
+                                           KVQ_DEV_SLOT_TIMEOUT))
                     break;
-                const uint32_t d_tmem = tmem_base + (uint32_t)sc * C::kAccStride;
+                const uint32_t d_tmem = tmem_base + (uint32_t)sc * C::kAccCols;
+                constexpr int kPasses = C::kSmallFirst ? C::kSplit : 1;   // passes over the tile's blocks
 #pragma unroll
-                for (int kb = 0; kb < kKBlocks; ++kb) {
-                    const int u = kKBlocks * j + kb, s = u % kRing;
-                    if (!wait_or_abort(smem_u32(&ctrl->in_full[s]), (uint32_t)(u / kRing) & 1u, abort_flag, status, KVQ_DEV_LOAD_TIMEOUT)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t a_lo_s = a_lo + (uint32_t)s * (kBlockBytes >> 4);
+                for (int ps = 0; ps < kPasses && ok; ++ps) {
 #pragma unroll
-                    for (int t = 0; t < (C::kStack ? 1 : C::kSplit); ++t) {   // stacked terms: one MMA per K-step computes both
-#pragma unroll
-                        for (int ks = 0; ks < 4; ++ks) {   // the four K steps of this block
-                            const uint64_t ad = ((uint64_t)a_hi << 32) | (uint64_t)(a_lo_s + (uint32_t)ks * 2u);
-                            const uint64_t bd = ((uint64_t)b_hi << 32) |
-                                                (uint64_t)(b_lo + (uint32_t)t * (C::kBTerm >> 4) + (uint32_t)kb * (C::kBBlock >> 4) + (uint32_t)ks * 2u);
-                            if (kb > 0 || t > 0 || ks > 0) umma_f16_ss<true>(d_tmem, ad, bd, C::kIdesc);
-                            else umma_f16_ss<false>(d_tmem, ad, bd, C::kIdesc);
+                    for (int kb = 0; kb < kKBlocks; ++kb) {
+                        const int u = kKBlocks * j + kb, s = u % kRing;
+                        if (ps == 0 && !wait_cluster_or_abort(smem_u32(&ctrl->in_full[s]), (uint32_t)(u / kRing) & 1u, abort_flag, status,
+                                                              KVQ_DEV_LOAD_TIMEOUT)) {
+                            ok = false;
+                            break;
                         }
+                        tc_fence_after();
+                        const uint32_t a_lo_s = a_lo + (uint32_t)s * (kBlockBytes >> 4);
+#pragma unroll
+                        for (int tt = 0; tt < (C::kSmallFirst ? 1 : C::kSplit); ++tt) {
+                            const int t = C::kSmallFirst ? C::kSplit - 1 - ps : tt;
+#pragma unroll
+                            for (int ks = 0; ks < 4; ++ks) {   // the four K steps of this block
+                                const uint64_t ad = ((uint64_t)a_hi << 32) | (uint64_t)(a_lo_s + (uint32_t)ks * 2u);
+                                const uint64_t bd = ((uint64_t)b_hi << 32) |
+                                                    (uint64_t)(b_lo + (uint32_t)t * (kBTerm >> 4) + (uint32_t)kb * (kBBlock >> 4) + (uint32_t)ks * 2u);
+                                if (ps > 0 || kb > 0 || tt > 0 || ks > 0) umma_f16_ss_pair<true>(d_tmem, ad, bd, C::kIdesc);
+                                else umma_f16_ss_pair<false>(d_tmem, ad, bd, C::kIdesc);
+                            }
+                        }
+                        if (ps == kPasses - 1) umma_commit_pair(smem_u32(&ctrl->in_empty[s]));   // the tensor core has read this block of x
                     }
-                    umma_commit(smem_u32(&ctrl->in_empty[s]));   // the tensor core has read this block of x
                 }
-                if (ok) umma_commit(smem_u32(&ctrl->acc_full[sc]));
+                if (ok) umma_commit_pair(smem_u32(&ctrl->acc_full[sc]));
             }
         }
     } else {
         // =========================== epilogue: accumulator -> scales, codes, nibbles ===========================
-        // Two sets of eight warps take alternate tiles, so that one set's waits (barrier, tensor-memory load)
-        // hide behind the other set's arithmetic.  Thread = (row, half row).
-        const int set = (warp - 2) >> 3;        // this set takes tiles set, set + 2, ...
+        // All sixteen warps on every tile, thread = (row, ROWS / 64 of the row's eight groups): the accumulator goes back after
+        // half the time that two sets on alternate tiles would hold it, and the tensor core has the other stages meanwhile.
+        constexpr int kTG = C::kThreadGroups;
         const int q = warp & 3;                 // tensor-memory lane quarter this warp may touch
-        const int h = ((warp - 2) >> 2) & 1;    // half of the row
-        const int r = q * 32 + lane;            // tile row of this thread
-        const int bw = (warp - 2) & 7;          // position within the set: 16 rows of B per warp when the set rebuilds B
-        const int g0 = 2 * h;                   // this thread's groups within the CTA's four: g0, g0 + 1
-        const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        // Group g (of this CTA's four) of this thread's row of accumulator stage sc; with stacked terms the sum of the two
-        // terms' columns.
-        auto load_group = [&](int sc, int g, uint32_t (&vb)[32]) {
-            tmem_ld32(t_addr + (uint32_t)sc * C::kAccStride + (uint32_t)(g * kGroup), vb);
-            if constexpr (C::kStack) {
-                uint32_t lo[32];
-                tmem_ld32(t_addr + (uint32_t)sc * C::kAccStride + (uint32_t)(kHalfN + g * kGroup), lo);
-                tmem_ld_wait();
-#pragma unroll
-                for (int i = 0; i < 32; ++i) vb[i] = __float_as_uint(__uint_as_float(vb[i]) + __uint_as_float(lo[i]));
-            } else {
-                tmem_ld_wait();
-            }
+        const int q_rows = q % (ROWS / 32);     // the 32 rows those lanes hold
+        const int r = q_rows * 32 + lane;       // row of this CTA's
+        const int col0 = ((warp - 2) >> 2) * (kTG * kGroup);                              // first accumulator column of this thread
+        const int g0 = (q / (ROWS / 32)) * (kG / 2) + ((warp - 2) >> 2) * kTG;            // and the group it belongs to
+        const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)col0;
+        auto load_group = [&](int sc, int gi, uint32_t (&vb)[32]) {   // this thread's group g0 + gi out of accumulator stage sc
+            tmem_ld32(t_addr + (uint32_t)sc * C::kAccCols + (uint32_t)(gi * kGroup), vb);
+            tmem_ld_wait();
         };
-        int64_t cached_seg = -1;
-        float unlift = 1.0f;
-        if (n_my > 0) {   // B for the CTA's first lambda row: D / 16 rows per warp, all sixteen warps
-            TileCursor first(tile_begin, tps);
-            const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : first.seg) * kD;
-            const float lift = lift_of<kD>(lam, prm.table_max, lane);
-            build_b_rows<BF16, CALIB>(sB, prm.e0, lam, lift, half, (warp - 2) * 8, (warp - 1) * 8, lane);
-            fence_proxy_async();   // B is read by the tensor core through the async proxy
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
-            unlift = 1.0f / lift;
-            cached_seg = first.seg;
-        }
-        float colmax[2] = {};   // calibration: lane i keeps the running maximum of column i of each of this thread's groups
-        TileCursor cur(tile_begin + set, tps);
-        for (int j = set; j < n_my; j += 2, cur.advance(2)) {
+        float lift_next = first_lift;
+        float colmax[kTG] = {};   // calibration: lane i keeps the running maximum of column i of each of this thread's groups
+        TileCursor cur(tile_begin, tps);
+        for (int j = 0; j < n_my; ++j, cur.advance(1)) {
             __syncwarp();
             const int64_t seg = cur.seg;
-            const int64_t off = cur.row_in_segment();
+            const int64_t off = cur.tin * (2 * ROWS) + rank * ROWS;
+            const float unlift = 1.0f / lift_next;
 
-            // ---- a new lambda row.  Every set needs its lift; the set that owns the row's first tile rebuilds B,
-            // ---- once every MMA that read the old B is complete (the previous tile's accumulator is full), and
-            // ---- tells the mma warp.
-            if (seg != cached_seg) {
-                const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : seg) * kD;
-                const float lift = lift_of<kD>(lam, prm.table_max, lane);
-                if (j > 0 && cur.first_of_segment()) {
-                    if (!wait_or_abort(smem_u32(&ctrl->acc_full[(j - 1) % C::kAccStages]), (uint32_t)((j - 1) / C::kAccStages) & 1u,
-                                       abort_flag, status, KVQ_DEV_MMA_TIMEOUT))
-                        break;
-                    build_b_rows<BF16, CALIB>(sB, prm.e0, lam, lift, half, bw * 16, (bw + 1) * 16, lane);
-                    fence_proxy_async();   // B is read by the tensor core through the async proxy
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_ready));
-                }
-                unlift = 1.0f / lift;
-                cached_seg = seg;
+            // ---- this tile's accumulator.  Where the next tile begins a new lambda row, every MMA that read the old B is complete
+            // ---- with it: B is rebuilt first, before this tile's own work, from table rows requested before the wait.
+            const int sc = j % kAccStages;
+            const bool rebuild = !CALIB && j + 1 < n_my && cur.tin + 1 == tps && prm.n_lambda > 1;
+            if (rebuild) {
+                const float *lam = prm.lambda + (seg + 1) * kD;
+                BuildRows<BF16, CALIB> rows;
+                rows.load(prm.e0, rank, (warp - 2) * 8, lane);
+                lift_next = lift_of<kD>(lam, prm.table_max, lane);
+                if (!wait_or_abort(smem_u32(&ctrl->acc_full[sc]), (uint32_t)(j / kAccStages) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
+                rows.store(sB, lam, lift_next, rank, (warp - 2) * 8, lane);
+                fence_proxy_async();   // B is read by the tensor core through the async proxy
+                __syncwarp();
+                if (lane == 0) cluster_mbar_arrive(cluster_map(smem_u32(&ctrl->b_ready), 0));
+            } else {
+                if (!wait_or_abort(smem_u32(&ctrl->acc_full[sc]), (uint32_t)(j / kAccStages) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
             }
-
-            const int sc = j % C::kAccStages;
-            if (!wait_or_abort(smem_u32(&ctrl->acc_full[sc]), (uint32_t)(j / C::kAccStages) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
             tc_fence_after();
 
             // ---- rows of the tile that exist: the segment (and with it the tensor) may end inside the tile
@@ -390,158 +362,85 @@ __device__ __forceinline__ void encode_d256_body(const UmmaEncode256Params &prm,
             if (seg_rows > rpl) seg_rows = rpl;
             const bool live = off + r < seg_rows;
             const int64_t orow = prm.out_map(seg * rpl + off + r);
-            const float Q = prm.bits == 4 ? 7.0f : 127.0f;   // largest code (warp-uniform)
-            // ---- one scale per vector: this thread's maximum over its 64 channels goes to both CTAs of the pair; the four
-            // ---- parties of a row (two half-row threads in each CTA) meet on a four-arrival barrier in each CTA, once per
-            // ---- tile; buffers alternate with the tile parity, so a party cannot overwrite what another still reads
-            float row_rs = 0.0f;
-            bool row_clamp = false;
+            const float Q = prm.bits == 4 ? 7.0f : 127.0f, inv_q = prm.bits == 4 ? 1.0f / 7.0f : 1.0f / 127.0f;   // largest code (warp-uniform)
+            // ---- one scale per vector: the row's maximum first (this thread's groups, then the others' through
+            // ---- shared memory), then a second pass over the accumulator for the codes; buffers alternate with the tile
+            // ---- parity, so a thread cannot overwrite what its partners still read
+            GroupScale row_scale;
             if constexpr (PERVEC) {
                 float m = 0.0f;
 #pragma unroll
-                for (int gi = 0; gi < 2; ++gi) {
+                for (int gi = 0; gi < kTG; ++gi) {
                     uint32_t vb[32];
-                    load_group(sc, g0 + gi, vb);
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) m = fmaxf(m, fabsf(__uint_as_float(vb[i])));
+                    load_group(sc, gi, vb);
+                    m = fmaxf(m, group_absmax(vb));
                 }
-                const int it = (j - set) >> 1;                       // this set's tile count
-                float *slot = rowmax + (((it & 1) * 2 + set) * 4) * kTile;   // [party][row] of this buffer
-                const int party = 2 * half + h;
-                slot[party * kTile + r] = m;
-                cluster_st_f32(cluster_map(smem_u32(slot + party * kTile + r), (uint32_t)(half ^ 1)), m);
-                asm volatile("fence.acq_rel.cluster;" ::: "memory");   // every lane's stores before lane 0's arrives
+                float *slot = rowmax + (j & 1) * C::kParties * ROWS;   // [party][row] of this buffer
+                slot[(g0 / kTG) * ROWS + r] = m;
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(smem_u32(&ctrl->quad[set][q]));
-                    cluster_mbar_arrive(cluster_map(smem_u32(&ctrl->quad[set][q]), (uint32_t)(half ^ 1)));
-                }
-                if (!wait_cluster_or_abort(smem_u32(&ctrl->quad[set][q]), (uint32_t)it & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
-                m = fmaxf(fmaxf(slot[r], slot[kTile + r]), fmaxf(slot[2 * kTile + r], slot[3 * kTile + r]));
-                const float amax = m * unlift;
-                const float sig = fminf(__fdiv_rn(amax, Q), 65504.0f);
-                const __half hs = __float2half_rn(sig);
-                const float sg = __half2float(hs);
-                const float rs1 = sg > 0.0f ? __frcp_rn(sg) : 0.0f;
-                row_clamp = !(amax * rs1 < Q + 0.25f);
-                row_rs = rs1 * unlift;
-                if (live && party == 0) prm.scales[orow] = __half_as_ushort(hs);
+                if (lane == 0) mbar_arrive(smem_u32(&ctrl->swap[q_rows]));
+                if (!wait_or_abort(smem_u32(&ctrl->swap[q_rows]), (uint32_t)j & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
+#pragma unroll
+                for (int i = 0; i < C::kParties; ++i) m = fmaxf(m, slot[i * ROWS + r]);
+                row_scale = group_scale(m, unlift, Q, inv_q);
+                if (live && g0 == 0) prm.scales[orow] = row_scale.half;
             }
+            uint32_t sc2 = 0u;   // the groups' fp16 scales
 #pragma unroll
-            for (int gi = 0; gi < 2; ++gi) {
-                const int g = g0 + gi;       // warp-uniform; group within this CTA's half
-                {
-                    uint32_t vb[32];
-                    load_group(sc, g, vb);
-                    if (gi == 1) {   // this thread's last group is in registers: hand the accumulator back
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty[sc]));
+            for (int gi = 0; gi < kTG; ++gi) {
+                const int g = g0 + gi;       // warp-uniform
+                uint32_t vb[32];
+                load_group(sc, gi, vb);
+                if (gi == kTG - 1) {   // this thread's last group is in registers: hand the accumulator back
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) cluster_mbar_arrive(cluster_map(smem_u32(&ctrl->acc_empty[sc]), 0));
+                }
+                if constexpr (CALIB) {
+                    // column maxima over the warp's 32 rows (rows past the end were filled with zeros by the TMA load)
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) {
+                        const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, vb[i] & 0x7FFFFFFFu);   // |v| orders like its bits
+                        if (lane == i) colmax[gi] = fmaxf(colmax[gi], __uint_as_float(m));
                     }
-                    if constexpr (CALIB) {
-                        // column maxima over the warp's 32 rows (rows past the end were filled with zeros by the TMA load)
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, vb[i] & 0x7FFFFFFFu);   // |v| orders like its bits
-                            if (lane == i) colmax[gi] = fmaxf(colmax[gi], __uint_as_float(m));
-                        }
-                        continue;
-                    }
-                    // ---- scale: sigma = fp16(absmax / 7); codes are taken against the stored value
-                    float rs = row_rs;
-                    bool clamp = row_clamp;
-                    __half hs = __float2half_rn(0.0f);
-                    if constexpr (!PERVEC) {
-                        float amax = 0.0f;
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(vb[i])));
-                        amax *= unlift;
-                        const float sig = fminf(__fdiv_rn(amax, Q), 65504.0f);
-                        hs = __float2half_rn(sig);
-                        const float sg = __half2float(hs);
-                        const float rs1 = sg > 0.0f ? __frcp_rn(sg) : 0.0f;
-                        clamp = !(amax * rs1 < Q + 0.25f);   // saturated or subnormal scale: codes could leave [-Q, Q]
-                        rs = rs1 * unlift;               // applies to the lifted accumulator values
-                    }
-
-                    const int gg = 4 * half + g;   // group within the row
-                    if (prm.bits == 8) {   // ---- round, bias to unsigned bytes, pack 4 codes per word
-                        uint32_t words[8];
-#pragma unroll
-                        for (int w = 0; w < 8; ++w) {
-                            uint32_t acc = 0;
-                            if (!clamp) {
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    acc += __float_as_uint(fmaf(__uint_as_float(vb[4 * w + e]), rs, kMagicRound8)) << (8 * e);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    acc += __float_as_uint(fminf(fmaxf(__uint_as_float(vb[4 * w + e]) * rs, -127.0f), 127.0f) + kMagicRound8) << (8 * e);
-                            }
-                            words[w] = (acc - kMagicSum8) ^ 0x80808080u;
-                        }
-                        if (live) {
-                            uint4 *dst = reinterpret_cast<uint4 *>(prm.packed + orow * kD + gg * 32);
-                            dst[0] = make_uint4(words[0], words[1], words[2], words[3]);
-                            dst[1] = make_uint4(words[4], words[5], words[6], words[7]);
-                            if constexpr (!PERVEC) prm.scales[orow * kG + gg] = __half_as_ushort(hs);
-                        }
-                        continue;
-                    }
-                    // ---- round, bias to unsigned nibbles, pack 8 codes per word
-                    uint32_t words[4];
-#pragma unroll
-                    for (int w = 0; w < 4; ++w) {
-                        uint32_t acc = 0;
-                        if (!clamp) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                acc += __float_as_uint(fmaf(__uint_as_float(vb[8 * w + e]), rs, kMagicRound)) << (4 * e);
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                acc += __float_as_uint(fminf(fmaxf(__uint_as_float(vb[8 * w + e]) * rs, -7.0f), 7.0f) + kMagicRound) << (4 * e);
-                        }
-                        words[w] = (acc - kMagicSum) ^ 0x88888888u;
-                    }
+                    continue;
+                }
+                const GroupScale gs = PERVEC ? row_scale : group_scale(group_absmax(vb), unlift, Q, inv_q);
+                sc2 |= (uint32_t)gs.half << (16 * gi);
+                if (prm.bits == 4) {
+                    const uint4 codes = pack_nibbles(vb, gs);
+                    if (live) *reinterpret_cast<uint4 *>(prm.packed + orow * (kD / 2) + g * 16) = codes;
+                } else {
+                    const uint4 first = pack_bytes(vb, gs), second = pack_bytes(vb + 16, gs);
                     if (live) {
-                        *reinterpret_cast<uint4 *>(prm.packed + orow * (kD / 2) + gg * 16) = make_uint4(words[0], words[1], words[2], words[3]);
-                        if constexpr (!PERVEC) prm.scales[orow * kG + gg] = __half_as_ushort(hs);
+                        uint4 *dst = reinterpret_cast<uint4 *>(prm.packed + orow * kD + g * 32);
+                        dst[0] = first, dst[1] = second;
                     }
                 }
             }
+            if constexpr (!CALIB && !PERVEC)
+                if (live) {
+                    if constexpr (kTG == 2) *reinterpret_cast<uint32_t *>(prm.scales + orow * kG + g0) = sc2;
+                    else prm.scales[orow * kG + g0] = (uint16_t)sc2;
+                }
         }
         if constexpr (CALIB) {   // this warp's maxima of its 32 rows of every tile -> the global column maxima
 #pragma unroll
-            for (int gi = 0; gi < 2; ++gi)
-                atomicMax(prm.amax_bits + (4 * half + g0 + gi) * kGroup + lane, __float_as_uint(colmax[gi] * unlift));
+            for (int gi = 0; gi < kTG; ++gi) atomicMax(prm.amax_bits + (g0 + gi) * kGroup + lane, __float_as_uint(colmax[gi] * (1.0f / first_lift)));
         }
     }
 
     grid_trigger();
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        if (*abort_flag) __nanosleep(20000);   // let tensor-core work that was already issued drain
-        tmem_dealloc(tmem_base, kTmemCols);
+    if (*abort_flag) {
+        // tell the partner, and let loads and tensor-core work that were already issued drain
+        if (lane == 0) cluster_st_u32(cluster_map(smem_u32(const_cast<uint32_t *>(&ctrl->abort)), (uint32_t)(rank ^ 1)), 1u);
+        __nanosleep(200000);
     }
-    if constexpr (PERVEC) cluster_sync_all();   // neither CTA leaves while the other may still store into its shared memory
-}
-
-template <bool BF16, bool CALIB>
-__global__ void __launch_bounds__(kThreads, 1)
-    kvq_encode_umma_d256_kernel(const __grid_constant__ UmmaEncode256Params prm, const __grid_constant__ CUtensorMap tm_x)
-{
-    encode_d256_body<BF16, CALIB, false>(prm, tm_x);
-}
-
-// one scale per vector: the same body with the CTA pair as a cluster (launched with a cluster dimension of 2)
-template <bool BF16>
-__global__ void __launch_bounds__(kThreads, 1)
-    kvq_encode_umma_d256_pv_kernel(const __grid_constant__ UmmaEncode256Params prm, const __grid_constant__ CUtensorMap tm_x)
-{
-    encode_d256_body<BF16, false, true>(prm, tm_x);
+    __syncwarp();
+    tc_fence_before();
+    cluster_sync_all();   // neither CTA leaves, or gives its tensor memory back, while the other may still use it
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc_pair(tmem_base, kTmemCols);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -549,31 +448,23 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ------------------------------------------------------------------------------------------------
 namespace {
 
-template <bool BF16, bool CALIB = false, bool PERVEC = false>
+template <bool BF16, bool CALIB, bool PERVEC, int ROWS>
 cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t stream, uint32_t *amax_bits = nullptr)
 {
-    using C = Cfg<BF16, CALIB, PERVEC>;
-    auto kern = [] {
-        if constexpr (PERVEC) return kvq_encode_umma_d256_pv_kernel<BF16>;
-        else return kvq_encode_umma_d256_kernel<BF16, CALIB>;
-    }();
+    using C = Cfg<BF16, CALIB, PERVEC, ROWS>;
+    auto kern = kvq_encode_umma_d256_kernel<BF16, CALIB, PERVEC, ROWS>;
     static DeviceSlots slots;
     int dev = 0;
     cudaError_t e = current_device_slot(&dev);
     if (e != cudaSuccess) return e;
-    int &sms = slots.sms[dev];
-    if (sms == 0) {
+    int &fit = slots.sms[dev];   // pairs resident at once (the SMs of a cluster share a GPC), looked up once per device
+    if (fit == 0) {
         int n = 0;
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        sms = n;
-    }
-    // one scale per vector: the pair is a cluster of two CTAs, as many pairs as the device holds at once (SMs of a
-    // cluster share a GPC); looked up once per device
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    if constexpr (PERVEC) {
-        cfg.gridDim = dim3((unsigned)sms, 1, 1);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        cfg.gridDim = dim3((unsigned)(n & ~1), 1, 1);
         cfg.blockDim = dim3(kThreads, 1, 1);
         cfg.dynamicSmemBytes = C::kSmemBytes;
         cfg.stream = stream;
@@ -583,18 +474,15 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        int &fit = slots.blocks_per_sm[dev];
-        if (fit == 0) {
-            int n = 0;
-            if ((e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg)) != cudaSuccess) return e;
-            if (n < 1) return cudaErrorLaunchOutOfResources;
-            fit = n;
-        }
+        if ((e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg)) != cudaSuccess) return e;
+        if (n < 1) return cudaErrorLaunchOutOfResources;
+        fit = n;
     }
     if (N == 0) return cudaSuccess;   // kvq_plan_prepare: the launch attributes are set, there is nothing to run
     if (N >= (int64_t)1 << 31) return cudaErrorInvalidValue;   // tensor-map coordinates are 32-bit
 
     UmmaEncode256Params prm;
+    prm.x = static_cast<const unsigned char *>(f.in);
     prm.lambda = f.lambda;
     prm.e0 = e0;
     prm.packed = static_cast<unsigned char *>(f.packed);
@@ -612,20 +500,28 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     CUtensorMap tm_x;
     const cuuint64_t dims[2] = {(cuuint64_t)kD, (cuuint64_t)N};
     const cuuint64_t strides[1] = {(cuuint64_t)(2 * kD)};
-    const cuuint32_t box[2] = {64, (cuuint32_t)kTile};
+    const cuuint32_t box[2] = {64, (cuuint32_t)ROWS};
     if (!make_tensor_map(&tm_x, BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, f.in, dims, strides, box,
                          CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
 
-    const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
-    int64_t pairs = tiles < sms / 2 ? tiles : sms / 2;
-    if constexpr (PERVEC) {
-        const int fit = slots.blocks_per_sm[dev];   // clusters resident at once
-        if (pairs > fit) pairs = fit;
+    const int64_t tiles = prm.n_seg * ((prm.rpl + 2 * ROWS - 1) / (2 * ROWS));
+    const unsigned pairs = (unsigned)(tiles < fit ? tiles : fit);
+    return launch_kernel(kern, 2 * pairs, kThreads, C::kSmemBytes, stream, 2, prm, tm_x);
+}
+
+// The tile height: 64 vectors per CTA where that gives no pair more than one tile.
+template <bool BF16, bool CALIB, bool PERVEC>
+cudaError_t launch_any(int64_t N, const FftParams &f, const float *e0, cudaStream_t stream, uint32_t *amax_bits = nullptr)
+{
+    if (N == 0) {   // kvq_plan_prepare: both heights
+        const cudaError_t e = launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits);
+        return e != cudaSuccess ? e : launch<BF16, CALIB, PERVEC, 128>(N, f, e0, stream, amax_bits);
     }
-    // the CTAs of a pair read the same tiles, the second one out of L2: they are to start together (212,992 bf16 vectors, 52 lambda
-    // rows: 65.5 us so, 67.2 us when they come up as the SMs of the kernel before fall free)
-    return launch_kernel<false>(kern, (unsigned)(2 * pairs), kThreads, C::kSmemBytes, stream, PERVEC ? 2 : 1, prm, tm_x);
+    const int64_t rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
+    const int64_t tiles = (N + rpl - 1) / rpl * ((rpl + 127) / 128);
+    return tiles <= kShortTiles ? launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits)
+                                : launch<BF16, CALIB, PERVEC, 128>(N, f, e0, stream, amax_bits);
 }
 
 }  // namespace
@@ -633,14 +529,14 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
 cudaError_t umma_encode_d256(bool bf16, bool per_vector, int64_t N, const FftParams &f, const float *e0, cudaStream_t stream)
 {
     if (!tensor_map_encode_fn()) return cudaErrorNotSupported;
-    if (per_vector) return bf16 ? launch<true, false, true>(N, f, e0, stream) : launch<false, false, true>(N, f, e0, stream);
-    return bf16 ? launch<true>(N, f, e0, stream) : launch<false>(N, f, e0, stream);
+    if (per_vector) return bf16 ? launch_any<true, false, true>(N, f, e0, stream) : launch_any<false, false, true>(N, f, e0, stream);
+    return bf16 ? launch_any<true, false, false>(N, f, e0, stream) : launch_any<false, false, false>(N, f, e0, stream);
 }
 
 cudaError_t umma_calibrate_d256(bool bf16, int64_t N, const FftParams &f, const float *e0, uint32_t *amax_bits, cudaStream_t stream)
 {
     if (!tensor_map_encode_fn()) return cudaErrorNotSupported;
-    return bf16 ? launch<true, true>(N, f, e0, stream, amax_bits) : launch<false, true>(N, f, e0, stream, amax_bits);
+    return bf16 ? launch_any<true, true, false>(N, f, e0, stream, amax_bits) : launch_any<false, true, false>(N, f, e0, stream, amax_bits);
 }
 
 }  // namespace kvq
