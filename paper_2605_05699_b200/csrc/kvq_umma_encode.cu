@@ -39,6 +39,7 @@
 // Every wait on an mbarrier is bounded: on a time-out the role records the reason in the status word,
 // raises the CTA's abort flag and leaves its loop; the CTA then frees its tensor memory and returns.
 #include "kvq_internal.h"
+#include "kvq_quantize.cuh"
 #include "kvq_umma.cuh"
 
 namespace kvq {
@@ -392,8 +393,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 uint32_t lo[32];
                 tmem_ld32(t_addr + (uint32_t)sc * C::kAccStride + (uint32_t)(D + g * kGroup), lo);
                 tmem_ld_wait();
-#pragma unroll
-                for (int i = 0; i < 32; ++i) vb[i] = __float_as_uint(__uint_as_float(vb[i]) + __uint_as_float(lo[i]));
+                add_group(vb, lo);
             } else {
                 tmem_ld_wait();
             }
@@ -433,11 +433,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (seg_rows > rpl) seg_rows = rpl;
             const bool live = off + r < seg_rows;
             const int64_t orow = prm.out_map(seg * rpl + off + r);
-            const float Q = prm.bits == 4 ? 7.0f : 127.0f;   // largest code (warp-uniform)
+            const float Q = prm.bits == 4 ? 7.0f : 127.0f, inv_q = prm.bits == 4 ? 1.0f / 7.0f : 1.0f / 127.0f;   // largest code (warp-uniform)
             // ---- one scale per vector: the row's maximum first (this thread's half, then the other half's through
             // ---- shared memory), then a second pass over the accumulator for the codes
-            float row_rs = 0.0f;
-            bool row_clamp = false;
+            GroupScale row_scale;
             if constexpr (PERVEC) {
                 float m = 0.0f;
 #pragma unroll
@@ -446,8 +445,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (g < g1) {
                         uint32_t vb[32];
                         load_group(sc, g, vb);
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) m = fmaxf(m, fabsf(__uint_as_float(vb[i])));
+                        m = fmaxf(m, group_absmax(vb));
                     }
                 }
                 const int it = (j - set) >> 1;   // this set's tile count: parity of the pair barrier and of the buffer
@@ -456,15 +454,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->pair[set][q]));
                 if (!wait_or_abort(smem_u32(&ctrl->pair[set][q]), (uint32_t)it & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
                 m = fmaxf(m, ctrl->rowmax[it & 1][set][h ^ 1][r]);
-                const float amax = m * unlift;
-                const float sig = fminf(__fdiv_rn(amax, Q), 65504.0f);
-                const __half hs = __float2half_rn(sig);
-                const float sg = __half2float(hs);
-                const float rs1 = sg > 0.0f ? __frcp_rn(sg) : 0.0f;
-                row_clamp = !(amax * rs1 < Q + 0.25f);
-                row_rs = rs1 * unlift;
-                if (live && h == 0) prm.scales[orow] = __half_as_ushort(hs);
+                row_scale = group_scale(m, unlift, Q, inv_q);
+                if (live && h == 0) prm.scales[orow] = row_scale.half;
             }
+            constexpr bool kPairScales = G == 4;   // two groups per thread, rows of 8 bytes: one 4-byte store
+            uint32_t scale_pair = 0u;
 #pragma unroll
             for (int gi = 0; gi < C::kGroupsPerPart; ++gi) {
                 const int g = g0 + gi;       // warp-uniform
@@ -485,65 +479,24 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                         continue;
                     }
-                    // ---- scale: sigma = fp16(absmax / 7); codes are taken against the stored value
-                    float rs = row_rs;
-                    bool clamp = row_clamp;
-                    __half hs = __float2half_rn(0.0f);
-                    if constexpr (!PERVEC) {
-                        float amax = 0.0f;
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(vb[i])));
-                        amax *= unlift;
-                        const float sig = fminf(__fdiv_rn(amax, Q), 65504.0f);
-                        hs = __float2half_rn(sig);
-                        const float sg = __half2float(hs);
-                        const float rs1 = sg > 0.0f ? __frcp_rn(sg) : 0.0f;
-                        clamp = !(amax * rs1 < Q + 0.25f);   // saturated or subnormal scale: codes could leave [-Q, Q]
-                        rs = rs1 * unlift;               // applies to the lifted accumulator values
-                    }
-
-                    // ---- round, bias to unsigned codes, pack: 8 nibbles or 4 bytes per word
+                    const GroupScale gs = PERVEC ? row_scale : group_scale(group_absmax(vb), unlift, Q, inv_q);
+                    if constexpr (!PERVEC && kPairScales) scale_pair |= (uint32_t)gs.half << (16 * gi);
                     if (prm.bits == 4) {
-                        uint32_t words[4];
-#pragma unroll
-                        for (int w = 0; w < 4; ++w) {
-                            uint32_t acc = 0;
-                            if (!clamp) {
-#pragma unroll
-                                for (int e = 0; e < 8; ++e)
-                                    acc += __float_as_uint(fmaf(__uint_as_float(vb[8 * w + e]), rs, kMagicRound)) << (4 * e);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 8; ++e)
-                                    acc += __float_as_uint(fminf(fmaxf(__uint_as_float(vb[8 * w + e]) * rs, -7.0f), 7.0f) + kMagicRound) << (4 * e);
-                            }
-                            words[w] = (acc - kMagicSum) ^ 0x88888888u;
-                        }
-                        if (live) *reinterpret_cast<uint4 *>(prm.packed + orow * (D / 2) + g * 16) = make_uint4(words[0], words[1], words[2], words[3]);
+                        const uint4 codes = pack_nibbles(vb, gs);
+                        if (live) *reinterpret_cast<uint4 *>(prm.packed + orow * (D / 2) + g * 16) = codes;
                     } else {
-                        uint32_t words[8];
-#pragma unroll
-                        for (int w = 0; w < 8; ++w) {
-                            uint32_t acc = 0;
-                            if (!clamp) {
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    acc += __float_as_uint(fmaf(__uint_as_float(vb[4 * w + e]), rs, kMagicRound8)) << (8 * e);
-                            } else {
-#pragma unroll
-                                for (int e = 0; e < 4; ++e)
-                                    acc += __float_as_uint(fminf(fmaxf(__uint_as_float(vb[4 * w + e]) * rs, -127.0f), 127.0f) + kMagicRound8) << (8 * e);
-                            }
-                            words[w] = (acc - kMagicSum8) ^ 0x80808080u;
-                        }
+                        const uint4 first = pack_bytes(vb, gs), second = pack_bytes(vb + 16, gs);
                         if (live) {
                             uint4 *dst = reinterpret_cast<uint4 *>(prm.packed + orow * D + g * 32);
-                            dst[0] = make_uint4(words[0], words[1], words[2], words[3]);
-                            dst[1] = make_uint4(words[4], words[5], words[6], words[7]);
+                            dst[0] = first, dst[1] = second;
                         }
                     }
-                    if (live) {
-                        if constexpr (!PERVEC) prm.scales[orow * G + g] = __half_as_ushort(hs);
+                    if constexpr (!PERVEC) {
+                        if (!kPairScales) {
+                            if (live) prm.scales[orow * G + g] = gs.half;
+                        } else if (gi == 1) {
+                            if (live) *reinterpret_cast<uint32_t *>(prm.scales + orow * G + g0) = scale_pair;
+                        }
                     }
                 }
             }
