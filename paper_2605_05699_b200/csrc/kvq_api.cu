@@ -345,6 +345,8 @@ kvq_status_t kvq_plan_prepare(kvq_plan_t *plan, kvq_dtype_t dtype)
     if (gemm_decode_ok(plan, bf16))
         also(plan->rot && plan->D == 256 ? umma_decode_d256_dense(bf16, 0, g, nullptr)
                                          : umma_decode(plan->D, bf16, plan->bits, 0, g, plan->sign_xor, nullptr, !plan->rot));
+    if (gemm_decode_ok(plan, bf16) && !plan->rot && plan->D != 256)   // the form that a rotation set later takes
+        also(umma_decode(plan->D, bf16, plan->bits, 0, g, plan->sign_xor, nullptr, false));
     if (umma_calibrate_supported(plan->D, bf16)) also(umma_calibrate(plan->D, bf16, 0, prm, plan->d_e0, nullptr, nullptr));
     also(matvec_encode(plan->D, plan->group, plan->bits, bf16, 0, prm, plan->d_b0, nullptr));
     also(matvec_decode(plan->D, plan->group, plan->bits, bf16, 0, prm, plan->d_e0, nullptr));

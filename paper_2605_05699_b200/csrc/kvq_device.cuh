@@ -222,25 +222,45 @@ struct TileCursor {
 
 // The contiguous share of a call's tiles that one CTA (or one CTA pair) of a persistent kernel takes: lambda segments of rpl
 // rows are cut into tiles of 128 rows (256 where a CTA pair works on one tile) (a segment's last tile may be short), n_seg * tps tiles in all, `parts` shares.
-// Contiguous, so that the B operand of a lambda row is rebuilt as rarely as possible.  A share that crosses into another
-// lambda row pays a rebuild of B, about one tile's time, so with several rows and at least eight tiles per share the shares
-// are equal in COST, each segment counting one unit more than its tiles (a share that would begin inside that unit begins
-// at the segment's first tile); otherwise they are equal in tiles.
+// Contiguous, so that the B operand of a lambda row is rebuilt as rarely as possible.  `segs` consecutive segments have one
+// lambda row (1, or the streams of a cache view that share theirs; the last row may have fewer).  A share that crosses into
+// another lambda row pays a rebuild of B on its critical path, about two tiles' time, so:
+//   * where no more lambda rows than shares exist and the longest share grows by no more than that, every share stays inside one
+//     lambda row (90,000 vectors under 30 rows, shares equal in tiles
+//     against this: encode D = 160 25.2 and 18.1 us, decode D = 128 bf16 14.5 and 12.0, D = 256 31.2 and 28.9);
+//   * else, with at least eight tiles per share, the shares are equal in COST, a lambda row counting one unit more than its
+//     tiles (a share that would begin inside that unit begins at the row's first tile);
+//   * else they are equal in tiles.
 struct TileShare {
     int64_t tps;     // tiles per segment
     int64_t begin;   // first tile of this share
     int n;           // tiles in this share
-    __device__ __forceinline__ TileShare(int64_t n_seg, int64_t rpl, unsigned part, unsigned parts, int tile_rows = 128)
+    __host__ __device__ __forceinline__ TileShare(int64_t n_seg, int64_t rpl, unsigned part, unsigned parts, int tile_rows = 128, int64_t segs = 1)
     {
         tps = (rpl + tile_rows - 1) / tile_rows;
         const int64_t n_tiles = n_seg * tps;
-        const int64_t R = (n_seg > 1 && n_tiles >= 8 * (int64_t)parts) ? 1 : 0;   // cost units of a rebuild
-        const int64_t C = tps + R, total = n_seg * C;
+        if (segs > n_seg) segs = n_seg;
+        const int64_t row_tiles = segs * tps, n_rows = (n_seg + segs - 1) / segs;
+        const int64_t even = (n_tiles + parts - 1) / parts;
+        if (n_rows <= (int64_t)parts) {
+            const int64_t k = parts / n_rows, per = (row_tiles + k - 1) / k;   // shares per lambda row, tiles per share
+            if (per <= even + 2 || n_rows == 1) {
+                const int64_t row = part / k, from = (part - row * k) * per;
+                int64_t end = from + per < row_tiles ? from + per : row_tiles;
+                begin = row * row_tiles + from;
+                end += row * row_tiles;
+                if (end > n_tiles) end = n_tiles;
+                n = row < n_rows && end > begin ? (int)(end - begin) : 0;
+                return;
+            }
+        }
+        const int64_t R = n_tiles >= 8 * (int64_t)parts ? 1 : 0;   // cost units of a rebuild
+        const int64_t C = row_tiles + R, total = n_tiles + n_rows * R;
         const int64_t per = (total + parts - 1) / parts;
         auto tile_of = [&](int64_t u) -> int64_t {
             if (u >= total) return n_tiles;
-            const int64_t seg = u / C, w = u - seg * C;
-            return seg * tps + (w > R ? w - R : 0);
+            const int64_t row = u / C, w = u - row * C;
+            return row * row_tiles + (w > R ? w - R : 0);
         };
         begin = tile_of((int64_t)part * per);
         const int64_t end = tile_of(((int64_t)part + 1) * per);

@@ -48,8 +48,7 @@ namespace {
 constexpr int kTile = 128;       // vectors per tile = MMA M
 constexpr int kThreads = 576;    // producer, mma, 2 x 4 dequant, 2 x 4 epilogue warps
 constexpr int kMaxInStages = 6;  // packed tiles in flight, at most
-constexpr int kAccStages = 2;    // accumulators in tensor memory
-constexpr int kCtrlBytes = 4608;   // barriers and flags, then eight tiles' worth of per-row output scales
+constexpr int kCtrlBytes = 5888;   // barriers and flags, eight tiles' worth of per-row output scales, two rows of reciprocals
 constexpr int kRowScaleSlots = 8;  // a dequant group is never more than seven tiles ahead of the epilogue that reads its slot
 constexpr uint32_t kTmemCols = 512;
 
@@ -59,18 +58,19 @@ constexpr uint32_t kTmemCols = 512;
 // W' = W_hi + W_lo, and x^ = a_hi W_hi + a_lo W_hi + a_hi W_lo accumulates in fp32 (a_lo W_lo is below 1e-7).
 // BITS: 4 (nibble pairs) or 8 (one two's-complement byte per code; scale = absmax / 127).  The byte path dequantises
 // pairs of neighbouring codes, so its K order is the natural one and the B operand is built to match.
-// R2: one radix-2 step of the transform is taken out of the GEMM (plans without a rotation; D = 128, 4-bit codes, either
-// output type).  Rows of M are cos / sin(2 pi k n / D), so n -> n + D / 2 multiplies a row by (-1)^k, and in the packing of Eq. 2
-// the parity of k is the parity of the channel c.  With E_n / O_n the sums over the even / odd channels (n < D / 2),
+// R2: one radix-2 step of the transform is taken out of the GEMM (plans without a rotation).  Rows of M are cos / sin(2 pi k n / D),
+// so n -> n + D / 2 multiplies a row by (-1)^k, and in the packing of Eq. 2 the parity of k is the parity of the channel c.  With
+// E_n / O_n the sums over the even / odd channels (n < D / 2),
 //     x^_n = s_n (E_n + O_n),        x^_{n + D/2} = s_{n + D/2} (E_n - O_n):
-// two 128 x 64 x 64 GEMMs per tile instead of one 128 x 128 x 128, half the tensor work, and an add, a subtract and half a
-// sign flip per output in the epilogue.  The kernel runs at the board's power limit, where tensor flops are what is left to
-// save: 147 -> 134 us per 2M-vector launch back to back (bf16 output: 215 -> 192 us).  The half2 nibble trick yields pairs
-// (c, c + 4) of equal parity, so routing codes to the two A operands is free.
+// two 128 x D/2 x D/2 GEMMs per tile instead of one 128 x D x D, half the tensor work and half the B operand to build and to hold, for
+// an add, a subtract and half a sign flip per output in the epilogue.  The half2 nibble trick yields pairs (c, c + 4) of equal
+// parity, a byte permute pairs (c, c + 2), so routing codes to the two A operands is free.  2M vectors at D = 128 back to back: 147 ->
+// 134 us (bf16 output: 215 -> 192).  At the other head dimensions, with the
+// quads of the table dealt out evenly and elect.sync, dense form -> this: D = 160 bf16 500,000 vectors 87.9 -> 65.0, 99,993 under three
+// lambda rows 37.9 -> 19.8; fp16 53.9 -> 45.9; D = 96 bf16 41.0 -> 34.9; D = 64 fp16 1M 42.7 -> 39.2; D = 128 bytes, bf16, 303,067: 36.2 -> 29.6.
 template <int D, bool BF16OUT, int BITS = 4, bool R2 = false>
 struct Cfg {
     static_assert(D % 32 == 0 && D >= 64 && D <= 160, "head dim not built");
-    static_assert(!R2 || (D == 128 && BITS == 4), "radix-2 form: D = 128, 4-bit codes");
     static_assert(!BF16OUT || BITS == 4 || D <= 128, "two-term operands with byte codes: shared memory holds them for D <= 128 only");
     static_assert(BITS == 4 || BITS == 8, "code width not built");
     static constexpr int kTerms = BF16OUT ? 2 : 1;         // W_hi (, W_lo); a_hi (, a_lo)
@@ -79,7 +79,8 @@ struct Cfg {
     static constexpr int kKBlocks = (D + 63) / 64;         // K blocks of 64 elements (the last one may be half used)
     static constexpr int kBBlock = D * 128;                // bytes of one K block: D rows x 128 B
     static constexpr int kBTerm = kKBlocks * kBBlock;
-    static constexpr int kBPart = (D / 2) * 128;           // R2: one parity's operand, D / 2 outputs x D / 2 channels
+    static constexpr int kBPartBlock = (D / 2) * 128;      // R2: one K block of one parity's operand, D / 2 outputs x 64 channels
+    static constexpr int kBPart = (D / 2 + 63) / 64 * kBPartBlock;   // D / 2 outputs x D / 2 channels
     static constexpr int kBBytes = R2 ? kTerms * 2 * kBPart : kTerms * kBTerm;   // R2: [term][parity]
     static constexpr int kInRow = D * BITS / 8;            // code bytes per row
     static constexpr int kInBytes = kTile * kInRow;        // bytes one TMA load brings
@@ -94,21 +95,27 @@ struct Cfg {
     static constexpr int kInStages = kRoom < kMaxInStages ? kRoom : kMaxInStages;
     static_assert(kInStages >= (D == 160 && BF16OUT ? 2 : 3), "too few packed tiles in flight");
     static constexpr int kSmemBytes = kBBytes + kInStages * kInPitch + kOutBytes + kCtrlBytes + 1024;
-    // tensor memory, D <= 128: two accumulators of D columns, then the A stages of D / 2 columns per term (a_lo 64 columns
-    // behind a_hi).  D = 160: an accumulator and an A term of 80 columns in each half of the 512 columns; with two-term
-    // operands the two halves hold a_hi and a_lo of ONE stage (the tile is tensor-bound: 3 x 10 K-steps per tile).
+    // tensor memory, D <= 128: two accumulators of up to 128 columns, then the A stages of D / 2 columns per term (a_lo 64 columns
+    // behind a_hi).  D = 160: an accumulator and an A term of 80 columns in each half of the 512 columns.  With two-term operands
+    // the dense form has a_hi and a_lo of ONE stage there; the radix-2 form, whose MMAs take a third of the time, has two A stages
+    // and one accumulator, which the epilogue hands back as soon as it is in registers.
+    static constexpr bool kOneAcc = R2 && D == 160 && BF16OUT;
+    static constexpr int kAccStages = kOneAcc ? 1 : 2;
     static constexpr uint32_t kAccStride = D <= 128 ? 128 : 256;
-    static constexpr int kAStages = BF16OUT ? (D <= 128 ? 2 : 1) : D <= 128 ? 4 : 2;
+    static constexpr uint32_t kOCol = D == 96 ? 64 : D == 160 ? 96 : D / 2;   // R2: the O columns of an accumulator (E at 0)
+    static constexpr int kAStages = kOneAcc ? 2 : BF16OUT ? (D <= 128 ? 2 : 1) : D <= 128 ? 4 : 2;
     // The "A full" / "A free" barriers form a ring of at least two, indexed by tile: the two dequant groups take alternate
     // tiles, and a parity wait only tells a phase from its neighbours, so a barrier must not be shared by both groups.
     // Tile j writes A stage j % kAStages once the MMAs of tile j - kAStages have completed (barrier (j - kAStages) % kABars).
+    // For the same reason the accumulator's barriers are a ring of two whatever the number of stages.
     static constexpr int kABars = kAStages < 2 ? 2 : kAStages;
-    static constexpr uint32_t kALo = D <= 128 ? 64 : 256;
+    static constexpr uint32_t kALo = kOneAcc ? 80 : D <= 128 ? 64 : 256;
     __host__ __device__ static constexpr uint32_t acc_col(int s) { return (uint32_t)s * kAccStride; }
     __host__ __device__ static constexpr uint32_t a_col(int s)
     {
-        return D <= 128 ? 256u + 64u * (uint32_t)kTerms * (uint32_t)s : 160u + 256u * (uint32_t)s;
+        return D <= 128 ? 256u + 64u * (uint32_t)kTerms * (uint32_t)s : kOneAcc ? 176u + 160u * (uint32_t)s : (R2 ? 176u : 160u) + 256u * (uint32_t)s;
     }
+    static constexpr int kQuads = D / 4;                   // float4 per table row
     static constexpr uint32_t kIdesc = umma_idesc_m128(R2 ? D / 2 : D, false);
     static constexpr int kBRows = R2 ? D / 2 : D;          // rows of the plan table that B is built from
 };
@@ -116,123 +123,123 @@ struct Cfg {
 struct Ctrl {
     uint64_t in_full[kMaxInStages], in_empty[kMaxInStages];
     uint64_t a_full[4], a_empty[4];
-    uint64_t acc_full[kAccStages], acc_empty[kAccStages];
+    uint64_t acc_full[2], acc_empty[2];
     uint64_t b_first;
     uint32_t tmem_base;
     volatile uint32_t abort;
     volatile uint32_t any_wide;   // some lambda row of this CTA's tiles is too wide for the fp16 B operand: redone in fp32 at the end
+    alignas(16) float recip[2][160];                      // 1 / (max(lambda, 1e-6) rho) of the row a dequant group builds B for
     float row_scale[kRowScaleSlots][kTile];   // what the epilogue multiplies a row by (1 unless its scales left fp16's comfort zone)
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 
-// Rows [n0, n1) of the B operand, by one warp: a lane reads four table entries b0[n][4 i .. 4 i + 3] (coalesced
-// rows), scales them, trades two values with its neighbour so that each lane holds two K-ordered pairs, and
-// writes 8 bytes of the swizzled row.
-template <int D, bool BF16OUT, int BITS>
-__device__ __forceinline__ void build_b_quad(unsigned char *sB, float4 m, const RecipLambda<D> &rl, int n, int p, int lane)
+// One quad of the B operand, the table entries m of row n and channels 4 i .. 4 i + 3 times the reciprocals rc, and its place in the
+// swizzled K-major row.  4-bit codes: neighbouring lanes hold the two quads of a word of eight codes and trade two values, so that
+// each holds two K-ordered pairs of the dense form (K order of a word: 0, 4, 1, 5, 2, 6, 3, 7), or one pair of each parity of
+// the radix-2 form (even lane 8w + p and 8w + p + 4, odd lane 8w + p + 2 and 8w + p + 6): the order in which the dequant threads
+// write the codes.  Byte codes: the natural order, per parity pairs (c, c + 2).  Every lane calls it (shuffles); `live` ones store.
+template <int D, bool BF16OUT, int BITS, bool R2>
+__device__ __forceinline__ void build_b_quad(unsigned char *sB, float4 m, float4 rc, int n, int i, bool live)
 {
-    using C = Cfg<D, BF16OUT, BITS>;
-    const bool odd = lane & 1;
-    const int i = lane + 32 * p;
-    const bool live = i < D / 4;
+    using C = Cfg<D, BF16OUT, BITS, R2>;
+    const bool odd = i & 1;
     auto sat = [](float v) { return fminf(fmaxf(v, -65504.0f), 65504.0f); };
-    float vx = sat(m.x * rl.r[p].x), vy = sat(m.y * rl.r[p].y), vz = sat(m.z * rl.r[p].z), vw = sat(m.w * rl.r[p].w);
-    const int w = i >> 1;   // word of 8 codes = 16-byte chunk w of the K-major row: K block w / 8, chunk w % 8
-    unsigned char *dst = sB + (w >> 3) * C::kBBlock + n * 128 + (((w & 7) ^ (n & 7)) << 4) + (odd ? 8 : 0);
+    const float v[4] = {sat(m.x * rc.x), sat(m.y * rc.y), sat(m.z * rc.z), sat(m.w * rc.w)};
+    if constexpr (R2) {
+        const int at = BITS == 4 ? 8 * (i >> 1) + (odd ? 4 : 0) : 4 * i;   // byte of the pair within a parity's K-major row
+        unsigned char *dst = sB + (at >> 7) * C::kBPartBlock + n * 128 + ((((at >> 4) & 7) ^ (n & 7)) << 4) + (at & 15);
 #pragma unroll
-    for (int t = 0; t < C::kTerms; ++t) {
-        uint2 o;
-        if constexpr (BITS == 4) {
-            // even lane holds codes 8w .. 8w+3, odd lane 8w+4 .. 8w+7; K order of the word is (0,4,1,5,2,6,3,7)
-            const float r0 = __shfl_xor_sync(0xFFFFFFFFu, odd ? vx : vz, 1);
-            const float r1 = __shfl_xor_sync(0xFFFFFFFFu, odd ? vy : vw, 1);
-            o.x = odd ? narrow2<false>(r0, vz) : narrow2<false>(vx, r0);   // odd: (2, 6)   even: (0, 4)
-            o.y = odd ? narrow2<false>(r1, vw) : narrow2<false>(vy, r1);   // odd: (3, 7)   even: (1, 5)
-        } else {   // byte codes: natural K order, this lane's four channels side by side
-            o.x = narrow2<false>(vx, vy);
-            o.y = narrow2<false>(vz, vw);
+        for (int p = 0; p < 2; ++p) {
+            float w0 = v[p], w1 = v[p + 2];
+            if constexpr (BITS == 4) {
+                const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? v[p] : v[p + 2], 1);
+                w0 = odd ? got : v[p], w1 = odd ? v[p + 2] : got;
+            }
+#pragma unroll
+            for (int t = 0; t < C::kTerms; ++t) {
+                const uint32_t h = narrow2<false>(w0, w1);
+                if (live) *reinterpret_cast<uint32_t *>(dst + p * C::kBPart + t * (2 * C::kBPart)) = h;
+                if (t + 1 < C::kTerms) {   // what the fp16 term left behind (exact in fp32)
+                    const float2 a = widen2<false>(h);
+                    w0 -= a.x, w1 -= a.y;
+                }
+            }
         }
-        if (live) *reinterpret_cast<uint2 *>(dst + t * C::kBTerm) = o;
-        if (t + 1 < C::kTerms) {   // what the fp16 term left behind (exact in fp32)
-            vx -= __half2float(__float2half_rn(vx)), vy -= __half2float(__float2half_rn(vy));
-            vz -= __half2float(__float2half_rn(vz)), vw -= __half2float(__float2half_rn(vw));
-        }
-    }
-}
-
-// Radix-2 form, row n < D / 2 of both parities' operands.  The lane's four channels 4 i .. 4 i + 3 alternate in parity;
-// per parity p the even lane assembles the pair (8w + p, 8w + p + 4) and the odd lane (8w + p + 2, 8w + p + 6), each from
-// one value of its own and one of its neighbour's: the K order in which the dequant threads write the codes of parity p.
-template <int D, int TERMS>
-__device__ __forceinline__ void build_b_quad_r2(unsigned char *sB, float4 m, const RecipLambda<D> &rl, int n, int lane)
-{
-    static_assert(D == 128, "one pass of 32 lanes covers the row");
-    constexpr int kPart = (D / 2) * 128;
-    const bool odd = lane & 1;
-    auto sat = [](float v) { return fminf(fmaxf(v, -65504.0f), 65504.0f); };
-    const float v[4] = {sat(m.x * rl.r[0].x), sat(m.y * rl.r[0].y), sat(m.z * rl.r[0].z), sat(m.w * rl.r[0].w)};
-    const int w = lane >> 1;   // word of 8 codes; its parity-p codes take bytes 8 w .. 8 w + 7 of the parity's K-major row
+    } else {
+        float vx = v[0], vy = v[1], vz = v[2], vw = v[3];
+        const int w = i >> 1;   // 16-byte chunk w of the K-major row: K block w / 8, chunk w % 8
+        unsigned char *dst = sB + (w >> 3) * C::kBBlock + n * 128 + (((w & 7) ^ (n & 7)) << 4) + (odd ? 8 : 0);
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? v[p] : v[p + 2], 1);
-        float w0 = odd ? got : v[p], w1 = odd ? v[p + 2] : got;
-        unsigned char *dst = sB + p * kPart + n * 128 + ((((w >> 1) ^ (n & 7))) << 4) + ((w & 1) ? 8 : 0) + (odd ? 4 : 0);
-#pragma unroll
-        for (int t = 0; t < TERMS; ++t) {
-            const uint32_t h = narrow2<false>(w0, w1);
-            *reinterpret_cast<uint32_t *>(dst + t * (2 * kPart)) = h;
-            if (t + 1 < TERMS) {   // what the fp16 term left behind (exact in fp32)
-                const float2 a = widen2<false>(h);
-                w0 -= a.x, w1 -= a.y;
+        for (int t = 0; t < C::kTerms; ++t) {
+            uint2 o;
+            if constexpr (BITS == 4) {
+                const float r0 = __shfl_xor_sync(0xFFFFFFFFu, odd ? vx : vz, 1);
+                const float r1 = __shfl_xor_sync(0xFFFFFFFFu, odd ? vy : vw, 1);
+                o.x = odd ? narrow2<false>(r0, vz) : narrow2<false>(vx, r0);   // odd: (2, 6)   even: (0, 4)
+                o.y = odd ? narrow2<false>(r1, vw) : narrow2<false>(vy, r1);   // odd: (3, 7)   even: (1, 5)
+            } else {
+                o.x = narrow2<false>(vx, vy);
+                o.y = narrow2<false>(vz, vw);
+            }
+            if (live) *reinterpret_cast<uint2 *>(dst + t * C::kBTerm) = o;
+            if (t + 1 < C::kTerms) {   // what the fp16 term left behind (exact in fp32)
+                vx -= __half2float(__float2half_rn(vx)), vy -= __half2float(__float2half_rn(vy));
+                vz -= __half2float(__float2half_rn(vz)), vw -= __half2float(__float2half_rn(vw));
             }
         }
     }
 }
 
-template <int D, bool BF16OUT, int BITS, bool R2>
-__device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__restrict__ b0, const RecipLambda<D> &rl, int n0, int n1,
-                                             int lane)
-{
-#pragma unroll 4
-    for (int n = n0; n < n1; ++n) {
-#pragma unroll
-        for (int p = 0; p < RecipLambda<D>::kPasses; ++p) {
-            const int i = lane + 32 * p;
-            float4 m = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (i < D / 4) m = __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)n * D) + i);
-            if constexpr (R2) build_b_quad_r2<D, Cfg<D, BF16OUT, BITS, R2>::kTerms>(sB, m, rl, n, lane);
-            else build_b_quad<D, BF16OUT, BITS>(sB, m, rl, n, p, lane);
-        }
-    }
-}
-
-// The first build of a CTA: its D / 16 table rows per warp are requested at kernel entry, all at once, and turned
-// into B rows here, once lambda has arrived too: one round trip to L2 instead of one per batch of rows.
-template <int D, bool BF16OUT, int BITS, bool R2>
-struct FirstRows {
-    static constexpr int kRows = (R2 ? D / 2 : D) / 16, kPasses = RecipLambda<D>::kPasses;
-    float4 m[kRows][kPasses];
-    __device__ __forceinline__ void load(const float *__restrict__ b0, int n0, int lane)
+// The B operand by W warps: the table's quads, row after row, dealt out to all their lanes, so that no lane idles where a row is not
+// a multiple of 32 quads, in batches of up to 16 that are requested together (load) and turned into B rows once the reciprocals
+// are in shared memory and the old operand is free (store): one round trip to L2 per batch, the first one before the wait.
+template <int D, bool BF16OUT, int BITS, bool R2, int W>
+struct BuildB {
+    using C = Cfg<D, BF16OUT, BITS, R2>;
+    static constexpr int kTotal = C::kBRows * C::kQuads;
+    static constexpr int kPerLane = (kTotal + 32 * W - 1) / (32 * W);
+    static constexpr int kBatches = (kPerLane + 15) / 16;
+    static constexpr int kBatch = (kPerLane + kBatches - 1) / kBatches;
+    float4 m[kBatch];
+    static __device__ __forceinline__ int quad(int batch, int k, int w, int lane) { return ((batch * kBatch + k) * W + w) * 32 + lane; }
+    __device__ __forceinline__ void load(const float *__restrict__ b0, int batch, int w, int lane)
     {
 #pragma unroll
-        for (int k = 0; k < kRows; ++k)
-#pragma unroll
-            for (int p = 0; p < kPasses; ++p) {
-                const int i = lane + 32 * p;
-                m[k][p] = i < D / 4 ? __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)(n0 + k) * D) + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
+        for (int k = 0; k < kBatch; ++k) {
+            const int f = quad(batch, k, w, lane);
+            m[k] = f < kTotal ? __ldg(reinterpret_cast<const float4 *>(b0) + f) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
     }
-    __device__ __forceinline__ void build(unsigned char *sB, const RecipLambda<D> &rl, int n0, int lane) const
+    __device__ __forceinline__ void store(unsigned char *sB, const float *recip, int batch, int w, int lane) const
     {
 #pragma unroll
-        for (int k = 0; k < kRows; ++k)
+        for (int k = 0; k < kBatch; ++k) {
+            const int f = quad(batch, k, w, lane), n = f / C::kQuads, i = f - n * C::kQuads;   // kQuads is even: lane pairs stay in one row
+            const bool live = f < kTotal;
+            const float4 rc = *reinterpret_cast<const float4 *>(recip + 4 * i);
+            build_b_quad<D, BF16OUT, BITS, R2>(sB, m[k], rc, live ? n : 0, i, live);
+        }
+    }
+    // batches from the second on, after store(0)
+    __device__ __forceinline__ void rest(unsigned char *sB, const float *__restrict__ b0, const float *recip, int w, int lane)
+    {
 #pragma unroll
-            for (int p = 0; p < kPasses; ++p) {
-                if constexpr (R2) build_b_quad_r2<D, Cfg<D, BF16OUT, BITS, R2>::kTerms>(sB, m[k][p], rl, n0 + k, lane);
-                else build_b_quad<D, BF16OUT, BITS>(sB, m[k][p], rl, n0 + k, p, lane);
-            }
+        for (int b = 1; b < kBatches; ++b) {
+            load(b0, b, w, lane);
+            store(sB, recip, b, w, lane);
+        }
     }
 };
+
+// every warp that builds writes the whole row itself (the same values) and so needs no more than its own lanes to be done
+template <int D>
+__device__ __forceinline__ void post_reciprocals(float *recip, const RecipLambda<D> &rl, int lane)
+{
+#pragma unroll
+    for (int p = 0; p < RecipLambda<D>::kPasses; ++p)
+        if (lane + 32 * p < D / 4) *reinterpret_cast<float4 *>(recip + 4 * (lane + 32 * p)) = rl.r[p];
+    __syncwarp();
+}
 
 // The D / 32 fp16 group scales of one row, as packed 16-bit pairs.
 template <int G>
@@ -260,9 +267,10 @@ struct UmmaDecodeParams {
     GemmParams g;
     int64_t rpl;        // rows per lambda segment (N when there is one lambda row)
     int64_t n_seg;      // segments
+    int64_t segs;       // consecutive segments with one lambda row: 1, or what a cache view's streams share
     int64_t n_full;     // segments of exactly rpl rows, covered by the main output maps; a shorter last one uses the tail maps
     int64_t phys_rows;  // rows of the packed / scales arrays (N, or the whole cache for a cache view)
-    uint32_t flip2[32]; // radix-2 form: sign-bit masks of s_n s_{n + 64} for the output pairs (n, n + 1), n = 0, 2, .. 62
+    uint32_t flip2[40]; // radix-2 form: sign-bit masks of s_n s_{n + D/2} for the output pairs (n, n + 1), n = 0, 2, .. D/2 - 2
 };
 
 struct UmmaDecodeMaps {
@@ -271,12 +279,38 @@ struct UmmaDecodeMaps {
     CUtensorMap slim, slim_tail;   // output, boxes of 32 columns x 32 rows (64-byte swizzle), used when D / 32 is odd
 };
 
+// The group that meets a lambda row's first tile rebuilds B.  Kept out of line: rare, and the loop around it stays small.
+template <int D, bool BF16OUT, int BITS, bool R2>
+__device__ __noinline__ bool rebuild_b(unsigned char *sB, Ctrl *ctrl, const float *__restrict__ b0, const RecipLambda<D> &rl, int grp, int q, int lane,
+                                       int j, uint32_t *status)
+{
+    using C = Cfg<D, BF16OUT, BITS, R2>;
+    BuildB<D, BF16OUT, BITS, R2, 4> rows;
+    rows.load(b0, 0, q, lane);
+    post_reciprocals<D>(ctrl->recip[grp], rl, lane);
+    // Every MMA issued so far has read B: the commit of the previous tile (the other group's) covers them
+    // all.  A parity wait can only tell a phase from its neighbours, and the other group may lag by more
+    // than one of its tiles, so first wait for this group's own last tile (its barrier is at most one
+    // phase behind, this group waited on it before writing that tile): MMAs complete in order, so after it
+    // the previous tile's barrier is at most one phase behind too.
+    if (j >= 2 && !wait_or_abort(smem_u32(&ctrl->a_empty[(j - 2) % C::kABars]), (uint32_t)((j - 2) / C::kABars) & 1u, &ctrl->abort, status,
+                                 KVQ_DEV_MMA_TIMEOUT))
+        return false;
+    if (!wait_or_abort(smem_u32(&ctrl->a_empty[(j - 1) % C::kABars]), (uint32_t)((j - 1) / C::kABars) & 1u, &ctrl->abort, status,
+                       KVQ_DEV_MMA_TIMEOUT))
+        return false;
+    rows.store(sB, ctrl->recip[grp], 0, q, lane);
+    rows.rest(sB, b0, ctrl->recip[grp], q, lane);
+    fence_proxy_async();   // B is read by the tensor core through the async proxy
+    return true;
+}
+
 template <int D, bool BF16OUT, int BITS, bool R2>
 __global__ void __launch_bounds__(kThreads, 1)
     kvq_decode_umma_kernel(const __grid_constant__ UmmaDecodeParams prm, const __grid_constant__ UmmaDecodeMaps maps)
 {
     using C = Cfg<D, BF16OUT, BITS, R2>;
-    constexpr int G = C::G, kInStages = C::kInStages;
+    constexpr int G = C::G, kInStages = C::kInStages, kAccStages = C::kAccStages;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char *sB = smem;
@@ -295,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(smem_u32(&ctrl->a_full[s]), 4);
             mbar_init(smem_u32(&ctrl->a_empty[s]), 1);
         }
-        for (int s = 0; s < kAccStages; ++s) {
+        for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&ctrl->acc_full[s]), 1);
             mbar_init(smem_u32(&ctrl->acc_empty[s]), 4);
         }
@@ -309,13 +343,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range of tiles
     // ---- per CTA, so that the B operand is rebuilt as rarely as possible
     const int64_t N = prm.g.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x);
+    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x, kTile, prm.segs);
     const int64_t tps = share.tps, tile_begin = share.begin;
     const int n_my = share.n;
     const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * D; };
 
-    // ---- B for the first tile's lambda row: the sixteen dequant and epilogue warps build D / 16 rows each while the
+    // ---- B for the first tile's lambda row: the sixteen dequant and epilogue warps build it while the
     // ---- producer's first loads are in flight; the mma warp waits for all of them.  Table rows and lambda are
     // ---- requested before the set-up barrier, so that their latency runs under it.
     // ---- The dequant warps also request the scales of their first tile here and keep rho, so that neither costs a round
@@ -325,8 +359,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
     for (int i = 0; i < (G + 1) / 2; ++i) sc_first[i] = 0u;
     if (n_my > 0 && warp >= 2) {
-        FirstRows<D, BF16OUT, BITS, R2> rows;
-        rows.load(prm.g.b0, (warp - 2) * (C::kBRows / 16), lane);
+        BuildB<D, BF16OUT, BITS, R2, 16> rows;
+        rows.load(prm.g.b0, 0, warp - 2, lane);
         grid_wait();
         if (warp < 10 && ((warp - 2) >> 2) < n_my) {   // dequant group g's first tile is tile_begin + g
             const TileCursor first(tile_begin + ((warp - 2) >> 2), tps);
@@ -349,7 +383,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         __syncthreads();
         tc_fence_after();
         if (rl.wide) ctrl->any_wide = 1u;
-        rows.build(sB, rl, (warp - 2) * (C::kBRows / 16), lane);
+        post_reciprocals<D>(ctrl->recip[0], rl, lane);
+        rows.store(sB, ctrl->recip[0], 0, warp - 2, lane);
+        rows.rest(sB, prm.g.b0, ctrl->recip[0], warp - 2, lane);
         fence_proxy_async();   // B is read by the tensor core through the async proxy
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
@@ -389,7 +425,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 1) {
         // =========================== mma issuer ===========================
-        if (lane == 0) {
+        // (elect.sync, not lane 0: the compiler then knows that one thread issues.  128 x 64 x 16 with A in tensor memory: 32 cycles, else 45)
+        if (elect_one()) {
             const uint64_t b_desc = smem_desc_sw128(smem_u32(sB));
             const uint32_t b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
             int n_mma = n_my;
@@ -397,9 +434,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int j = 0; j < n_mma; ++j) {
                 const int sa = j % C::kAStages, sb = j % C::kABars, sc = j % kAccStages;
                 if (!wait_or_abort(smem_u32(&ctrl->a_full[sb]), (uint32_t)(j / C::kABars) & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
-                if (!wait_or_abort(smem_u32(&ctrl->acc_empty[sc]), ((uint32_t)(j / kAccStages) & 1u) ^ 1u, abort_flag, status,
-                                   KVQ_DEV_SLOT_TIMEOUT))
-                    break;
+                if (j >= kAccStages) {   // the epilogue has taken the tile that used this accumulator last
+                    const int jp = j - kAccStages;
+                    if (!wait_or_abort(smem_u32(&ctrl->acc_empty[jp & 1]), (uint32_t)(jp >> 1) & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
+                }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + C::acc_col(sc);
                 const uint32_t a_tmem = tmem_base + C::a_col(sa);
@@ -411,8 +449,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                             for (int ks = 0; ks < D / 32; ++ks) {
                                 const uint32_t b_set = b_lo + (set == 2 ? (uint32_t)((2 * C::kBPart) >> 4) : 0u) + (uint32_t)p * (C::kBPart >> 4);
-                                const uint64_t bd = ((uint64_t)b_hi << 32) | (uint64_t)(b_set + (uint32_t)ks * 2u);
-                                const uint32_t dp = d_tmem + (uint32_t)p * (D / 2);
+                                const uint64_t bd = ((uint64_t)b_hi << 32) | (uint64_t)(b_set + (uint32_t)(ks >> 2) * (C::kBPartBlock >> 4) + (uint32_t)(ks & 3) * 2u);
+                                const uint32_t dp = d_tmem + (uint32_t)p * C::kOCol;
                                 const uint32_t ap = a_tmem + (set == 1 ? C::kALo : 0u) + (uint32_t)p * (D / 4) + (uint32_t)ks * 8u;
                                 if (set > 0 || ks > 0) umma_f16_ts<true>(dp, ap, bd, C::kIdesc);
                                 else umma_f16_ts<false>(dp, ap, bd, C::kIdesc);
@@ -433,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         else umma_f16_ts<false>(d_tmem, a_set, bd, C::kIdesc);
                     }
                 }
-                umma_commit(smem_u32(&ctrl->acc_full[sc]));
+                umma_commit(smem_u32(&ctrl->acc_full[j & 1]));
                 umma_commit(smem_u32(&ctrl->a_empty[sb]));
             }
         }
@@ -447,7 +485,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                              : C::kInSwizzleBits == 2 ? (uint32_t)((r >> 1) & 3)
                              : C::kInSwizzleBits == 1 ? (uint32_t)((r >> 2) & 1)
                                                       : 0u;
-        int64_t cached_seg = n_my > 0 ? seg_first : -1;   // B holds this row's table (built above)
+        int64_t cached_row = n_my > 0 ? prm.g.lambda_index(seg_first) : -1;   // the lambda row that B holds (built above)
         float rho = rho_first;
 
         TileCursor cur(tile_begin + grp, tps), ahead(tile_begin + grp, tps);   // this tile; the tile whose scales are fetched
@@ -480,26 +518,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t seg = cur.seg;
 
             // ---- a new lambda row: this group needs its rho; the group that meets the row's first tile rebuilds B
-            if (seg != cached_seg) {
+            const int64_t row_of_seg = prm.g.lambda_index(seg);
+            if (row_of_seg != cached_row) {
                 const RecipLambda<D> rl(lambda_row(seg), lane);
                 rho = rl.rho;
                 if (rl.wide) ctrl->any_wide = 1u;
-                if (cur.first_of_segment()) {
-                    // Every MMA issued so far has read B: the commit of the previous tile (the other group's) covers them
-                    // all.  A parity wait can only tell a phase from its neighbours, and the other group may lag by more
-                    // than one of its tiles, so first wait for this group's own last tile (its barrier is at most one
-                    // phase behind, this group waited on it before writing that tile): MMAs complete in order, so after it
-                    // the previous tile's barrier is at most one phase behind too.
-                    if (j >= 2 && !wait_or_abort(smem_u32(&ctrl->a_empty[(j - 2) % C::kABars]), (uint32_t)((j - 2) / C::kABars) & 1u,
-                                                 abort_flag, status, KVQ_DEV_MMA_TIMEOUT))
-                        break;
-                    if (!wait_or_abort(smem_u32(&ctrl->a_empty[(j - 1) % C::kABars]), (uint32_t)((j - 1) / C::kABars) & 1u, abort_flag,
-                                       status, KVQ_DEV_MMA_TIMEOUT))
-                        break;
-                    build_b_rows<D, BF16OUT, BITS, R2>(sB, prm.g.b0, rl, q * (C::kBRows / 4), (q + 1) * (C::kBRows / 4), lane);
-                    fence_proxy_async();   // B is read by the tensor core through the async proxy
+                if (cur.first_of_segment() && prm.g.lambda_index(seg - 1) != row_of_seg) {
+                    if (!rebuild_b<D, BF16OUT, BITS, R2>(sB, ctrl, prm.g.b0, rl, grp, q, lane, j, status)) break;
                 }
-                cached_seg = seg;
+                cached_row = row_of_seg;
             }
 
             // ---- this tile's packed rows have landed; the A stage is free again
@@ -564,10 +591,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
                             const uint32_t u = words[i] ^ 0x80808080u;                 // bytes now hold q + 128
-                            const uint32_t m01 = __byte_perm(u, 0x64646464u, 0x4140);   // {1024 + b0, 1024 + b1} as fp16 bit patterns
-                            const uint32_t m23 = __byte_perm(u, 0x64646464u, 0x4342);
-                            put(8 * hc + 2 * i, __hsub2(*reinterpret_cast<const __half2 *>(&m01), h1152));       // exact q
-                            put(8 * hc + 2 * i + 1, __hsub2(*reinterpret_cast<const __half2 *>(&m23), h1152));
+                            // {1024 + b, 1024 + b'} as fp16 bit patterns: bytes 0, 1 and 2, 3, or 0, 2 (even channels) and 1, 3 (odd)
+                            const uint32_t ma = __byte_perm(u, 0x64646464u, R2 ? 0x4240 : 0x4140);
+                            const uint32_t mb = __byte_perm(u, 0x64646464u, R2 ? 0x4341 : 0x4342);
+                            put(R2 ? 4 * hc + i : 8 * hc + 2 * i, __hsub2(*reinterpret_cast<const __half2 *>(&ma), h1152));       // exact q
+                            put(R2 ? 8 + 4 * hc + i : 8 * hc + 2 * i + 1, __hsub2(*reinterpret_cast<const __half2 *>(&mb), h1152));
                         }
                     }
                 }
@@ -606,7 +634,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         TileCursor cur(tile_begin + grp, tps);
         for (int j = grp; j < n_my; j += 2, cur.advance(2)) {
             const int sc = j % kAccStages;
-            if (!wait_or_abort(smem_u32(&ctrl->acc_full[sc]), (uint32_t)(j / kAccStages) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
+            if (!wait_or_abort(smem_u32(&ctrl->acc_full[j & 1]), (uint32_t)(j >> 1) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
             tc_fence_after();
             if (lane == 0) bulk_wait_read_all();   // this warp's previous stores have read the staging tile
             __syncwarp();
@@ -614,11 +642,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             const bool rescale = __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
             if constexpr (R2) {
 #pragma unroll
-                for (int h = 0; h < 4; ++h) {   // E and O columns 16 h .. 16 h + 15 -> outputs 16 h .. and D / 2 + 16 h ..
+                for (int h = 0; h < D / 32; ++h) {   // E and O columns 16 h .. 16 h + 15 -> outputs 16 h .. and D / 2 + 16 h ..
                     uint32_t ev[16], ov[16];
                     tmem_ld16(lane_addr + C::acc_col(sc) + (uint32_t)h * 16u, ev);
-                    tmem_ld16(lane_addr + C::acc_col(sc) + (uint32_t)(D / 2) + (uint32_t)h * 16u, ov);
+                    tmem_ld16(lane_addr + C::acc_col(sc) + C::kOCol + (uint32_t)h * 16u, ov);
                     tmem_ld_wait();
+                    if (h == D / 32 - 1) {   // the last values are in registers: hand the accumulator back
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty[j & 1]));
+                    }
                     if (rescale) {
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
@@ -637,9 +670,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                             lo[p2] = narrow2<BF16OUT>(e0 + o0, e1 + o1);                                     // s_n is already in E and O
                             hi[p2] = narrow2<BF16OUT>(e0 - o0, e1 - o1) ^ prm.flip2[8 * h + 4 * k + p2];     // times s_n s_{n + D/2}
                         }
-                        const int chunk = 2 * h + k;   // both halves of the row are 64-column boxes: [32 rows][128 B], 128-byte swizzle
-                        *reinterpret_cast<uint4 *>(stg + lane * 128 + ((chunk ^ (lane & 7)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                        *reinterpret_cast<uint4 *>(stg + 32 * 128 + lane * 128 + ((chunk ^ (lane & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                        // 16-byte chunk c of the row: a 64-column box [32 rows][128 B] of 128-byte swizzle, or the last, 32-column one
+                        auto at = [&](int c) -> uint4 * {
+                            unsigned char *box = stg + (c >> 3) * (32 * 128);
+                            return reinterpret_cast<uint4 *>((c >> 3) < G / 2 ? box + lane * 128 + (((c & 7) ^ (lane & 7)) << 4)
+                                                                              : box + lane * 64 + (((c & 3) ^ ((lane >> 1) & 3)) << 4));
+                        };
+                        *at(2 * h + k) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                        *at(D / 16 + 2 * h + k) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                     }
                 }
             }
@@ -674,7 +712,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(smem_u32(&ctrl->acc_empty[sc]));
+                if constexpr (!R2) mbar_arrive(smem_u32(&ctrl->acc_empty[j & 1]));
                 const int64_t seg = cur.seg;
                 const int row_in_seg = (int)cur.row_in_segment() + q * 32;
                 const bool tail = seg >= prm.n_full;
@@ -732,12 +770,13 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const ui
     prm.g = g;
     prm.rpl = g.view.rows ? g.view.rows : g.n_lambda == 1 ? N : g.rows_per_lambda;   // a cache view: one segment per stream
     prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
+    prm.segs = g.n_lambda == 1 ? prm.n_seg : g.view.rows ? g.view.streams_per_lambda : 1;
     prm.n_full = N / prm.rpl;
     prm.phys_rows = g.view.rows ? prm.n_seg * g.view.stride : N;
     if (prm.phys_rows >= (int64_t)1 << 31) return cudaErrorInvalidValue;
     const int64_t seg_stride = g.view.rows ? g.view.stride : prm.rpl;   // rows from one segment's first row to the next's
     unsigned char *out0 = static_cast<unsigned char *>(g.out) + (size_t)(g.view.rows ? g.view.base : 0) * (2 * D);
-    for (int m = 0; m < 32; ++m) prm.flip2[m] = R2 && sign_xor ? sign_xor[m] ^ sign_xor[m + D / 4] : 0u;   // words hold two signs each
+    for (int m = 0; m < D / 4; ++m) prm.flip2[m] = R2 && sign_xor ? sign_xor[m] ^ sign_xor[m + D / 4] : 0u;   // words hold two signs each
 
     UmmaDecodeMaps maps;
     {
@@ -785,10 +824,26 @@ bool umma_decode_bits8_supported(int D, bool bf16) { return !(D == 160 && bf16) 
 cudaError_t umma_decode(int D, bool bf16, int bits, int64_t N, const GemmParams &g, const uint32_t *sign_xor, cudaStream_t stream,
                         bool radix2)
 {
-    // the radix-2 form needs the transform's even / odd structure: the caller asks for it on plans without a rotation
-    if (radix2 && D == 128 && bits == 4 && sign_xor)
-        return bf16 ? launch<128, true, 4, true>(N, g, stream, sign_xor) : launch<128, false, 4, true>(N, g, stream, sign_xor);
     if (D == 256 && sign_xor) return umma_decode_d256(bf16, bits, N, g, sign_xor, stream);   // its own kernel: radix-2 split, split operands for bf16
+    // the radix-2 form needs the transform's even / odd structure: the caller asks for it on plans without a rotation
+    if (radix2 && sign_xor) {
+        if (bits == 8) {
+            switch (D) {
+                case 64: return bf16 ? launch<64, true, 8, true>(N, g, stream, sign_xor) : launch<64, false, 8, true>(N, g, stream, sign_xor);
+                case 96: return bf16 ? launch<96, true, 8, true>(N, g, stream, sign_xor) : launch<96, false, 8, true>(N, g, stream, sign_xor);
+                case 128: return bf16 ? launch<128, true, 8, true>(N, g, stream, sign_xor) : launch<128, false, 8, true>(N, g, stream, sign_xor);
+                case 160: return bf16 ? cudaErrorInvalidValue : launch<160, false, 8, true>(N, g, stream, sign_xor);
+            }
+            return cudaErrorInvalidValue;
+        }
+        switch (D) {
+            case 64: return bf16 ? launch<64, true, 4, true>(N, g, stream, sign_xor) : launch<64, false, 4, true>(N, g, stream, sign_xor);
+            case 96: return bf16 ? launch<96, true, 4, true>(N, g, stream, sign_xor) : launch<96, false, 4, true>(N, g, stream, sign_xor);
+            case 128: return bf16 ? launch<128, true, 4, true>(N, g, stream, sign_xor) : launch<128, false, 4, true>(N, g, stream, sign_xor);
+            case 160: return bf16 ? launch<160, true, 4, true>(N, g, stream, sign_xor) : launch<160, false, 4, true>(N, g, stream, sign_xor);
+        }
+        return cudaErrorInvalidValue;
+    }
     if (bits == 8) {
         switch (D) {
             case 64: return bf16 ? launch<64, true, 8>(N, g, stream) : launch<64, false, 8>(N, g, stream);

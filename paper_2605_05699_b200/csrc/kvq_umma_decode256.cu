@@ -131,6 +131,7 @@ struct UmmaDecode256Params {
     GemmParams g;
     int64_t rpl;        // rows per lambda segment (N when there is one lambda row)
     int64_t n_seg;      // segments
+    int64_t segs;       // consecutive segments with one lambda row: 1, or what a cache view's streams share
     int64_t n_full;     // segments of exactly rpl rows, covered by the main output map; a shorter last one uses the tail map
     int64_t phys_rows;  // rows of the packed / scales arrays (N, or the whole cache for a cache view)
     uint32_t sign_xor[128];   // word m: bit 15 set if s_{2m} = -1, bit 31 set if s_{2m+1} = -1
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range of tiles per CTA
     const int64_t N = prm.g.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x);
+    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x, kTile, prm.segs);
     const int64_t tps = share.tps, tile_begin = share.begin;
     const int n_my = share.n;
     const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
@@ -251,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 1) {
         // =========================== mma issuer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             const uint64_t b_desc = smem_desc_sw128(smem_u32(sB));
             const uint32_t b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
             int n_mma = n_my;
@@ -294,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3;                 // tensor-memory lane quarter this warp may touch
         const int r = q * 32 + lane;            // tile row and tensor-memory lane of this thread
         const uint4 *scales = static_cast<const uint4 *>(prm.g.scales);   // 8 fp16 scales per row
-        int64_t cached_seg = n_my > 0 ? seg_first : -1;   // B holds this row's table (built above)
+        int64_t cached_row = n_my > 0 ? prm.g.lambda_index(seg_first) : -1;   // the lambda row that B holds (built above)
         float rho = rho_first;
 
         TileCursor cur(tile_begin, tps), ahead(tile_begin, tps);
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
             // ---- a new lambda row: new rho, and this group rebuilds the B operand of its own GEMM once every MMA of that
             // ---- GEMM issued so far is complete: the previous tile's, on this group's own barriers (it sees every phase)
-            if (seg != cached_seg) {
+            if (prm.g.lambda_index(seg) != cached_row) {
                 const RecipLambda<kD> rl(lambda_row(seg), lane);
                 if (rl.wide) ctrl->any_wide = 1u;
                 rho = rl.rho;
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     break;
                 build_b_rows<kTerms>(sB, prm.g.b0, rl, p, q * 32, q * 32 + 32, lane);
                 fence_proxy_async();   // B is read by the tensor core through the async proxy
-                cached_seg = seg;
+                cached_row = prm.g.lambda_index(seg);
             }
 
             // ---- this tile's packed rows have landed
@@ -525,6 +526,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cud
     prm.g = g;
     prm.rpl = g.view.rows ? g.view.rows : g.n_lambda == 1 ? N : g.rows_per_lambda;   // a cache view: one segment per stream
     prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
+    prm.segs = g.n_lambda == 1 ? prm.n_seg : g.view.rows ? g.view.streams_per_lambda : 1;
     prm.n_full = N / prm.rpl;
     prm.phys_rows = g.view.rows ? prm.n_seg * g.view.stride : N;
     if (prm.phys_rows >= (int64_t)1 << 31) return cudaErrorInvalidValue;

@@ -1,0 +1,50 @@
+"""The split of a call's tiles over the CTAs of a persistent kernel (TileShare), run on the host: every tile belongs to exactly one
+share, shares follow one another, and no share is more than two tiles longer than an even split's."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2605_05699_b200", "csrc")
+SOURCE = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "kvq_device.cuh"
+int main()
+{
+    srand(1);
+    for (long it = 0; it < 200000; ++it) {
+        const long n_seg = 1 + rand() % (it % 3 ? 12 : 400), rpl = 1 + rand() % (it % 2 ? 400 : 9000), segs = 1 + rand() % (it % 5 ? 1 : 20);
+        const unsigned parts = 1 + rand() % 150;
+        const int rows = it % 7 ? 128 : 256;
+        const long tps = (rpl + rows - 1) / rows, tiles = n_seg * tps, even = (tiles + parts - 1) / parts;
+        long at = 0;
+        for (unsigned p = 0; p < parts; ++p) {
+            const kvq::TileShare s(n_seg, rpl, p, parts, rows, segs);
+            if (s.n == 0) continue;
+            if (s.tps != tps || s.begin != at || s.n < 0 || s.n > even + 2) {
+                printf("n_seg %ld rpl %ld segs %ld parts %u: share %u begins at %ld (%ld), %d tiles of %ld\n", n_seg, rpl, segs, parts, p,
+                       (long)s.begin, at, s.n, even);
+                return 1;
+            }
+            at += s.n;
+        }
+        if (at != tiles) {
+            printf("n_seg %ld rpl %ld segs %ld parts %u: %ld of %ld tiles\n", n_seg, rpl, segs, parts, at, tiles);
+            return 1;
+        }
+    }
+    return 0;
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("nvcc") is None, reason="no nvcc")
+def test_every_tile_belongs_to_one_share(tmp_path):
+    src, exe = tmp_path / "share.cu", tmp_path / "share"
+    src.write_text(SOURCE)
+    subprocess.run(["nvcc", "-std=c++17", "--expt-relaxed-constexpr", "-gencode", "arch=compute_100a,code=sm_100a", "-I", CSRC, "-o", str(exe), str(src)],
+                   check=True, capture_output=True, text=True)
+    run = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert run.returncode == 0, run.stdout
