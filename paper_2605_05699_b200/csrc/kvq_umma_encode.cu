@@ -124,9 +124,6 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
     return __uint_as_float((uint32_t)(127 + 13 - e) << 23);
 }
 
-// Rows [c0, c1) of every split term of the B operand, by one warp: a lane reads four table entries
-// e0[c][4 i .. 4 i + 3] (coalesced rows), scales them by lambda_c 2^k, peels off 16-bit terms and writes
-// 8 bytes of each term's swizzled row.
 // One quad of row c of every split term: the four table entries m scaled by f = lambda_c 2^k, 16-bit terms peeled
 // off one after the other, 8 bytes of each term's swizzled row written.
 template <int D, bool BF16, bool THREE>
@@ -147,53 +144,47 @@ __device__ __forceinline__ void build_b_quad(unsigned char *sB, float4 m, float 
     }
 }
 
-template <int D, bool BF16, bool THREE>
-__device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__restrict__ e0, const float *__restrict__ lam, float lift,
-                                             int c0, int c1, int lane)
-{
-#pragma unroll 4
-    for (int c = c0; c < c1; ++c) {
-        const float f = lam ? __ldg(lam + c) * lift : lift;
+// The B operand by W warps: the table's quads, row after row, dealt out to all their lanes, so that no lane idles where a row is not
+// a multiple of 32 quads, in batches of up to 16 that are requested together (load) and turned into B rows once the lift is
+// known and the old operand is free (store): one round trip to L2 per batch, the first one before the wait.
+template <int D, bool BF16, bool THREE, int W>
+struct BuildB {
+    static constexpr int kQuads = D / 4, kTotal = D * kQuads;
+    static constexpr int kPerLane = (kTotal + 32 * W - 1) / (32 * W);
+    static constexpr int kBatches = (kPerLane + 15) / 16;
+    static constexpr int kBatch = (kPerLane + kBatches - 1) / kBatches;
+    float4 m[kBatch];
+    static __device__ __forceinline__ int quad(int batch, int k, int w, int lane) { return ((batch * kBatch + k) * W + w) * 32 + lane; }
+    __device__ __forceinline__ void load(const float *__restrict__ e0, int batch, int w, int lane)
+    {
 #pragma unroll
-        for (int p = 0; p < (D / 4 + 31) / 32; ++p) {
-            const int i = lane + 32 * p;
-            if (i < D / 4) build_b_quad<D, BF16, THREE>(sB, __ldg(reinterpret_cast<const float4 *>(e0 + (size_t)c * D) + i), f, c, i);
+        for (int k = 0; k < kBatch; ++k) {
+            const int f = quad(batch, k, w, lane);
+            m[k] = f < kTotal ? __ldg(reinterpret_cast<const float4 *>(e0) + f) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
     }
-}
-
-// The first build of a CTA: a warp's D / 16 table rows and their lambda entries are requested at kernel entry, all at
-// once, and turned into B rows once the lift is known: one round trip to L2 instead of one per batch of rows.
-template <int D, bool BF16, bool THREE>
-struct FirstRows {
-    static constexpr int kRows = D / 16, kPasses = (D / 4 + 31) / 32;
-    float4 m[kRows][kPasses];
-    float lam_c[kRows];
-    __device__ __forceinline__ void load_table(const float *__restrict__ e0, int c0, int lane)
+    __device__ __forceinline__ void store(unsigned char *sB, const float *__restrict__ lam, float lift, int batch, int w, int lane) const
     {
+        float fc[kBatch];
 #pragma unroll
-        for (int k = 0; k < kRows; ++k) {
+        for (int k = 0; k < kBatch; ++k) {
+            const int f = quad(batch, k, w, lane);
+            fc[k] = lam ? (f < kTotal ? __ldg(lam + f / kQuads) * lift : 0.0f) : lift;
+        }
 #pragma unroll
-            for (int p = 0; p < kPasses; ++p) {
-                const int i = lane + 32 * p;
-                m[k][p] = i < D / 4 ? __ldg(reinterpret_cast<const float4 *>(e0 + (size_t)(c0 + k) * D) + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
+        for (int k = 0; k < kBatch; ++k) {
+            const int f = quad(batch, k, w, lane), c = f / kQuads;
+            if (f < kTotal) build_b_quad<D, BF16, THREE>(sB, m[k], fc[k], c, f - c * kQuads);
         }
     }
-    __device__ __forceinline__ void load_lambda(const float *__restrict__ lam, int c0)
+    // batches from the second on, after store(0)
+    __device__ __forceinline__ void rest(unsigned char *sB, const float *__restrict__ e0, const float *__restrict__ lam, float lift, int w, int lane)
     {
 #pragma unroll
-        for (int k = 0; k < kRows; ++k) lam_c[k] = lam ? __ldg(lam + c0 + k) : 1.0f;
-    }
-    __device__ __forceinline__ void build(unsigned char *sB, float lift, int c0, int lane) const
-    {
-#pragma unroll
-        for (int k = 0; k < kRows; ++k)
-#pragma unroll
-            for (int p = 0; p < kPasses; ++p) {
-                const int i = lane + 32 * p;
-                if (i < D / 4) build_b_quad<D, BF16, THREE>(sB, m[k][p], lam_c[k] * lift, c0 + k, i);
-            }
+        for (int b = 1; b < kBatches; ++b) {
+            load(e0, b, w, lane);
+            store(sB, lam, lift, b, w, lane);
+        }
     }
 };
 
@@ -207,6 +198,21 @@ __device__ __forceinline__ bool wait_first_operand(uint32_t bar, volatile uint32
     *abort_flag = 1u;
     atomicOr(status, (uint32_t)KVQ_DEV_SLOT_TIMEOUT);
     return false;
+}
+
+// A set's rebuild of B, once the MMAs that read the old one are complete (phase `parity` of barrier `full_bar`).  Kept out of line:
+// rare, and the loop around it stays small.
+template <int D, bool BF16, bool THREE>
+__device__ __noinline__ bool rebuild_b(unsigned char *sB, const float *__restrict__ e0, const float *__restrict__ lam, float lift, int w, int lane,
+                                       uint32_t full_bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status)
+{
+    BuildB<D, BF16, THREE, kEpiWarps / 2> rows;
+    rows.load(e0, 0, w, lane);
+    if (!wait_or_abort(full_bar, parity, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) return false;
+    rows.store(sB, lam, lift, 0, w, lane);
+    rows.rest(sB, e0, lam, lift, w, lane);
+    fence_proxy_async();   // B is read by the tensor core through the async proxy
+    return true;
 }
 
 }  // namespace
@@ -263,23 +269,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t tps = share.tps, tile_begin = share.begin;
     const int n_my = share.n;
 
-    // ---- B for the CTA's first lambda row: D / 16 rows per epilogue warp.  Table rows and lambda are requested before
+    // ---- B for the CTA's first lambda row, by all epilogue warps.  Table and lambda are requested before
     // ---- the set-up barrier, so that their latency runs under it and under the first x loads.
     float first_lift = 1.0f;
     int64_t first_seg = -1;
     if (n_my > 0 && warp >= 2) {
         first_seg = tile_begin / tps;
         const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : first_seg) * D;
-        FirstRows<D, BF16, CALIB || WIDE> rows;
-        rows.load_table(prm.e0, (warp - 2) * (D / 16), lane);
+        BuildB<D, BF16, CALIB || WIDE, kEpiWarps> rows;
+        rows.load(prm.e0, 0, warp - 2, lane);
         grid_wait();
-        rows.load_lambda(lam, (warp - 2) * (D / 16));
         first_lift = lift_of<D>(lam, prm.table_max, lane);
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        rows.build(sB, first_lift, (warp - 2) * (D / 16), lane);
+        rows.store(sB, lam, first_lift, 0, warp - 2, lane);
+        rows.rest(sB, prm.e0, lam, first_lift, warp - 2, lane);
         fence_proxy_async();   // B is read by the tensor core through the async proxy
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
@@ -326,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 1) {
         // =========================== mma issuer ===========================
-        if (lane == 0) {
+        if (elect_one()) {
             // A limit shortened by the host (kvq_plan_set_wait_limit) is spent here, straight after the set-up barrier, when
             // the builders have only just begun to store: this thread has issued nothing yet and can leave at once.
             bool first_ok = true;
@@ -362,7 +368,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int ks = 0; ks < C::kKSteps; ++ks) {
                         // (bytes >> 4) of K-step ks inside the x tile and inside a split term
                         const uint32_t a_off = (uint32_t)(ks >> 2) * (kBlockBytes >> 4) + (uint32_t)(ks & 3) * 2u;
-                        const uint32_t b_off = (uint32_t)t * (C::kBTerm >> 4) + (uint32_t)(ks >> 2) * (C::kBBlock >> 4) + (uint32_t)(ks & 3) * 2u;
+                        // the small terms first: their sums are then complete before anything large is in the accumulator
+                        const uint32_t b_off = (uint32_t)(C::kStack ? 0 : C::kSplit - 1 - t) * (C::kBTerm >> 4) + (uint32_t)(ks >> 2) * (C::kBBlock >> 4) + (uint32_t)(ks & 3) * 2u;
                         const uint64_t ad = ((uint64_t)a_hi << 32) | (uint64_t)(a_lo_s + a_off);
                         const uint64_t bd = ((uint64_t)b_hi << 32) | (uint64_t)(b_lo + b_off);
                         if (t > 0 || ks > 0) umma_f16_ss<true>(d_tmem, ad, bd, C::kIdesc);
@@ -412,11 +419,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : seg) * D;
                 const float lift = lift_of<D>(lam, prm.table_max, lane);
                 if (j > 0 && cur.first_of_segment()) {
-                    if (!wait_or_abort(smem_u32(&ctrl->acc_full[(j - 1) % kFullBars]), (uint32_t)((j - 1) / kFullBars) & 1u,
-                                       abort_flag, status, KVQ_DEV_MMA_TIMEOUT))
+                    if (!rebuild_b<D, BF16, CALIB || WIDE>(sB, prm.e0, lam, lift, bw, lane, smem_u32(&ctrl->acc_full[(j - 1) % kFullBars]),
+                                                           (uint32_t)((j - 1) / kFullBars) & 1u, abort_flag, status))
                         break;
-                    build_b_rows<D, BF16, CALIB || WIDE>(sB, prm.e0, lam, lift, bw * (D / 8), (bw + 1) * (D / 8), lane);
-                    fence_proxy_async();   // B is read by the tensor core through the async proxy
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_ready));
                 }

@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 1) {
         // =========================== mma issuer (leader) ===========================
-        if (rank == 0 && lane == 0) {
+        if (rank == 0 && elect_one()) {
             // Descriptors differ only in their 14-bit start-address field (bytes >> 4): one base per operand, one add per MMA.
             const uint64_t b_desc = smem_desc_sw128(smem_u32(sB));
             const uint64_t a_desc = smem_desc_sw128(smem_u32(sIn));
