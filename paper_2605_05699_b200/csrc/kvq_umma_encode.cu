@@ -11,16 +11,16 @@
 //                                             scales then differ from the fp64 evaluation, all at rounding ties;
 //                                             the calibration pass adds a third term)
 // every product x_n W_i[c, n] is exact in fp32, and the terms are summed in fp32: for D <= 128 the two terms are stacked
-// along N (one MMA of N = 2 D per K-step fills two halves of the accumulator, which the epilogue adds: an MMA
-// instruction costs about 117 cycles whatever N <= 128 it carries and 176 at N = 256, so half the instructions is
-// worth more than the flops); D = 160 and the three-term forms accumulate all terms in one accumulator.  A term costs as much energy as the same GEMM in a library (0.6 pJ per flop), and the kernel runs
-// at the board's power cap, so a term more is 20 % less throughput.  2^k lifts the small terms clear of fp16's subnormal range; the epilogue undoes it in
-// the scale computation, at no cost per element.
+// along N (one MMA of N = 2 D per K-step fills two halves of the accumulator, which the epilogue adds: x is then read from
+// shared memory once for both terms); D = 160 and the three-term forms accumulate all terms in one accumulator, the smallest
+// first, so that the small sums are complete before anything large is in it.  A term costs as much energy as the same GEMM in a
+// library (0.6 pJ per flop), and on long calls the kernel runs at the board's power cap, so a term more is 20 % less throughput.
+// 2^k lifts the small terms clear of fp16's subnormal range; the epilogue undoes it in the scale computation, at no cost per element.
 //
 //   warp 0        producer   one TMA tensor load per K block of 64 elements and tile of 128 vectors (128-byte
 //                            swizzle): x lands in shared memory in the tensor core's canonical K-major
 //                            layout, several tiles in flight, no thread touches it
-//   warp 1        mma        one thread issues D / 16 K-steps (per split term where the terms are not stacked) into
+//   warp 1        mma        one elected thread issues D / 16 K-steps (per split term where the terms are not stacked) into
 //                            one accumulator stage, then commits once: the epilogue reads it as "accumulator full", the producer as
 //                            "x stage free"
 //   warps 2-17    epilogue   two sets of eight warps on alternate tiles; thread = (row, half row).  Per group
@@ -72,9 +72,8 @@ struct Cfg {
     static constexpr int kXBytes = kKBlocks * kBlockBytes;      // one x tile
     // Two terms and D <= 128: the terms are STACKED along N, rows [0, D) of a K block the first term's, rows [D, 2 D) the
     // second's, and one MMA of N = 2 D computes x W_hi into accumulator columns [0, D) and x W_lo into [D, 2 D); the
-    // epilogue adds the two.  An MMA of M 128, N 128, K 16 costs about 120 cycles here, one of N = 256 about 176 (measured,
-    // both operands in shared memory, accumulating into one tile; the nominal rates are 68 and 135): the per-instruction
-    // overhead is paid once for both terms, and the x tile is read from shared memory once instead of twice.
+    // epilogue adds the two.  Alone on the SM an MMA of M 128, K 16 takes 64 cycles at N = 128 and 128 at N = 256, but at N = 128 it
+    // reads 8 KB of shared memory in those 64 cycles, all that there is, while x arrives by TMA; at N = 256 it is 12 KB in 128.
     static constexpr bool kStack = kSplit == 2 && D <= 128;
     static constexpr int kNmma = kStack ? 2 * D : D;            // N of one MMA
     static constexpr int kBBlock = kNmma * 128;                 // one K block of B: kNmma rows x 128 B
