@@ -593,9 +593,11 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const bool bf16 = dtype == KVQ_BF16;
     // A large block of a plan without a rotation: the tensor-core decode, reading and writing the window [pos0, pos0 + rows)
-    // of every stream's cache in place through a cache view (tiles of 128 rows per stream, so blocks of 64 rows and more;
+    // of every stream's cache in place through a cache view (tiles of 128 rows per stream, so blocks of 64 rows and more, and
+    // shorter ones where the call has no more tiles than the device has SMs: a tile's time is then all it takes, whatever part of
+    // the tile is used (64 streams x 17 rows, D = 256: 28.1 us with the register FFT, 21.0 so; 64 x 33, D = 128: 15.1 and 13.9);
     // the whole cache must fit 32-bit tensor-map coordinates).
-    if (!mv && plan->dec_impl != KVQ_IMPL_FFT && gemm_decode_ok(plan, bf16) && (rows >= 64 || plan->dec_impl == KVQ_IMPL_GEMM) &&
+    if (!mv && plan->dec_impl != KVQ_IMPL_FFT && gemm_decode_ok(plan, bf16) && (rows >= 64 || S <= 148 || plan->dec_impl == KVQ_IMPL_GEMM) &&
         S <= (((int64_t)1 << 31) - 1) / T_max) {
         GemmParams g;
         g.packed = packed_cache;

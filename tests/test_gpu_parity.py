@@ -445,6 +445,16 @@ def test_flush_block_fills_the_int4_and_the_dequantized_caches(D, dtype, S, T_ma
     plan.close()
 
 
+@pytest.mark.parametrize("D,dtype,S,T_max,spl,blocks", [
+    (256, "bf16", 128, 64, 40, (17, 33)), (128, "f16", 100, 90, 30, (25, 41)), (96, "bf16", 148, 70, 148, (20, 9)),
+    (64, "f16", 130, 40, 1, (33,)),
+    (160, "f16", 149, 60, 3, (20,)),   # one stream more than the rule takes: the register FFT
+])
+def test_flush_of_short_blocks_of_many_streams(D, dtype, S, T_max, spl, blocks):
+    """Blocks above the small-call limit and under 64 rows: one partly used tile per stream."""
+    test_flush_block_fills_the_int4_and_the_dequantized_caches(D, dtype, S, T_max, spl, blocks)
+
+
 @pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("group,nbits", [(G, 4), (0, 4), (G, 8)])
