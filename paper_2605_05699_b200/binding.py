@@ -122,12 +122,14 @@ def _check(status: int, where: str):
         raise KvqError(status, where)
 
 
+_DTYPE_CODES = {torch.float16: KVQ_F16, torch.bfloat16: KVQ_BF16}
+
+
 def _dtype_code(t: torch.Tensor) -> int:
-    if t.dtype == torch.float16:
-        return KVQ_F16
-    if t.dtype == torch.bfloat16:
-        return KVQ_BF16
-    raise TypeError("expected a float16 or bfloat16 tensor, got %s" % t.dtype)
+    code = _DTYPE_CODES.get(t.dtype)
+    if code is None:
+        raise TypeError("expected a float16 or bfloat16 tensor, got %s" % t.dtype)
+    return code
 
 
 def _dev(t: torch.Tensor, what: str) -> int:
@@ -149,27 +151,21 @@ def _stream(stream, device: torch.device = None) -> int:
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
-class _on_device:
-    """Makes ``device`` current for the call (a plan's tables live on the device of its first use) and restores the
-    previous one; costs one query when it already is current, which is the usual case."""
-    __slots__ = ("idx", "prev")
+_current_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
 
-    def __init__(self, device: torch.device):
-        self.idx = device.index
-        self.prev = -1
 
-    def __enter__(self):
-        if self.idx is not None:
-            cur = torch.cuda.current_device()
-            if cur != self.idx:
-                self.prev = cur
-                torch.cuda.set_device(self.idx)
-        return self
-
-    def __exit__(self, *exc):
-        if self.prev >= 0:
-            torch.cuda.set_device(self.prev)
-        return False
+def _call(fn, where: str, device: torch.device, *args) -> None:
+    """One compute call with ``device`` current (a plan's tables live on the device of its first use), the previous one restored
+    after it.  A small call's time is the host's: no context manager and one query where the device already is the current one,
+    which is the usual case."""
+    idx = device.index
+    if idx is None or idx == _current_device():
+        st = fn(*args)
+    else:
+        with torch.cuda.device(idx):
+            st = fn(*args)
+    if st != KVQ_OK:
+        raise KvqError(st, where)
 
 
 # ---- C entry points, same names ---------------------------------------------------------
@@ -242,7 +238,7 @@ def kvq_plan_prepare(plan: int, dtype: torch.dtype, device=None) -> None:
     current one), so that later calls with tensors of ``dtype`` allocate nothing and never block."""
     code = KVQ_F16 if dtype == torch.float16 else KVQ_BF16 if dtype == torch.bfloat16 else -1
     dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
-    with _on_device(dev):
+    with torch.cuda.device(dev):
         _check(lib().kvq_plan_prepare(plan, code), "kvq_plan_prepare")
 
 
@@ -259,10 +255,9 @@ def kvq_encode(plan: int, x: torch.Tensor, lam: torch.Tensor, packed: torch.Tens
     D = x.shape[-1]
     N = x.numel() // D
     n_lambda = lam.numel() // D
-    with _on_device(x.device):
-        _check(lib().kvq_encode(plan, _dev(x, "x"), _dtype_code(x), N, _dev(lam, "lambda"), n_lambda,
-                                rows_per_lambda, _dev(packed, "packed"), _dev(scales, "scales"), _stream(stream, x.device)),
-               "kvq_encode")
+    dev = x.device
+    _call((_lib or lib()).kvq_encode, "kvq_encode", dev, plan, _dev(x, "x"), _dtype_code(x), N, _dev(lam, "lambda"),
+          n_lambda, rows_per_lambda, _dev(packed, "packed"), _dev(scales, "scales"), _stream(stream, dev))
 
 
 def kvq_decode(plan: int, packed: torch.Tensor, scales: torch.Tensor, lam: torch.Tensor, out: torch.Tensor,
@@ -270,10 +265,9 @@ def kvq_decode(plan: int, packed: torch.Tensor, scales: torch.Tensor, lam: torch
     D = out.shape[-1]
     N = out.numel() // D
     n_lambda = lam.numel() // D
-    with _on_device(out.device):
-        _check(lib().kvq_decode(plan, _dev(packed, "packed"), _dev(scales, "scales"), N, _dev(lam, "lambda"),
-                                n_lambda, rows_per_lambda, _dev(out, "out"), _dtype_code(out), _stream(stream, out.device)),
-               "kvq_decode")
+    dev = out.device
+    _call((_lib or lib()).kvq_decode, "kvq_decode", dev, plan, _dev(packed, "packed"), _dev(scales, "scales"), N,
+          _dev(lam, "lambda"), n_lambda, rows_per_lambda, _dev(out, "out"), _dtype_code(out), _stream(stream, dev))
 
 
 def kvq_append(plan: int, x_new: torch.Tensor, lam: torch.Tensor, packed_cache: torch.Tensor,
@@ -282,11 +276,10 @@ def kvq_append(plan: int, x_new: torch.Tensor, lam: torch.Tensor, packed_cache: 
     S = x_new.numel() // D
     T_max = packed_cache.shape[-2]
     n_lambda = lam.numel() // D
-    with _on_device(x_new.device):
-        _check(lib().kvq_append(plan, _dev(x_new, "x_new"), _dtype_code(x_new), S, _dev(lam, "lambda"), n_lambda,
-                                streams_per_lambda, _dev(packed_cache, "packed_cache"),
-                                _dev(scales_cache, "scales_cache"), T_max, pos, _stream(stream, x_new.device)),
-               "kvq_append")
+    dev = x_new.device
+    _call((_lib or lib()).kvq_append, "kvq_append", dev, plan, _dev(x_new, "x_new"), _dtype_code(x_new), S,
+          _dev(lam, "lambda"), n_lambda, streams_per_lambda, _dev(packed_cache, "packed_cache"),
+          _dev(scales_cache, "scales_cache"), T_max, pos, _stream(stream, dev))
 
 
 def kvq_decode_static(plan: int, packed: torch.Tensor, scales: torch.Tensor, lam: torch.Tensor, out: torch.Tensor,
@@ -300,11 +293,10 @@ def kvq_decode_static(plan: int, packed: torch.Tensor, scales: torch.Tensor, lam
     N = out.numel() // D
     n_lambda = lam.numel() // D
     sw = None if status_word is None else _dev(status_word, "status_word")
-    with _on_device(out.device):
-        _check(lib().kvq_decode_static(plan, _dev(packed, "packed"), _dev(scales, "scales"), N, _dev(lam, "lambda"),
-                                       n_lambda, rows_per_lambda, _dev(out, "out"), _dtype_code(out), sw,
-                                       _stream(stream, out.device)),
-               "kvq_decode_static")
+    dev = out.device
+    _call((_lib or lib()).kvq_decode_static, "kvq_decode_static", dev, plan, _dev(packed, "packed"),
+          _dev(scales, "scales"), N, _dev(lam, "lambda"), n_lambda, rows_per_lambda, _dev(out, "out"),
+          _dtype_code(out), sw, _stream(stream, dev))
 
 
 def kvq_flush_block(plan: int, x_block: torch.Tensor, lam: torch.Tensor, packed_cache: torch.Tensor, scales_cache: torch.Tensor,
@@ -312,11 +304,11 @@ def kvq_flush_block(plan: int, x_block: torch.Tensor, lam: torch.Tensor, packed_
     S, rows, D = x_block.shape
     T_max = packed_cache.shape[-2]
     n_lambda = lam.numel() // D
-    with _on_device(x_block.device):
-        _check(lib().kvq_flush_block(plan, _dev(x_block, "x_block"), _dtype_code(x_block), S, rows, _dev(lam, "lambda"), n_lambda,
-                                     streams_per_lambda, _dev(packed_cache, "packed_cache"), _dev(scales_cache, "scales_cache"),
-                                     _dev(dq_cache, "dq_cache"), T_max, pos0, _stream(stream, x_block.device)),
-               "kvq_flush_block")
+    dev = x_block.device
+    _call((_lib or lib()).kvq_flush_block, "kvq_flush_block", dev, plan, _dev(x_block, "x_block"),
+          _dtype_code(x_block), S, rows, _dev(lam, "lambda"), n_lambda, streams_per_lambda,
+          _dev(packed_cache, "packed_cache"), _dev(scales_cache, "scales_cache"), _dev(dq_cache, "dq_cache"), T_max,
+          pos0, _stream(stream, dev))
 
 
 def _pos_word(pos_device: torch.Tensor):
@@ -332,11 +324,10 @@ def kvq_append_at(plan: int, x_new: torch.Tensor, lam: torch.Tensor, packed_cach
     S = x_new.numel() // D
     T_max = packed_cache.shape[-2]
     n_lambda = lam.numel() // D
-    with _on_device(x_new.device):
-        _check(lib().kvq_append_at(plan, _dev(x_new, "x_new"), _dtype_code(x_new), S, _dev(lam, "lambda"), n_lambda,
-                                   streams_per_lambda, _dev(packed_cache, "packed_cache"), _dev(scales_cache, "scales_cache"),
-                                   T_max, _pos_word(pos_device), _stream(stream, x_new.device)),
-               "kvq_append_at")
+    dev = x_new.device
+    _call((_lib or lib()).kvq_append_at, "kvq_append_at", dev, plan, _dev(x_new, "x_new"), _dtype_code(x_new), S,
+          _dev(lam, "lambda"), n_lambda, streams_per_lambda, _dev(packed_cache, "packed_cache"),
+          _dev(scales_cache, "scales_cache"), T_max, _pos_word(pos_device), _stream(stream, dev))
 
 
 def kvq_flush_block_at(plan: int, x_block: torch.Tensor, lam: torch.Tensor, packed_cache: torch.Tensor, scales_cache: torch.Tensor,
@@ -345,19 +336,19 @@ def kvq_flush_block_at(plan: int, x_block: torch.Tensor, lam: torch.Tensor, pack
     S, rows, D = x_block.shape
     T_max = packed_cache.shape[-2]
     n_lambda = lam.numel() // D
-    with _on_device(x_block.device):
-        _check(lib().kvq_flush_block_at(plan, _dev(x_block, "x_block"), _dtype_code(x_block), S, rows, _dev(lam, "lambda"), n_lambda,
-                                        streams_per_lambda, _dev(packed_cache, "packed_cache"), _dev(scales_cache, "scales_cache"),
-                                        _dev(dq_cache, "dq_cache"), T_max, _pos_word(pos0_device), _stream(stream, x_block.device)),
-               "kvq_flush_block_at")
+    dev = x_block.device
+    _call((_lib or lib()).kvq_flush_block_at, "kvq_flush_block_at", dev, plan, _dev(x_block, "x_block"),
+          _dtype_code(x_block), S, rows, _dev(lam, "lambda"), n_lambda, streams_per_lambda,
+          _dev(packed_cache, "packed_cache"), _dev(scales_cache, "scales_cache"), _dev(dq_cache, "dq_cache"), T_max,
+          _pos_word(pos0_device), _stream(stream, dev))
 
 
 def kvq_calibrate_lambda(plan: int, x: torch.Tensor, lambda_out: torch.Tensor, stream=None) -> None:
     D = x.shape[-1]
     N = x.numel() // D
-    with _on_device(x.device):
-        _check(lib().kvq_calibrate_lambda(plan, _dev(x, "x"), _dtype_code(x), N, _dev(lambda_out, "lambda_out"), _stream(stream, x.device)),
-               "kvq_calibrate_lambda")
+    dev = x.device
+    _call((_lib or lib()).kvq_calibrate_lambda, "kvq_calibrate_lambda", dev, plan, _dev(x, "x"), _dtype_code(x), N,
+          _dev(lambda_out, "lambda_out"), _stream(stream, dev))
 
 
 class Plan:
