@@ -287,7 +287,6 @@ __device__ __noinline__ bool rebuild_b(unsigned char *sB, Ctrl *ctrl, const floa
     using C = Cfg<D, BF16OUT, BITS, R2>;
     BuildB<D, BF16OUT, BITS, R2, 4> rows;
     rows.load(b0, 0, q, lane);
-    post_reciprocals<D>(ctrl->recip[grp], rl, lane);
     // Every MMA issued so far has read B: the commit of the previous tile (the other group's) covers them
     // all.  A parity wait can only tell a phase from its neighbours, and the other group may lag by more
     // than one of its tiles, so first wait for this group's own last tile (its barrier is at most one
@@ -299,6 +298,10 @@ __device__ __noinline__ bool rebuild_b(unsigned char *sB, Ctrl *ctrl, const floa
     if (!wait_or_abort(smem_u32(&ctrl->a_empty[(j - 1) % C::kABars]), (uint32_t)((j - 1) / C::kABars) & 1u, &ctrl->abort, status,
                        KVQ_DEV_MMA_TIMEOUT))
         return false;
+    // The reciprocals go to shared memory only now that nobody reads the ones before them: the MMAs of tile j - 2 were issued after
+    // all four warps of this group had arrived for it, done with what they built there, and those of any tile after the first
+    // build, by all sixteen warps, out of recip[0].
+    post_reciprocals<D>(ctrl->recip[grp], rl, lane);
     rows.store(sB, ctrl->recip[grp], 0, q, lane);
     rows.rest(sB, b0, ctrl->recip[grp], q, lane);
     fence_proxy_async();   // B is read by the tensor core through the async proxy

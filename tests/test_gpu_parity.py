@@ -218,6 +218,30 @@ def test_d256_encode_at_the_edges_of_a_cta_pair_tile(dtype, N, n_lambda, rpl):
     assert enc["mismatches"] <= max(2, int(1e-4 * N * 256))
 
 
+@pytest.mark.parametrize("D,dtype,nbits", [(64, "f16", 4), (96, "bf16", 4), (128, "f16", 4), (128, "bf16", 8), (160, "f16", 4), (160, "bf16", 4), (256, "f16", 4)])
+@pytest.mark.parametrize("rpl,n_lambda", [(104, 450), (200, 450), (504, 230)])
+def test_decode_under_lambda_rows_of_a_few_tiles_equals_one_call_per_row(D, dtype, nbits, rpl, n_lambda):
+    """Shares of several lambda rows of one, two or four tiles: a group rebuilds the operand again while other warps are behind it.
+    The same kernel on each lambda row alone builds it once per CTA; the rows must be equal bit for bit."""
+    N = rpl * n_lambda - 37
+    plan = kb.Plan(D, G, 23, nbits)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_AUTO, kb.KVQ_IMPL_GEMM)
+    lam = wl.make_lambda(n_lambda, D, 24).cuda()
+    packed, scales = plan.empty_packed(N), plan.empty_scales(N)
+    kb.kvq_encode(plan.handle, wl.make_vectors(N, D, dtype, "lognormal", 25).cuda(), lam, packed, scales, rpl)
+    want = torch.empty(N, D, dtype=wl.torch_dtype(dtype), device="cuda")
+    for i in range(n_lambda):
+        a, b = i * rpl, min(N, (i + 1) * rpl)
+        kb.kvq_decode(plan.handle, packed[a:b], scales[a:b], lam[i], want[a:b])
+    out = torch.empty_like(want)
+    for _ in range(20):
+        out.zero_()
+        kb.kvq_decode(plan.handle, packed, scales, lam, out, rpl)
+        assert torch.equal(out, want)
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    plan.close()
+
+
 # ---- static lambda calibration (Sec. 7.1): lambda_c = 1 / max over the calibration vectors of |SRFT(x)_c|
 
 @pytest.mark.parametrize("D,dtype", [(64, "f16"), (96, "f16"), (128, "f16"), (128, "bf16"), (160, "f16"), (256, "f16"), (256, "bf16")])
