@@ -55,7 +55,7 @@ __device__ __noinline__ void decode_rows_fp32(const GemmParams &g, const float *
                     q = (int)static_cast<signed char>(packed[row * D + c]);
                 }
                 const float sig = __half2float(__ushort_as_half(scales[g.per_vector ? row : row * G + (c >> 5)]));
-                u = __fdiv_rn((float)q * sig, fmaxf(__ldg(lam + c), 1e-6f));
+                u = __fdiv_rn((float)q * sig, fmaxf(load_input(lam + c), 1e-6f));
             }
             su[i] = u;
         }

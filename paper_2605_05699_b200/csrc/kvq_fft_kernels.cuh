@@ -321,7 +321,7 @@ __device__ __forceinline__ void fill_lambda(float *cache, const float *__restric
 {
 #pragma unroll
     for (int c = lane; c < D; c += 32) {
-        float l = __ldg(lam + lr * D + c);
+        float l = load_input(lam + lr * D + c);
         cache[c] = RECIP ? __frcp_rn(fmaxf(l, 1e-6f)) : l;
     }
 }
@@ -465,21 +465,21 @@ __global__ void __launch_bounds__(WARPS * 32) kvq_decode_fft_kernel(const __grid
             if constexpr ((G * 2) % 16 == 0) {
 #pragma unroll
                 for (int j = 0; j < G / 8; ++j) {
-                    uint4 q = __ldg(reinterpret_cast<const uint4 *>(sp) + j);
+                    uint4 q = load_input(reinterpret_cast<const uint4 *>(sp) + j);
                     sb[4 * j] = q.x, sb[4 * j + 1] = q.y, sb[4 * j + 2] = q.z, sb[4 * j + 3] = q.w;
                 }
             } else if constexpr ((G * 2) % 8 == 0) {
 #pragma unroll
                 for (int j = 0; j < G / 4; ++j) {
-                    uint2 q = __ldg(reinterpret_cast<const uint2 *>(sp) + j);
+                    uint2 q = load_input(reinterpret_cast<const uint2 *>(sp) + j);
                     sb[2 * j] = q.x, sb[2 * j + 1] = q.y;
                 }
             } else if constexpr ((G * 2) % 4 == 0) {
 #pragma unroll
-                for (int j = 0; j < G / 2; ++j) sb[j] = __ldg(reinterpret_cast<const uint32_t *>(sp) + j);
+                for (int j = 0; j < G / 2; ++j) sb[j] = load_input(reinterpret_cast<const uint32_t *>(sp) + j);
             } else {
 #pragma unroll
-                for (int j = 0; j < G; ++j) sb[j / 2] |= (uint32_t)__ldg(sp + j) << (16 * (j & 1));
+                for (int j = 0; j < G; ++j) sb[j / 2] |= (uint32_t)load_input(sp + j) << (16 * (j & 1));
             }
         }
     };

@@ -50,7 +50,7 @@ __device__ __forceinline__ bool resolve_out_map(const MatvecParams &prm, RowMap 
 {
     map = prm.out_map;
     if (prm.pos_dev) {
-        const int64_t p = __ldg(prm.pos_dev);
+        const int64_t p = load_input(prm.pos_dev);
         if (p < 0 || p > prm.pos_limit) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(prm.status, KVQ_DEV_POSITION);
             return false;
@@ -172,7 +172,7 @@ __device__ __forceinline__ void encode_batch(const MatvecParams &prm, const RowM
     for (int p = 0; p < P; ++p) {
         const int i = lane + 32 * p;
         lam4[p] = (r < prm.N && i < D / 4)
-                      ? __ldg(reinterpret_cast<const float4 *>(prm.lambda + lambda_row(r, prm.n_lambda, prm.rows_per_lambda) * D) + i)
+                      ? load_input(reinterpret_cast<const float4 *>(prm.lambda + lambda_row(r, prm.n_lambda, prm.rows_per_lambda) * D) + i)
                       : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
 
@@ -181,7 +181,7 @@ __device__ __forceinline__ void encode_batch(const MatvecParams &prm, const RowM
     for (int idx = threadIdx.x; idx < kV * (D / 2); idx += kWarps * 32) {
         const int v = idx / (D / 2), j = idx % (D / 2);
         const int64_t r = v0 + v;
-        const float2 f = widen2<BF16>(r < prm.N ? __ldg(x + r * (D / 2) + j) : 0u);
+        const float2 f = widen2<BF16>(r < prm.N ? load_input(x + r * (D / 2) + j) : 0u);
         xs[v * D + 2 * j] = f.x, xs[v * D + 2 * j + 1] = f.y;
     }
     __syncthreads();
@@ -328,16 +328,16 @@ __device__ __forceinline__ void decode_batch(const MatvecParams &prm, float4 (&t
             const int64_t irow = prm.in_map(r);
             int q[4];
             if (prm.bits == 4) {
-                const uint32_t w = __ldg(reinterpret_cast<const uint16_t *>(pk + irow * (D / 2) + 2 * i));
+                const uint32_t w = load_input(reinterpret_cast<const uint16_t *>(pk + irow * (D / 2) + 2 * i));
 #pragma unroll
                 for (int e = 0; e < 4; ++e) q[e] = (int)(((w >> (4 * e)) & 0xFu) ^ 8u) - 8;
             } else {
-                const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(pk + irow * D + 4 * i));
+                const uint32_t w = load_input(reinterpret_cast<const uint32_t *>(pk + irow * D + 4 * i));
 #pragma unroll
                 for (int e = 0; e < 4; ++e) q[e] = (int)(signed char)((w >> (8 * e)) & 0xFFu);
             }
-            const float sig = __half2float(__ushort_as_half(__ldg(scl + irow * G + (4 * i) / prm.group)));
-            const float4 l = __ldg(reinterpret_cast<const float4 *>(prm.lambda + lambda_row(r, prm.n_lambda, prm.rows_per_lambda) * D) + i);
+            const float sig = __half2float(__ushort_as_half(load_input(scl + irow * G + (4 * i) / prm.group)));
+            const float4 l = load_input(reinterpret_cast<const float4 *>(prm.lambda + lambda_row(r, prm.n_lambda, prm.rows_per_lambda) * D) + i);
             o.x = (float)q[0] * (sig * __frcp_rn(fmaxf(l.x, 1e-6f)));
             o.y = (float)q[1] * (sig * __frcp_rn(fmaxf(l.y, 1e-6f)));
             o.z = (float)q[2] * (sig * __frcp_rn(fmaxf(l.z, 1e-6f)));

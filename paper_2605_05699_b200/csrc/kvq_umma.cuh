@@ -256,7 +256,7 @@ struct RecipLambda {
             const int i = lane + 32 * p;
             r[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (i < D / 4) {
-                const float4 l = __ldg(reinterpret_cast<const float4 *>(lam) + i);
+                const float4 l = load_input(reinterpret_cast<const float4 *>(lam) + i);
                 r[p] = make_float4(__frcp_rn(fmaxf(l.x, 1e-6f)), __frcp_rn(fmaxf(l.y, 1e-6f)), __frcp_rn(fmaxf(l.z, 1e-6f)),
                                    __frcp_rn(fmaxf(l.w, 1e-6f)));
             }

@@ -246,18 +246,18 @@ template <int G>
 __device__ __forceinline__ void load_row_scales(const uint16_t *__restrict__ sp, uint32_t (&sb)[(G + 1) / 2])
 {
     if constexpr (G == 8) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(sp));
+        const uint4 v = load_input(reinterpret_cast<const uint4 *>(sp));
         sb[0] = v.x, sb[1] = v.y, sb[2] = v.z, sb[3] = v.w;
     } else if constexpr (G == 4) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(sp));
+        const uint2 v = load_input(reinterpret_cast<const uint2 *>(sp));
         sb[0] = v.x, sb[1] = v.y;
     } else if constexpr (G == 2) {
-        sb[0] = __ldg(reinterpret_cast<const uint32_t *>(sp));
+        sb[0] = load_input(reinterpret_cast<const uint32_t *>(sp));
     } else {   // rows of 6 or 10 bytes are only 2-byte aligned
 #pragma unroll
         for (int j = 0; j < (G + 1) / 2; ++j) sb[j] = 0;
 #pragma unroll
-        for (int j = 0; j < G; ++j) sb[j / 2] |= (uint32_t)__ldg(sp + j) << (16 * (j & 1));
+        for (int j = 0; j < G; ++j) sb[j / 2] |= (uint32_t)load_input(sp + j) << (16 * (j & 1));
     }
 }
 
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint16_t *scales = static_cast<const uint16_t *>(prm.g.scales);
             if (row < prm.phys_rows) {
                 if (prm.g.per_vector) {
-                    const uint32_t s1 = (uint32_t)__ldg(scales + row);
+                    const uint32_t s1 = (uint32_t)load_input(scales + row);
 #pragma unroll
                     for (int i = 0; i < (G + 1) / 2; ++i) sc_first[i] = s1 | (s1 << 16);
                 } else {
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int64_t row = prm.g.phys_row(ahead.seg, ahead.row_in_segment(), rpl) + r;
                 if (row < prm.phys_rows) {
                     if (prm.g.per_vector) {   // one scale per vector: the same value in every group's slot
-                        const uint32_t s1 = (uint32_t)__ldg(scales + row);
+                        const uint32_t s1 = (uint32_t)load_input(scales + row);
 #pragma unroll
                         for (int i = 0; i < (G + 1) / 2; ++i) sc_next[i] = s1 | (s1 << 16);
                     } else {

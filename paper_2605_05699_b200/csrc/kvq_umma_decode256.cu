@@ -210,10 +210,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
             if (row < prm.phys_rows) {
                 if (prm.g.per_vector) {
-                    const uint32_t s1 = (uint32_t)__ldg(static_cast<const uint16_t *>(prm.g.scales) + row);
+                    const uint32_t s1 = (uint32_t)load_input(static_cast<const uint16_t *>(prm.g.scales) + row);
                     sc_first = make_uint4(s1 | (s1 << 16), s1 | (s1 << 16), s1 | (s1 << 16), s1 | (s1 << 16));
                 } else {
-                    sc_first = __ldg(static_cast<const uint4 *>(prm.g.scales) + row);
+                    sc_first = load_input(static_cast<const uint4 *>(prm.g.scales) + row);
                 }
             }
         }
@@ -304,11 +304,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t row = prm.g.phys_row(ahead.seg, ahead.row_in_segment(), rpl) + r;
             if (row >= prm.phys_rows) return make_uint4(0u, 0u, 0u, 0u);
             if (prm.g.per_vector) {   // one scale per vector: the same value in every group's slot
-                const uint32_t s1 = (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(prm.g.scales) + row);
+                const uint32_t s1 = (uint32_t)load_input(reinterpret_cast<const uint16_t *>(prm.g.scales) + row);
                 const uint32_t s2 = s1 | (s1 << 16);
                 return make_uint4(s2, s2, s2, s2);
             }
-            return __ldg(scales + row);
+            return load_input(scales + row);
         };
         uint4 sc_next = sc_first;   // requested before the first B build
         for (int j = 0; j < n_my; ++j, cur.advance(1)) {

@@ -269,11 +269,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t row = ahead.seg * rpl + ahead.row_in_segment() + r;
             if (row >= N) return make_uint4(0u, 0u, 0u, 0u);
             if (prm.g.per_vector) {   // one scale per vector: the same value in every group's slot
-                const uint32_t s1 = (uint32_t)__ldg(reinterpret_cast<const uint16_t *>(prm.g.scales) + row);
+                const uint32_t s1 = (uint32_t)load_input(reinterpret_cast<const uint16_t *>(prm.g.scales) + row);
                 const uint32_t s2 = s1 | (s1 << 16);
                 return make_uint4(s2, s2, s2, s2);
             }
-            return __ldg(scales + row);
+            return load_input(scales + row);
         };
         uint4 sc_next = fetch_scales(grp);
         bool ok = true;

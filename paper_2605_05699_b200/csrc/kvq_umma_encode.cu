@@ -112,7 +112,7 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
     for (int p = 0; p < (D / 4 + 31) / 32; ++p) {
         const int i = lane + 32 * p;
         if (lam && i < D / 4) {
-            const float4 l = __ldg(reinterpret_cast<const float4 *>(lam) + i);
+            const float4 l = load_input(reinterpret_cast<const float4 *>(lam) + i);
             mx = fmaxf(mx, fmaxf(fmaxf(fabsf(l.x), fabsf(l.y)), fmaxf(fabsf(l.z), fabsf(l.w))));
         }
     }
@@ -168,7 +168,7 @@ struct BuildB {
 #pragma unroll
         for (int k = 0; k < kBatch; ++k) {
             const int f = quad(batch, k, w, lane);
-            fc[k] = lam ? (f < kTotal ? __ldg(lam + f / kQuads) * lift : 0.0f) : lift;
+            fc[k] = lam ? (f < kTotal ? load_input(lam + f / kQuads) * lift : 0.0f) : lift;
         }
 #pragma unroll
         for (int k = 0; k < kBatch; ++k) {

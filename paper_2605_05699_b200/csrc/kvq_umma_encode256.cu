@@ -97,7 +97,7 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
     for (int p = 0; p < (D / 4 + 31) / 32; ++p) {
         const int i = lane + 32 * p;
         if (lam && i < D / 4) {
-            const float4 l = __ldg(reinterpret_cast<const float4 *>(lam) + i);
+            const float4 l = load_input(reinterpret_cast<const float4 *>(lam) + i);
             mx = fmaxf(mx, fmaxf(fmaxf(fabsf(l.x), fabsf(l.y)), fmaxf(fabsf(l.z), fabsf(l.w))));
         }
     }
@@ -127,7 +127,7 @@ struct BuildRows {
         using C = Cfg<BF16, CALIB>;
         float f[kBuildRows];
 #pragma unroll
-        for (int k = 0; k < kBuildRows; ++k) f[k] = lam ? __ldg(lam + half * kHalfN + c0 + k) * lift : lift;
+        for (int k = 0; k < kBuildRows; ++k) f[k] = lam ? load_input(lam + half * kHalfN + c0 + k) * lift : lift;
 #pragma unroll
         for (int k = 0; k < kBuildRows; ++k) {
             const int c = c0 + k;

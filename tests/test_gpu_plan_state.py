@@ -145,3 +145,63 @@ def test_a_call_queued_behind_another_sees_all_that_it_wrote(D, dtype, group, nb
     del graph
     assert kb.kvq_plan_device_status(plan.handle) == 0
     plan.close()
+
+
+@pytest.mark.parametrize("D,dtype", [(64, "bf16"), (96, "f16"), (128, "f16"), (128, "bf16"), (160, "f16"), (256, "f16"), (256, "bf16")])
+@pytest.mark.parametrize("small", [False, True])
+def test_a_call_queued_behind_another_reads_the_lambda_and_the_rows_that_it_wrote(D, dtype, small):
+    """What a grid reads right behind its wait is written by the grid ahead: a calibration's lambda (new vectors, other values, each
+    turn; one turn with a channel so small that the decode takes its fp32 form), appended rows, their codes.  Small calls take
+    the matrix-vector kernels.  Queued without a wait, on a side stream and as a replayed graph, against one by one."""
+    N, S, T = (900, 300, 3) if small else (128 * 148 + 77, 1871, 10)
+    plan = kb.Plan(D, G, 5)
+    dt = wl.torch_dtype(dtype)
+    kb.kvq_plan_prepare(plan.handle, dt)
+    samples = [wl.make_vectors(2500, D, dtype, kind, 20 + i, device="cuda") for i, kind in enumerate(("lognormal", "gaussian", "k_outlier"))]
+    samples.append(torch.zeros_like(samples[0]))
+    samples[3][:, 0] = 60000.0                                     # |z_c| above 5000 on the cosine channels, 0 on the sine ones: lambda 1
+    xs = [wl.make_vectors(N, D, dtype, "k_outlier", 30 + i, device="cuda") for i in range(len(samples))]
+
+    def buffers():
+        z = lambda *shape, dtype: torch.zeros(*shape, dtype=dtype, device="cuda")
+        return [z(D, dtype=torch.float32), z(N, D // 2, dtype=torch.uint8), z(N, D // G, dtype=torch.float16), z(N, D, dtype=dt)]
+
+    def chain(b, wait):
+        lam, packed, scales, out = b
+        pc, sc = packed[:S * T].view(S, T, -1), scales[:S * T].view(S, T, -1)
+        for i, x in enumerate(xs):
+            kb.kvq_calibrate_lambda(plan.handle, samples[i], lam)
+            wait()
+            kb.kvq_encode(plan.handle, x, lam, packed, scales)
+            wait()
+            kb.kvq_decode(plan.handle, packed, scales, lam, out)
+            wait()
+            for pos in range(T):                                   # the decoded rows go back in, one per stream and call
+                kb.kvq_append(plan.handle, out[pos * S:(pos + 1) * S], lam, pc, sc, pos)
+                wait()
+                kb.kvq_decode(plan.handle, packed, scales, lam, out)
+                wait()
+
+    want = buffers()
+    chain(want, torch.cuda.synchronize)
+    same = lambda got: all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(got, want))
+    side = torch.cuda.Stream()
+    for _ in range(4):
+        got = buffers()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            chain(got, lambda: None)
+        torch.cuda.current_stream().wait_stream(side)
+        assert same(got)
+    got = buffers()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain(got, lambda: None)
+    for _ in range(3):
+        for b in got:
+            b.zero_()
+        graph.replay()
+        assert same(got)
+    del graph
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    plan.close()

@@ -30,3 +30,18 @@ def test_decode_rebuild_writes_its_reciprocals_after_both_waits():
     waits = [m.start() for m in re.finditer(r"wait_or_abort\(", b)]
     post = b.index("post_reciprocals")
     assert len(waits) == 2 and max(waits) < post < b.index("rows.store") < b.index("rows.rest")
+
+
+def test_non_coherent_loads_read_the_plans_tables_only():
+    """The grid ahead on the stream may still be writing x, lambda, codes, scales and positions when a kernel comes up: they are read
+    by load_input, behind grid_wait, and never by __ldg."""
+    tables = r"(b0|e0|table|brow)\b"
+    for name in sorted(os.listdir(CSRC)):
+        text = source(name)
+        for m in re.finditer(r"__ldg\(", text):
+            line = text[m.end():text.index("\n", m.end())]
+            assert re.match(r"(reinterpret_cast<const float4 \*>\()?\(?" + tables, line), "%s: __ldg(%s" % (name, line)
+        for kernel in re.finditer(r"__global__ void [^;{]*?(kvq_\w+_kernel)\(", text, re.S):
+            b = body(text, kernel.group(1) + "(")
+            if "load_input" in b:
+                assert 0 <= b.find("grid_wait()") < b.index("load_input"), "%s: %s reads an input before grid_wait" % (name, kernel.group(1))
