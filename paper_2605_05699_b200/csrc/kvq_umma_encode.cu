@@ -164,16 +164,10 @@ struct BuildB {
     }
     __device__ __forceinline__ void store(unsigned char *sB, const float *__restrict__ lam, float lift, int batch, int w, int lane) const
     {
-        float fc[kBatch];
-#pragma unroll
-        for (int k = 0; k < kBatch; ++k) {
-            const int f = quad(batch, k, w, lane);
-            fc[k] = lam ? (f < kTotal ? load_input(lam + f / kQuads) * lift : 0.0f) : lift;
-        }
 #pragma unroll
         for (int k = 0; k < kBatch; ++k) {
             const int f = quad(batch, k, w, lane), c = f / kQuads;
-            if (f < kTotal) build_b_quad<D, BF16, THREE>(sB, m[k], fc[k], c, f - c * kQuads);
+            if (f < kTotal) build_b_quad<D, BF16, THREE>(sB, m[k], lam ? load_input(lam + c) * lift : lift, c, f - c * kQuads);
         }
     }
     // batches from the second on, after store(0)
