@@ -139,6 +139,20 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar)
                  "h"((uint16_t)3)
                  : "memory");
 }
+// Both CTAs of a pair load block after block, in order, into the same ring of slots.  The leader's barrier of a slot counts the bytes
+// of both: its producer arms it for two loads together with its own.  Where the producers have stopped early, after leader and partner
+// blocks, the leader owes the barriers of the last `ring` blocks what follows, and each phase then ends when the
+// loads that are under way have landed.  (A producer is at most one ring ahead of the other: a slot is free once block u - ring is used.)
+struct PairDrain {
+    int leader, partner, ring;
+    __host__ __device__ __forceinline__ int end() const { return leader > partner ? leader : partner; }
+    __host__ __device__ __forceinline__ int begin() const { return end() > ring ? end() - ring : 0; }
+    __host__ __device__ __forceinline__ bool owes_arrival(int u) const { return u >= leader; }    // the partner's load alone: armed by nobody
+    __host__ __device__ __forceinline__ bool owes_bytes(int u) const { return u >= partner; }     // the leader's load alone: armed for two
+    __host__ __device__ __forceinline__ int slot(int u) const { return u % ring; }
+    __host__ __device__ __forceinline__ uint32_t parity(int u) const { return (uint32_t)(u / ring) & 1u; }
+};
+
 // TMA tensor load into this CTA's shared memory that completes on an mbarrier of the leader (a shared::cluster address)
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst_smem, const CUtensorMap *tm, int c0, int c1, uint32_t leader_bar)
 {

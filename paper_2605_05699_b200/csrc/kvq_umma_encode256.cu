@@ -81,8 +81,11 @@ struct Ctrl {
     uint64_t acc_full[kMaxAcc], acc_empty[kMaxAcc];
     uint64_t b_first, b_ready;
     uint64_t swap[4];           // one scale per vector: the warps that share 32 rows
+    uint64_t drain;             // after an abort: every MMA issued is complete
     uint32_t tmem_base;
     volatile uint32_t abort;
+    uint32_t mma_stopped;       // the mma role left its loop early (both CTAs' copies)
+    uint32_t issued[2];         // leader's copy: K blocks that each CTA's producer asked for
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 
@@ -199,7 +202,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(smem_u32(&ctrl->b_first), 2 * kEpiWarps);   // first B: all epilogue warps of both CTAs build it
         mbar_init(smem_u32(&ctrl->b_ready), 2 * kEpiWarps);   // later rebuilds
         for (int qq = 0; qq < 4; ++qq) mbar_init(smem_u32(&ctrl->swap[qq]), C::kParties);
+        mbar_init(smem_u32(&ctrl->drain), 1);
         ctrl->abort = 0u;
+        ctrl->mma_stopped = 0u;
         mbar_init_fence();
     }
     if (warp == 0) tmem_alloc_pair(smem_u32(&ctrl->tmem_base), kTmemCols);
@@ -239,6 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // =========================== producer ===========================
         if (lane == 0) {
             bool ok = true;
+            int issued = 0;
             TileCursor cur(tile_begin, tps), ahead(tile_begin, tps);
             ahead.advance(1);
             for (int j = 0; j < n_my && ok; ++j, cur.advance(1), ahead.advance(1)) {
@@ -257,8 +263,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (!ok) break;
                     if (rank == 0) mbar_arrive_expect_tx(smem_u32(&ctrl->in_full[s]), 2 * kBlockBytes);   // this CTA's block and the partner's
                     tma_load_2d_pair(smem_u32(sIn + s * kBlockBytes), &tm_x, 64 * kb, (int)row0, cluster_map(smem_u32(&ctrl->in_full[s]), 0));
+                    issued = u + 1;
                 }
             }
+            cluster_st_u32(cluster_map(smem_u32(&ctrl->issued[rank]), 0), (uint32_t)issued);
         }
     } else if (warp == 1) {
         // =========================== mma issuer (leader) ===========================
@@ -274,14 +282,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int j = 0; j < n_my && ok; ++j, cur.advance(1)) {
                 const int sc = j % kAccStages;
                 if (j == 0) {   // the epilogue warps build the first B while the first x blocks are in flight
-                    if (!wait_cluster_or_abort(smem_u32(&ctrl->b_first), 0u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
+                    ok = wait_cluster_or_abort(smem_u32(&ctrl->b_first), 0u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT);
                 } else if (!CALIB && prm.n_lambda > 1 && cur.first_of_segment()) {   // the epilogue warps rebuild B for this lambda row
-                    if (!wait_cluster_or_abort(smem_u32(&ctrl->b_ready), builds & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
+                    ok = wait_cluster_or_abort(smem_u32(&ctrl->b_ready), builds & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT);
                     ++builds;
                 }
-                if (!wait_cluster_or_abort(smem_u32(&ctrl->acc_empty[sc]), ((uint32_t)(j / kAccStages) & 1u) ^ 1u, abort_flag, status,
-                                           KVQ_DEV_SLOT_TIMEOUT))
-                    break;
+                ok = ok && wait_cluster_or_abort(smem_u32(&ctrl->acc_empty[sc]), ((uint32_t)(j / kAccStages) & 1u) ^ 1u, abort_flag, status,
+                                                 KVQ_DEV_SLOT_TIMEOUT);
+                if (!ok) break;
                 const uint32_t d_tmem = tmem_base + (uint32_t)sc * C::kAccCols;
                 constexpr int kPasses = C::kSmallFirst ? C::kSplit : 1;   // passes over the tile's blocks
 #pragma unroll
@@ -312,6 +320,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 if (ok) umma_commit_pair(smem_u32(&ctrl->acc_full[sc]));
+            }
+            if (!ok) {   // the abort flag is up: both CTAs take the drain below
+                umma_commit_pair(smem_u32(&ctrl->drain));
+                ctrl->mma_stopped = 1u;
+                cluster_st_u32(cluster_map(smem_u32(&ctrl->mma_stopped), 1), 1u);
             }
         }
     } else {
@@ -431,15 +444,34 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 
     grid_trigger();
-    if (*abort_flag) {
-        // tell the partner, and let loads and tensor-core work that were already issued drain
-        if (lane == 0) cluster_st_u32(cluster_map(smem_u32(const_cast<uint32_t *>(&ctrl->abort)), (uint32_t)(rank ^ 1)), 1u);
-        __nanosleep(200000);
-    }
+    __syncwarp();
+    if (lane == 0 && *abort_flag)   // tell the partner
+        cluster_st_u32(cluster_map(smem_u32(const_cast<uint32_t *>(&ctrl->abort)), (uint32_t)(rank ^ 1)), 1u);
     __syncwarp();
     tc_fence_before();
     cluster_sync_all();   // neither CTA leaves, or gives its tensor memory back, while the other may still use it
     tc_fence_after();
+    if (*abort_flag) {   // up in both CTAs or in neither: whoever raises it tells the other before the barrier
+        if (threadIdx.x == 0) {
+            // MMAs that were issued (they complete in order: after the last tile's, or the commit that the mma role left with, all
+            // are) and loads that are under way get a bounded time to end before shared and tensor memory go back.
+            if (ctrl->mma_stopped)
+                (void)mbar_wait_bounded(smem_u32(&ctrl->drain), 0u, 1u << 16);
+            else if (n_my > 0)
+                (void)mbar_wait_bounded(smem_u32(&ctrl->acc_full[(n_my - 1) % kAccStages]), (uint32_t)((n_my - 1) / kAccStages) & 1u, 1u << 16);
+            if (rank == 0) {
+                const PairDrain d{(int)ctrl->issued[0], (int)ctrl->issued[1], kRing};
+                for (int u = d.begin(); u < d.end(); ++u) {
+                    const uint32_t bar = smem_u32(&ctrl->in_full[d.slot(u)]);
+                    if (d.owes_arrival(u)) mbar_arrive_expect_tx(bar, kBlockBytes);
+                    if (d.owes_bytes(u)) mbar_complete_tx(bar, kBlockBytes);
+                    (void)mbar_wait_bounded(bar, d.parity(u), 1u << 16);
+                }
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();   // the partner stays until its loads, which arrive on the leader's barriers, have landed
+    }
     if (warp == 0) tmem_dealloc_pair(tmem_base, kTmemCols);
 }
 
