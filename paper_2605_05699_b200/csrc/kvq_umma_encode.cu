@@ -145,14 +145,19 @@ __device__ __forceinline__ void build_b_quad(unsigned char *sB, float4 m, float 
 
 // The B operand by W warps: the table's quads, row after row, dealt out to all their lanes, so that no lane idles where a row is not
 // a multiple of 32 quads, in batches of up to 16 that are requested together (load) and turned into B rows once the lift is
-// known and the old operand is free (store): one round trip to L2 per batch, the first one before the wait.
+// known and the old operand is free (store): one round trip to L2 per batch, the first one before the wait.  The lambda entries of a
+// batch are requested by one lane each (load_lambda, behind grid_wait) and handed round by shuffles: loads that cannot move across
+// the stores to shared memory cost 100 cycles a quad in their place (5120 vectors under 160 lambda rows, D = 128: 9.5 and 11.4 us).
 template <int D, bool BF16, bool THREE, int W>
 struct BuildB {
     static constexpr int kQuads = D / 4, kTotal = D * kQuads;
     static constexpr int kPerLane = (kTotal + 32 * W - 1) / (32 * W);
     static constexpr int kBatches = (kPerLane + 15) / 16;
     static constexpr int kBatch = (kPerLane + kBatches - 1) / kBatches;
+    static constexpr int kRowsPerPass = (31 + kQuads - 1) / kQuads + 1;   // table rows that 32 neighbouring quads can touch
+    static_assert(kBatch * kRowsPerPass <= 32, "a lane per lambda entry of a batch");
     float4 m[kBatch];
+    float l;   // lane k kRowsPerPass + d: lambda of the d-th table row of pass k
     static __device__ __forceinline__ int quad(int batch, int k, int w, int lane) { return ((batch * kBatch + k) * W + w) * 32 + lane; }
     __device__ __forceinline__ void load(const float *__restrict__ e0, int batch, int w, int lane)
     {
@@ -162,12 +167,19 @@ struct BuildB {
             m[k] = f < kTotal ? __ldg(reinterpret_cast<const float4 *>(e0) + f) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
     }
-    __device__ __forceinline__ void store(unsigned char *sB, const float *__restrict__ lam, float lift, int batch, int w, int lane) const
+    __device__ __forceinline__ void load_lambda(const float *__restrict__ lam, int batch, int w, int lane)
     {
+        const int k = lane / kRowsPerPass, c = quad(batch, k, w, 0) / kQuads + lane % kRowsPerPass;
+        l = lam && k < kBatch && c < D ? load_input(lam + c) : 1.0f;
+    }
+    __device__ __forceinline__ void store(unsigned char *sB, float lift, int batch, int w, int lane) const
+    {
+        const float lifted = l * lift;
 #pragma unroll
         for (int k = 0; k < kBatch; ++k) {
             const int f = quad(batch, k, w, lane), c = f / kQuads;
-            if (f < kTotal) build_b_quad<D, BF16, THREE>(sB, m[k], lam ? load_input(lam + c) * lift : lift, c, f - c * kQuads);
+            const float lc = __shfl_sync(0xFFFFFFFFu, lifted, k * kRowsPerPass + c - quad(batch, k, w, 0) / kQuads);
+            if (f < kTotal) build_b_quad<D, BF16, THREE>(sB, m[k], lc, c, f - c * kQuads);
         }
     }
     // batches from the second on, after store(0)
@@ -176,7 +188,8 @@ struct BuildB {
 #pragma unroll
         for (int b = 1; b < kBatches; ++b) {
             load(e0, b, w, lane);
-            store(sB, lam, lift, b, w, lane);
+            load_lambda(lam, b, w, lane);
+            store(sB, lift, b, w, lane);
         }
     }
 };
@@ -201,8 +214,9 @@ __device__ __noinline__ bool rebuild_b(unsigned char *sB, const float *__restric
 {
     BuildB<D, BF16, THREE, kEpiWarps / 2> rows;
     rows.load(e0, 0, w, lane);
+    rows.load_lambda(lam, 0, w, lane);
     if (!wait_or_abort(full_bar, parity, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) return false;
-    rows.store(sB, lam, lift, 0, w, lane);
+    rows.store(sB, lift, 0, w, lane);
     rows.rest(sB, e0, lam, lift, w, lane);
     fence_proxy_async();   // B is read by the tensor core through the async proxy
     return true;
@@ -272,12 +286,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         BuildB<D, BF16, CALIB || WIDE, kEpiWarps> rows;
         rows.load(prm.e0, 0, warp - 2, lane);
         grid_wait();
+        rows.load_lambda(lam, 0, warp - 2, lane);
         first_lift = lift_of<D>(lam, prm.table_max, lane);
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        rows.store(sB, lam, first_lift, 0, warp - 2, lane);
+        rows.store(sB, first_lift, 0, warp - 2, lane);
         rows.rest(sB, prm.e0, lam, first_lift, warp - 2, lane);
         fence_proxy_async();   // B is read by the tensor core through the async proxy
         __syncwarp();

@@ -118,6 +118,7 @@ constexpr int kBuildRows = 8;
 template <bool BF16, bool CALIB>
 struct BuildRows {
     float4 m[kBuildRows][2];
+    float l;   // lane k: lambda of row c0 + k (load_lambda, behind grid_wait)
     __device__ __forceinline__ void load(const float *__restrict__ e0, int half, int c0, int lane)
     {
 #pragma unroll
@@ -125,19 +126,22 @@ struct BuildRows {
 #pragma unroll
             for (int p = 0; p < 2; ++p) m[k][p] = __ldg(reinterpret_cast<const float4 *>(e0 + (size_t)(half * kHalfN + c0 + k) * kD) + lane + 32 * p);
     }
-    __device__ __forceinline__ void store(unsigned char *sB, const float *__restrict__ lam, float lift, int half, int c0, int lane) const
+    __device__ __forceinline__ void load_lambda(const float *__restrict__ lam, int half, int c0, int lane)
+    {
+        l = lam ? load_input(lam + half * kHalfN + c0 + lane % kBuildRows) : 1.0f;
+    }
+    __device__ __forceinline__ void store(unsigned char *sB, float lift, int c0, int lane) const
     {
         using C = Cfg<BF16, CALIB>;
-        float f[kBuildRows];
-#pragma unroll
-        for (int k = 0; k < kBuildRows; ++k) f[k] = lam ? load_input(lam + half * kHalfN + c0 + k) * lift : lift;
+        const float lifted = l * lift;
 #pragma unroll
         for (int k = 0; k < kBuildRows; ++k) {
             const int c = c0 + k;
+            const float f = __shfl_sync(0xFFFFFFFFu, lifted, k);
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 const int i = lane + 32 * p;
-                float w[4] = {m[k][p].x * f[k], m[k][p].y * f[k], m[k][p].z * f[k], m[k][p].w * f[k]};
+                float w[4] = {m[k][p].x * f, m[k][p].y * f, m[k][p].z * f, m[k][p].w * f};
                 const int ch = i >> 1;   // 16-byte chunk of the K-major row: K block ch / 8, chunk ch % 8
                 const uint32_t off = (uint32_t)((ch >> 3) * kBBlock + c * 128 + (((ch & 7) ^ (c & 7)) << 4) + ((i & 1) ? 8 : 0));
 #pragma unroll
@@ -222,11 +226,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         BuildRows<BF16, CALIB> rows;
         rows.load(prm.e0, rank, (warp - 2) * 8, lane);
         grid_wait();
+        rows.load_lambda(lam, rank, (warp - 2) * 8, lane);
         first_lift = lift_of<kD>(lam, prm.table_max, lane);
         tc_fence_before();
         cluster_sync_all();   // both CTAs' barriers exist and both have their tensor memory
         tc_fence_after();
-        rows.store(sB, lam, first_lift, rank, (warp - 2) * 8, lane);
+        rows.store(sB, first_lift, (warp - 2) * 8, lane);
         fence_proxy_async();   // B is read by the tensor core through the async proxy
         __syncwarp();
         if (lane == 0) cluster_mbar_arrive(cluster_map(smem_u32(&ctrl->b_first), 0));
@@ -359,9 +364,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float *lam = prm.lambda + (seg + 1) * kD;
                 BuildRows<BF16, CALIB> rows;
                 rows.load(prm.e0, rank, (warp - 2) * 8, lane);
+                rows.load_lambda(lam, rank, (warp - 2) * 8, lane);
                 lift_next = lift_of<kD>(lam, prm.table_max, lane);
                 if (!wait_or_abort(smem_u32(&ctrl->acc_full[sc]), (uint32_t)(j / kAccStages) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
-                rows.store(sB, lam, lift_next, rank, (warp - 2) * 8, lane);
+                rows.store(sB, lift_next, (warp - 2) * 8, lane);
                 fence_proxy_async();   // B is read by the tensor core through the async proxy
                 __syncwarp();
                 if (lane == 0) cluster_mbar_arrive(cluster_map(smem_u32(&ctrl->b_ready), 0));
