@@ -593,11 +593,11 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const bool bf16 = dtype == KVQ_BF16;
     // A large block of a plan without a rotation: the tensor-core decode, reading and writing the window [pos0, pos0 + rows)
-    // of every stream's cache in place through a cache view (tiles of 128 rows per stream, so blocks of 64 rows and more, and
-    // shorter ones where the call has no more tiles than the device has SMs: a tile's time is then all it takes, whatever part of
-    // the tile is used (64 streams x 17 rows, D = 256: 28.1 us with the register FFT, 21.0 so; 64 x 33, D = 128: 15.1 and 13.9);
-    // the whole cache must fit 32-bit tensor-map coordinates).
-    if (!mv && plan->dec_impl != KVQ_IMPL_FFT && gemm_decode_ok(plan, bf16) && (rows >= 64 || S <= 148 || plan->dec_impl == KVQ_IMPL_GEMM) &&
+    // of every stream's cache in place through a cache view (tiles of 128 rows per stream, so blocks of 64 rows and more; the whole
+    // cache must fit 32-bit tensor-map coordinates).  Shorter blocks stay in fp32: the tensor cores take 64 x 17 rows at D = 256 in
+    // 21.0 us instead of 28.1, but with operands of 16 bits (fp16 output: relative error 3.4e-4 instead of the output rounding's
+    // 2.1e-4; bf16: two to four times as many outputs off their correct rounding, 1.0e-3 of them at D = 128 instead of 3.8e-4).
+    if (!mv && plan->dec_impl != KVQ_IMPL_FFT && gemm_decode_ok(plan, bf16) && (rows >= 64 || plan->dec_impl == KVQ_IMPL_GEMM) &&
         S <= (((int64_t)1 << 31) - 1) / T_max) {
         GemmParams g;
         g.packed = packed_cache;

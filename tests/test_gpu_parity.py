@@ -472,11 +472,33 @@ def test_flush_block_fills_the_int4_and_the_dequantized_caches(D, dtype, S, T_ma
 @pytest.mark.parametrize("D,dtype,S,T_max,spl,blocks", [
     (256, "bf16", 128, 64, 40, (17, 33)), (128, "f16", 100, 90, 30, (25, 41)), (96, "bf16", 148, 70, 148, (20, 9)),
     (64, "f16", 130, 40, 1, (33,)),
-    (160, "f16", 149, 60, 3, (20,)),   # one stream more than the rule takes: the register FFT
+    (160, "f16", 149, 60, 3, (20,)),
 ])
 def test_flush_of_short_blocks_of_many_streams(D, dtype, S, T_max, spl, blocks):
-    """Blocks above the small-call limit and under 64 rows: one partly used tile per stream."""
+    """Blocks above the small-call limit and under 64 rows: the register FFT."""
     test_flush_block_fills_the_int4_and_the_dequantized_caches(D, dtype, S, T_max, spl, blocks)
+
+
+@pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+def test_flush_of_short_blocks_dequantizes_in_fp32(D, dtype):
+    """Blocks above the small-call limit and under 64 rows keep 32-bit operands: bit for bit what the register FFT gives, however many
+    streams there are."""
+    rows = 41
+    lam = wl.make_lambda(2, D, 92).cuda()
+    for S in (60, 148, 149):
+        x = wl.make_vectors(S * rows, D, dtype, "gaussian", 93).view(S, rows, D).cuda()
+        got = []
+        for impl in (kb.KVQ_IMPL_AUTO, kb.KVQ_IMPL_FFT):
+            plan = kb.Plan(D, G, 91)
+            kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_AUTO, impl)
+            packed = torch.zeros(S, rows, D // 2, dtype=torch.uint8, device="cuda")
+            scales = torch.zeros(S, rows, D // G, dtype=torch.float16, device="cuda")
+            got.append(torch.zeros(S, rows, D, dtype=wl.torch_dtype(dtype), device="cuda"))
+            kb.kvq_flush_block(plan.handle, x, lam, packed, scales, got[-1], 0, (S + 1) // 2)
+            torch.cuda.synchronize()
+            plan.close()
+        assert torch.equal(got[0], got[1]), S
 
 
 @pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
