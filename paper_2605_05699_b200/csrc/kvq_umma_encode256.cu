@@ -10,16 +10,17 @@
 // What bounds it: 32 MMAs of 128 cycles per tile (2.1 us per 128 vectors and SM at 1965 MHz; the bytes take 1.9), and, back to
 // back, the board's power limit.  The form before this one gave each CTA 128 channels of the same 128 vectors: every x block was
 // fetched by both CTAs, the ring beside B held less than the latency of its loads, and both split terms were added up in the
-// epilogue.  Before -> now, back to back: 212,992 bf16 vectors under 52 lambda rows 62.4 -> 58.6 us, 1,064,960 under one
-// 287 -> 266, one scale per vector 73.8 -> 64.0, calibration of 200,000 fp16 vectors 65.0 -> 51.9, 9000 vectors 10.3 -> 9.5.
-// Between 38,000 and 60,000 vectors, where a pair's three or four tall tiles take the place of five to seven, 5 to 9 % slower.
+// epilogue.  Before -> now, back to back, both on one box (which vary by 5 %): 212,992 bf16 vectors under 52 lambda rows 63.7 -> 58.6 us,
+// under one 59.6 -> 54.1, one scale per vector 69.7 -> 55.8; 9000 fp16 vectors 10.3 -> 9.7, 24,000: 14.4 -> 13.2, 42,000: 17.7 -> 17.0;
+// 300 lambda rows of 300 vectors 47.1 -> 43.8.  Slower by 2 to 3 % where the last of many tall tiles is nearly
+// empty (95,000 fp16 vectors 28.1 -> 28.8; 52 x 2048 31.6 -> 32.5).
 //
 //   warp 0        producer   (both CTAs) one TMA tensor load per K block of 64 columns into a ring of blocks; the
 //                            loads of both CTAs complete on the leader's barrier
 //   warp 1        mma        (leader) per tile every K step of the small term first, then of the large one: the small sums are
 //                            then added up before anything large is in the accumulator, so that each rounding of the fp32
 //                            accumulator is counted once per K step of the large term alone.  A block is released
-//                            in the second pass.  (Three terms: block by block, all terms; the ring holds two blocks.)
+//                            in the second pass.  (Three terms: block by block, all terms; the ring holds one tile.)
 //   warps 2-17    epilogue   (both CTAs) all sixteen warps on every tile, thread = (row, two of the row's eight groups, or one)
 //
 // Byte codes (fp16 input) are a run-time switch of the epilogue.  Every wait is bounded.
@@ -46,13 +47,10 @@ constexpr int kBBlock = kHalfN * 128;      // one K block of one term of B: 128 
 constexpr int kBTerm = kKBlocks * kBBlock; // one split term of B: 128 rows x K = 256, 64 KB
 constexpr int kMaxRing = 12;
 constexpr int kMaxAcc = 4;
-constexpr int64_t kShortTiles = 74;        // tiles of 128 vectors up to which a tile has 64 vectors per CTA: one per pair of SMs
 
 // CALIB: the calibration pass keeps a third bf16 term (it runs once; its result is compared at 1e-6 of the vector norm)
 // PERVEC: one scale per vector: the four threads of a row trade their maxima through shared memory
-// ROWS: vectors per CTA and tile; a pair's tile has twice as many = MMA M.  128, or 64 where a call has no more than one tile of
-// 128 vectors per pair: its MMAs cost 1.3 us per tile instead of 2.1 and twice as many SMs take part (9000 vectors: 11.1 -> 9.5 us;
-// on long calls they are the dearer ones, 62 -> 71 us at 212,992 vectors).
+// ROWS: vectors per CTA and tile; a pair's tile has twice as many = MMA M.  128, or 64 where that ends earlier (short_is_faster).
 template <bool BF16, bool CALIB = false, bool PERVEC = false, int ROWS = 128>
 struct Cfg {
     static_assert(ROWS == 64 || ROWS == 128, "tile heights");
@@ -68,7 +66,7 @@ struct Cfg {
     static constexpr int kMaxBytes = PERVEC ? 2 * kParties * ROWS * (int)sizeof(float) : 0;   // one scale per vector: [tile parity][party][row]
     static constexpr int kRoom = (kSmemLimit - 1024 - kCtrlBytes - kMaxBytes - kBBytes) / kBlockBytes;
     static constexpr int kWant = 6 * 128 / ROWS;
-    static constexpr int kRing = kRoom < kWant ? kRoom : kWant;   // K blocks of x in flight: 6 (12 short ones), one less with kMaxBytes, 2 beside three terms
+    static constexpr int kRing = kRoom < kWant ? kRoom : kWant;   // K blocks of x in flight: 6 (12 short ones), one less with kMaxBytes, 4 short ones beside three terms
     static_assert(kRing >= 2, "no room for the x ring");
     static constexpr bool kSmallFirst = kRing > kKBlocks;   // a whole tile stays in the ring for two passes over it
     static constexpr int kSmemBytes = kBBytes + kRing * kBlockBytes + kCtrlBytes + kMaxBytes + 1024;
@@ -486,8 +484,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ------------------------------------------------------------------------------------------------
 namespace {
 
+// Sets the kernel's launch attributes; fit: pairs resident at once (the SMs of a cluster share a GPC).  Looked up once per device.
 template <bool BF16, bool CALIB, bool PERVEC, int ROWS>
-cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t stream, uint32_t *amax_bits = nullptr)
+cudaError_t resident_pairs(int *fit)
 {
     using C = Cfg<BF16, CALIB, PERVEC, ROWS>;
     auto kern = kvq_encode_umma_d256_kernel<BF16, CALIB, PERVEC, ROWS>;
@@ -495,8 +494,7 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     int dev = 0;
     cudaError_t e = current_device_slot(&dev);
     if (e != cudaSuccess) return e;
-    int &fit = slots.sms[dev];   // pairs resident at once (the SMs of a cluster share a GPC), looked up once per device
-    if (fit == 0) {
+    if (slots.sms[dev] == 0) {
         int n = 0;
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -505,7 +503,6 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
         cfg.gridDim = dim3((unsigned)(n & ~1), 1, 1);
         cfg.blockDim = dim3(kThreads, 1, 1);
         cfg.dynamicSmemBytes = C::kSmemBytes;
-        cfg.stream = stream;
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 2;
         attr[0].val.clusterDim.y = 1;
@@ -514,8 +511,35 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
         cfg.numAttrs = 1;
         if ((e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg)) != cudaSuccess) return e;
         if (n < 1) return cudaErrorLaunchOutOfResources;
-        fit = n;
+        slots.sms[dev] = n;
     }
+    *fit = slots.sms[dev];
+    return cudaSuccess;
+}
+
+int64_t tiles_of(int64_t n_seg, int64_t rpl, int rows) { return n_seg * ((rpl + rows - 1) / rows); }
+
+// A pair's time is 7.1 us and 1.93 us per short tile (128 vectors), or 8.3 and 2.97 per tall one (256): short where
+// 2 n_short <= 3 n_tall + 1.  Back to back, fp16, short and tall: 9000 vectors 9.6 and 11.2 us, 18,944: 11.6, 12.1; 24,000: 13.0, 14.5;
+// 36,000: 15.0, 14.6; 46,000: 17.0, 17.3; 54,000: 18.9, 17.4; 212,992: 62.4, 53.5.  bf16 and one scale per vector lie alike.
+// Calibration from fp16: 9000 vectors 14.6 and 16.4, 57,000: 22.9, 26.6; 170,000: 41.9, 43.0; 200,000: 52.2, 49.9; 500,000: 116, 105.
+// (From bf16 its three terms leave a tall tile two x blocks beside B, and short ones are as fast or faster throughout: 9000 vectors 16.5
+// and 20.5, 57,000: 26.7, 30.8; 212,992: 63.9, 66.0; 500,000: 146.5, 145.1.  The tall form is not built.)
+template <bool CALIB>
+bool short_is_faster(int64_t n_seg, int64_t rpl, int fit)
+{
+    const int64_t n_short = (tiles_of(n_seg, rpl, 128) + fit - 1) / fit, n_tall = (tiles_of(n_seg, rpl, 256) + fit - 1) / fit;
+    if (CALIB) return n_short <= 18;
+    return 2 * n_short <= 3 * n_tall + 1;
+}
+
+template <bool BF16, bool CALIB, bool PERVEC, int ROWS>
+cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t stream, uint32_t *amax_bits)
+{
+    using C = Cfg<BF16, CALIB, PERVEC, ROWS>;
+    int fit = 0;
+    const cudaError_t e = resident_pairs<BF16, CALIB, PERVEC, ROWS>(&fit);
+    if (e != cudaSuccess) return e;
     if (N == 0) return cudaSuccess;   // kvq_plan_prepare: the launch attributes are set, there is nothing to run
     if (N >= (int64_t)1 << 31) return cudaErrorInvalidValue;   // tensor-map coordinates are 32-bit
 
@@ -543,23 +567,28 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
                          CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
 
-    const int64_t tiles = prm.n_seg * ((prm.rpl + 2 * ROWS - 1) / (2 * ROWS));
+    const int64_t tiles = tiles_of(prm.n_seg, prm.rpl, 2 * ROWS);
     const unsigned pairs = (unsigned)(tiles < fit ? tiles : fit);
-    return launch_kernel(kern, 2 * pairs, kThreads, C::kSmemBytes, stream, 2, prm, tm_x);
+    return launch_kernel(kvq_encode_umma_d256_kernel<BF16, CALIB, PERVEC, ROWS>, 2 * pairs, kThreads, C::kSmemBytes, stream, 2, prm, tm_x);
 }
 
-// The tile height: 64 vectors per CTA where that gives no pair more than one tile.
 template <bool BF16, bool CALIB, bool PERVEC>
 cudaError_t launch_any(int64_t N, const FftParams &f, const float *e0, cudaStream_t stream, uint32_t *amax_bits = nullptr)
 {
-    if (N == 0) {   // kvq_plan_prepare: both heights
-        const cudaError_t e = launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits);
-        return e != cudaSuccess ? e : launch<BF16, CALIB, PERVEC, 128>(N, f, e0, stream, amax_bits);
+    if constexpr (BF16 && CALIB) {
+        return launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits);
+    } else {
+        if (N == 0) {   // kvq_plan_prepare: both heights
+            const cudaError_t e = launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits);
+            return e != cudaSuccess ? e : launch<BF16, CALIB, PERVEC, 128>(N, f, e0, stream, amax_bits);
+        }
+        const int64_t rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
+        int fit = 0;
+        const cudaError_t e = resident_pairs<BF16, CALIB, PERVEC, 128>(&fit);
+        if (e != cudaSuccess) return e;
+        return short_is_faster<CALIB>((N + rpl - 1) / rpl, rpl, fit) ? launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits)
+                                                                     : launch<BF16, CALIB, PERVEC, 128>(N, f, e0, stream, amax_bits);
     }
-    const int64_t rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
-    const int64_t tiles = (N + rpl - 1) / rpl * ((rpl + 127) / 128);
-    return tiles <= kShortTiles ? launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits)
-                                : launch<BF16, CALIB, PERVEC, 128>(N, f, e0, stream, amax_bits);
 }
 
 }  // namespace

@@ -208,11 +208,20 @@ def test_gemm_kernels_d256(dtype, N, n_lambda, rpl, kind):
 
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("N,n_lambda,rpl", [(3 * 74 * 128, 1, 0), (3 * 74 * 128 + 1, 1, 0), (3 * 74 * 128 + 129, 1, 0), (38001, 1, 0),
+                                            (30000, 2, 15000), (30720, 60, 512), (76800, 150, 512)])
+def test_d256_encode_where_the_tile_height_changes(dtype, N, n_lambda, rpl):
+    """74 pairs: three short tiles each, then two tall ones, then five short ones; tall tiles under many lambda rows, one or several per share."""
+    enc, _ = run_case(256, dtype, N, "k_outlier", 4500 + N, n_lambda=n_lambda, rows_per_lambda=rpl, enc_impl="gemm")
+    assert enc["mismatches"] <= max(2, int(1e-4 * N * 256))
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("N,n_lambda,rpl", [(63, 1, 0), (65, 1, 0), (129, 1, 0), (74 * 128, 1, 0), (74 * 128 + 1, 1, 0), (640, 5, 128),
                                             (770, 3, 257), (19200, 75, 256), (19300, 76, 257), (58001, 4, 15001)])
 def test_d256_encode_at_the_edges_of_a_cta_pair_tile(dtype, N, n_lambda, rpl):
-    """128 vectors per tile, 64 per CTA, up to 74 tiles, then 256 and 128: tiles that end in the first CTA's half, at its end, one
-    row into the second's; the last size of the short tiles and the first of the tall ones; a new lambda row at every tile, and
+    """128 vectors per tile, 64 per CTA, or 256 and 128: tiles that end in the first CTA's half, at its end, one
+    row into the second's; one and two short tiles per pair; a new lambda row at every tile, and
     inside a pair's share."""
     enc, _ = run_case(256, dtype, N, "k_outlier", 4400 + N, n_lambda=n_lambda, rows_per_lambda=rpl, enc_impl="gemm")
     assert enc["mismatches"] <= max(2, int(1e-4 * N * 256))
