@@ -124,8 +124,7 @@ void count_launch();
 
 // Launches a kernel that takes grid_trigger() / grid_wait() (kvq_device.cuh): its blocks may be brought up, its barriers set up
 // and its table rows requested, while the previous kernel of the stream runs out.  cluster: CTAs per thread-block cluster.
-// overlap = false: an ordinary launch, for kernels whose CTAs gain from starting together.
-template <bool overlap = true, class... P, class... A>
+template <class... P, class... A>
 cudaError_t launch_kernel(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream, unsigned cluster,
                           const A &...args)
 {
@@ -136,10 +135,8 @@ cudaError_t launch_kernel(void (*kern)(P...), unsigned grid, unsigned threads, s
     cfg.blockDim = dim3(threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    if (overlap) {
-        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[n++].val.programmaticStreamSerializationAllowed = 1;
-    }
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
     if (cluster > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
         attr[n].val.clusterDim.x = cluster;
