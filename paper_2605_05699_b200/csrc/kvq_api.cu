@@ -630,12 +630,10 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
 static __global__ void kvq_calibrate_finish_kernel(float *lambda, int D)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    grid_trigger();
     grid_wait();
-    if (c < D) {
-        const float a = lambda[c];
-        lambda[c] = a > 0.0f ? 1.0f / a : 1.0f;
-    }
+    const float a = c < D ? lambda[c] : 0.0f;
+    grid_trigger();
+    if (c < D) lambda[c] = a > 0.0f ? 1.0f / a : 1.0f;
 }
 
 kvq_status_t kvq_calibrate_lambda(kvq_plan_t *plan, const void *x, kvq_dtype_t dtype, int64_t N, float *lambda_out, void *cuda_stream)

@@ -188,13 +188,16 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 
 // Programmatic dependent launch.  The kernels of this library are launched with the attribute that lets a grid's blocks come up
 // while its predecessor on the stream runs out (launch_kernel in kvq_internal.h): the launch, the set-up of barriers and tensor
-// memory and the requests for table rows then run under the predecessor's last tiles.  grid_trigger() allows the successor;
-// grid_wait() returns once every grid ahead on the stream is complete and its writes are visible, and stands before the first
-// access to anything but the plan's tables (which only host calls and kernels without an early trigger write).  Every thread
-// takes the wait, so that no grid is complete before the grids ahead of it.  A block triggers when it has read the last of its
-// inputs, not at entry: what it cached of a buffer that its successor reads is then older than the successor's launch, and blocks
-// brought up on the SMs that a call leaves idle, long before the rest of their grid, cost more than they hid (encode + decode of 99,993 vectors, D = 160, bf16: 78.7 us without any of this, 83.5 us with the
-// trigger at entry, 76.5 us with it at the end; 5120 appends at D = 128: 12.3 -> 9.0 us).
+// memory and the requests for table rows then run under the predecessor's last tiles.  grid_wait() returns once every grid ahead on
+// the stream is complete and its writes are visible, and stands before the first access to anything but the plan's tables (which
+// only host calls and kernels without an early trigger write).  Every thread takes the wait, so that no grid is complete before the
+// grids ahead of it.  Results rest on that wait alone.  grid_trigger() only says when the successor's blocks may come up: once every
+// block has had a thread there or has ended.  It stands where a block's last input is on its way or in, in the tensor-core kernels
+// behind the producer's last load (a tile that is decoded again in fp32 is read later), in the register-FFT kernels where a block's
+// first warp is done.  At entry it costs more than it hides, blocks then sit on SMs that a call leaves idle long before the
+// rest of their grid (encode + decode of 99,993 vectors, D = 160, bf16: 78.7 us without any of this, 83.5 us with the trigger at entry,
+// 76.5 us so; 5120 appends at D = 128, back to back: 12.3 -> 9.5 us).  A call gains where it follows one of this library's: other kernels
+// do not trigger early.
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

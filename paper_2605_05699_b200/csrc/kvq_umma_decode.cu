@@ -426,6 +426,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     (void)mbar_wait_bounded(smem_u32(&ctrl->in_full[j % kInStages]), (uint32_t)(j / kInStages) & 1u, 1u << 16);
             }
         }
+        __syncwarp();
+        grid_trigger();   // the last load is on its way
     } else if (warp == 1) {
         // =========================== mma issuer ===========================
         // (elect.sync, not lane 0: the compiler then knows that one thread issues.  128 x 64 x 16 with A in tensor memory: 32 cycles, else 45)
@@ -733,7 +735,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) bulk_wait_all();
     }
 
-    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {

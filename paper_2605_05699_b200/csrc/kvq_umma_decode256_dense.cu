@@ -200,6 +200,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     (void)mbar_wait_bounded(smem_u32(&ctrl->in_full[j % kInStages]), (uint32_t)(j / kInStages) & 1u, 1u << 16);
             }
         }
+        __syncwarp();
+        grid_trigger();   // the last load is on its way
     } else if (warp == 1) {
         // =========================== mma issuer ===========================
         if (lane == 0) {
@@ -425,7 +427,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) bulk_wait_all();
     }
 
-    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {

@@ -338,6 +338,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     (void)mbar_wait_bounded(smem_u32(&ctrl->in_full[j % kInStages]), (uint32_t)(j / kInStages) & 1u, 1u << 16);
             }
         }
+        __syncwarp();
+        grid_trigger();   // the last load is on its way
     } else if (warp == 1) {
         // =========================== mma issuer ===========================
         if (elect_one()) {
@@ -521,7 +523,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
 
-    grid_trigger();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {

@@ -271,6 +271,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             cluster_st_u32(cluster_map(smem_u32(&ctrl->issued[rank]), 0), (uint32_t)issued);
         }
+        __syncwarp();
+        grid_trigger();   // the last load is on its way
     } else if (warp == 1) {
         // =========================== mma issuer (leader) ===========================
         if (rank == 0 && elect_one()) {
@@ -447,7 +449,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     }
 
-    grid_trigger();
     __syncwarp();
     if (lane == 0 && *abort_flag)   // tell the partner
         cluster_st_u32(cluster_map(smem_u32(const_cast<uint32_t *>(&ctrl->abort)), (uint32_t)(rank ^ 1)), 1u);
