@@ -281,12 +281,12 @@ struct TileCursor {
 // rows are cut into tiles of 128 rows (256 where a CTA pair works on one tile) (a segment's last tile may be short), n_seg * tps tiles in all, `parts` shares.
 // Contiguous, so that the B operand of a lambda row is rebuilt as rarely as possible.  `segs` consecutive segments have one
 // lambda row (1, or the streams of a cache view that share theirs; the last row may have fewer).  A share that crosses into
-// another lambda row pays a rebuild of B on its critical path, about two tiles' time, so:
+// another lambda row pays a rebuild of B on its critical path, one to two tiles' time, so:
 //   * where no more lambda rows than shares exist and the longest share grows by no more than that, every share stays inside one
 //     lambda row (90,000 vectors under 30 rows, shares equal in tiles
 //     against this: encode D = 160 25.2 and 18.1 us, decode D = 128 bf16 14.5 and 12.0, D = 256 31.2 and 28.9);
-//   * else, with at least eight tiles per share, the shares are equal in COST, a lambda row counting one unit more than its
-//     tiles (a share that would begin inside that unit begins at the row's first tile);
+//   * else, with at least eight tiles per share, the shares are equal in COST, a lambda row counting one unit, the price's lower end,
+//     more than its tiles (a share that would begin inside that unit begins at the row's first tile);
 //   * else they are equal in tiles.
 struct TileShare {
     int64_t tps;     // tiles per segment

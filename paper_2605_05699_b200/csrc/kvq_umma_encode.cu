@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3;                 // tensor-memory lane quarter this warp may touch
         const int h = ((warp - 2) >> 2) & 1;    // half of the row
         const int r = q * 32 + lane;            // tile row of this thread
-        const int bw = (warp - 2) & 7;          // position within the set: D / 8 rows of B per warp when the set rebuilds B
+        const int bw = (warp - 2) & 7;          // position within the set, for the quads of a rebuild of B
         const int g0 = h * C::kGroupsPerPart;                                        // this thread's groups: g0 .. g1 - 1
         const int g1 = h == 0 ? C::kGroupsPerPart : G;
         const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16);

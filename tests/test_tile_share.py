@@ -1,5 +1,6 @@
 """The split of a call's tiles over the CTAs of a persistent kernel (TileShare), run on the host: every tile belongs to exactly one
-share, shares follow one another, and no share is more than two tiles longer than an even split's."""
+share, shares follow one another, no share is more than two tiles longer than an even split's, and none holds tiles of two lambda rows
+where the rows can have shares of their own within that length."""
 import os
 import shutil
 import subprocess
@@ -19,6 +20,8 @@ int main()
         const unsigned parts = 1 + rand() % 150;
         const int rows = it % 7 ? 128 : 256;
         const long tps = (rpl + rows - 1) / rows, tiles = n_seg * tps, even = (tiles + parts - 1) / parts;
+        const long row_tiles = (segs < n_seg ? segs : n_seg) * tps, n_rows = (tiles + row_tiles - 1) / row_tiles;
+        const bool apart = n_rows <= (long)parts && (n_rows == 1 || (row_tiles + (long)parts / n_rows - 1) / ((long)parts / n_rows) <= even + 2);
         long at = 0;
         for (unsigned p = 0; p < parts; ++p) {
             const kvq::TileShare s(n_seg, rpl, p, parts, rows, segs);
@@ -26,6 +29,11 @@ int main()
             if (s.tps != tps || s.begin != at || s.n < 0 || s.n > even + 2) {
                 printf("n_seg %ld rpl %ld segs %ld parts %u: share %u begins at %ld (%ld), %d tiles of %ld\n", n_seg, rpl, segs, parts, p,
                        (long)s.begin, at, s.n, even);
+                return 1;
+            }
+            if (apart && s.begin / row_tiles != (s.begin + s.n - 1) / row_tiles) {
+                printf("n_seg %ld rpl %ld segs %ld parts %u: share %u (%d tiles from %ld) crosses a lambda row of %ld tiles\n", n_seg, rpl, segs,
+                       parts, p, s.n, (long)s.begin, row_tiles);
                 return 1;
             }
             at += s.n;
