@@ -238,8 +238,7 @@ def kvq_plan_prepare(plan: int, dtype: torch.dtype, device=None) -> None:
     current one), so that later calls with tensors of ``dtype`` allocate nothing and never block."""
     code = KVQ_F16 if dtype == torch.float16 else KVQ_BF16 if dtype == torch.bfloat16 else -1
     dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
-    with torch.cuda.device(dev):
-        _check(lib().kvq_plan_prepare(plan, code), "kvq_plan_prepare")
+    _call(lib().kvq_plan_prepare, "kvq_plan_prepare", dev, plan, code)
 
 
 def kvq_plan_set_wait_limit(plan: int, polls: int) -> None:

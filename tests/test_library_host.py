@@ -172,6 +172,22 @@ def test_status_strings_and_launch_counter():
     assert kb.kvq_launch_count() >= 0
 
 
+def test_prepare_takes_a_device_without_an_index_as_the_current_one(monkeypatch):
+    """A device that names no ordinal, of whatever kind, changes nothing: the library prepares the plan where it is called."""
+    seen = []
+
+    class Fake:
+        @staticmethod
+        def kvq_plan_prepare(plan, code):
+            seen.append((plan, code))
+            return kb.KVQ_OK
+
+    monkeypatch.setattr(kb, "lib", lambda: Fake)
+    kb.kvq_plan_prepare(7, torch.float16, "cpu")
+    kb.kvq_plan_prepare(7, torch.bfloat16, torch.device("cuda"))
+    assert seen == [(7, kb.KVQ_F16), (7, kb.KVQ_BF16)]
+
+
 def test_compute_without_a_device_fails_loudly_never_silently():
     import torch
 
