@@ -15,8 +15,8 @@
 //                            half2 instruction, stored straight into TENSOR MEMORY as the A operand
 //                            (tcgen05.st); the group scales come by plain loads, one tile ahead.
 //                            The group that meets the first tile of a new lambda row rebuilds B.
-//   warp 1        mma        one thread issues D / 16 K-steps of tcgen05.mma (A from tensor memory, B
-//                            from shared memory) into one of two accumulator stages and commits
+//   warp 1        mma        one thread issues the K-steps of tcgen05.mma (A from tensor memory, B from shared memory; D / 16 of
+//                            them, or D / 32 per parity of the radix-2 form) into an accumulator stage and commits
 //   warps 10-17   epilogue   two groups of four warps, alternate tiles.  Thread t reads accumulator
 //                            row t (tcgen05.ld), rounds to fp16, writes a swizzled staging tile; one
 //                            lane per warp issues the TMA tensor stores (32 rows x 128 B boxes, plus a
@@ -28,7 +28,7 @@
 //   A [128 vectors, K = D]   fp16 in tensor memory: lane = vector, D / 2 columns of two codes each
 //   B [N = D outputs, K]     fp16 in shared memory, K-major, 128-byte swizzle, K blocks of 64:
 //                            W'[n, c] = s_n M[c, n] / max(lambda_c, 1e-6) / rho, rho a power of two
-//   D [128, D]               fp32 accumulator in tensor memory, two stages
+//   D [128, D]               fp32 accumulator in tensor memory, two stages (one at D = 160 with bf16 output in the radix-2 form)
 //
 // The K order inside a word of 8 codes is (0,4,1,5,2,6,3,7): that is how the half2 nibble trick
 // delivers them, and B is built in the same order, so no instruction is spent on reordering.
