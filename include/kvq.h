@@ -225,7 +225,8 @@ kvq_status_t kvq_append(kvq_plan_t *plan, const void *x_new /* [S, D] */, kvq_dt
  * fp16 window; when it is full the block is quantized, and the already dequantized prefix is kept, so that a decode step
  * costs O(new rows) instead of O(prefix)).  Quantizes `rows` new vectors of each of S streams into rows
  * [pos0, pos0 + rows) of the int4 caches (exactly what `rows` kvq_append calls would store) and writes the dequantized
- * values of those rows (exactly what kvq_decode of the caches would give there) into the same rows of dq_cache.
+ * values of those rows (what kvq_decode of the caches gives there, bit for bit where both calls take the same kernel
+ * family) into the same rows of dq_cache.
  *   x_block       device, [S, rows, D] row-major, fp16 or bf16 per `dtype`; 16-byte aligned.
  *   lambda, n_lambda, streams_per_lambda, packed_cache [S, T_max, D/2], scales_cache [S, T_max, D/group]: as in kvq_append.
  *   dq_cache      device out, [S, T_max, D] of the same 16-bit type; 16-byte aligned.  Only rows [pos0, pos0 + rows) are written.
