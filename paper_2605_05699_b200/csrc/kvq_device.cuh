@@ -196,8 +196,8 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 // behind the producer's last load (a tile that is decoded again in fp32 is read later), in the register-FFT kernels where a block's
 // first warp is done.  At entry it costs more than it hides, blocks then sit on SMs that a call leaves idle long before the
 // rest of their grid (encode + decode of 99,993 vectors, D = 160, bf16: 78.7 us without any of this, 83.5 us with the trigger at entry,
-// 76.5 us so; 5120 appends at D = 128, back to back: 12.3 -> 9.5 us).  A call gains where it follows one of this library's: other kernels
-// do not trigger early.
+// 76.5 us so; 5120 appends at D = 128, back to back: 12.3 -> 9.7 us).  Behind another program's kernel, which does not trigger early, a
+// call gains less (those appends behind a small elementwise kernel: 12.3 -> 11.3 us).
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
