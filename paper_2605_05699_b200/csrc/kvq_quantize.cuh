@@ -4,7 +4,8 @@
 // These kernels run at the board's power limit, where a warp instruction costs about a nanojoule, so the count is what matters:
 // the magnitudes take one instruction each (max.xorsign.abs carries the absolute value for free), sums and products of
 // neighbouring values go in pairs (add / fma.f32x2, rounded like the single ones), the codes are gathered by byte permutes.
-// Encode of 2,097,152 vectors at D = 128, back to back: 183.1 -> 180.2 us; D = 160, 700,000: 97.5 -> 93.4; D = 256, 1,064,960: 269 -> 266.
+// Encode of 2,097,152 vectors at D = 128, back to back: 183.1 -> 180.2 us (another box: 182.7 -> 181.1, inside the spread); D = 160, 700,000:
+// 97.5 -> 93.4; D = 256, 1,064,960: 269 -> 266.
 #pragma once
 
 #include "kvq_device.cuh"
