@@ -46,6 +46,7 @@ EXPORTS = (
 )
 
 _lib = None
+_native = None   # kvq_call, the calls' host side in native code, once the library is loaded; None where it has not been built
 
 
 class KvqError(RuntimeError):
@@ -56,7 +57,7 @@ class KvqError(RuntimeError):
 
 def lib() -> ctypes.CDLL:
     """Loads libkvq.so (once).  Raises if it has not been built: there is no fallback."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(
@@ -105,6 +106,13 @@ def lib() -> ctypes.CDLL:
         L.kvq_status_string.argtypes = [i32]
         L.kvq_launch_count.restype = u64
         L.kvq_launch_count.argtypes = []
+        try:
+            from . import kvq_call
+        except ImportError:
+            kvq_call = None
+        if kvq_call is not None:
+            kvq_call.bind(*(ctypes.cast(f, vp).value for f in (L.kvq_encode, L.kvq_decode, L.kvq_append, L.kvq_append_at, L.kvq_flush_block)))
+        _native = kvq_call
         _lib = L
     return _lib
 
@@ -166,6 +174,13 @@ def _call(fn, where: str, device: torch.device, *args) -> None:
             st = fn(*args)
     if st != KVQ_OK:
         raise KvqError(st, where)
+
+
+def _done(status: int, where: str) -> bool:
+    """Whether a native call was made (-1: not taken, the general way below has it); raises for its errors."""
+    if status > 0:
+        raise KvqError(status, where)
+    return status == 0
 
 
 # ---- C entry points, same names ---------------------------------------------------------
@@ -251,6 +266,8 @@ def kvq_plan_clear_device_status(plan: int) -> None:
 
 def kvq_encode(plan: int, x: torch.Tensor, lam: torch.Tensor, packed: torch.Tensor, scales: torch.Tensor,
                rows_per_lambda: int = 0, stream=None) -> None:
+    if stream is None and _native is not None and _done(_native.encode(plan, x, lam, packed, scales, rows_per_lambda), "kvq_encode"):
+        return
     D = x.shape[-1]
     N = x.numel() // D
     n_lambda = lam.numel() // D
@@ -261,6 +278,8 @@ def kvq_encode(plan: int, x: torch.Tensor, lam: torch.Tensor, packed: torch.Tens
 
 def kvq_decode(plan: int, packed: torch.Tensor, scales: torch.Tensor, lam: torch.Tensor, out: torch.Tensor,
                rows_per_lambda: int = 0, stream=None) -> None:
+    if stream is None and _native is not None and _done(_native.decode(plan, packed, scales, lam, out, rows_per_lambda), "kvq_decode"):
+        return
     D = out.shape[-1]
     N = out.numel() // D
     n_lambda = lam.numel() // D
@@ -271,6 +290,8 @@ def kvq_decode(plan: int, packed: torch.Tensor, scales: torch.Tensor, lam: torch
 
 def kvq_append(plan: int, x_new: torch.Tensor, lam: torch.Tensor, packed_cache: torch.Tensor,
                scales_cache: torch.Tensor, pos: int, streams_per_lambda: int = 0, stream=None) -> None:
+    if stream is None and _native is not None and _done(_native.append(plan, x_new, lam, packed_cache, scales_cache, pos, streams_per_lambda), "kvq_append"):
+        return
     D = x_new.shape[-1]
     S = x_new.numel() // D
     T_max = packed_cache.shape[-2]
@@ -300,6 +321,9 @@ def kvq_decode_static(plan: int, packed: torch.Tensor, scales: torch.Tensor, lam
 
 def kvq_flush_block(plan: int, x_block: torch.Tensor, lam: torch.Tensor, packed_cache: torch.Tensor, scales_cache: torch.Tensor,
                     dq_cache: torch.Tensor, pos0: int, streams_per_lambda: int = 0, stream=None) -> None:
+    if stream is None and _native is not None and _done(
+            _native.flush_block(plan, x_block, lam, packed_cache, scales_cache, dq_cache, pos0, streams_per_lambda), "kvq_flush_block"):
+        return
     S, rows, D = x_block.shape
     T_max = packed_cache.shape[-2]
     n_lambda = lam.numel() // D
@@ -319,6 +343,9 @@ def _pos_word(pos_device: torch.Tensor):
 def kvq_append_at(plan: int, x_new: torch.Tensor, lam: torch.Tensor, packed_cache: torch.Tensor, scales_cache: torch.Tensor,
                   pos_device: torch.Tensor, streams_per_lambda: int = 0, stream=None) -> None:
     """kvq_append with the row to write read from ``pos_device`` (one int64 on the device) when the kernel runs."""
+    if stream is None and _native is not None and _done(
+            _native.append_at(plan, x_new, lam, packed_cache, scales_cache, pos_device, streams_per_lambda), "kvq_append_at"):
+        return
     D = x_new.shape[-1]
     S = x_new.numel() // D
     T_max = packed_cache.shape[-2]

@@ -7,12 +7,15 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkvq.so")
+CALL_SRC = os.path.join(CSRC, "kvq_call.cpp")
+CALL = os.path.join(HERE, "kvq_call.so")   # the binding's native half: a Python extension on torch's own headers and libraries
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 NVCC_FLAGS = [
@@ -49,8 +52,25 @@ def _compile(src: str, force: bool, newest: float) -> str:
     return obj
 
 
+def _build_call(force: bool) -> None:
+    if not force and os.path.exists(CALL) and os.path.getmtime(CALL) >= max(os.path.getmtime(CALL_SRC), os.path.getmtime(os.path.join(INCLUDE, "kvq.h"))):
+        return
+    import torch
+
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = CALL + ".tmp.%d" % os.getpid()
+    subprocess.check_call([
+        "g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+        "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+        "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), CALL_SRC, "-o", tmp,
+        "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    os.replace(tmp, CALL)
+
+
 def build(force: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
+    _build_call(force)
     newest = _deps_mtime()
     srcs = _sources()
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
