@@ -18,6 +18,7 @@
 // same order), so the two families agree wherever fp32 rounding of the transform does not decide a code.
 #include "kvq_internal.h"
 #include "kvq_device.cuh"
+#include "kvq_umma.cuh"
 
 namespace kvq {
 
@@ -308,15 +309,11 @@ __global__ void __launch_bounds__(kWarps * 32) kvq_encode_matvec_kernel(const __
 // ------------------------------------------------------------------------------------------------
 // decode: codes and scales -> x^  (Sec. 3.1: Eq. 2 undone, inverse real DFT, signs last; 1 / max(lambda, 1e-6) of Sec. 5.1)
 // ------------------------------------------------------------------------------------------------
-template <int D, bool BF16>
-__device__ __forceinline__ void decode_batch(const MatvecParams &prm, float4 (&t)[Geo<D>::CH][Geo<D>::P], float *zs, float *red, int warp,
-                                             int lane, int64_t batch, bool last)
+// the CTA's stored vectors, dequantised: q sigma / max(lambda, 1e-6), four coordinates per thread and pass
+template <int D>
+__device__ __forceinline__ void dequantise_batch(const MatvecParams &prm, float *zs, int64_t batch)
 {
-    using Gm = Geo<D>;
-    constexpr int P = Gm::P;
     const int64_t v0 = batch * kV;
-
-    // ---- the CTA's stored vectors, dequantised: q sigma / max(lambda, 1e-6), four coordinates per thread and pass
     const unsigned char *pk = static_cast<const unsigned char *>(prm.packed);
     const uint16_t *scl = static_cast<const uint16_t *>(prm.scales);
     const int G = D / prm.group;
@@ -345,6 +342,17 @@ __device__ __forceinline__ void decode_batch(const MatvecParams &prm, float4 (&t
         }
         *reinterpret_cast<float4 *>(zs + v * D + 4 * i) = o;
     }
+}
+
+template <int D, bool BF16>
+__device__ __forceinline__ void decode_batch(const MatvecParams &prm, float4 (&t)[Geo<D>::CH][Geo<D>::P], float *zs, float *red, int warp,
+                                             int lane, int64_t batch, bool last)
+{
+    using Gm = Geo<D>;
+    constexpr int P = Gm::P;
+    const int64_t v0 = batch * kV;
+
+    dequantise_batch<D>(prm, zs, batch);
     __syncthreads();
     if (last) grid_trigger();   // nothing but the table is read from here on
 
@@ -382,7 +390,186 @@ __global__ void __launch_bounds__(kWarps * 32) kvq_decode_matvec_kernel(const __
     }
 }
 
+// ------------------------------------------------------------------------------------------------
+// the smallest calls: the output coordinates of a batch over several CTAs
+// ------------------------------------------------------------------------------------------------
+// A call of a few batches leaves most of the chip idle while a CTA reads a whole table (64 KB at D = 128, 256 KB at D = 256, there in two
+// passes) and makes 8 D^2 multiply-adds.  Here a CTA has 32 output coordinates of its batch, 64 at D = 256; 8 (16) lanes cover
+// its part of a table row, and each quarter (half) of a warp takes two (four) of the eight vectors, so that every sum has the same terms
+// in the same order: the results are those of the form above bit for bit.  Append of 64 vectors, back to
+// back: D = 128 3.2 -> 2.6 us, 256 6.9 -> 3.6; 200 at D = 160 6.0 -> 3.0; 200 at D = 256 with one scale per vector 6.9 -> 4.4; decode of 64 at
+// D = 256 6.8 -> 3.7; window flush of 8 x 15 rows at D = 256 12.3 -> 7.0.
+// A group of 32 lies inside a slice.  What crosses slices, the row maximum of a plan with one scale per vector and the
+// dequantized values of the window flush, goes through distributed shared memory; the CTAs of a batch are then a cluster (two or four:
+// D = 96 and 160 would be three and five, and stay with the form above there).
+// A CTA takes one batch, and the form is taken while the device holds all of them at once; beyond that the copies of
+// the staging and the barriers cost more than they save.
+template <int D>
+struct Slice {
+    static constexpr int W = D == 256 ? 64 : 32, kSlices = D / W;   // coordinates per slice
+    static constexpr bool kCluster = kSlices == 2 || kSlices == 4;
+    static constexpr int Q = W / 4, kSub = 32 / Q, kSubV = kV / kSub;   // lanes per table row; parts of a warp, vectors of each
+    static constexpr int KW = D / kWarps;                   // contraction indices per warp
+    static constexpr int kSmemBytes = (2 * kV * D + kWarps * kV * W + kSlices * kV) * (int)sizeof(float);
+};
+
+template <int D>
+__device__ __forceinline__ void slice_rows(const float *__restrict__ table, int slice, int warp, int lane, float4 (&t)[Slice<D>::KW])
+{
+    using S = Slice<D>;
+#pragma unroll
+    for (int k = 0; k < S::KW; ++k)
+        t[k] = __ldg(reinterpret_cast<const float4 *>(table + (size_t)(warp * S::KW + k) * D + slice * S::W) + lane % S::Q);
+}
+
+// the sums of vector `warp`, coordinates 4 (lane % Q) .. + 3 of the slice, in every part of the warp
+template <int D>
+__device__ __forceinline__ float4 slice_matvec(const float4 (&t)[Slice<D>::KW], const float *xs, float *red, int warp, int lane)
+{
+    using S = Slice<D>;
+    const int sub = lane / S::Q, i = lane % S::Q;
+#pragma unroll
+    for (int v = 0; v < S::kSubV; ++v) {
+        const int vec = sub * S::kSubV + v;
+        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < S::KW; ++k) {
+            const float xk = xs[vec * D + warp * S::KW + k];
+            a.x = fmaf(t[k].x, xk, a.x), a.y = fmaf(t[k].y, xk, a.y), a.z = fmaf(t[k].z, xk, a.z), a.w = fmaf(t[k].w, xk, a.w);
+        }
+        *reinterpret_cast<float4 *>(red + (warp * kV + vec) * S::W + 4 * i) = a;
+    }
+    __syncthreads();
+    float4 y = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const float4 a = *reinterpret_cast<const float4 *>(red + (w * kV + warp) * S::W + 4 * i);
+        y.x += a.x, y.y += a.y, y.z += a.z, y.w += a.w;
+    }
+    return y;
+}
+
+template <int D, bool BF16, bool FLUSH>
+__global__ void __launch_bounds__(kWarps * 32, D == 256 ? 1 : 2) kvq_encode_matvec_sliced_kernel(const __grid_constant__ MatvecParams prm)
+{
+    using S = Slice<D>;
+    extern __shared__ __align__(16) float sm[];
+    float *xs = sm, *back = xs + kV * D, *red = back + kV * D, *peak = red + kWarps * kV * S::W;   // peak: [slice][vector]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = lane % S::Q, sub = lane / S::Q;
+    const int slice = (int)blockIdx.x % S::kSlices, c0 = slice * S::W + 4 * i;   // this lane's coordinates
+    const bool per_vector = prm.group == D, cluster = FLUSH || per_vector;
+
+    float4 t[S::KW];
+    slice_rows<D>(prm.table, slice, warp, lane, t);
+    if (cluster) cluster_arrive();   // all four have begun: waited for in front of the first access to a partner's memory
+    grid_wait();
+    RowMap out_map;
+    const bool ok = resolve_out_map(prm, out_map);   // uniform over the grid
+    if (cluster) cluster_wait();
+    if (!ok) return;
+    const int64_t batch = blockIdx.x / S::kSlices;
+    const int64_t r = batch * kV + warp;   // the vector this warp finishes
+    const bool live = r < prm.N;
+    const float4 l = load_input(reinterpret_cast<const float4 *>(prm.lambda + lambda_row(live ? r : prm.N - 1, prm.n_lambda, prm.rows_per_lambda) * D + c0));
+    const uint32_t *x = static_cast<const uint32_t *>(prm.in);
+    for (int idx = threadIdx.x; idx < kV * (D / 2); idx += kWarps * 32) {
+        const int64_t row = batch * kV + idx / (D / 2);
+        const float2 f = widen2<BF16>(row < prm.N ? load_input(x + row * (D / 2) + idx % (D / 2)) : 0u);   // rows past the end are zeros
+        xs[2 * idx] = f.x, xs[2 * idx + 1] = f.y;
+    }
+    __syncthreads();
+    grid_trigger();   // nothing but the tables is read from here on
+    float4 z = slice_matvec<D>(t, xs, red, warp, lane);
+
+    // ---- warp w finishes this slice of vector w: the quantizer of encode_batch
+    z.x *= l.x, z.y *= l.y, z.z *= l.z, z.w *= l.w;
+    float amax = fmaxf(fmaxf(fabsf(z.x), fabsf(z.y)), fmaxf(fabsf(z.z), fabsf(z.w)));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));   // 8 lanes are a group
+    if (per_vector) {
+#pragma unroll
+        for (int o = 8; o < S::Q; o <<= 1) amax = fmaxf(amax, __shfl_xor_sync(0xFFFFFFFFu, amax, o));
+        float *to = peak + slice * kV + warp;
+        if (lane < S::kSlices) cluster_st_u32(cluster_map(smem_u32(to), (uint32_t)lane), __float_as_uint(amax));
+        cluster_sync_all();
+#pragma unroll
+        for (int s = 0; s < S::kSlices; ++s) amax = fmaxf(amax, peak[s * kV + warp]);
+    }
+    const int64_t orow = live ? out_map(r) : 0;
+    const float Q = prm.bits == 4 ? 7.0f : 127.0f;
+    const __half hs = __float2half_rn(fminf(__fdiv_rn(amax, Q), 65504.0f));   // codes are taken against the stored value
+    const float sg = __half2float(hs);
+    const float rs = sg > 0.0f ? __frcp_rn(sg) : 0.0f;
+    const bool clamp = !(amax * rs < Q + 0.25f);   // saturated or subnormal scale: codes could leave [-Q, Q]
+    const bool stores = live && sub == 0;
+    if (stores && (per_vector ? c0 == 0 : (i & 7) == 0)) static_cast<uint16_t *>(prm.scales)[orow * (D / prm.group) + (per_vector ? 0 : c0 >> 5)] = __half_as_ushort(hs);
+    const float zz[4] = {z.x, z.y, z.z, z.w};
+    uint32_t code[4];
+    float qf[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float v = clamp ? fminf(fmaxf(zz[e] * rs, -Q), Q) + 12582912.0f : fmaf(zz[e], rs, 12582912.0f);
+        code[e] = __float_as_uint(v);   // low bits: q in two's complement (1.5 * 2^23 + q)
+        qf[e] = v - 12582912.0f;        // q itself, exactly
+    }
+    if (stores) {
+        unsigned char *pk = static_cast<unsigned char *>(prm.packed);
+        if (prm.bits == 4) {
+            const uint32_t w = (code[0] & 0xFu) | ((code[1] & 0xFu) << 4) | ((code[2] & 0xFu) << 8) | ((code[3] & 0xFu) << 12);
+            *reinterpret_cast<uint16_t *>(pk + orow * (D / 2) + c0 / 2) = (uint16_t)w;
+        } else {
+            const uint32_t w = (code[0] & 0xFFu) | ((code[1] & 0xFFu) << 8) | ((code[2] & 0xFFu) << 16) | (code[3] << 24);
+            *reinterpret_cast<uint32_t *>(pk + orow * D + c0) = w;
+        }
+    }
+    if constexpr (FLUSH) {   // the way back starts from the stored values
+        const float o[4] = {qf[0] * (sg * __frcp_rn(fmaxf(l.x, 1e-6f))), qf[1] * (sg * __frcp_rn(fmaxf(l.y, 1e-6f))),
+                            qf[2] * (sg * __frcp_rn(fmaxf(l.z, 1e-6f))), qf[3] * (sg * __frcp_rn(fmaxf(l.w, 1e-6f)))};
+        float4 t2[S::KW];
+        slice_rows<D>(prm.table2, slice, warp, lane, t2);   // in flight across the barrier
+        for (int s = sub; s < S::kSlices; s += S::kSub) {   // every CTA of the cluster needs all of the vector
+            const uint32_t to = cluster_map(smem_u32(back + warp * D + c0), (uint32_t)s);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) cluster_st_u32(to + 4 * e, live ? __float_as_uint(o[e]) : 0u);
+        }
+        __syncwarp();
+        cluster_sync_all();
+        const float4 y = slice_matvec<D>(t2, back, red, warp, lane);
+        if (stores)
+            *reinterpret_cast<uint2 *>(static_cast<unsigned char *>(prm.out) + orow * (2 * D) + 2 * c0) = make_uint2(narrow2<BF16>(y.x, y.y), narrow2<BF16>(y.z, y.w));
+    }
+}
+
+template <int D, bool BF16>
+__global__ void __launch_bounds__(kWarps * 32, D == 256 ? 1 : 2) kvq_decode_matvec_sliced_kernel(const __grid_constant__ MatvecParams prm)
+{
+    using S = Slice<D>;
+    extern __shared__ __align__(16) float sm[];
+    float *zs = sm, *red = sm + 2 * kV * D;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int slice = (int)blockIdx.x % S::kSlices;
+    float4 t[S::KW];
+    slice_rows<D>(prm.table, slice, warp, lane, t);   // in flight while the codes are fetched and dequantised
+    grid_wait();
+    const int64_t batch = blockIdx.x / S::kSlices;
+    dequantise_batch<D>(prm, zs, batch);
+    __syncthreads();
+    grid_trigger();   // nothing but the table is read from here on
+    const float4 y = slice_matvec<D>(t, zs, red, warp, lane);
+    const int64_t r = batch * kV + warp;
+    if (r < prm.N && lane < S::Q)
+        *reinterpret_cast<uint2 *>(static_cast<unsigned char *>(prm.out) + prm.out_map(r) * (2 * D) + 2 * (slice * S::W + 4 * lane)) =
+            make_uint2(narrow2<BF16>(y.x, y.y), narrow2<BF16>(y.z, y.w));
+}
+
 // MODE: 0 decode, 1 encode, 2 encode + decode of the same rows (window flush)
+template <int D, bool BF16, int MODE>
+constexpr auto sliced_kernel()
+{
+    if constexpr (MODE == 0) return &kvq_decode_matvec_sliced_kernel<D, BF16>;
+    else return &kvq_encode_matvec_sliced_kernel<D, BF16, MODE == 2>;
+}
+
 template <int D, bool BF16, int MODE>
 cudaError_t launch(const MatvecParams &prm, cudaStream_t stream)
 {
@@ -390,17 +577,31 @@ cudaError_t launch(const MatvecParams &prm, cudaStream_t stream)
     int dev = 0;
     cudaError_t e = current_device_slot(&dev);
     if (e != cudaSuccess) return e;
+    constexpr bool kSliced = MODE != 2 || Slice<D>::kCluster;
     auto kern = MODE == 0 ? kvq_decode_matvec_kernel<D, BF16> : MODE == 1 ? kvq_encode_matvec_kernel<D, BF16, false> : kvq_encode_matvec_kernel<D, BF16, true>;
     if (slots.sms[dev] == 0) {   // slots.sms: the CTAs of this kernel that the device holds at once
         int sms = 0, per_sm = 0;
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<D>::kSmemBytes)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, Geo<D>::kSmemBytes)) != cudaSuccess) return e;
+        if constexpr (kSliced) {   // slots.blocks_per_sm: the CTAs of the sliced form that the device holds at once
+            int sliced_per_sm = 0;
+            auto sliced = sliced_kernel<D, BF16, MODE>();
+            if ((e = cudaFuncSetAttribute(sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, Slice<D>::kSmemBytes)) != cudaSuccess) return e;
+            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sliced_per_sm, sliced, kWarps * 32, Slice<D>::kSmemBytes)) != cudaSuccess) return e;
+            slots.blocks_per_sm[dev] = sms * (sliced_per_sm < 2 ? sliced_per_sm : 2);
+        }
         slots.sms[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
     if (prm.N == 0) return cudaSuccess;   // kvq_plan_prepare: the launch attributes are set, there is nothing to run
     const int64_t batches = (prm.N + kV - 1) / kV;
     if (batches > 0x7FFFFFFF) return cudaErrorInvalidValue;
+    if constexpr (kSliced) {
+        constexpr int kSlices = Slice<D>::kSlices;
+        const bool cluster = MODE == 2 || (MODE == 1 && prm.group == D);
+        if (batches * kSlices <= slots.blocks_per_sm[dev] && (Slice<D>::kCluster || !cluster))
+            return launch_kernel(sliced_kernel<D, BF16, MODE>(), (unsigned)(batches * kSlices), kWarps * 32, Slice<D>::kSmemBytes, stream, cluster ? kSlices : 1, prm);
+    }
     // one resident wave of CTAs that loop over batches where the kernel does; else a CTA per batch
     const int ctas = (int)(Geo<D>::kLoops && batches > slots.sms[dev] ? slots.sms[dev] : batches);
     return launch_kernel(kern, (unsigned)ctas, kWarps * 32, Geo<D>::kSmemBytes, stream, 1, prm);

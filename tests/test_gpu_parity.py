@@ -744,6 +744,44 @@ def test_matvec_kernels_all_dims(D, dtype):
     run_case(D, dtype, 5, "gaussian", 7100 + D, enc_impl="matvec", dec_impl="matvec")
 
 
+@pytest.mark.parametrize("D,dtype,per_vector,nbits,most", [(64, "f16", True, 4, 1184), (96, "bf16", False, 8, 784), (128, "f16", False, 4, 592), (128, "bf16", True, 8, 592),
+                                                           (160, "bf16", False, 4, 472), (160, "f16", True, 4, 472), (256, "f16", False, 4, 296),
+                                                           (256, "bf16", True, 4, 296)])
+def test_matvec_kernels_sliced_over_several_ctas(D, dtype, per_vector, nbits, most):
+    """A batch of 8 vectors, one vector more under lambda rows of one; the most whose slices the device holds at once, and one more: encode and
+    decode against the oracle and, bit for bit, against one call that is too long for slices; the fused flush, whose dequantized rows are
+    bit for bit the decode of what it stored."""
+    odt = DT[dtype]
+    plan = kb.Plan(D, D if per_vector else G, 31, bits=nbits)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_MATVEC, kb.KVQ_IMPL_MATVEC)
+    x = wl.make_vectors(2400, D, dtype, "k_outlier", 33)
+    lam1 = wl.make_lambda(1, D, 32)
+    xd = x.cuda()
+    p_all, s_all = gpu_encode(plan, xd, lam1.cuda())
+    o_all = gpu_decode(plan, p_all, s_all, lam1.cuda(), dtype)
+    for N, n_lambda, rpl in ((8, 1, 0), (9, 9, 1), (most, 1, 0), (most + 1, 1, 0)):
+        lam = lam1 if n_lambda == 1 else wl.make_lambda(n_lambda, D, 34)
+        lamd = lam.cuda()
+        packed, scales = gpu_encode(plan, xd[:N], lamd, rpl)
+        out = gpu_decode(plan, packed, scales, lamd, dtype, rpl)
+        if n_lambda == 1:
+            assert torch.equal(packed, p_all[:N]) and torch.equal(scales, s_all[:N]) and torch.equal(out.view(torch.int16), o_all[:N].view(torch.int16))
+        ora = ko.encode(bits(x[:N]), odt, plan.signs(), lam.numpy(), plan.group, rpl, want_v=True, bits=nbits)
+        pk, sb = packed.cpu().numpy(), bits(scales)
+        parity.check_encode(pk, sb, ora, plan.group, "sliced encode", bits=nbits, min_agree=0.9995)
+        ob, o64 = ko.decode(pk, sb, plan.signs(), lam.numpy(), plan.group, odt, rpl, want_f64=True, bits=nbits)
+        parity.check_decode(bits(out), ob, o64, odt, "sliced decode")
+        p2, s2, dq = torch.zeros_like(packed), torch.zeros_like(scales), torch.zeros_like(out)
+        pos0 = torch.zeros(1, dtype=torch.int64, device="cuda")
+        n0 = kb.kvq_launch_count()
+        kb.kvq_flush_block_at(plan.handle, xd[:N].view(N, 1, D), lamd, p2.view(N, 1, -1), s2.view(N, 1, -1), dq.view(N, 1, D), pos0, rpl or N)
+        assert kb.kvq_launch_count() - n0 == 1
+        torch.cuda.synchronize()
+        assert kb.kvq_plan_device_status(plan.handle) == 0
+        assert torch.equal(p2, packed) and torch.equal(s2, scales) and torch.equal(dq.view(torch.int16), out.view(torch.int16))
+    plan.close()
+
+
 def test_small_calls_take_the_matvec_kernels_and_agree_with_the_fft():
     # AUTO below 2048 rows is the matrix-vector kernel; its codes agree with the register FFT except at rounding ties
     D, N = 128, 1500
