@@ -108,41 +108,35 @@ static kvq_status_t ensure_device(kvq_plan *p)
     }
     if (p->device == dev) return KVQ_OK;
     if (p->device >= 0) return KVQ_ERR_INVALID_ARG;   // a plan stays on the device of its first use
-    uint32_t *st = nullptr;
-    if (cudaMalloc(&st, 256) != cudaSuccess) {
+    // one allocation: the status word, then the tables of the tensor-core and matrix-vector kernels
+    constexpr size_t kStatusBytes = 256;
+    const bool tables = umma_encode_supported(p->D, false) || umma_decode_supported(p->D, false);
+    const size_t bytes = tables ? sizeof(float) * (size_t)p->D * p->D : 0, total = kStatusBytes + (tables ? 2 * bytes + operand_bytes(p->D) : 0);
+    std::vector<float> b0, e0;
+    if (tables && !make_tables(p, b0, e0)) return KVQ_ERR_NOMEM;
+    unsigned char *mem = nullptr;
+    if (cudaMalloc(&mem, total) != cudaSuccess) {
         (void)cudaGetLastError();
         return KVQ_ERR_NOMEM;
     }
-    if (cudaMemset(st, 0, 256) != cudaSuccess) {
+    float *db = reinterpret_cast<float *>(mem + kStatusBytes), *de = reinterpret_cast<float *>(mem + kStatusBytes + bytes);
+    unsigned char *dw = mem + kStatusBytes + 2 * bytes;
+    bool ok = cudaMemset(mem, 0, kStatusBytes) == cudaSuccess;
+    if (ok && tables)
+        ok = cudaMemcpy(db, b0.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
+             cudaMemcpy(de, e0.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess && build_encode_operands(p->D, de, p->table_max, dw) == cudaSuccess;
+    if (!ok) {
         (void)cudaGetLastError();
-        cudaFree(st);
+        cudaFree(mem);
         return KVQ_ERR_CUDA;
     }
-    p->d_status = st;
-    p->table_bytes = 256;
-    if (umma_encode_supported(p->D, false) || umma_decode_supported(p->D, false)) {   // tables of the tensor-core kernels
-        const size_t bytes = sizeof(float) * (size_t)p->D * p->D;
-        std::vector<float> b0, e0;
-        float *db = nullptr, *de = nullptr;
-        bool ok = make_tables(p, b0, e0) && cudaMalloc(&db, bytes) == cudaSuccess && cudaMalloc(&de, bytes) == cudaSuccess;
-        kvq_status_t why = KVQ_ERR_NOMEM;
-        if (ok) {
-            ok = cudaMemcpy(db, b0.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
-                 cudaMemcpy(de, e0.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess;
-            why = KVQ_ERR_CUDA;
-        }
-        if (!ok) {
-            (void)cudaGetLastError();
-            if (db) cudaFree(db);
-            if (de) cudaFree(de);
-            cudaFree(st);
-            p->d_status = nullptr;
-            return why;
-        }
+    p->d_status = reinterpret_cast<uint32_t *>(mem);
+    if (tables) {
         p->d_b0 = db;
         p->d_e0 = de;
-        p->table_bytes += 2 * bytes;
+        p->d_operands = dw;
     }
+    p->table_bytes = total;
     p->device = dev;
     return KVQ_OK;
 }
@@ -186,6 +180,7 @@ static void fill_params(const kvq_plan *p, FftParams &prm, int64_t N, const floa
     prm.table_max = p->table_max;
     prm.first_wait_polls = p->first_wait_polls;
     prm.bits = p->bits;
+    prm.operands = p->d_operands;
     std::memcpy(prm.sign_xor, p->sign_xor, sizeof(prm.sign_xor));
 }
 
@@ -212,6 +207,7 @@ kvq_status_t kvq_plan_create_ex(int D, int group, int bits, uint64_t seed, kvq_p
     p->d_status = nullptr;
     p->d_b0 = nullptr;
     p->d_e0 = nullptr;
+    p->d_operands = nullptr;
     p->table_bytes = 0;
     p->rot = nullptr;
     p->table_max = (float)std::sqrt(2.0 / D);
@@ -232,12 +228,6 @@ kvq_status_t kvq_plan_destroy(kvq_plan_t *plan)
     if (!plan) return KVQ_OK;
     if (plan->d_status) {
         if (cudaFree(plan->d_status) != cudaSuccess) (void)cudaGetLastError();
-    }
-    if (plan->d_b0) {
-        if (cudaFree(plan->d_b0) != cudaSuccess) (void)cudaGetLastError();
-    }
-    if (plan->d_e0) {
-        if (cudaFree(plan->d_e0) != cudaSuccess) (void)cudaGetLastError();
     }
     delete[] plan->rot;
     delete plan;
@@ -277,7 +267,8 @@ kvq_status_t kvq_plan_set_rotation(kvq_plan_t *plan, const float *R_host)
     if (!make_tables(plan, b0, e0)) return KVQ_ERR_NOMEM;
     const size_t bytes = sizeof(float) * n;
     if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(plan->d_b0, b0.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(plan->d_e0, e0.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaMemcpy(plan->d_e0, e0.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+        build_encode_operands(plan->D, plan->d_e0, plan->table_max, plan->d_operands) != cudaSuccess) {
         (void)cudaGetLastError();
         return KVQ_ERR_CUDA;
     }
@@ -403,7 +394,7 @@ static bool flush_decode_is_matvec(const kvq_plan_t *plan, int64_t N)
 static kvq_status_t encode_common(kvq_plan_t *plan, const void *x, kvq_dtype_t dtype, int64_t N, const float *lambda,
                                   int64_t n_lambda, int64_t rows_per_lambda, uint8_t *packed, void *scales,
                                   const RowMap &out_map, void *cuda_stream, void *dq = nullptr, bool *fused = nullptr,
-                                  const DevicePos *pos = nullptr)
+                                  const DevicePos *pos = nullptr, bool append = false)
 {
     if (!plan || N < 0) return KVQ_ERR_INVALID_ARG;
     if (dtype != KVQ_F16 && dtype != KVQ_BF16) return KVQ_ERR_INVALID_ARG;
@@ -427,6 +418,7 @@ static kvq_status_t encode_common(kvq_plan_t *plan, const void *x, kvq_dtype_t d
     prm.packed = packed;
     prm.scales = scales;
     prm.out_map = out_map;
+    prm.append = append;
     // AUTO: the matrix-vector kernel for small calls (latency), beyond that the tensor-core kernel (measured faster than
     // the register FFT at every size above the matrix-vector limit), the register FFT where no tensor-core kernel is
     // built.  A rotated plan has no FFT path: matrix-vector wherever the tensor-core kernel does not apply.
@@ -464,7 +456,7 @@ kvq_status_t kvq_append(kvq_plan_t *plan, const void *x_new, kvq_dtype_t dtype, 
 {
     if (T_max < 1 || pos < 0 || pos >= T_max) return KVQ_ERR_INVALID_ARG;
     return encode_common(plan, x_new, dtype, S, lambda, n_lambda, streams_per_lambda, packed_cache, scales_cache,
-                         RowMap{1, T_max, pos}, cuda_stream);
+                         RowMap{1, T_max, pos}, cuda_stream, nullptr, nullptr, nullptr, true);
 }
 
 kvq_status_t kvq_decode(kvq_plan_t *plan, const uint8_t *packed, const void *scales, int64_t N, const float *lambda,

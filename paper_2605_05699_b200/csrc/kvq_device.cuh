@@ -352,6 +352,44 @@ __device__ __forceinline__ uint32_t narrow2(float lo, float hi)
 }
 
 // ---------------------------------------------------------------------------
+// two fp32 values in one 64-bit register: sums and differences of both in one instruction, each rounded like the single one
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+
+__device__ __forceinline__ float2 unpack_f32x2(uint64_t v)
+{
+    float2 f;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+    return f;
+}
+
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+__device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %2, %3, %1;" : "=l"(d) : "l"(a), "l"(b), "l"(0xBF800000BF800000ull));   // a - 1 b, one rounding
+    return d;
+}
+
+// ---------------------------------------------------------------------------
 // round-to-nearest-even codes by the magic-number trick (Sec. 3.2 step 4): v / sigma + 1.5 * 2^23 (+ bias) has the
 // biased code in its low mantissa bits, so eight nibbles (four bytes) are gathered with shifts and one subtraction
 // ---------------------------------------------------------------------------

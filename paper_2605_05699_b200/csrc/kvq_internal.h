@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <mutex>
 
 #include "../../include/kvq.h"
@@ -38,8 +39,15 @@ struct FftParams {
     float table_max;            // tensor-core encode: largest |entry| of the plan's forward table (sqrt(2/D) without a rotation)
     uint32_t first_wait_polls;  // tensor-core encode, D <= 160: polls the mma role gives its first operand build (0: the default)
     int bits;                   // tensor-core encode: 4 or 8 (the register-FFT launchers take it as an argument)
+    const unsigned char *operands;   // tensor-core append: the plan's split operands (build_encode_operands)
+    int append;                 // the call is an append: one new row per stream
     uint32_t sign_xor[128];     // word m: bit 15 set if s_{2m} = -1, bit 31 set if s_{2m+1} = -1
 };
+
+// The split operands of the append kernel: two fp16 terms of e0 2^k, each one block of [D rows][128 B] per 64 columns, 128-byte
+// swizzle.
+__host__ __device__ constexpr size_t operand_bytes(int D) { return 2 * (size_t)((D + 63) / 64) * (size_t)D * 128; }
+cudaError_t build_encode_operands(int D, const float *e0, float table_max, unsigned char *out);   // complete when it returns
 
 // A decode whose rows live in a cache laid out [stream][T][...]: the call's N = S * rows logical rows are rows
 // [base, base + rows) of each of S streams, `stride` cache rows apart, in packed, scales and out alike; the lambda row of
@@ -88,6 +96,10 @@ cudaError_t umma_decode_d256_dense(bool bf16, int64_t N, const GemmParams &prm, 
 bool umma_encode_per_vector_supported(int D, bool bf16);
 bool umma_encode_bits8_supported(int D, bool bf16);
 cudaError_t umma_encode(int D, bool bf16, bool per_vector, int64_t N, const FftParams &prm, const float *e0, cudaStream_t stream);
+
+// the append of many streams (kvq_umma_append.cu), which umma_encode takes where it is built and pays
+bool umma_append_pays(int D, bool bf16, bool per_vector, int64_t N, const FftParams &prm);
+cudaError_t umma_append(int D, bool per_vector, int64_t N, const FftParams &prm, cudaStream_t stream);
 
 // fp32 matrix-vector kernels for small calls (kvq_matvec.cu): every layout, dtype and D; b0 / e0 are the plan's tables
 // A cache position that lives in device memory (read when the kernel runs): the base row of the output row map; it must
@@ -163,9 +175,10 @@ struct kvq_plan {
     // device state, created on first use
     std::mutex mu;
     int device;            // -1 until initialised
-    uint32_t *d_status;    // device status word
+    uint32_t *d_status;    // device status word; the tables stand behind it in the same allocation
     float *d_b0;           // [D, D] fp32 inverse-transform matrix with the signs folded in (GEMM decode), or null
     float *d_e0;           // [D, D] fp32 forward-transform matrix with the signs folded in (GEMM encode), or null
+    unsigned char *d_operands;   // split operands of the append kernel, or null
     size_t table_bytes;
     double *rot;           // host, [D, D] row-major: the rotation between the transform and lambda, or null
     float table_max;       // largest |entry| of the forward table

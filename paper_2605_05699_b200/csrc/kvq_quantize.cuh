@@ -31,13 +31,6 @@ __device__ __forceinline__ float group_absmax(const uint32_t (&v)[32])
     return fmaxf(a, 0.0f);   // 0 where every value is a NaN
 }
 
-__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi)
-{
-    uint64_t d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-
 // v[i] += w[i], two at a time
 __device__ __forceinline__ void add_group(uint32_t (&v)[32], const uint32_t (&w)[32])
 {
@@ -49,6 +42,14 @@ __device__ __forceinline__ void add_group(uint32_t (&v)[32], const uint32_t (&w)
             "mov.b64 {%0, %1}, a;\n\t}"
             : "+r"(v[i]), "+r"(v[i + 1])
             : "r"(w[i]), "r"(w[i + 1]));
+}
+
+// v[0 .. 3] *= l, two at a time
+__device__ __forceinline__ void mul_quad(uint32_t *v, float4 l)
+{
+    const float2 a = unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[0]), __uint_as_float(v[1])), pack_f32x2(l.x, l.y)));
+    const float2 b = unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(v[2]), __uint_as_float(v[3])), pack_f32x2(l.z, l.w)));
+    v[0] = __float_as_uint(a.x), v[1] = __float_as_uint(a.y), v[2] = __float_as_uint(b.x), v[3] = __float_as_uint(b.y);
 }
 
 // bit patterns of v0 rs + magic, v1 rs + magic

@@ -191,6 +191,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
         : "memory");
 }
 
+// Says behind a tmem_ld_wait() that these values have arrived: what uses them stays behind it, also where other work stands between
+// the request and the wait.
+template <int N>
+__device__ __forceinline__ void tmem_loaded(uint32_t (&r)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; i += 4) asm volatile("" : "+r"(r[i]), "+r"(r[i + 1]), "+r"(r[i + 2]), "+r"(r[i + 3]));
+}
+
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // 16 consecutive columns of this thread's tensor-memory lane

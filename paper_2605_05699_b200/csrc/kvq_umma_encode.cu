@@ -610,6 +610,10 @@ bool umma_encode_bits8_supported(int D, bool bf16) { return !(D == 256 && bf16) 
 cudaError_t umma_encode(int D, bool bf16, bool per_vector, int64_t N, const FftParams &f, const float *e0, cudaStream_t stream)
 {
     if (!tensor_map_encode_fn()) return cudaErrorNotSupported;
+    if (umma_append_pays(D, bf16, per_vector, N, f)) {
+        const cudaError_t e = umma_append(D, per_vector, N, f, stream);
+        if (N > 0 || e != cudaSuccess) return e;   // kvq_plan_prepare: both
+    }
     if (D == 256) return umma_encode_d256(bf16, per_vector, N, f, e0, stream);   // its own kernel: CTA pairs, x through a ring of K blocks
     if (bf16 && f.bits == 8) {   // three bf16 terms
         switch (D) {

@@ -227,6 +227,38 @@ def test_d256_encode_at_the_edges_of_a_cta_pair_tile(dtype, N, n_lambda, rpl):
     assert enc["mismatches"] <= max(2, int(1e-4 * N * 256))
 
 
+def run_append(D, S, n_lambda, spl, per_vector=False, nbits=4):
+    """An fp16 append on the tensor cores into row 1 of three, against the oracle."""
+    plan = kb.Plan(D, D if per_vector else G, 6, bits=nbits)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_AUTO)
+    x, lam = wl.make_vectors(S, D, "f16", "k_outlier", 19 + S), wl.make_lambda(n_lambda, D, 20)
+    packed = torch.full((S, 3, D * nbits // 8), 0xAB, dtype=torch.uint8, device="cuda")
+    scales = torch.full((S, 3, D // plan.group), 1.25, dtype=torch.float16, device="cuda")
+    kb.kvq_append(plan.handle, x.cuda(), lam.cuda(), packed, scales, 1, spl)
+    torch.cuda.synchronize()
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    assert bool((packed[:, [0, 2]] == 0xAB).all()) and bool((scales[:, [0, 2]] == 1.25).all())
+    ora = ko.encode(bits(x), ko.F16, plan.signs(), lam.numpy(), plan.group, spl, want_v=True, bits=nbits)
+    parity.check_encode(packed[:, 1].contiguous().cpu().numpy(), bits(scales[:, 1].contiguous()), ora, plan.group, "append", bits=nbits, min_agree=0.9995)
+    plan.close()
+
+
+@pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
+@pytest.mark.parametrize("S,n_lambda,spl", [(1, 1, 0), (127, 127, 1), (129, 4, 33), (300, 2, 299), (148 * 128, 1, 0), (148 * 128 + 1, 300, 64),
+                                            (2 * 148 * 128 + 65, 3, 12700)])
+def test_append_at_the_edges_of_its_tiles(D, S, n_lambda, spl):
+    """Lambda rows of one vector, of a part of a warp, that end inside tiles; a tile per CTA, one more, three for one of them."""
+    run_append(D, S, n_lambda, spl)
+
+
+@pytest.mark.parametrize("D,per_vector,nbits,tiles", [(64, False, 4, 370), (64, True, 4, 222), (96, True, 8, 370), (160, False, 8, 592), (160, True, 4, 370),
+                                                      (256, True, 4, 100)])
+def test_append_on_both_sides_of_its_limit(D, per_vector, nbits, tiles):
+    """The longest call of the append kernel and one vector more, and a layout that it is not built for."""
+    for S in (tiles * 128, tiles * 128 + 1):
+        run_append(D, S, 1, 0, per_vector, nbits)
+
+
 @pytest.mark.parametrize("D,dtype,nbits", [(64, "f16", 4), (96, "bf16", 4), (128, "f16", 4), (128, "bf16", 8), (160, "f16", 4), (160, "bf16", 4), (256, "f16", 4)])
 @pytest.mark.parametrize("rpl,n_lambda", [(104, 450), (200, 450), (504, 230)])
 def test_decode_under_lambda_rows_of_a_few_tiles_equals_one_call_per_row(D, dtype, nbits, rpl, n_lambda):
