@@ -2,21 +2,22 @@
 // tcgen05.ld delivers them -> largest magnitude -> fp16 scale -> round-to-nearest-even codes -> packed words.
 //
 // These kernels run at the board's power limit, where a warp instruction costs about a nanojoule, so the count is what matters:
-// the magnitudes take one instruction each (max.xorsign.abs carries the absolute value for free), sums and products of
+// the magnitudes take half an instruction each (max.abs of three: the absolute values are free), sums and products of
 // neighbouring values go in pairs (add / fma.f32x2, rounded like the single ones), the codes are gathered by byte permutes.
 // Encode of 2,097,152 vectors at D = 128, back to back: 183.1 -> 180.2 us (another box: 182.7 -> 181.1, inside the spread); D = 160, 700,000:
-// 97.5 -> 93.4; D = 256, 1,064,960: 269 -> 266.
+// 97.5 -> 93.4; D = 256, 1,064,960: 269 -> 266.  With the maxima three at a time instead of two: 2,097,152 at D = 128 179.5 -> 177.8,
+// 212,992 bf16 under 52 lambda rows at D = 256 59.6 -> 59.2.
 #pragma once
 
 #include "kvq_device.cuh"
 
 namespace kvq {
 
-// max(|a|, |b|) with a meaningless sign; like fmaxf a NaN yields the other operand
-__device__ __forceinline__ float max_magnitude(float a, float b)
+// max(|a|, |b|, |c|); like fmaxf a NaN yields to the other operands
+__device__ __forceinline__ float max_magnitude(uint32_t a, uint32_t b, uint32_t c)
 {
     float d;
-    asm("max.xorsign.abs.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(__uint_as_float(a)), "f"(__uint_as_float(b)), "f"(__uint_as_float(c)));
     return d;
 }
 
@@ -24,11 +25,14 @@ __device__ __forceinline__ float group_absmax(const uint32_t (&v)[32])
 {
     float m[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) m[i] = max_magnitude(__uint_as_float(v[i]), __uint_as_float(v[i + 4]));   // four chains of eight
+    for (int i = 0; i < 4; ++i) m[i] = max_magnitude(v[i], v[i + 4], v[i + 8]);   // four chains of eight
 #pragma unroll
-    for (int i = 8; i < 32; ++i) m[i & 3] = max_magnitude(m[i & 3], __uint_as_float(v[i]));
-    const float a = fabsf(max_magnitude(max_magnitude(m[0], m[1]), max_magnitude(m[2], m[3])));
-    return fmaxf(a, 0.0f);   // 0 where every value is a NaN
+    for (int i = 12; i < 28; i += 8)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) m[k] = max_magnitude(__float_as_uint(m[k]), v[i + k], v[i + 4 + k]);
+    m[0] = max_magnitude(__float_as_uint(m[0]), v[28], v[29]);
+    m[1] = max_magnitude(__float_as_uint(m[1]), v[30], v[31]);
+    return fmaxf(max_magnitude(__float_as_uint(m[0]), __float_as_uint(m[1]), __float_as_uint(fmaxf(m[2], m[3]))), 0.0f);   // 0 where every value is a NaN
 }
 
 // v[i] += w[i], two at a time
