@@ -80,19 +80,20 @@ static double build_b0(const kvq_plan *p, float *b0)
     return tmax;
 }
 
-// Host copies of both tables: b0 [n][c] for the decode kernels, its transpose e0 [c][n] for the encode kernels.
-static bool make_tables(kvq_plan *p, std::vector<float> &b0, std::vector<float> &e0)
+// Host copy of both tables, one behind the other as on the device: b0 [n][c] for the decode kernels, its transpose e0 [c][n] for the
+// encode kernels.
+static bool make_tables(kvq_plan *p, std::vector<float> &both)
 {
     const size_t D = (size_t)p->D;
     try {
-        b0.resize(D * D);
-        e0.resize(D * D);
+        both.resize(2 * D * D);
+        float *b0 = both.data(), *e0 = b0 + D * D;
+        p->table_max = (float)build_b0(p, b0);
+        for (size_t n = 0; n < D; ++n)
+            for (size_t c = 0; c < D; ++c) e0[c * D + n] = b0[n * D + c];
     } catch (...) {
         return false;
     }
-    p->table_max = (float)build_b0(p, b0.data());
-    for (size_t n = 0; n < D; ++n)
-        for (size_t c = 0; c < D; ++c) e0[c * D + n] = b0[n * D + c];
     return true;
 }
 
@@ -112,8 +113,8 @@ static kvq_status_t ensure_device(kvq_plan *p)
     constexpr size_t kStatusBytes = 256;
     const bool tables = umma_encode_supported(p->D, false) || umma_decode_supported(p->D, false);
     const size_t bytes = tables ? sizeof(float) * (size_t)p->D * p->D : 0, total = kStatusBytes + (tables ? 2 * bytes + operand_bytes(p->D) : 0);
-    std::vector<float> b0, e0;
-    if (tables && !make_tables(p, b0, e0)) return KVQ_ERR_NOMEM;
+    std::vector<float> host;
+    if (tables && !make_tables(p, host)) return KVQ_ERR_NOMEM;
     unsigned char *mem = nullptr;
     if (cudaMalloc(&mem, total) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -123,8 +124,7 @@ static kvq_status_t ensure_device(kvq_plan *p)
     unsigned char *dw = mem + kStatusBytes + 2 * bytes;
     bool ok = cudaMemset(mem, 0, kStatusBytes) == cudaSuccess;
     if (ok && tables)
-        ok = cudaMemcpy(db, b0.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
-             cudaMemcpy(de, e0.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess && build_encode_operands(p->D, de, p->table_max, dw) == cudaSuccess;
+        ok = cudaMemcpy(db, host.data(), 2 * bytes, cudaMemcpyHostToDevice) == cudaSuccess && build_encode_operands(p->D, de, p->table_max, dw) == cudaSuccess;
     if (!ok) {
         (void)cudaGetLastError();
         cudaFree(mem);
@@ -263,11 +263,9 @@ kvq_status_t kvq_plan_set_rotation(kvq_plan_t *plan, const float *R_host)
         (void)cudaGetLastError();
         return KVQ_ERR_INVALID_ARG;
     }
-    std::vector<float> b0, e0;
-    if (!make_tables(plan, b0, e0)) return KVQ_ERR_NOMEM;
-    const size_t bytes = sizeof(float) * n;
-    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(plan->d_b0, b0.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(plan->d_e0, e0.data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess ||
+    std::vector<float> host;
+    if (!make_tables(plan, host)) return KVQ_ERR_NOMEM;
+    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(plan->d_b0, host.data(), 2 * sizeof(float) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
         build_encode_operands(plan->D, plan->d_e0, plan->table_max, plan->d_operands) != cudaSuccess) {
         (void)cudaGetLastError();
         return KVQ_ERR_CUDA;
