@@ -118,6 +118,15 @@ struct Cfg {
     static constexpr int kQuads = D / 4;                   // float4 per table row
     static constexpr uint32_t kIdesc = umma_idesc_m128(R2 ? D / 2 : D, false);
     static constexpr int kBRows = R2 ? D / 2 : D;          // rows of the plan table that B is built from
+    // The radix-2 epilogue's sums and differences two at a time (add / fma.f32x2): 2,097,152 fp16 vectors at D = 128 128.3 -> 126.0 us,
+    // 300,000: 21.0 -> 20.4.  With bf16 output, where a CTA waits for its operands and not for its instructions, single ones: 60,000 vectors
+    // at D = 96 9.1, in pairs 9.3; 1,000,000 at D = 160 117 and 123.
+    static constexpr bool kPairs = !BF16OUT;
+    // The dequant and epilogue loops rolled: five unrolled groups of two-term operands stream a warp through more code than the instruction
+    // caches hold beside the other roles' (a warp waits for an instruction 1.2 to 1.4 times per issue).  D = 160, bf16, 18,944 vectors
+    // 10.9 -> 10.1 us, 300,000: 40.6 -> 39.4, 1,000,000: 117 -> 108; encode + decode of 99,993 under three lambda rows 38.0 -> 35.7.
+    // (60,000 and 128,000 in a row of decodes alone: the same within 1 %.)  The other forms' loops are short enough: rolled they are 2 to 5 % slower.
+    static constexpr bool kRolled = R2 && BF16OUT && D == 160;
 };
 
 struct Ctrl {
@@ -538,8 +547,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int s = j % kInStages, sa = j % C::kAStages, sb = j % C::kABars;
             if (!wait_or_abort(smem_u32(&ctrl->in_full[s]), (uint32_t)(j / kInStages) & 1u, abort_flag, status, KVQ_DEV_LOAD_TIMEOUT)) break;
             const unsigned char *row = sIn + s * C::kInPitch + r * C::kInRow;
-            uint4 pk[BITS == 4 ? G : 1];
-            if constexpr (BITS == 4) {
+            constexpr bool kAllCodes = BITS == 4 && !C::kRolled;   // the whole row's codes at once, or group by group
+            uint4 pk[kAllCodes ? G : 1];
+            if constexpr (kAllCodes) {
 #pragma unroll
                 for (int c = 0; c < G; ++c) pk[c] = *reinterpret_cast<const uint4 *>(row + (((uint32_t)c ^ swz) << 4));
                 __syncwarp();
@@ -562,9 +572,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- nibbles -> fp16 codes -> times sigma * rho, two codes per instruction
             const uint32_t a_row = tmem_base + ((uint32_t)(q * 32) << 16) + C::a_col(sa);
             const __half2 h1032 = __float2half2_rn(1032.0f);
-#pragma unroll
+#pragma unroll(C::kRolled ? 1 : G)
             for (int c = 0; c < G; ++c) {   // chunk c = group c: 32 codes, 16 tensor-memory columns
-                const float sig = __half2float(__ushort_as_half((unsigned short)((sc[c >> 1] >> (16 * (c & 1))) & 0xFFFFu)));
+                uint32_t sc16 = sc[0];
+                if constexpr (C::kRolled) {
+#pragma unroll
+                    for (int i = 0; i < (G + 1) / 2; ++i) sc[i] = (sc[i] >> 16) | (i + 1 < (G + 1) / 2 ? sc[i + 1] << 16 : 0u);   // the next group's to the front
+                } else {
+                    sc16 = sc[c >> 1] >> (16 * (c & 1));
+                }
+                const float sig = __half2float(__ushort_as_half((unsigned short)(sc16 & 0xFFFFu)));
                 const __half2 s2 = __float2half2_rn(sig * rho * pw);
                 uint32_t a[16], al[BF16OUT ? 16 : 1];
                 auto put = [&](int k, __half2 q2) {   // K-pair k of the group: one rounding, and what it left behind
@@ -576,7 +593,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 };
                 if constexpr (BITS == 4) {
-                    const uint32_t words[4] = {pk[c].x, pk[c].y, pk[c].z, pk[c].w};
+                    uint4 pc;
+                    if constexpr (kAllCodes) pc = pk[c];
+                    else pc = *reinterpret_cast<const uint4 *>(row + (((uint32_t)c ^ swz) << 4));
+                    const uint32_t words[4] = {pc.x, pc.y, pc.z, pc.w};
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const uint32_t u = words[i] ^ 0x88888888u;   // nibbles now hold q + 8
@@ -620,7 +640,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if constexpr (BF16OUT) tmem_st16(a_row + C::kALo + 16u * (uint32_t)c, al);
                 }
             }
-            if constexpr (BITS == 8) {   // the packed rows were read group by group: only now is their stage free
+            if constexpr (!kAllCodes) {   // the packed rows were read group by group: only now is their stage free
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->in_empty[s]));
             }
@@ -646,7 +666,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const float row_inv = ctrl->row_scale[j & (kRowScaleSlots - 1)][q * 32 + lane];
             const bool rescale = __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
             if constexpr (R2) {
-#pragma unroll
+#pragma unroll(C::kRolled ? 1 : D / 32)
                 for (int h = 0; h < D / 32; ++h) {   // E and O columns 16 h .. 16 h + 15 -> outputs 16 h .. and D / 2 + 16 h ..
                     uint32_t ev[16], ov[16];
                     tmem_ld16(lane_addr + C::acc_col(sc) + (uint32_t)h * 16u, ev);
@@ -670,10 +690,17 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                         for (int p2 = 0; p2 < 4; ++p2) {
                             const int i = 8 * k + 2 * p2;
-                            const float e0 = __uint_as_float(ev[i]), e1 = __uint_as_float(ev[i + 1]);
-                            const float o0 = __uint_as_float(ov[i]), o1 = __uint_as_float(ov[i + 1]);
-                            lo[p2] = narrow2<BF16OUT>(e0 + o0, e1 + o1);                                     // s_n is already in E and O
-                            hi[p2] = narrow2<BF16OUT>(e0 - o0, e1 - o1) ^ prm.flip2[8 * h + 4 * k + p2];     // times s_n s_{n + D/2}
+                            const float2 e = make_float2(__uint_as_float(ev[i]), __uint_as_float(ev[i + 1]));
+                            const float2 o = make_float2(__uint_as_float(ov[i]), __uint_as_float(ov[i + 1]));
+                            float2 sum, diff;
+                            if constexpr (C::kPairs) {
+                                const uint64_t ep = pack_f32x2(e.x, e.y), op = pack_f32x2(o.x, o.y);
+                                sum = unpack_f32x2(add_f32x2(ep, op)), diff = unpack_f32x2(sub_f32x2(ep, op));
+                            } else {
+                                sum = make_float2(e.x + o.x, e.y + o.y), diff = make_float2(e.x - o.x, e.y - o.y);
+                            }
+                            lo[p2] = narrow2<BF16OUT>(sum.x, sum.y);                                          // s_n is already in E and O
+                            hi[p2] = narrow2<BF16OUT>(diff.x, diff.y) ^ prm.flip2[8 * h + 4 * k + p2];       // times s_n s_{n + D/2}
                         }
                         // 16-byte chunk c of the row: a 64-column box [32 rows][128 B] of 128-byte swizzle, or the last, 32-column one
                         auto at = [&](int c) -> uint4 * {
