@@ -189,11 +189,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * kD; };
 
-    grid_wait();
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    grid_wait();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile uint32_t *abort_flag = &ctrl->abort;
     uint32_t *status = prm.g.status;

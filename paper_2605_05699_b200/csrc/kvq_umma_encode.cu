@@ -116,8 +116,7 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
             mx = fmaxf(mx, fmaxf(fmaxf(fabsf(l.x), fabsf(l.y)), fmaxf(fabsf(l.z), fabsf(l.w))));
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    mx = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx)));   // non-negative: ordered like its bits
     mx = fminf(fmaxf(mx * table_max, 1e-30f), 1e30f);   // table_max: largest |entry| of the table
     const int e = (int)((__float_as_uint(mx) >> 23) & 0xFFu) - 127;      // floor(log2 mx)
     return __uint_as_float((uint32_t)(127 + 13 - e) << 23);
