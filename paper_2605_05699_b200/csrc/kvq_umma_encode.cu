@@ -97,7 +97,7 @@ struct Ctrl {
     uint32_t tmem_base;
     volatile uint32_t abort;
     uint32_t pad[2];
-    float rowmax[2][2][2][kTile];   // [tile parity within the set][set][half row][row]
+    float rowmax[8 * kTile];    // [tile parity within the set][set][half row][row], or [quarter][row] of a CTA's only tile
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 
@@ -256,6 +256,16 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+    // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range per CTA
+    const int64_t N = prm.N, rpl = prm.rpl;
+    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x);
+    const int64_t tps = share.tps, tile_begin = share.begin;
+    const int n_my = share.n;
+    // One tile: both sets of epilogue warps share it, four threads to a row.  Back to back, 8000 vectors: D = 96 5.0 -> 4.4 us, 128 5.9 -> 5.3,
+    // 160 7.1 -> 6.6 (one scale per vector 7.2 -> 6.8); 18,944: 6.2 -> 5.7, 7.1 -> 6.7, 8.7 -> 8.1.  Not at D = 64, which has two groups, one for
+    // each half row, as it is, nor with one scale per vector at D = 128, where calls of seven tiles per CTA lose 2 % to the longer loop.
+    const bool solo = D > 64 && !(PERVEC && D == 128) && n_my == 1;
+
     if (threadIdx.x == 0) {
         for (int s = 0; s < kInStages; ++s) mbar_init(smem_u32(&ctrl->in_full[s]), 1);
         for (int s = 0; s < kFullBars; ++s) mbar_init(smem_u32(&ctrl->acc_full[s]), 1);
@@ -263,17 +273,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(smem_u32(&ctrl->b_first), kEpiWarps);       // first B: all epilogue warps build it
         mbar_init(smem_u32(&ctrl->b_ready), kEpiWarps / 2);   // later rebuilds: the set that owns the tile
         for (int s = 0; s < 2; ++s)
-            for (int qq = 0; qq < 4; ++qq) mbar_init(smem_u32(&ctrl->pair[s][qq]), 2);
+            for (int qq = 0; qq < 4; ++qq) mbar_init(smem_u32(&ctrl->pair[s][qq]), solo ? 4 : 2);
         ctrl->abort = 0u;
         mbar_init_fence();
     }
     if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
-
-    // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range per CTA
-    const int64_t N = prm.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x);
-    const int64_t tps = share.tps, tile_begin = share.begin;
-    const int n_my = share.n;
 
     // ---- B for the CTA's first lambda row, by all epilogue warps.  The table is requested and the set-up barrier passed in front of the
     // ---- grid wait, under the grid ahead; lambda and the first x loads follow it side by side.  (With the barrier behind lambda, its round
@@ -388,13 +392,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         // =========================== epilogue: accumulator -> scales, codes, nibbles ===========================
         // Two sets of eight warps take alternate tiles, so that one set's waits (barrier, tensor-memory load)
         // hide behind the other set's arithmetic.  Thread = (row, half row).
-        const int set = (warp - 2) >> 3;        // this set takes tiles set, set + 2, ...
+        const int set = solo ? 0 : (warp - 2) >> 3;   // this set takes tiles set, set + 2, ...
         const int q = warp & 3;                 // tensor-memory lane quarter this warp may touch
-        const int h = ((warp - 2) >> 2) & 1;    // half of the row
+        const int h = solo ? (warp - 2) >> 2 : ((warp - 2) >> 2) & 1;   // half of the row (a quarter of it)
         const int r = q * 32 + lane;            // tile row of this thread
         const int bw = (warp - 2) & 7;          // position within the set, for the quads of a rebuild of B
-        const int g0 = h * C::kGroupsPerPart;                                        // this thread's groups: g0 .. g1 - 1
-        const int g1 = h == 0 ? C::kGroupsPerPart : G;
+        const int g0 = solo ? h * G / 4 : h * C::kGroupsPerPart;                      // this thread's groups: g0 .. g1 - 1
+        const int g1 = solo ? (h + 1) * G / 4 : h == 0 ? C::kGroupsPerPart : G;
         const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16);
         int64_t cached_seg = first_seg;           // B holds this row's table (built above)
         float unlift = 1.0f / first_lift;
@@ -459,11 +463,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 const int it = (j - set) >> 1;   // this set's tile count: parity of the pair barrier and of the buffer
-                ctrl->rowmax[it & 1][set][h][r] = m;
+                float *slot = &ctrl->rowmax[((it & 1) * 2 + set) * 2 * kTile + r];   // this row's of the half rows (the quarters: all of them)
+                slot[h * kTile] = m;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&ctrl->pair[set][q]));
                 if (!wait_or_abort(smem_u32(&ctrl->pair[set][q]), (uint32_t)it & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
-                m = fmaxf(m, ctrl->rowmax[it & 1][set][h ^ 1][r]);
+                m = fmaxf(slot[0], slot[kTile]);
+                if (solo) m = fmaxf(m, fmaxf(slot[2 * kTile], slot[3 * kTile]));
                 row_scale = group_scale(m, unlift, Q, inv_q);
                 if (live && h == 0) prm.scales[orow] = row_scale.half;
             }
@@ -475,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (g < g1) {
                     uint32_t vb[32];
                     load_group(sc, g, vb);
-                    if (g == g1 - 1) {   // this thread's last group is in registers: hand the accumulator back
+                    if (g == g1 - 1 && !solo) {   // this thread's last group is in registers: hand the accumulator back
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty[sc]));
@@ -502,7 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                     }
                     if constexpr (!PERVEC) {
-                        if (!kPairScales) {
+                        if (!kPairScales || solo) {
                             if (live) prm.scales[orow * G + g] = gs.half;
                         } else if (gi == 1) {
                             if (live) *reinterpret_cast<uint32_t *>(prm.scales + orow * G + g0) = scale_pair;

@@ -259,6 +259,21 @@ def test_append_on_both_sides_of_its_limit(D, per_vector, nbits, tiles):
         run_append(D, S, 1, 0, per_vector, nbits)
 
 
+@pytest.mark.parametrize("D,dtype,per_vector,nbits", [(64, "f16", False, 4), (64, "bf16", True, 4), (96, "f16", True, 8), (96, "bf16", False, 4),
+                                                      (128, "f16", False, 8), (128, "bf16", True, 4), (160, "f16", True, 4), (160, "bf16", False, 4)])
+@pytest.mark.parametrize("N,n_lambda,rpl", [(1, 1, 0), (148 * 128, 1, 0), (148 * 128 + 1, 1, 0), (9000, 150, 60)])
+def test_encode_of_one_tile_per_cta(D, dtype, per_vector, nbits, N, n_lambda, rpl):
+    """A CTA's only tile is shared by all epilogue warps, a CTA with two gives each set one: one row, a tile for every CTA, two for one
+    of them; a short tile per lambda row, for some CTAs two."""
+    plan = kb.Plan(D, D if per_vector else G, 91, bits=nbits)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_AUTO)
+    lam, x = wl.make_lambda(n_lambda, D, 92), wl.make_vectors(N, D, dtype, "k_outlier", 93 + N)
+    packed, scales = gpu_encode(plan, x.cuda(), lam.cuda(), rpl)
+    ora = ko.encode(bits(x), DT[dtype], plan.signs(), lam.numpy(), plan.group, rpl, want_v=True, bits=nbits)
+    parity.check_encode(packed.cpu().numpy(), bits(scales), ora, plan.group, "one tile per CTA", bits=nbits, min_agree=0.999 if N == 1 else 0.9995)
+    plan.close()
+
+
 @pytest.mark.parametrize("D,dtype,nbits", [(64, "f16", 4), (96, "bf16", 4), (128, "f16", 4), (128, "bf16", 8), (160, "f16", 4), (160, "bf16", 4), (256, "f16", 4)])
 @pytest.mark.parametrize("rpl,n_lambda", [(104, 450), (200, 450), (504, 230)])
 def test_decode_under_lambda_rows_of_a_few_tiles_equals_one_call_per_row(D, dtype, nbits, rpl, n_lambda):
