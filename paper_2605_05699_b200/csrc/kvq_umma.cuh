@@ -265,11 +265,12 @@ __device__ __forceinline__ float operand_rescue(const uint32_t (&sc)[(G + 1) / 2
     return __uint_as_float((uint32_t)(127 + 7 - e) << 23);
 }
 
-// 1 / max(lambda, 1e-6) for the channels this lane covers (4 i .. 4 i + 3, i = lane and, for D > 128, lane + 32),
-// divided by rho, the power of two that brings the row's largest reciprocal into [1, 2).  Every lane gets rho.
-template <int D>
+// 1 / max(lambda, 1e-6) for the channels this lane covers (4 i .. 4 i + 3, i = lane and, for D > 128, lane + 32; NEIGHBOURS: i = 2 lane and
+// 2 lane + 1), divided by rho, the power of two that brings the row's largest reciprocal into [1, 2).  Every lane gets rho.
+template <int D, bool NEIGHBOURS = false>
 struct RecipLambda {
     static constexpr int kPasses = (D / 4 + 31) / 32;
+    static_assert(!NEIGHBOURS || D == 256, "two quads for every lane");
     float4 r[kPasses];
     float rho;
     bool wide;   // the reciprocals span more than 2^8: B, which carries them in fp16 next to each other, loses bits on the small ones
@@ -278,7 +279,7 @@ struct RecipLambda {
         float mx = 0.0f, mn = 3.0e38f;
 #pragma unroll
         for (int p = 0; p < kPasses; ++p) {
-            const int i = lane + 32 * p;
+            const int i = NEIGHBOURS ? 2 * lane + p : lane + 32 * p;
             r[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (i < D / 4) {
                 const float4 l = load_input(reinterpret_cast<const float4 *>(lam) + i);

@@ -86,42 +86,63 @@ struct Ctrl {
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 
-// Rows [n0, n1) (outputs n < 128) of the B operand of parity p (0: E GEMM, even channels; 1: O GEMM), by one warp.
-// The table row b0[n][c] = s_n M[c][n] is used as it is: the accumulators then hold s_n E_n and s_n O_n.  Lanes 2w and 2w + 1 hold
-// channels 8w .. 8w + 7; the K order inside a word is the one the nibble trick produces, pairs (c, c + 4): the even
-// lane assembles the pair (8w + p, 8w + p + 4), the odd lane (8w + p + 2, 8w + p + 6), each from one value of its
-// own and one of its neighbour's.  Terms: fp16(W'), then what that left behind.
+// Row n (output n < 128) of the B operand of parity p (0: E GEMM, even channels; 1: O GEMM), by one warp: lane w has channels 8w .. 8w + 7 of
+// the table row b0[n][c] = s_n M[c][n] in m0 and m1.  The table is used as it is: the accumulators then hold s_n E_n and s_n O_n.  The K
+// order inside a word of eight codes is the one the nibble trick produces: pairs (8w + p, 8w + p + 4), (8w + p + 2, 8w + p + 6).
+// Terms: fp16(W'), then what that left behind.
+typedef RecipLambda<kD, true> Recip;
+
 template <int TERMS>
-__device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__restrict__ b0, const RecipLambda<kD> &rl, int p, int n0, int n1, int lane)
+__device__ __forceinline__ void put_b_row(unsigned char *sB, const float4 m0, const float4 m1, const Recip &rl, int p, int n, int lane)
 {
-    const bool odd = lane & 1;
+    auto sat = [](float v) { return fminf(fmaxf(v, -65504.0f), 65504.0f); };
+    const float4 r0 = rl.r[0], r1 = rl.r[1];
+    float w[4] = {sat(p ? m0.y * r0.y : m0.x * r0.x), sat(p ? m1.y * r1.y : m1.x * r1.x), sat(p ? m0.w * r0.w : m0.z * r0.z), sat(p ? m1.w * r1.w : m1.z * r1.z)};
+    const int ch = lane >> 1;   // 16-byte chunk of the K-major row: K block ch / 8, chunk ch % 8
+    unsigned char *dst = sB + p * kBPart + (ch >> 3) * kBBlock + n * 128 + (((ch & 7) ^ (n & 7)) << 4) + (lane & 1) * 8;
+#pragma unroll
+    for (int t = 0; t < TERMS; ++t) {
+        const uint32_t h0 = narrow2<false>(w[0], w[1]), h1 = narrow2<false>(w[2], w[3]);
+        *reinterpret_cast<uint2 *>(dst + t * (2 * kBPart)) = make_uint2(h0, h1);
+        if (t + 1 < TERMS) {   // what the fp16 term left behind (exact in fp32)
+            const float2 a = widen2<false>(h0), b = widen2<false>(h1);
+            w[0] -= a.x, w[1] -= a.y, w[2] -= b.x, w[3] -= b.y;
+        }
+    }
+}
+
+// The first B: eight rows of both parities per builder warp, requested in front of the grid wait and all together.  (Before, a warp took
+// sixteen rows of one parity in two round trips behind lambda, and every row crossed L2 for each parity.  Back to back, 1500 fp16
+// vectors 9.7 -> 7.6 us, 10,000: 10.3 -> 8.9; bf16 11.1 -> 9.5, 12.0 -> 11.0; 212,992: 36.9 -> 33.9, 48.9 -> 46.9.)
+constexpr int kFirstRows = kHalf / 16;
+struct FirstRows {
+    float4 m[kFirstRows][2];
+    __device__ __forceinline__ void load(const float *__restrict__ b0, int n0, int lane)
+    {
+#pragma unroll
+        for (int k = 0; k < kFirstRows; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) m[k][h] = __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)(n0 + k) * kD) + 2 * lane + h);
+    }
+    template <int TERMS>
+    __device__ __forceinline__ void store(unsigned char *sB, const Recip &rl, int n0, int lane) const
+    {
+#pragma unroll
+        for (int k = 0; k < kFirstRows; ++k)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) put_b_row<TERMS>(sB, m[k][0], m[k][1], rl, p, n0 + k, lane);
+    }
+};
+
+// Rows [n0, n1) of one parity, by one warp: a dequant group's rebuild of its own operand.
+template <int TERMS>
+__device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__restrict__ b0, const Recip &rl, int p, int n0, int n1, int lane)
+{
 #pragma unroll 8   // 16 row quads in flight per lane: the build is a chain of L2 round trips, not arithmetic
     for (int n = n0; n < n1; ++n) {
-#pragma unroll
-        for (int ps = 0; ps < 2; ++ps) {
-            const int i = lane + 32 * ps;
-            const float4 m = __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)n * kD) + i);
-            auto sat = [](float v) { return fminf(fmaxf(v, -65504.0f), 65504.0f); };
-            // this lane's two channels of parity p: 4 i + p and 4 i + p + 2
-            const float v0 = sat((p ? m.y : m.x) * (p ? rl.r[ps].y : rl.r[ps].x));
-            const float v2 = sat((p ? m.w : m.z) * (p ? rl.r[ps].w : rl.r[ps].z));
-            // even lane (channels 8w ..): keeps v0 = 8w + p, needs the odd lane's v0 = 8w + p + 4
-            // odd lane (channels 8w + 4 ..): keeps v2 = 8w + p + 6, needs the even lane's v2 = 8w + p + 2
-            const float got = __shfl_xor_sync(0xFFFFFFFFu, odd ? v0 : v2, 1);
-            float w0 = odd ? got : v0, w1 = odd ? v2 : got;
-            const int wd = i >> 1;   // word of 8 codes: columns 2 wd (even lane) and 2 wd + 1 (odd lane) of the K-major row
-            const int ch = wd >> 1;  // 16-byte chunk: K block ch / 8, chunk ch % 8
-            const uint32_t off = (uint32_t)(p * kBPart + (ch >> 3) * kBBlock + n * 128 + (((ch & 7) ^ (n & 7)) << 4) + ((wd & 1) ? 8 : 0) + (odd ? 4 : 0));
-#pragma unroll
-            for (int t = 0; t < TERMS; ++t) {
-                const uint32_t h = narrow2<false>(w0, w1);
-                *reinterpret_cast<uint32_t *>(sB + t * (2 * kBPart) + off) = h;
-                if (t + 1 < TERMS) {   // what the fp16 term left behind (exact in fp32)
-                    const float2 a = widen2<false>(h);
-                    w0 -= a.x, w1 -= a.y;
-                }
-            }
-        }
+        const float4 m0 = __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)n * kD) + 2 * lane);
+        const float4 m1 = __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)n * kD) + 2 * lane + 1);
+        put_b_row<TERMS>(sB, m0, m1, rl, p, n, lane);
     }
 }
 
@@ -189,6 +210,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * kD; };
 
+    FirstRows rows;
+    const bool builds_first = n_my > 0 && warp >= 2;
+    if (builds_first) rows.load(prm.g.b0, (warp - 2) * kFirstRows, lane);
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
@@ -198,13 +222,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile uint32_t *abort_flag = &ctrl->abort;
     uint32_t *status = prm.g.status;
 
-    // ---- B for the first tile's lambda row: of the sixteen dequant and epilogue warps, eight build the E operand
-    // ---- and eight the O operand, sixteen rows each
+    // ---- B for the first tile's lambda row, by the sixteen dequant and epilogue warps
     // ---- (the dequant warps request their first tile's scales before the build and keep rho from it, so that neither
     // ---- costs a round trip to L2 after it)
     float rho_first = 1.0f;
     uint4 sc_first = make_uint4(0u, 0u, 0u, 0u);
-    if (n_my > 0 && warp >= 2) {
+    if (builds_first) {
         if (warp < 10) {
             const TileCursor first(tile_begin, tps);
             const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
@@ -217,11 +240,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
-        const RecipLambda<kD> rl(lambda_row(seg_first), lane);
+        const Recip rl(lambda_row(seg_first), lane);
         rho_first = rl.rho;
         if (rl.wide) ctrl->any_wide = 1u;
-        const int bp = ((warp - 2) >> 2) & 1, bw = ((warp - 2) & 3) + 4 * ((warp - 2) >> 3);   // parity, position among its eight
-        build_b_rows<kTerms>(sB, prm.g.b0, rl, bp, bw * 16, bw * 16 + 16, lane);
+        rows.store<kTerms>(sB, rl, (warp - 2) * kFirstRows, lane);
         fence_proxy_async();   // B is read by the tensor core through the async proxy
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
@@ -324,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- a new lambda row: new rho, and this group rebuilds the B operand of its own GEMM once every MMA of that
             // ---- GEMM issued so far is complete: the previous tile's, on this group's own barriers (it sees every phase)
             if (prm.g.lambda_index(seg) != cached_row) {
-                const RecipLambda<kD> rl(lambda_row(seg), lane);
+                const Recip rl(lambda_row(seg), lane);
                 if (rl.wide) ctrl->any_wide = 1u;
                 rho = rl.rho;
                 if (!wait_or_abort(smem_u32(&ctrl->a_empty[p][(j - 1) % C::kAStages]), (uint32_t)((j - 1) / C::kAStages) & 1u, abort_flag,
