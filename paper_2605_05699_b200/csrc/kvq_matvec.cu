@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(kWarps * 32) kvq_decode_matvec_kernel(const __
 // dequantized values of the window flush, goes through distributed shared memory; the CTAs of a batch are then a cluster (two or four:
 // D = 96 and 160 would be three and five, and stay with the form above there).
 // A CTA takes one batch, and the form is taken while the device holds all of them at once; beyond that the copies of
-// the staging and the barriers cost more than they save.
+// the staging and the barriers cost more than they save.  sliced_tenths says where that is.
 template <int D>
 struct Slice {
     static constexpr int W = D == 256 ? 64 : 32, kSlices = D / W;   // coordinates per slice
@@ -563,6 +563,18 @@ __global__ void __launch_bounds__(kWarps * 32, D == 256 ? 1 : 2) kvq_decode_matv
 }
 
 // MODE: 0 decode, 1 encode, 2 encode + decode of the same rows (window flush)
+
+// CTAs of the sliced form per ten SMs up to which a call takes it.  Two per SM fit (D = 256: one), and without clusters that is the
+// limit but for the decode at D = 64, whose two halves share little (528 vectors 2.58 -> 2.21 us, 648 2.59 -> 2.52, 824 2.60 -> 2.69).  Clusters are
+// placed inside a GPC and do not fill the last SMs; a second one on an SM waits for partners that run beside others: window flush at D = 64,
+// 528 vectors 4.22 -> 3.95 us, 648 4.23 -> 4.31, 944 4.25 -> 5.39; D = 128, 176: 5.00 -> 4.85, 264: 4.99 -> 5.29, 592: 5.05 -> 10.4; D = 256, 264:
+// 12.3 -> 8.0, 272: 12.3 -> 13.5; append with one scale per vector at D = 128, 264: 3.34 -> 3.28, 320: 3.34 -> 3.68; at D = 64 never (2.67 -> 2.85 at 112).
+template <int D, int MODE>
+constexpr int sliced_tenths(bool cluster, bool per_vector)
+{
+    return !cluster ? ((D == 64 && MODE == 0) || D == 256 ? 10 : 20) : D == 64 && per_vector ? 0 : D == 128 && MODE == 2 ? 6 : 9;
+}
+
 template <int D, bool BF16, int MODE>
 constexpr auto sliced_kernel()
 {
@@ -584,12 +596,12 @@ cudaError_t launch(const MatvecParams &prm, cudaStream_t stream)
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<D>::kSmemBytes)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, Geo<D>::kSmemBytes)) != cudaSuccess) return e;
-        if constexpr (kSliced) {   // slots.blocks_per_sm: the CTAs of the sliced form that the device holds at once
+        if constexpr (kSliced) {   // slots.blocks_per_sm: the SMs, where the sliced form fits as often as it is meant to
             int sliced_per_sm = 0;
             auto sliced = sliced_kernel<D, BF16, MODE>();
             if ((e = cudaFuncSetAttribute(sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, Slice<D>::kSmemBytes)) != cudaSuccess) return e;
             if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sliced_per_sm, sliced, kWarps * 32, Slice<D>::kSmemBytes)) != cudaSuccess) return e;
-            slots.blocks_per_sm[dev] = sms * (sliced_per_sm < 2 ? sliced_per_sm : 2);
+            slots.blocks_per_sm[dev] = sliced_per_sm >= (D == 256 ? 1 : 2) ? sms : 0;
         }
         slots.sms[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
@@ -599,7 +611,7 @@ cudaError_t launch(const MatvecParams &prm, cudaStream_t stream)
     if constexpr (kSliced) {
         constexpr int kSlices = Slice<D>::kSlices;
         const bool cluster = MODE == 2 || (MODE == 1 && prm.group == D);
-        if (batches * kSlices <= slots.blocks_per_sm[dev] && (Slice<D>::kCluster || !cluster))
+        if (10 * batches * kSlices <= (int64_t)sliced_tenths<D, MODE>(cluster, prm.group == D) * slots.blocks_per_sm[dev] && (Slice<D>::kCluster || !cluster))
             return launch_kernel(sliced_kernel<D, BF16, MODE>(), (unsigned)(batches * kSlices), kWarps * 32, Slice<D>::kSmemBytes, stream, cluster ? kSlices : 1, prm);
     }
     // one resident wave of CTAs that loop over batches where the kernel does; else a CTA per batch

@@ -791,11 +791,11 @@ def test_matvec_kernels_all_dims(D, dtype):
     run_case(D, dtype, 5, "gaussian", 7100 + D, enc_impl="matvec", dec_impl="matvec")
 
 
-@pytest.mark.parametrize("D,dtype,per_vector,nbits,most", [(64, "f16", True, 4, 1184), (96, "bf16", False, 8, 784), (128, "f16", False, 4, 592), (128, "bf16", True, 8, 592),
-                                                           (160, "bf16", False, 4, 472), (160, "f16", True, 4, 472), (256, "f16", False, 4, 296),
-                                                           (256, "bf16", True, 4, 296)])
+@pytest.mark.parametrize("D,dtype,per_vector,nbits,most", [(64, "f16", True, 4, 592), (64, "bf16", False, 4, 528), (96, "bf16", False, 8, 784), (128, "f16", False, 4, 592),
+                                                           (128, "f16", False, 4, 176), (128, "bf16", True, 8, 264), (160, "bf16", False, 4, 472),
+                                                           (160, "f16", True, 4, 472), (256, "f16", False, 4, 296), (256, "bf16", True, 4, 264)])
 def test_matvec_kernels_sliced_over_several_ctas(D, dtype, per_vector, nbits, most):
-    """A batch of 8 vectors, one vector more under lambda rows of one; the most whose slices the device holds at once, and one more: encode and
+    """A batch of 8 vectors, one vector more under lambda rows of one; the most that one of the sliced kernels takes, and one more: encode and
     decode against the oracle and, bit for bit, against one call that is too long for slices; the fused flush, whose dequantized rows are
     bit for bit the decode of what it stored."""
     odt = DT[dtype]
