@@ -116,7 +116,10 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
             mx = fmaxf(mx, fmaxf(fmaxf(fabsf(l.x), fabsf(l.y)), fmaxf(fabsf(l.z), fabsf(l.w))));
         }
     }
-    mx = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx)));   // non-negative: ordered like its bits
+    if (lam) mx = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx)));   // non-negative: ordered like its bits
+    else   // the same 1 everywhere, but without the shuffles the calibration's loop is laid out worse: 400,000 vectors at D = 128 33.4 -> 34.0 us
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
     mx = fminf(fmaxf(mx * table_max, 1e-30f), 1e30f);   // table_max: largest |entry| of the table
     const int e = (int)((__float_as_uint(mx) >> 23) & 0xFFu) - 127;      // floor(log2 mx)
     return __uint_as_float((uint32_t)(127 + 13 - e) << 23);
@@ -256,6 +259,17 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kInStages; ++s) mbar_init(smem_u32(&ctrl->in_full[s]), 1);
+        for (int s = 0; s < kFullBars; ++s) mbar_init(smem_u32(&ctrl->acc_full[s]), 1);
+        for (int s = 0; s < kAccStages; ++s) mbar_init(smem_u32(&ctrl->acc_empty[s]), kEpiWarps / 2);
+        mbar_init(smem_u32(&ctrl->b_first), kEpiWarps);       // first B: all epilogue warps build it
+        mbar_init(smem_u32(&ctrl->b_ready), kEpiWarps / 2);   // later rebuilds: the set that owns the tile
+        ctrl->abort = 0u;
+        mbar_init_fence();
+    }
+    if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
+
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range per CTA
     const int64_t N = prm.N, rpl = prm.rpl;
     const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x);
@@ -264,20 +278,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     // One tile: both sets of epilogue warps share it, four threads to a row.  Back to back, 8000 vectors: D = 96 5.0 -> 4.4 us, 128 5.9 -> 5.3,
     // 160 7.1 -> 6.6 (one scale per vector 7.2 -> 6.8); 18,944: 6.2 -> 5.7, 7.1 -> 6.7, 8.7 -> 8.1.  Not at D = 64, which has two groups, one for
     // each half row, as it is, nor with one scale per vector at D = 128, where calls of seven tiles per CTA lose 2 % to the longer loop.
-    const bool solo = D > 64 && !(PERVEC && D == 128) && n_my == 1;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kInStages; ++s) mbar_init(smem_u32(&ctrl->in_full[s]), 1);
-        for (int s = 0; s < kFullBars; ++s) mbar_init(smem_u32(&ctrl->acc_full[s]), 1);
-        for (int s = 0; s < kAccStages; ++s) mbar_init(smem_u32(&ctrl->acc_empty[s]), kEpiWarps / 2);
-        mbar_init(smem_u32(&ctrl->b_first), kEpiWarps);       // first B: all epilogue warps build it
-        mbar_init(smem_u32(&ctrl->b_ready), kEpiWarps / 2);   // later rebuilds: the set that owns the tile
+    // Nor in the calibration, which waits for its column maxima, not for a set: 60,000 vectors at D = 128 16.4 -> 18.1 us, 400,000 33.2 -> 39.4.
+    const bool solo = !CALIB && D > 64 && !(PERVEC && D == 128) && n_my == 1;
+    if (PERVEC && threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s)
             for (int qq = 0; qq < 4; ++qq) mbar_init(smem_u32(&ctrl->pair[s][qq]), solo ? 4 : 2);
-        ctrl->abort = 0u;
         mbar_init_fence();
     }
-    if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
 
     // ---- B for the CTA's first lambda row, by all epilogue warps.  The table is requested and the set-up barrier passed in front of the
     // ---- grid wait, under the grid ahead; lambda and the first x loads follow it side by side.  (With the barrier behind lambda, its round
