@@ -2,7 +2,10 @@
 
 Argument marshalling only: every step of the quantizer runs in the library's CUDA
 kernels.  PyTorch provides device memory and streams.  If the library has not
-been built the binding raises; there is no other code path.
+been built the binding raises; there is no other code path.  The calls of a
+decode loop (encode, decode, append, append_at, flush_block) on plain tensors
+and the current stream marshal the same arguments in native code (``kvq_call``);
+what that does not take, every error among it, goes the way written out here.
 
 The functions carry the names of the C entry points: ``kvq_plan_create``,
 ``kvq_encode``, ``kvq_decode``, ``kvq_append`` ...  ``Plan`` is a small
