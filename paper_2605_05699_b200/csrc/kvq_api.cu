@@ -112,7 +112,7 @@ static kvq_status_t ensure_device(kvq_plan *p)
     // one allocation: the status word, then the tables of the tensor-core and matrix-vector kernels
     constexpr size_t kStatusBytes = 256;
     const bool tables = umma_encode_supported(p->D, false) || umma_decode_supported(p->D, false);
-    const size_t bytes = tables ? sizeof(float) * (size_t)p->D * p->D : 0, total = kStatusBytes + (tables ? 2 * bytes + operand_bytes(p->D) : 0);
+    const size_t bytes = tables ? sizeof(float) * (size_t)p->D * p->D : 0, total = kStatusBytes + (tables ? 2 * bytes + operand_room(p->D) : 0);
     std::vector<float> host;
     if (tables && !make_tables(p, host)) return KVQ_ERR_NOMEM;
     unsigned char *mem = nullptr;

@@ -39,14 +39,16 @@ struct FftParams {
     float table_max;            // tensor-core encode: largest |entry| of the plan's forward table (sqrt(2/D) without a rotation)
     uint32_t first_wait_polls;  // tensor-core encode, D <= 160: polls the mma role gives its first operand build (0: the default)
     int bits;                   // tensor-core encode: 4 or 8 (the register-FFT launchers take it as an argument)
-    const unsigned char *operands;   // tensor-core append: the plan's split operands (build_encode_operands)
+    const unsigned char *operands;   // tensor-core append: the plan's split operands and 2^-k (build_encode_operands)
     int append;                 // the call is an append: one new row per stream
     uint32_t sign_xor[128];     // word m: bit 15 set if s_{2m} = -1, bit 31 set if s_{2m+1} = -1
 };
 
 // The split operands of the append kernel: two fp16 terms of e0 2^k, each one block of [D rows][128 B] per 64 columns, 128-byte
-// swizzle.
+// swizzle; behind them 2^-k as a float, in operand_room bytes in all.  k follows the table's largest entry, so the kernel reads it where
+// it reads the operands: a recorded launch finds both as the last rotation left them.
 __host__ __device__ constexpr size_t operand_bytes(int D) { return 2 * (size_t)((D + 63) / 64) * (size_t)D * 128; }
+constexpr size_t operand_room(int D) { return operand_bytes(D) + 16; }
 cudaError_t build_encode_operands(int D, const float *e0, float table_max, unsigned char *out);   // complete when it returns
 
 // A decode whose rows live in a cache laid out [stream][T][...]: the call's N = S * rows logical rows are rows

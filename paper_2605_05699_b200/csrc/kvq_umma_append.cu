@@ -87,14 +87,13 @@ __device__ __forceinline__ void load_b(unsigned char *sB, const unsigned char *w
 
 struct UmmaAppendParams {
     const float *lambda;   // [n_lambda, D] fp32
-    const unsigned char *w;   // split terms of W 2^k: [term][K block][D rows][128 B], swizzled (build_encode_operands)
+    const unsigned char *w;   // split terms of W 2^k: [term][K block][D rows][128 B], swizzled, then 2^-k (build_encode_operands)
     unsigned char *packed; // [*, D bits / 8] bytes out
     uint16_t *scales;      // [*, D/32] (one scale per vector: [*, 1]) fp16 out
     uint32_t N;            // below 2^31
     uint32_t rpl;          // rows per lambda row
     int64_t n_lambda;
     RowMap out_map;        // output row of input row r
-    float unlift;          // 2^-k
     int bits;              // 4: nibble pairs; 8: one two's-complement byte per code, scale = absmax / 127
     uint32_t *status;
     uint32_t first_wait_polls;  // polls the mma role gives the B operand before it gives up (kvq_plan_set_wait_limit)
@@ -226,7 +225,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int r = q * 32 + lane;            // tile row of this thread
         const int p = (warp - 2) >> 2;          // this thread's groups: p, p + 4
         const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        const float unlift = prm.unlift, Q = prm.bits == 4 ? 7.0f : 127.0f, inv_q = prm.bits == 4 ? 1.0f / 7.0f : 1.0f / 127.0f;
+        const float unlift = load_input(reinterpret_cast<const float *>(prm.w + operand_bytes(D)));
+        const float Q = prm.bits == 4 ? 7.0f : 127.0f, inv_q = prm.bits == 4 ? 1.0f / 7.0f : 1.0f / 127.0f;
         // lambda of this thread's row and CTA's channels (the same for the whole warp where lambda rows are long: a broadcast out of L1)
         auto lambda_of = [&](uint32_t row) -> const float4 * {
             const uint32_t at = prm.n_lambda > 1 ? (row < N ? row : N - 1u) / prm.rpl : 0u;
@@ -350,6 +350,7 @@ __global__ void kvq_build_encode_operands_kernel(const float *e0, int D, float l
         }
         *reinterpret_cast<uint4 *>(dst + (t ? operand_bytes(D) / 2 : 0)) = make_uint4(o[0], o[1], o[2], o[3]);
     }
+    if (i == 0) *reinterpret_cast<float *>(out + operand_bytes(D)) = 1.0f / lift;
 }
 
 // 2^k, what brings the table's largest entry into [2^13, 2^14): the first fp16 term stays below fp16's maximum and the second above its
@@ -388,7 +389,6 @@ cudaError_t launch(int64_t N, const FftParams &f, cudaStream_t stream)
     prm.rpl = (uint32_t)(f.rows_per_lambda < N ? f.rows_per_lambda : N);
     prm.n_lambda = f.n_lambda;
     prm.out_map = f.out_map;
-    prm.unlift = 1.0f / operand_lift(f.table_max);
     prm.bits = f.bits;
     prm.status = f.status;
     prm.first_wait_polls = f.first_wait_polls ? f.first_wait_polls : kWaitPolls;

@@ -52,6 +52,45 @@ def test_prepared_plan_is_captured_without_a_warm_call(D, dtype, N):
     plan.close()
 
 
+def inverse_transform(D):
+    """The rotation that undoes the transform: the plan's forward table becomes the sign diagonal, entries of 1 among zeros."""
+    n, k = np.arange(D), np.arange(1, D // 2)
+    m = np.empty((D, D))
+    m[0], m[D // 2] = D ** -0.5, (-1.0) ** n * D ** -0.5
+    m[1:D // 2] = np.sqrt(2 / D) * np.cos(2 * np.pi * np.outer(k, n) / D)
+    m[D // 2 + 1:] = -np.sqrt(2 / D) * np.sin(2 * np.pi * np.outer(k, n) / D)
+    return torch.from_numpy(m.T.copy()).to(torch.float32)
+
+
+@pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
+def test_a_recorded_append_follows_the_plans_rotation(D):
+    """A rotation rewrites the plan's tables in place, and the power of two that the append kernel's operands carry moves with the largest
+    table entry: what a recorded append takes out again has to be the tables' own, not that of the recording."""
+    S, T, rpl = 2500, 3, 32
+    plan = kb.Plan(D, G, 60 + D)
+    sg = plan.signs()
+    x, lam = wl.make_vectors(S, D, "f16", "k_outlier", 61), wl.make_lambda(-(-S // rpl), D, 62)
+    xd, lamd = x.cuda(), lam.cuda()
+    packed = torch.zeros(S, T, D // 2, dtype=torch.uint8, device="cuda")
+    scales = torch.zeros(S, T, D // G, dtype=torch.float16, device="cuda")
+    kb.kvq_plan_prepare(plan.handle, torch.float16)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        kb.kvq_append(plan.handle, xd, lamd, packed, scales, 1, rpl)
+    for R in (None, wl.make_rotation(D, 63), wl.make_rotation(D, 64, 0.02), inverse_transform(D), None):
+        plan.set_rotation(R)
+        packed.zero_(), scales.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        ora = ko.encode(wl.raw_bits(x), ko.F16, sg, lam.numpy(), G, rpl, want_v=True, rot=None if R is None else R.numpy().astype(np.float64))
+        parity.check_encode(packed[:, 1].contiguous().cpu().numpy(), wl.raw_bits(scales[:, 1].contiguous()), ora, G, "replayed append", min_agree=0.9995)
+        assert not bool(packed[:, [0, 2]].any()) and not bool(scales[:, [0, 2]].any())
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    del graph
+    plan.close()
+
+
 def test_prepare_checks_its_arguments_first():
     L = kb.lib()
     p = kb.Plan(128, G, 1)
