@@ -80,15 +80,18 @@ static double build_b0(const kvq_plan *p, float *b0)
     return tmax;
 }
 
-// Host copy of both tables, one behind the other as on the device: b0 [n][c] for the decode kernels, its transpose e0 [c][n] for the
-// encode kernels.
+// Floats of both tables and of what stands behind them, and their host copy, as on the device: b0 [n][c] for the decode kernels, its
+// transpose e0 [c][n] for the encode kernels, then the largest |entry|.  The encode kernels read it there: a recorded launch finds the one that
+// belongs to the tables as they are when it runs.
+static size_t table_floats(int D) { return 2 * (size_t)D * D + 4; }
+
 static bool make_tables(kvq_plan *p, std::vector<float> &both)
 {
     const size_t D = (size_t)p->D;
     try {
-        both.resize(2 * D * D);
+        both.assign(table_floats(p->D), 0.0f);
         float *b0 = both.data(), *e0 = b0 + D * D;
-        p->table_max = (float)build_b0(p, b0);
+        both[2 * D * D] = p->table_max = (float)build_b0(p, b0);
         for (size_t n = 0; n < D; ++n)
             for (size_t c = 0; c < D; ++c) e0[c * D + n] = b0[n * D + c];
     } catch (...) {
@@ -112,7 +115,7 @@ static kvq_status_t ensure_device(kvq_plan *p)
     // one allocation: the status word, then the tables of the tensor-core and matrix-vector kernels
     constexpr size_t kStatusBytes = 256;
     const bool tables = umma_encode_supported(p->D, false) || umma_decode_supported(p->D, false);
-    const size_t bytes = tables ? sizeof(float) * (size_t)p->D * p->D : 0, total = kStatusBytes + (tables ? 2 * bytes + operand_room(p->D) : 0);
+    const size_t bytes = tables ? sizeof(float) * table_floats(p->D) : 0, total = kStatusBytes + (tables ? bytes + operand_room(p->D) : 0);
     std::vector<float> host;
     if (tables && !make_tables(p, host)) return KVQ_ERR_NOMEM;
     unsigned char *mem = nullptr;
@@ -120,11 +123,11 @@ static kvq_status_t ensure_device(kvq_plan *p)
         (void)cudaGetLastError();
         return KVQ_ERR_NOMEM;
     }
-    float *db = reinterpret_cast<float *>(mem + kStatusBytes), *de = reinterpret_cast<float *>(mem + kStatusBytes + bytes);
-    unsigned char *dw = mem + kStatusBytes + 2 * bytes;
+    float *db = reinterpret_cast<float *>(mem + kStatusBytes), *de = db + (size_t)p->D * p->D;
+    unsigned char *dw = mem + kStatusBytes + bytes;
     bool ok = cudaMemset(mem, 0, kStatusBytes) == cudaSuccess;
     if (ok && tables)
-        ok = cudaMemcpy(db, host.data(), 2 * bytes, cudaMemcpyHostToDevice) == cudaSuccess && build_encode_operands(p->D, de, p->table_max, dw) == cudaSuccess;
+        ok = cudaMemcpy(db, host.data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess && build_encode_operands(p->D, de, p->table_max, dw) == cudaSuccess;
     if (!ok) {
         (void)cudaGetLastError();
         cudaFree(mem);
@@ -177,7 +180,6 @@ static void fill_params(const kvq_plan *p, FftParams &prm, int64_t N, const floa
     prm.out_map = RowMap{1, 1, 0};
     prm.in_map = RowMap{1, 1, 0};
     prm.status = p->d_status;
-    prm.table_max = p->table_max;
     prm.first_wait_polls = p->first_wait_polls;
     prm.bits = p->bits;
     prm.operands = p->d_operands;
@@ -265,7 +267,7 @@ kvq_status_t kvq_plan_set_rotation(kvq_plan_t *plan, const float *R_host)
     }
     std::vector<float> host;
     if (!make_tables(plan, host)) return KVQ_ERR_NOMEM;
-    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(plan->d_b0, host.data(), 2 * sizeof(float) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
+    if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(plan->d_b0, host.data(), sizeof(float) * host.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
         build_encode_operands(plan->D, plan->d_e0, plan->table_max, plan->d_operands) != cudaSuccess) {
         (void)cudaGetLastError();
         return KVQ_ERR_CUDA;

@@ -36,7 +36,6 @@ struct FftParams {
     RowMap out_map;             // row of packed / scales (encode) or of out (decode) that row r goes to
     RowMap in_map;              // decode: row of packed / scales that row r comes from
     uint32_t *status;           // per-plan device status word
-    float table_max;            // tensor-core encode: largest |entry| of the plan's forward table (sqrt(2/D) without a rotation)
     uint32_t first_wait_polls;  // tensor-core encode, D <= 160: polls the mma role gives its first operand build (0: the default)
     int bits;                   // tensor-core encode: 4 or 8 (the register-FFT launchers take it as an argument)
     const unsigned char *operands;   // tensor-core append: the plan's split operands and 2^-k (build_encode_operands)
@@ -83,7 +82,7 @@ struct GemmParams {
 
 // tcgen05 DFT-as-GEMM kernels (kvq_umma_decode.cu, kvq_umma_encode.cu): which (D, 16-bit type) pairs are built, and the
 // launchers.  Encode takes the register-FFT argument block (its sign words are unused) and the plan table e0 [D, D]
-// fp32, e0[c][n] = M[c][n] s_n; decode takes the table b0 = e0 transposed through GemmParams.
+// fp32, e0[c][n] = M[c][n] s_n, with its largest |entry| behind it; decode takes the table b0 = e0 transposed through GemmParams.
 bool umma_decode_supported(int D, bool bf16);
 bool umma_encode_supported(int D, bool bf16);
 bool umma_calibrate_supported(int D, bool bf16);
@@ -179,7 +178,7 @@ struct kvq_plan {
     int device;            // -1 until initialised
     uint32_t *d_status;    // device status word; the tables stand behind it in the same allocation
     float *d_b0;           // [D, D] fp32 inverse-transform matrix with the signs folded in (GEMM decode), or null
-    float *d_e0;           // [D, D] fp32 forward-transform matrix with the signs folded in (GEMM encode), or null
+    float *d_e0;           // [D, D] fp32 forward-transform matrix with the signs folded in (GEMM encode), then its largest |entry|, or null
     unsigned char *d_operands;   // split operands of the append kernel, or null
     size_t table_bytes;
     double *rot;           // host, [D, D] row-major: the rotation between the transform and lambda, or null

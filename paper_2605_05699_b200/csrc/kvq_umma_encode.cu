@@ -105,8 +105,9 @@ static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 // the first split term of W 2^k stays below fp16's maximum and the later ones above its subnormals.
 // Every lane of the warp gets the same value.
 template <int D>
-__device__ __forceinline__ float lift_of(const float *__restrict__ lam, float table_max, int lane)
+__device__ __forceinline__ float lift_of(const float *__restrict__ lam, const float *__restrict__ e0, int lane)
 {
+    const float table_max = __ldg(e0 + D * D);   // largest |entry| of the table
     float mx = lam ? 0.0f : 1.0f;   // no lambda row (calibration): lambda = 1
 #pragma unroll
     for (int p = 0; p < (D / 4 + 31) / 32; ++p) {
@@ -120,7 +121,7 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
     else   // the same 1 everywhere, but without the shuffles the calibration's loop is laid out worse: 400,000 vectors at D = 128 33.4 -> 34.0 us
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    mx = fminf(fmaxf(mx * table_max, 1e-30f), 1e30f);   // table_max: largest |entry| of the table
+    mx = fminf(fmaxf(mx * table_max, 1e-30f), 1e30f);
     const int e = (int)((__float_as_uint(mx) >> 23) & 0xFFu) - 127;      // floor(log2 mx)
     return __uint_as_float((uint32_t)(127 + 13 - e) << 23);
 }
@@ -236,7 +237,6 @@ struct UmmaEncodeParams {
     int64_t rpl;           // rows per lambda segment (N when there is one lambda row)
     int64_t n_seg;
     RowMap out_map;        // output row of input row r
-    float table_max;       // largest |entry| of e0
     int bits;              // 4: nibble pairs; 8: one two's-complement byte per code, scale = absmax / 127
     uint32_t *status;
     uint32_t *amax_bits;        // calibration only: [D] running column maxima as fp32 bit patterns (start at zero)
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         first_seg = tile_begin / tps;
         const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : first_seg) * D;
         rows.load_lambda(lam, 0, warp - 2, lane);
-        first_lift = lift_of<D>(lam, prm.table_max, lane);
+        first_lift = lift_of<D>(lam, prm.e0, lane);
         rows.store(sB, first_lift, 0, warp - 2, lane);
         rows.rest(sB, prm.e0, lam, first_lift, warp - 2, lane);
         fence_proxy_async();   // B is read by the tensor core through the async proxy
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- tells the mma warp.
             if (seg != cached_seg) {
                 const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : seg) * D;
-                const float lift = lift_of<D>(lam, prm.table_max, lane);
+                const float lift = lift_of<D>(lam, prm.e0, lane);
                 if (j > 0 && cur.first_of_segment()) {
                     if (!rebuild_b<D, BF16, CALIB || WIDE>(sB, prm.e0, lam, lift, bw, lane, smem_u32(&ctrl->acc_full[(j - 1) % kFullBars]),
                                                            (uint32_t)((j - 1) / kFullBars) & 1u, abort_flag, status))
@@ -581,7 +581,6 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     prm.rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
     prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
     prm.out_map = f.out_map;
-    prm.table_max = f.table_max;
     prm.bits = f.bits;
     prm.status = f.status;
     prm.amax_bits = amax_bits;

@@ -91,8 +91,9 @@ static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 // the first split term of W 2^k stays below fp16's maximum and the later ones above its subnormals.
 // Every lane of the warp gets the same value.
 template <int D>
-__device__ __forceinline__ float lift_of(const float *__restrict__ lam, float table_max, int lane)
+__device__ __forceinline__ float lift_of(const float *__restrict__ lam, const float *__restrict__ e0, int lane)
 {
+    const float table_max = __ldg(e0 + D * D);   // largest |entry| of the table
     float mx = lam ? 0.0f : 1.0f;   // no lambda row (calibration): lambda = 1
 #pragma unroll
     for (int p = 0; p < (D / 4 + 31) / 32; ++p) {
@@ -103,7 +104,7 @@ __device__ __forceinline__ float lift_of(const float *__restrict__ lam, float ta
         }
     }
     mx = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx)));   // non-negative: ordered like its bits
-    mx = fminf(fmaxf(mx * table_max, 1e-30f), 1e30f);   // table_max: largest |entry| of the table
+    mx = fminf(fmaxf(mx * table_max, 1e-30f), 1e30f);
     const int e = (int)((__float_as_uint(mx) >> 23) & 0xFFu) - 127;      // floor(log2 mx)
     return __uint_as_float((uint32_t)(127 + 13 - e) << 23);
 }
@@ -168,7 +169,6 @@ struct UmmaEncode256Params {
     int64_t rpl;           // rows per lambda segment (N when there is one lambda row)
     int64_t n_seg;
     RowMap out_map;        // output row of input row r
-    float table_max;       // largest |entry| of e0
     uint32_t *status;
     uint32_t *amax_bits;        // calibration only: [D] running column maxima as fp32 bit patterns (start at zero)
     int bits;                   // 4: nibble pairs; 8 (fp16 input): one two's-complement byte per code, scale = absmax / 127
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         rows.load(prm.e0, rank, (warp - 2) * 8, lane);
         grid_wait();
         rows.load_lambda(lam, rank, (warp - 2) * 8, lane);
-        first_lift = lift_of<kD>(lam, prm.table_max, lane);
+        first_lift = lift_of<kD>(lam, prm.e0, lane);
         tc_fence_before();
         cluster_sync_all();   // both CTAs' barriers exist and both have their tensor memory
         tc_fence_after();
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 BuildRows<BF16, CALIB> rows;
                 rows.load(prm.e0, rank, (warp - 2) * 8, lane);
                 rows.load_lambda(lam, rank, (warp - 2) * 8, lane);
-                lift_next = lift_of<kD>(lam, prm.table_max, lane);
+                lift_next = lift_of<kD>(lam, prm.e0, lane);
                 if (!wait_or_abort(smem_u32(&ctrl->acc_full[sc]), (uint32_t)(j / kAccStages) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
                 rows.store(sB, lift_next, (warp - 2) * 8, lane);
                 fence_proxy_async();   // B is read by the tensor core through the async proxy
@@ -554,7 +554,6 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     prm.rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
     prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
     prm.out_map = f.out_map;
-    prm.table_max = f.table_max;
     prm.status = f.status;
     prm.amax_bits = amax_bits;
     prm.bits = f.bits;

@@ -63,6 +63,34 @@ def inverse_transform(D):
 
 
 @pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
+@pytest.mark.parametrize("dtype,group", [("f16", 32), ("bf16", 32), ("f16", 0)])
+def test_a_recorded_encode_follows_the_plans_rotation(D, dtype, group):
+    """The encode kernels scale their operands by the table's largest entry: it too has to be that of the tables as they are.  (A limit
+    kept from the recording takes fp16 operands out of range where a rotation makes it more than four times as large.)"""
+    N, rpl = 3000, 1100
+    plan = kb.Plan(D, group or D, 70 + D)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_AUTO)
+    sg = plan.signs()
+    x, lam = wl.make_vectors(N, D, dtype, "k_outlier", 71), wl.make_lambda(3, D, 72)
+    xd, lamd = x.cuda(), lam.cuda()
+    packed, scales = plan.empty_packed(N), plan.empty_scales(N)
+    kb.kvq_plan_prepare(plan.handle, wl.torch_dtype(dtype))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        kb.kvq_encode(plan.handle, xd, lamd, packed, scales, rpl)
+    for R in (None, wl.make_rotation(D, 73), inverse_transform(D), None):
+        plan.set_rotation(R)
+        graph.replay()
+        torch.cuda.synchronize()
+        ora = ko.encode(wl.raw_bits(x), DT[dtype], sg, lam.numpy(), plan.group, rpl, want_v=True, rot=None if R is None else R.numpy().astype(np.float64))
+        parity.check_encode(packed.cpu().numpy(), wl.raw_bits(scales), ora, plan.group, "replayed encode", min_agree=0.9995)
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    del graph
+    plan.close()
+
+
+@pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
 def test_a_recorded_append_follows_the_plans_rotation(D):
     """A rotation rewrites the plan's tables in place, and the power of two that the append kernel's operands carry moves with the largest
     table entry: what a recorded append takes out again has to be the tables' own, not that of the recording."""
