@@ -199,3 +199,20 @@ def test_compute_without_a_device_fails_loudly_never_silently():
     assert L.kvq_encode(p.handle, A, 0, 8, A, 1, 0, A, A, None) == kb.KVQ_ERR_CUDA
     assert L.kvq_decode(p.handle, A, A, 8, A, 1, 0, A, 0, None) == kb.KVQ_ERR_CUDA
     p.close()
+
+
+def test_the_library_is_built_also_where_the_bindings_native_half_cannot_be(tmp_path, monkeypatch):
+    """libkvq.so needs nvcc alone.  Without g++ (or torch's or Python's headers) the native half is left out, with a warning, and no file
+    of an earlier source stays behind to be loaded in its place."""
+    old = tmp_path / "kvq_call.so"
+    old.write_bytes(b"of an earlier source")
+    os.utime(old, (1, 1))
+    monkeypatch.setattr(kbuild, "CALL", str(old))
+
+    def no_compiler(cmd, *a, **k):
+        raise FileNotFoundError("g++")
+
+    monkeypatch.setattr(kbuild.subprocess, "check_call", no_compiler)
+    with pytest.warns(RuntimeWarning, match="kvq_call has not been built"):
+        assert kbuild.build() == kbuild.LIB
+    assert os.path.exists(kbuild.LIB) and not old.exists()
