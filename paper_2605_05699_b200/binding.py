@@ -113,6 +113,8 @@ def lib() -> ctypes.CDLL:
             from . import kvq_call
         except ImportError:
             kvq_call = None
+        if kvq_call is not None and getattr(kvq_call, "torch_version", None) != torch.__version__:
+            kvq_call = None   # compiled against other class layouts
         if kvq_call is not None:
             kvq_call.bind(*(ctypes.cast(f, vp).value for f in (L.kvq_encode, L.kvq_decode, L.kvq_append, L.kvq_append_at, L.kvq_flush_block)))
         _native = kvq_call

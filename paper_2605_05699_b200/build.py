@@ -16,7 +16,8 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkvq.so")
 CALL_SRC = os.path.join(CSRC, "kvq_call.cpp")
-CALL = os.path.join(HERE, "kvq_call.so")   # the binding's native half: a Python extension on torch's own headers and libraries
+# the binding's native half: a Python extension on torch's own headers and libraries, good for the Python in its name and the torch it says
+CALL = os.path.join(HERE, "kvq_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 NVCC_FLAGS = [
@@ -54,21 +55,29 @@ def _compile(src: str, force: bool, newest: float) -> str:
 
 
 def _build_call(force: bool) -> None:
-    if not force and os.path.exists(CALL) and os.path.getmtime(CALL) >= max(os.path.getmtime(CALL_SRC), os.path.getmtime(os.path.join(INCLUDE, "kvq.h"))):
+    import torch
+
+    stamp = os.path.join(OBJ, os.path.basename(CALL) + ".torch")   # the torch that CALL was compiled against
+    built_for = None
+    if os.path.exists(CALL) and os.path.exists(stamp):
+        with open(stamp) as f:
+            built_for = f.read()
+    if not force and built_for == torch.__version__ and os.path.getmtime(CALL) >= max(os.path.getmtime(CALL_SRC), os.path.getmtime(os.path.join(INCLUDE, "kvq.h"))):
         return
     if os.path.exists(CALL):   # out of date: not left behind where the compiler fails
         os.remove(CALL)
-    import torch
-
     root = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = CALL + ".tmp.%d" % os.getpid()
     subprocess.check_call([
         "g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+        '-DKVQ_TORCH="%s"' % torch.__version__,
         "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
         "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), CALL_SRC, "-o", tmp,
         "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
     os.replace(tmp, CALL)
+    with open(stamp, "w") as f:
+        f.write(torch.__version__)
 
 
 def _build_library(force: bool) -> str:

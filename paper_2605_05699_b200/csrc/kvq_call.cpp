@@ -183,4 +183,13 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "kvq_call", nullptr, -1, methods, n
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit_kvq_call() { return PyModule_Create(&module); }
+// torch_version: the torch whose class layouts are compiled in; binding.py takes the module under no other.
+PyMODINIT_FUNC PyInit_kvq_call()
+{
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "torch_version", KVQ_TORCH) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

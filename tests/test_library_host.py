@@ -216,3 +216,48 @@ def test_the_library_is_built_also_where_the_bindings_native_half_cannot_be(tmp_
     with pytest.warns(RuntimeWarning, match="kvq_call has not been built"):
         assert kbuild.build() == kbuild.LIB
     assert os.path.exists(kbuild.LIB) and not old.exists()
+
+
+def test_the_bindings_native_half_is_rebuilt_for_another_torch_or_python(tmp_path, monkeypatch):
+    """It is compiled against torch's C++ classes and Python's ABI: the file name says which Python, a stamp which torch."""
+    import sysconfig
+
+    suffix = sysconfig.get_config_var("EXT_SUFFIX")
+    assert kbuild.CALL.endswith("kvq_call" + suffix) and "cpython" in suffix
+    call = tmp_path / ("kvq_call" + suffix)
+    monkeypatch.setattr(kbuild, "CALL", str(call))
+    monkeypatch.setattr(kbuild, "OBJ", str(tmp_path))
+    compiled = []
+
+    def compiler(cmd, *a, **k):
+        compiled.append(cmd)
+        with open(cmd[cmd.index("-o") + 1], "wb") as f:
+            f.write(b"module")
+
+    monkeypatch.setattr(kbuild.subprocess, "check_call", compiler)
+    for found, times in ((None, 1), ("0.0", 1), (torch.__version__, 0)):
+        call.write_bytes(b"found")
+        stamp = tmp_path / (call.name + ".torch")
+        if found:
+            stamp.write_text(found)
+        del compiled[:]
+        kbuild._build_call(False)
+        assert len(compiled) == times and stamp.read_text() == torch.__version__, found
+        assert call.read_bytes() == (b"module" if times else b"found")
+
+
+def test_a_native_half_for_another_torch_is_not_used(monkeypatch):
+    import types
+
+    import paper_2605_05699_b200 as package
+
+    kb.lib()
+    assert kb._native is not None and kb._native.torch_version == torch.__version__
+    for other in (types.SimpleNamespace(torch_version="0.0", bind=None), types.SimpleNamespace(bind=None)):   # (and one that does not say)
+        with monkeypatch.context() as m:
+            m.setattr(kb, "_lib", None)
+            m.setattr(kb, "_native", kb._native)
+            m.setattr(package, "kvq_call", other)
+            kb.lib()
+            assert kb._native is None
+    assert kb._native is not None
