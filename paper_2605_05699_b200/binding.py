@@ -15,6 +15,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 
 import torch
 
@@ -111,10 +112,13 @@ def lib() -> ctypes.CDLL:
         L.kvq_launch_count.argtypes = []
         try:
             from . import kvq_call
-        except ImportError:
-            kvq_call = None
+            why = "compiled against torch %s" % getattr(kvq_call, "torch_version", "of an unknown version")
+        except ImportError as e:
+            kvq_call, why = None, str(e)
         if kvq_call is not None and getattr(kvq_call, "torch_version", None) != torch.__version__:
-            kvq_call = None   # compiled against other class layouts
+            kvq_call = None   # other class layouts
+        if kvq_call is None:
+            warnings.warn("kvq_call is not used, calls take the general way, some microseconds longer each: %s" % why, RuntimeWarning, stacklevel=2)
         if kvq_call is not None:
             kvq_call.bind(*(ctypes.cast(f, vp).value for f in (L.kvq_encode, L.kvq_decode, L.kvq_append, L.kvq_append_at, L.kvq_flush_block)))
         _native = kvq_call

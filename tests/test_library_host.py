@@ -3,6 +3,7 @@ declares, builds plans, and rejects bad arguments before touching CUDA."""
 import ctypes
 import os
 import re
+import sys
 
 import numpy as np
 import pytest
@@ -246,6 +247,7 @@ def test_the_bindings_native_half_is_rebuilt_for_another_torch_or_python(tmp_pat
         assert call.read_bytes() == (b"module" if times else b"found")
 
 
+@pytest.mark.filterwarnings("ignore:kvq_call is not used")
 def test_a_native_half_for_another_torch_is_not_used(monkeypatch):
     import types
 
@@ -261,3 +263,26 @@ def test_a_native_half_for_another_torch_is_not_used(monkeypatch):
             kb.lib()
             assert kb._native is None
     assert kb._native is not None
+
+
+def test_a_native_half_that_is_not_used_is_said_so(monkeypatch):
+    """Every call is some microseconds longer without it: a warning when the library is loaded, with the reason."""
+    import types
+
+    import paper_2605_05699_b200 as package
+
+    kb.lib()
+    with monkeypatch.context() as m:
+        m.setattr(kb, "_lib", None)
+        m.setattr(kb, "_native", kb._native)
+        m.setattr(package, "kvq_call", types.SimpleNamespace(torch_version="0.0", bind=None))
+        with pytest.warns(RuntimeWarning, match="kvq_call is not used.*compiled against torch 0.0"):
+            kb.lib()
+    with monkeypatch.context() as m:
+        m.setattr(kb, "_lib", None)
+        m.setattr(kb, "_native", kb._native)
+        m.delattr(package, "kvq_call")
+        m.setitem(sys.modules, package.__name__ + ".kvq_call", None)   # what an import that fails looks like
+        with pytest.warns(RuntimeWarning, match="kvq_call is not used"):
+            kb.lib()
+        assert kb._native is None
