@@ -36,19 +36,21 @@ struct FftParams {
     RowMap out_map;             // row of packed / scales (encode) or of out (decode) that row r goes to
     RowMap in_map;              // decode: row of packed / scales that row r comes from
     uint32_t *status;           // per-plan device status word
-    uint32_t first_wait_polls;  // tensor-core encode, D <= 160: polls the mma role gives its first operand build (0: the default)
+    uint32_t first_wait_polls;  // tensor-core encode of D <= 160 and append: polls the mma role gives its first operands (0: the default)
     int bits;                   // tensor-core encode: 4 or 8 (the register-FFT launchers take it as an argument)
-    const unsigned char *operands;   // tensor-core append: the plan's split operands and 2^-k (build_encode_operands)
+    const unsigned char *operands;   // tensor-core append: the plan's split operands (build_encode_operands), or null: a table outside [kOperandMin, kOperandMax)
     int append;                 // the call is an append: one new row per stream
     uint32_t sign_xor[128];     // word m: bit 15 set if s_{2m} = -1, bit 31 set if s_{2m+1} = -1
 };
 
-// The split operands of the append kernel: two fp16 terms of e0 2^k, each one block of [D rows][128 B] per 64 columns, 128-byte
-// swizzle; behind them 2^-k as a float, in operand_room bytes in all.  k follows the table's largest entry, so the kernel reads it where
-// it reads the operands: a recorded launch finds both as the last rotation left them.
+// The split operands of the append kernel: two fp16 terms of e0 2^14, each one block of [D rows][128 B] per 64 columns, 128-byte
+// swizzle.  The same power of two for every table, so that a recorded launch takes out what any later rotation's operands carry: an orthogonal
+// table's entries are at most 1, the plain transform's at least 0.002, and 0.002 2^14 = 35 still has a second term of full precision (what
+// a rotation makes smaller loses less than 2^-39).  An orthogonal table's largest entry lies between D^-1/2 and 1; the appends of a table far from
+// that, outside fp16's range or in its subnormals, stay with the encode kernels.
+constexpr float kOperandLift = 16384.0f, kOperandMin = 0.06f, kOperandMax = 3.9f;
 __host__ __device__ constexpr size_t operand_bytes(int D) { return 2 * (size_t)((D + 63) / 64) * (size_t)D * 128; }
-constexpr size_t operand_room(int D) { return operand_bytes(D) + 16; }
-cudaError_t build_encode_operands(int D, const float *e0, float table_max, unsigned char *out);   // complete when it returns
+cudaError_t build_encode_operands(int D, const float *e0, unsigned char *out);   // complete when it returns
 
 // A decode whose rows live in a cache laid out [stream][T][...]: the call's N = S * rows logical rows are rows
 // [base, base + rows) of each of S streams, `stride` cache rows apart, in packed, scales and out alike; the lambda row of

@@ -5,7 +5,7 @@
 // decode step, Sec. 7.2): a tile or two per CTA, and a lambda row for every few dozen of its vectors.  So lambda stands in the epilogue,
 // half a multiply per channel (mul.f32x2), and not in the B operand:
 //
-//   * B = M diag(s) 2^k is the plan's alone: split and swizzled once (build_encode_operands), fetched by bulk copies while the grid ahead
+//   * B = M diag(s) 2^14 is the plan's alone: split and swizzled once (build_encode_operands), fetched by bulk copies while the grid ahead
 //     on the stream runs out.  The kernels above build it from the fp32 table and lambda at the start of every call and again at every
 //     lambda row: 2 us of a call of one tile per CTA.
 //   * A tile is any 128 consecutive vectors, whatever lambda rows they have: 160 lambda rows of 32 vectors are 40 full tiles, not 160.
@@ -87,13 +87,14 @@ __device__ __forceinline__ void load_b(unsigned char *sB, const unsigned char *w
 
 struct UmmaAppendParams {
     const float *lambda;   // [n_lambda, D] fp32
-    const unsigned char *w;   // split terms of W 2^k: [term][K block][D rows][128 B], swizzled, then 2^-k (build_encode_operands)
+    const unsigned char *w;   // split terms of W 2^14: [term][K block][D rows][128 B], swizzled (build_encode_operands)
     unsigned char *packed; // [*, D bits / 8] bytes out
     uint16_t *scales;      // [*, D/32] (one scale per vector: [*, 1]) fp16 out
     uint32_t N;            // below 2^31
     uint32_t rpl;          // rows per lambda row
     int64_t n_lambda;
     RowMap out_map;        // output row of input row r
+    float unlift;          // 1 / kOperandLift (as an immediate, or read from device memory: 5120 vectors at D = 128, calls one after another, 4.36 -> 4.41 us)
     int bits;              // 4: nibble pairs; 8: one two's-complement byte per code, scale = absmax / 127
     uint32_t *status;
     uint32_t first_wait_polls;  // polls the mma role gives the B operand before it gives up (kvq_plan_set_wait_limit)
@@ -225,8 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int r = q * 32 + lane;            // tile row of this thread
         const int p = (warp - 2) >> 2;          // this thread's groups: p, p + 4
         const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        const float unlift = load_input(reinterpret_cast<const float *>(prm.w + operand_bytes(D)));
-        const float Q = prm.bits == 4 ? 7.0f : 127.0f, inv_q = prm.bits == 4 ? 1.0f / 7.0f : 1.0f / 127.0f;
+        const float unlift = prm.unlift, Q = prm.bits == 4 ? 7.0f : 127.0f, inv_q = prm.bits == 4 ? 1.0f / 7.0f : 1.0f / 127.0f;
         // lambda of this thread's row and CTA's channels (the same for the whole warp where lambda rows are long: a broadcast out of L1)
         auto lambda_of = [&](uint32_t row) -> const float4 * {
             const uint32_t at = prm.n_lambda > 1 ? (row < N ? row : N - 1u) / prm.rpl : 0u;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 namespace {
 
 // The operands out of the forward table, once per plan (and rotation): 16 bytes of both terms' swizzled rows per thread.
-__global__ void kvq_build_encode_operands_kernel(const float *e0, int D, float lift, unsigned char *out)
+__global__ void kvq_build_encode_operands_kernel(const float *e0, int D, unsigned char *out)
 {
     const int chunks = (D + 63) / 64 * 8, i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= D * chunks) return;
@@ -338,7 +338,7 @@ __global__ void kvq_build_encode_operands_kernel(const float *e0, int D, float l
     unsigned char *dst = out + ((size_t)(ch >> 3) * D + c) * 128 + (((ch & 7) ^ (c & 7)) << 4);
     float w[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) w[k] = 8 * ch + k < D ? e0[(size_t)c * D + 8 * ch + k] * lift : 0.0f;
+    for (int k = 0; k < 8; ++k) w[k] = 8 * ch + k < D ? e0[(size_t)c * D + 8 * ch + k] * kOperandLift : 0.0f;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
         uint32_t o[4];
@@ -350,16 +350,6 @@ __global__ void kvq_build_encode_operands_kernel(const float *e0, int D, float l
         }
         *reinterpret_cast<uint4 *>(dst + (t ? operand_bytes(D) / 2 : 0)) = make_uint4(o[0], o[1], o[2], o[3]);
     }
-    if (i == 0) *reinterpret_cast<float *>(out + operand_bytes(D)) = 1.0f / lift;
-}
-
-// 2^k, what brings the table's largest entry into [2^13, 2^14): the first fp16 term stays below fp16's maximum and the second above its
-// subnormals
-float operand_lift(float table_max)
-{
-    int e = 0;
-    (void)std::frexp(std::fmin(std::fmax(table_max, 1e-30f), 1e30f), &e);   // table_max = m 2^e, m in [1/2, 1)
-    return std::ldexp(1.0f, 14 - e);
 }
 
 template <int D, bool PERVEC>
@@ -389,6 +379,7 @@ cudaError_t launch(int64_t N, const FftParams &f, cudaStream_t stream)
     prm.rpl = (uint32_t)(f.rows_per_lambda < N ? f.rows_per_lambda : N);
     prm.n_lambda = f.n_lambda;
     prm.out_map = f.out_map;
+    prm.unlift = 1.0f / kOperandLift;
     prm.bits = f.bits;
     prm.status = f.status;
     prm.first_wait_polls = f.first_wait_polls ? f.first_wait_polls : kWaitPolls;
@@ -406,10 +397,10 @@ cudaError_t launch(int64_t N, const FftParams &f, cudaStream_t stream)
 
 }  // namespace
 
-cudaError_t build_encode_operands(int D, const float *e0, float table_max, unsigned char *out)
+cudaError_t build_encode_operands(int D, const float *e0, unsigned char *out)
 {
     const int n = D * ((D + 63) / 64 * 8);
-    kvq_build_encode_operands_kernel<<<(n + 127) / 128, 128>>>(e0, D, operand_lift(table_max), out);
+    kvq_build_encode_operands_kernel<<<(n + 127) / 128, 128>>>(e0, D, out);
     const cudaError_t e = cudaGetLastError();
     return e != cudaSuccess ? e : cudaStreamSynchronize(nullptr);
 }
@@ -427,7 +418,7 @@ bool umma_append_pays(int D, bool bf16, bool per_vector, int64_t N, const FftPar
 {
     if (bf16 || (D == 256 && per_vector)) return false;
     if (N == 0) return true;
-    if (!f.append) return false;
+    if (!f.append || !f.operands) return false;
     static DeviceSlots slots;
     int dev = 0;
     if (current_device_slot(&dev) != cudaSuccess) return false;
