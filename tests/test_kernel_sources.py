@@ -45,3 +45,15 @@ def test_non_coherent_loads_read_the_plans_tables_only():
             b = body(text, kernel.group(1) + "(")
             if "load_input" in b:
                 assert 0 <= b.find("grid_wait()") < b.index("load_input"), "%s: %s reads an input before grid_wait" % (name, kernel.group(1))
+
+
+def test_a_warp_is_together_at_the_instructions_that_want_it_so():
+    """Cluster barriers and tensor-memory allocation are .aligned: every lane of the warp executes them together.  Callers come out of branches
+    that some lanes take (a row maximum sent by the first lanes, a status bit raised or barriers set up by one thread)."""
+    text = source("kvq_umma.cuh")
+    for helper in ("cluster_arrive", "cluster_wait", "cluster_sync_all", "tmem_alloc", "tmem_alloc_pair"):
+        b = body(text, "void %s(" % helper)
+        assert re.match(r"\{\s*__syncwarp\(\);\s*asm volatile", b), helper
+    for name in sorted(os.listdir(CSRC)):   # and nobody goes past the helpers
+        if name != "kvq_umma.cuh":
+            assert not re.search(r"barrier\.cluster|tcgen05\.alloc", source(name)), name
