@@ -20,8 +20,9 @@
  *   - every data pointer is a DEVICE pointer owned by the caller unless it says "host".
  *     The library owns only the plan and the small device tables hanging off it.
  *   - calls are asynchronous on the given CUDA stream (a cudaStream_t passed as void*,
- *     NULL = default stream).  The first use of a plan on a device allocates its small tables and
- *     copies them with a blocking copy; kvq_plan_prepare does that, and the per-kernel set-up,
+ *     NULL = default stream).  The first use of a plan on a device allocates its small tables, copies
+ *     them with a blocking copy and waits for a small kernel on the legacy default stream that derives
+ *     one of them; kvq_plan_prepare does that, and the per-kernel set-up,
  *     ahead of time, after which the compute calls allocate nothing and never synchronize.
  *   - every function returns a kvq_status_t; nothing throws across the boundary.
  *     Arguments are validated on the host before any CUDA call is made.
@@ -66,7 +67,8 @@ typedef enum {
                            a rotation) and the encode from fp16.  At most 2^31 - 1 rows per call (AUTO falls back
                            to the register FFT beyond).
                            Elsewhere the compute calls return KVQ_ERR_UNSUPPORTED_DIM. */
-    KVQ_IMPL_MATVEC = 3 /* fp32 matrix-vector product with the plan's D x D table, a CTA per 8 vectors: every D, dtype
+    KVQ_IMPL_MATVEC = 3 /* fp32 matrix-vector product with the plan's D x D table, a CTA per 8 vectors (in the smallest
+                           calls, up to a few hundred vectors, two to five CTAs, with the same results): every D, dtype
                            and layout, rotated plans included; meant for small calls, correct (and slow) at any size */
 } kvq_impl_t;
 
@@ -109,6 +111,11 @@ kvq_status_t kvq_plan_create_ex(int D, int group, int bits, uint64_t seed, kvq_p
  * UNSUPPORTED_DIM.
  * If the plan's device tables already exist they are rewritten after a device synchronisation: call it with the
  * plan's device current and no call using the plan in flight on another thread.
+ * CUDA graphs recorded before the call: kvq_encode and kvq_append where a tensor-core or matrix-vector kernel serves
+ * them, and kvq_append_at, read the tables as they are when they run and so follow the rotation (an R that takes the
+ * largest entry of R times the transform out of [0.06, 3.9), as no rotation does, excepted).  A recorded call keeps
+ * its kernel, though, and the others may hold one that is for plans without a rotation (the register FFT, the tensor-core
+ * decode that uses the plain transform's symmetry): record kvq_decode and kvq_flush_block again.
  * Errors: INVALID_ARG (null plan, non-finite entry, wrong device), NOMEM, CUDA.
  */
 kvq_status_t kvq_plan_set_rotation(kvq_plan_t *plan, const float *R_host /* [D, D] or NULL */);
@@ -132,8 +139,9 @@ kvq_status_t kvq_plan_set_impl(kvq_plan_t *plan, kvq_impl_t encode_impl, kvq_imp
 
 /*
  * kvq_plan_prepare -- everything a compute call would otherwise do on its first use, done now, on the
- * device that is current: allocates the plan's device tables (a status word; two [D, D] fp32 tables
- * where a tensor-core or matrix-vector kernel serves the plan), fills them with blocking copies, and
+ * device that is current: allocates the plan's device tables in one piece (a status word; two [D, D] fp32 tables;
+ * the tensor-core append's operands, 256 D ceil(D / 64) bytes), fills the tables with a blocking copy and the operands by
+ * a small kernel on the legacy default stream, which it waits for, and
  * sets the launch attributes (shared-memory size, occupancy look-ups) of every kernel that a call with
  * this plan and this 16-bit type can take, whichever family kvq_plan_set_impl or AUTO picks later.
  *   dtype   the type of x / out in the calls that follow; call once per type that will be used.
@@ -148,14 +156,16 @@ kvq_status_t kvq_plan_set_impl(kvq_plan_t *plan, kvq_impl_t encode_impl, kvq_imp
 kvq_status_t kvq_plan_prepare(kvq_plan_t *plan, kvq_dtype_t dtype);
 
 /*
- * kvq_plan_set_wait_limit -- how long the tensor-core encode kernel (D <= 160) lets its first wait run.
+ * kvq_plan_set_wait_limit -- how long the tensor-core encode kernel of D <= 160 and the tensor-core append kernel (fp16
+ * appends of many streams, every D) let their first wait run.
  * Every device-side wait in the library is bounded (about 2^22 polls, seconds of wall time) and ends in
  * a status bit instead of a hang.  This knob shortens ONE of them, the wait of the role that issues the
- * tensor-core instructions for the kernel's first operand build, a point at which that role has
- * nothing in flight: with a limit of a few polls the launch gives up at once, writes nothing, frees
- * what it holds and raises bit 2 of the status word, so that an integration can see KVQ_ERR_TIMEOUT
+ * tensor-core instructions for the kernel's first operands (built by the encode kernel, copied by the append kernel), a
+ * point at which that role has nothing in flight: with a limit of a few polls the launch gives up at once, writes nothing,
+ * frees what it holds and raises bit 2 of the status word, so that an integration can see KVQ_ERR_TIMEOUT
  * reported and cleared without a fault.
- *   polls   0 restores the default.  Takes effect for later kvq_encode / kvq_append calls on this plan.
+ *   polls   0 restores the default.  Takes effect for later kvq_encode / kvq_append / kvq_flush_block calls on this plan that
+ *           those kernels serve.
  */
 kvq_status_t kvq_plan_set_wait_limit(kvq_plan_t *plan, uint32_t polls);
 
@@ -214,6 +224,10 @@ kvq_status_t kvq_decode(kvq_plan_t *plan, const uint8_t *packed, const void *sca
  * caches laid out packed_cache [S, T_max, D/2] and scales_cache [S, T_max, D/group].
  * Stream i uses lambda row i / streams_per_lambda (row 0 when n_lambda == 1).  No other row
  * of the caches is touched.  Requires 0 <= pos < T_max.
+ * The same vectors stored by kvq_append, kvq_append_at, kvq_encode and kvq_flush_block give the same bytes where the
+ * same kernel serves the calls.  The kernels (matrix-vector; tensor-core encode; tensor-core append, for fp16 appends
+ * of many streams) round the transform and lambda at different places, so between them a few codes in a
+ * million, those at a rounding tie, lie one step apart, and up to two scales in a thousand by one fp16 step.
  */
 kvq_status_t kvq_append(kvq_plan_t *plan, const void *x_new /* [S, D] */, kvq_dtype_t dtype, int64_t S,
                         const float *lambda, int64_t n_lambda, int64_t streams_per_lambda,
@@ -224,7 +238,7 @@ kvq_status_t kvq_append(kvq_plan_t *plan, const void *x_new /* [S, D] */, kvq_dt
  * kvq_flush_block -- the residual-window flush with the dequantized-prefix cache (Sec. 7.2: new tokens wait in a short
  * fp16 window; when it is full the block is quantized, and the already dequantized prefix is kept, so that a decode step
  * costs O(new rows) instead of O(prefix)).  Quantizes `rows` new vectors of each of S streams into rows
- * [pos0, pos0 + rows) of the int4 caches (exactly what `rows` kvq_append calls would store) and writes the dequantized
+ * [pos0, pos0 + rows) of the int4 caches (what `rows` kvq_append calls would store; see there for ties) and writes the dequantized
  * values of those rows (what kvq_decode of the caches gives there, bit for bit where both calls take the same kernel
  * family) into the same rows of dq_cache.
  *   x_block       device, [S, rows, D] row-major, fp16 or bf16 per `dtype`; 16-byte aligned.
@@ -249,7 +263,8 @@ kvq_status_t kvq_flush_block(kvq_plan_t *plan, const void *x_block, kvq_dtype_t 
  *                 kernel runs, so the same call -- or a CUDA graph that holds it -- serves successive positions once
  *                 the caller updates that word on the same stream.  A value outside [0, T_max - 1] (append) or
  *                 [0, T_max - rows] (flush) writes nothing and raises bit 4 of the plan's device status word.
- * Everything else as in kvq_append / kvq_flush_block (same stored bytes, same dequantized rows).  Both always take the
+ * Everything else as in kvq_append / kvq_flush_block (the same stored bytes and dequantized rows where those take the
+ * matrix-vector kernels too; else see kvq_append for ties).  Both always take the
  * matrix-vector kernels, one launch whatever S and rows are (kvq_plan_set_impl is not consulted).  The first call of an
  * entry point for a given plan layout and dtype on a device allocates the plan's tables and sets the kernel's launch
  * attributes; every later one makes no CUDA call but the launch, and so can be recorded into a CUDA graph: make one call
@@ -313,7 +328,8 @@ kvq_status_t kvq_decode_static(kvq_plan_t *plan, const uint8_t *packed, const vo
 /* Static, human-readable name of a status code. */
 const char *kvq_status_string(kvq_status_t status);
 
-/* Number of kernels the library has launched in this process (all plans, all streams). */
+/* Number of kernels that compute calls have launched in this process (all plans, all streams).  What prepares a plan's
+ * tables (its first use, kvq_plan_prepare, kvq_plan_set_rotation) is not counted. */
 uint64_t kvq_launch_count(void);
 
 #ifdef __cplusplus
