@@ -1,4 +1,6 @@
 """GPU parity: the CUDA path, called through the C ABI, against the fp64 oracle on the same seeded inputs."""
+import re
+
 import numpy as np
 import pytest
 import torch
@@ -227,6 +229,25 @@ def test_d256_encode_at_the_edges_of_a_cta_pair_tile(dtype, N, n_lambda, rpl):
     assert enc["mismatches"] <= max(2, int(1e-4 * N * 256))
 
 
+def served_by(call):
+    """Names of the kernels that `call` launches, as a recording of it holds them (what it needs besides has been set up by then)."""
+    from cuda.bindings import driver
+
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    nodes = driver.cuGraphGetNodes(driver.CUgraph(graph.raw_cuda_graph()), 8)
+    names = []
+    for node in nodes[1][:nodes[-1]]:
+        err, kernel = driver.cuGraphKernelNodeGetParams(node)
+        assert int(err) == 0, err
+        names += re.findall(r"kvq_(?:(?!kvq_)\w)*?_kernel", driver.cuFuncGetName(kernel.func)[1].decode())
+    del graph
+    return names
+
+
 def run_append(D, S, n_lambda, spl, per_vector=False, nbits=4):
     """An fp16 append on the tensor cores into row 1 of three, against the oracle."""
     plan = kb.Plan(D, D if per_vector else G, 6, bits=nbits)
@@ -257,6 +278,122 @@ def test_append_on_both_sides_of_its_limit(D, per_vector, nbits, tiles):
     """The longest call of the append kernel and one vector more, and a layout that it is not built for."""
     for S in (tiles * 128, tiles * 128 + 1):
         run_append(D, S, 1, 0, per_vector, nbits)
+
+
+@pytest.mark.parametrize("D,per_vector,nbits", [(64, False, 4), (64, True, 8), (96, True, 4), (128, False, 8), (128, True, 4), (160, False, 4), (256, False, 4), (256, False, 8)])
+def test_append_of_a_plan_whose_rotation_comes_and_goes(D, per_vector, nbits):
+    """The append kernel's operands are split from the table with the rotation in it: set before the tables exist, another one on the
+    tables, none."""
+    S, rpl = 2 * 128 + 5, 100
+    plan = kb.Plan(D, D if per_vector else G, 6, bits=nbits)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_AUTO)
+    x, lam = wl.make_vectors(S, D, "f16", "k_outlier", 51), wl.make_lambda(3, D, 52)
+    xd, lamd = x.cuda(), lam.cuda()
+    packed = torch.zeros(S, 2, D * nbits // 8, dtype=torch.uint8, device="cuda")
+    scales = torch.zeros(S, 2, D // plan.group, dtype=torch.float16, device="cuda")
+    call = lambda: kb.kvq_append(plan.handle, xd, lamd, packed, scales, 1, rpl)
+    for R in (wl.make_rotation(D, 53), wl.make_rotation(D, 54, 0.02), None):
+        plan.set_rotation(R)
+        packed.zero_(), scales.zero_()
+        call()
+        torch.cuda.synchronize()
+        ora = ko.encode(bits(x), ko.F16, plan.signs(), lam.numpy(), plan.group, rpl, want_v=True, bits=nbits,
+                        rot=None if R is None else R.numpy().astype(np.float64))
+        parity.check_encode(packed[:, 1].contiguous().cpu().numpy(), bits(scales[:, 1].contiguous()), ora, plan.group, "rotated append", bits=nbits, min_agree=0.9995)
+        assert not bool(packed[:, 0].any()) and not bool(scales[:, 0].any())
+    assert served_by(call) == ["kvq_append_umma_kernel"]
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    plan.close()
+
+
+@pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
+def test_append_of_degenerate_rows(D):
+    """Zero, subnormal, saturating and single-spike rows against the oracle; rows with infinities and NaN among them change no other row's
+    bytes and store codes in range and scales that are numbers."""
+    x = _degenerate_rows(D, "f16")
+    S = x.shape[0]
+    wild = x.clone()
+    bad = torch.arange(5, S, 37)
+    wild[bad, torch.arange(len(bad)) % D] = torch.tensor([float("inf"), float("-inf"), float("nan")], dtype=torch.float16).repeat(len(bad))[:len(bad)]
+    wild[bad[-1]] = float("nan")
+    keep = torch.ones(S, dtype=torch.bool)
+    keep[bad] = False
+    for lam in (torch.ones(1, D), wl.make_lambda(1, D, 18), 16.0 * wl.make_lambda(1, D, 19)):
+        plan = kb.Plan(D, G, 17)
+        kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_AUTO)
+
+        def append(rows):
+            packed, scales = torch.zeros(S, 1, D // 2, dtype=torch.uint8, device="cuda"), torch.zeros(S, 1, D // G, dtype=torch.float16, device="cuda")
+            xd, lamd = rows.cuda(), lam.cuda()
+            call = lambda: kb.kvq_append(plan.handle, xd, lamd, packed, scales, 0)
+            assert served_by(call) == ["kvq_append_umma_kernel"]
+            call()
+            torch.cuda.synchronize()
+            return packed[:, 0].cpu(), scales[:, 0].cpu()
+
+        packed, scales = append(x)
+        assert bool(torch.isfinite(scales).all())
+        ora = ko.encode(bits(x), ko.F16, plan.signs(), lam.numpy(), G, want_v=True)
+        parity.check_encode(packed.contiguous().numpy(), bits(scales), ora, G, "degenerate append", min_agree=0.999)
+        assert not packed[0::13].any() and not scales[0::13].any()
+        pw, sw = append(wild)
+        assert torch.equal(pw[keep], packed[keep]) and torch.equal(sw[keep], scales[keep])
+        assert bool(torch.isfinite(sw).all()) and not bool(((pw & 15) == 8).any()) and not bool(((pw >> 4) == 8).any())
+        assert kb.kvq_plan_device_status(plan.handle) == 0
+        plan.close()
+
+
+@pytest.mark.parametrize("D,per_vector,half_tiles,per_row", [(64, False, 5, 2), (64, True, 3, 1), (96, False, 16, 4), (128, False, 20, 5), (128, True, 10, 2),
+                                                             (160, False, 8, 8), (160, True, 5, 4), (256, False, 14, 8)])
+def test_which_kernel_serves_an_append(D, per_vector, half_tiles, per_row):
+    """On both sides of the append kernel's limit, with one lambda row and with three, whatever the device's number of SMs."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    plan = kb.Plan(D, D if per_vector else G, 6)
+    kb.kvq_plan_prepare(plan.handle, torch.float16)
+    encode = "kvq_encode_umma_d256_kernel" if D == 256 else "kvq_encode_umma_kernel"
+    for rows in (1, 3):
+        most = 128 * ((half_tiles * sms + 2 * per_row * (rows - 1)) // 2)
+        x, lam = torch.zeros(most + 1, D, dtype=torch.float16, device="cuda"), torch.ones(rows, D, device="cuda")
+        packed, scales = plan.empty_packed(most + 1).view(most + 1, 1, -1), plan.empty_scales(most + 1).view(most + 1, 1, -1)
+        for S, kernel in ((most, "kvq_append_umma_kernel"), (most + 1, encode)):
+            assert served_by(lambda: kb.kvq_append(plan.handle, x[:S], lam, packed[:S], scales[:S], 0, -(-S // rows))) == [kernel], (rows, S)
+        assert served_by(lambda: kb.kvq_encode(plan.handle, x[:most], lam, packed[:most, 0], scales[:most, 0], -(-most // rows))) == [encode]
+    plan.close()
+
+
+@pytest.mark.parametrize("spread", ["calibrated", "wide", "flat"])
+@pytest.mark.parametrize("D", [64, 128, 256])
+def test_append_is_no_further_from_64_bits_than_the_encode(D, spread):
+    """The append kernel rounds lambda once, after the sum, the encode kernels fold it into 22 bits of every table entry.  Codes on the
+    other side of a tie and scales one fp16 step off, against 64 bits on the same vectors: no more of them than the encode's.  (Counts of
+    some tens and of some hundreds: four standard deviations of the difference of two such counts.)"""
+    S, rpl = 5120, 128
+    plan = kb.Plan(D, G, 7)
+    off, bytes_apart = np.zeros((2, 2), dtype=np.int64), 0
+    for i in range(6):
+        x = wl.make_vectors(S, D, "f16", "k_outlier", 90 + i)
+        lam = wl.make_lambda(S // rpl, D, 100 + i)
+        if spread == "wide":
+            g = torch.Generator().manual_seed(i)
+            lam = torch.exp(18.0 * torch.rand(S // rpl, D, generator=g) - 9.0)
+        elif spread == "flat":
+            lam = 1.0 + 1e-3 * (lam / lam.max())
+        xd, lamd = x.cuda(), lam.cuda()
+        a = torch.zeros(S, 1, D // 2, dtype=torch.uint8, device="cuda"), torch.zeros(S, 1, D // G, dtype=torch.float16, device="cuda")
+        append = lambda: kb.kvq_append(plan.handle, xd, lamd, *a, 0, rpl)
+        append()
+        e = gpu_encode(plan, xd, lamd, rpl)
+        ora = ko.encode(bits(x), ko.F16, plan.signs(), lam.numpy(), G, rpl, want_v=True)
+        for k, (p, s) in enumerate((a, e)):
+            p, s = p.view(S, -1).cpu().numpy(), bits(s.view(S, -1))
+            parity.check_encode(p, s, ora, G, "append" if k == 0 else "encode")
+            off[k] += (ko.unpack_nibbles(p) != ora["codes"]).sum(), (s != ora["scales"]).sum()
+        bytes_apart += int((a[0].view(S, -1) != e[0]).sum())
+    assert served_by(append) == ["kvq_append_umma_kernel"]
+    print("append, encode: codes, scales off 64 bits", off.tolist(), "of", 6 * S * D, 6 * S * D // G, "bytes apart", bytes_apart)
+    assert (off[0] <= off[1] + 4 * np.sqrt(off.sum(axis=0)) + 4).all()
+    assert bytes_apart <= 2e-5 * 3 * S * D
+    plan.close()
 
 
 @pytest.mark.parametrize("D,dtype,per_vector,nbits", [(64, "f16", False, 4), (64, "bf16", True, 4), (96, "f16", True, 8), (96, "bf16", False, 4),
@@ -826,6 +963,30 @@ def test_matvec_kernels_sliced_over_several_ctas(D, dtype, per_vector, nbits, mo
         torch.cuda.synchronize()
         assert kb.kvq_plan_device_status(plan.handle) == 0
         assert torch.equal(p2, packed) and torch.equal(s2, scales) and torch.equal(dq.view(torch.int16), out.view(torch.int16))
+    plan.close()
+
+
+@pytest.mark.parametrize("D,dtype,per_vector,op,tenths", [(64, "f16", False, "decode", 10), (64, "bf16", False, "append", 20), (64, "f16", True, "append", 0), (96, "bf16", True, "append", 0),
+                                                          (96, "f16", False, "append", 20), (128, "f16", False, "append", 20), (128, "bf16", True, "append", 9), (128, "f16", False, "flush", 6),
+                                                          (160, "f16", False, "decode", 20), (160, "f16", False, "flush", 0), (256, "f16", False, "append", 10), (256, "bf16", True, "append", 9),
+                                                          (256, "bf16", False, "flush", 9), (256, "f16", False, "decode", 10)])
+def test_which_matvec_kernel_serves_a_small_call(D, dtype, per_vector, op, tenths):
+    """On both sides of the sliced form's limit (CTAs per ten SMs), whatever the device's number of SMs."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    dt = wl.torch_dtype(dtype)
+    plan = kb.Plan(D, D if per_vector else G, 31)
+    kb.kvq_plan_prepare(plan.handle, dt)
+    most = 8 * (tenths * sms // 10 // (4 if D == 256 else D // 32))
+    x, lam = torch.zeros(most + 1, 1, D, dtype=dt, device="cuda"), torch.ones(1, D, device="cuda")
+    packed, scales = plan.empty_packed(most + 1).zero_().view(most + 1, 1, -1), plan.empty_scales(most + 1).zero_().view(most + 1, 1, -1)
+    dq = torch.zeros_like(x)
+    for N, kind in ((most, "_sliced"), (most + 1, "")):
+        if N == 0:
+            continue
+        b = packed[:N], scales[:N]
+        call = {"append": lambda: kb.kvq_append(plan.handle, x[:N, 0], lam, *b, 0), "flush": lambda: kb.kvq_flush_block(plan.handle, x[:N], lam, *b, dq[:N], 0),
+                "decode": lambda: kb.kvq_decode(plan.handle, b[0][:, 0], b[1][:, 0], lam, x[:N])}[op]
+        assert served_by(call) == ["kvq_%s_matvec%s_kernel" % ("decode" if op == "decode" else "encode", kind)], N
     plan.close()
 
 

@@ -182,6 +182,33 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_service_returns():
     plan.close()
 
 
+@pytest.mark.parametrize("D", [64, 128, 256])
+def test_the_append_kernels_first_wait_is_reported_and_service_returns(D):
+    """The same limit governs the append kernel's wait for its operands: they are then asked for when the wait begins, so that one poll is
+    over before they can be there."""
+    S = 100
+    plan = kb.Plan(D, G, 510)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_AUTO)
+    x, lam = wl.make_vectors(S, D, "f16", "gaussian", 511), wl.make_lambda(1, D, 512)
+    xd, lamd = x.cuda(), lam.cuda()
+    packed = torch.full((S, 2, D // 2), 0xAB, dtype=torch.uint8, device="cuda")
+    scales = torch.full((S, 2, D // G), 1.25, dtype=torch.float16, device="cuda")
+    kb.kvq_plan_set_wait_limit(plan.handle, 1)
+    kb.kvq_append(plan.handle, xd, lamd, packed, scales, 1)
+    torch.cuda.synchronize()
+    word = kb.kvq_plan_device_status(plan.handle)
+    assert word & 7 == 4, "status word %d" % word
+    assert bool((packed == 0xAB).all()) and bool((scales == 1.25).all())
+    kb.kvq_plan_clear_device_status(plan.handle)
+    kb.kvq_plan_set_wait_limit(plan.handle, 0)
+    kb.kvq_append(plan.handle, xd, lamd, packed, scales, 1)
+    torch.cuda.synchronize()
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    ora = ko.encode(wl.raw_bits(x), ko.F16, plan.signs(), lam.numpy(), G, want_v=True)
+    parity.check_encode(packed[:, 1].contiguous().cpu().numpy(), wl.raw_bits(scales[:, 1].contiguous()), ora, G, "append after a reported time-out", min_agree=0.9995)
+    plan.close()
+
+
 @pytest.mark.parametrize("D,dtype,group,nbits", [(64, "bf16", 32, 4), (96, "f16", 32, 4), (128, "f16", 32, 4), (128, "bf16", 128, 8),
                                                  (160, "bf16", 32, 4), (256, "bf16", 32, 4), (256, "f16", 256, 4), (256, "bf16", 32, 8)])
 def test_a_call_queued_behind_another_sees_all_that_it_wrote(D, dtype, group, nbits):
