@@ -585,23 +585,23 @@ constexpr auto sliced_kernel()
 template <int D, bool BF16, int MODE>
 cudaError_t launch(const MatvecParams &prm, cudaStream_t stream)
 {
-    static DeviceSlots slots;
+    static DeviceSlots slots, sliced_slots;   // CTAs of the kernel that the device holds at once; its SMs, 0 where the sliced form does not fit as often as it is meant to
     int dev = 0;
     cudaError_t e = current_device_slot(&dev);
     if (e != cudaSuccess) return e;
     constexpr bool kSliced = MODE != 2 || Slice<D>::kCluster;
     auto kern = MODE == 0 ? kvq_decode_matvec_kernel<D, BF16> : MODE == 1 ? kvq_encode_matvec_kernel<D, BF16, false> : kvq_encode_matvec_kernel<D, BF16, true>;
-    if (slots.sms[dev] == 0) {   // slots.sms: the CTAs of this kernel that the device holds at once
+    if (slots.sms[dev] == 0) {
         int sms = 0, per_sm = 0;
         if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<D>::kSmemBytes)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWarps * 32, Geo<D>::kSmemBytes)) != cudaSuccess) return e;
-        if constexpr (kSliced) {   // slots.blocks_per_sm: the SMs, where the sliced form fits as often as it is meant to
+        if constexpr (kSliced) {
             int sliced_per_sm = 0;
             auto sliced = sliced_kernel<D, BF16, MODE>();
             if ((e = cudaFuncSetAttribute(sliced, cudaFuncAttributeMaxDynamicSharedMemorySize, Slice<D>::kSmemBytes)) != cudaSuccess) return e;
             if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&sliced_per_sm, sliced, kWarps * 32, Slice<D>::kSmemBytes)) != cudaSuccess) return e;
-            slots.blocks_per_sm[dev] = sliced_per_sm >= (D == 256 ? 1 : 2) ? sms : 0;
+            sliced_slots.sms[dev] = sliced_per_sm >= (D == 256 ? 1 : 2) ? sms : 0;
         }
         slots.sms[dev] = sms * (per_sm > 0 ? per_sm : 1);
     }
@@ -611,7 +611,7 @@ cudaError_t launch(const MatvecParams &prm, cudaStream_t stream)
     if constexpr (kSliced) {
         constexpr int kSlices = Slice<D>::kSlices;
         const bool cluster = MODE == 2 || (MODE == 1 && prm.group == D);
-        if (10 * batches * kSlices <= (int64_t)sliced_tenths<D, MODE>(cluster, prm.group == D) * slots.blocks_per_sm[dev] && (Slice<D>::kCluster || !cluster))
+        if (10 * batches * kSlices <= (int64_t)sliced_tenths<D, MODE>(cluster, prm.group == D) * sliced_slots.sms[dev] && (Slice<D>::kCluster || !cluster))
             return launch_kernel(sliced_kernel<D, BF16, MODE>(), (unsigned)(batches * kSlices), kWarps * 32, Slice<D>::kSmemBytes, stream, cluster ? kSlices : 1, prm);
     }
     // one resident wave of CTAs that loop over batches where the kernel does; else a CTA per batch
