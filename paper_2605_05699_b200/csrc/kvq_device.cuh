@@ -205,7 +205,7 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 // which a volatile statement does not pass.  __ldg is neither: the non-coherent load is for memory that nobody writes
 // while the kernel runs, from its launch on, and the compiler may move it past the wait.  It is for the plan's tables.
 // (As ordinary loads of C++ the same reads hold up what stands around them more: 212,992 bf16 vectors decoded at D = 256 under 52
-// lambda rows 54.9 us, so 54.3, through __ldg 54.3.)
+// lambda rows 54.9 us, so 54.3, through __ldg 54.3, alternating on one box; boxes and what ran before move that call between 53 and 59.)
 __device__ __forceinline__ uint16_t load_input(const uint16_t *p)
 {
     uint16_t v;

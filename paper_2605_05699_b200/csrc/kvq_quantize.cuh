@@ -5,8 +5,8 @@
 // the magnitudes take half an instruction each (max.abs of three: the absolute values are free), sums and products of
 // neighbouring values go in pairs (add / fma.f32x2, rounded like the single ones), the codes are gathered by byte permutes.
 // Encode of 2,097,152 vectors at D = 128, back to back: 183.1 -> 180.2 us (another box: 182.7 -> 181.1, inside the spread); D = 160, 700,000:
-// 97.5 -> 93.4; D = 256, 1,064,960: 269 -> 266.  With the maxima three at a time instead of two: 2,097,152 at D = 128 179.5 -> 177.8,
-// 212,992 bf16 under 52 lambda rows at D = 256 59.6 -> 59.2.
+// 97.5 -> 93.4; D = 256, 1,064,960: 269 -> 266.  The maxima three at a time instead of two are 17 instructions per
+// group in place of 31; in time 1 % or less, inside the spread of repeated runs (2,097,152 at D = 128 179.5 -> 177.8).
 #pragma once
 
 #include "kvq_device.cuh"

@@ -304,8 +304,8 @@ struct RecipLambda {
         }
         // Positive: ordered like their bits, and one redux each in place of five dependent shuffles; the row is scaled by an exact
         // reciprocal, one division in place of four (eight).  This stands between lambda's arrival and the first MMA, and again at every lambda
-        // row: decode of 1500 fp16 vectors at D = 256 10.0 -> 9.6 us, of 7100 under four rows at D = 128 6.4 -> 6.25, of 212,992 under 52
-        // at D = 256 41.2 -> 40.0.
+        // row: decode of 1500 fp16 vectors at D = 256 10.0 -> 9.6 us, of 7100 under four rows at D = 128 6.4 -> 6.25 (one after another; with the D = 256
+        // decode's first operand as it was before FirstRows).
         mx = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(mx)));
         mn = __uint_as_float(__reduce_min_sync(0xFFFFFFFFu, __float_as_uint(mn)));
         rho = __uint_as_float(__float_as_uint(mx) & 0x7F800000u);   // 2^floor(log2 max): exact to divide by

@@ -10,8 +10,9 @@
 //     lambda row: 2 us of a call of one tile per CTA.
 //   * A tile is any 128 consecutive vectors, whatever lambda rows they have: 160 lambda rows of 32 vectors are 40 full tiles, not 160.
 //
-// Back to back, before -> now: D = 128, 5120 vectors under 160 lambda rows 9.4 -> 3.8 us, 4096 under one 5.8 -> 3.8; D = 256, 4950 under two
-// 9.4 -> 4.9.  What is left is the launch (2.2 us), one tile's way through the roles and the stores' drain.
+// Back to back, before -> now, caches of 2 rows per stream: D = 128, 5120 vectors under 160 lambda rows 9.4 -> 3.9 us, 4096 under one 6.1 -> 3.9; D = 256,
+// 4950 under two 9.5 -> 5.0.  Of 256 rows, each vector's bytes then on lines and pages of their own: 9.4 -> 4.4, 6.1 -> 4.4, 9.8 -> 5.3.
+// What is left is the launch (2.2 us), one tile's way through the roles and the stores' drain.
 // Appends alone take it.  Where lambda is rounded decides one to three codes in a million, those at a tie, and kvq_encode and the block
 // flush, whose rows are also compared dequantized, keep the rounding they have.  bf16 stays with the kernels above: with two bf16
 // terms, 16 bits, it would be ten times as many.

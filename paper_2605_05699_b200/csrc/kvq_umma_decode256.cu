@@ -113,7 +113,8 @@ __device__ __forceinline__ void put_b_row(unsigned char *sB, const float4 m0, co
 
 // The first B: eight rows of both parities per builder warp, requested in front of the grid wait and all together.  (Before, a warp took
 // sixteen rows of one parity in two round trips behind lambda, and every row crossed L2 for each parity.  Back to back, 1500 fp16
-// vectors 9.7 -> 7.6 us, 10,000: 10.3 -> 8.9; bf16 11.1 -> 9.5, 12.0 -> 11.0; 212,992: 36.9 -> 33.9, 48.9 -> 46.9.)
+// vectors 9.7 -> 7.6 us, 10,000: 10.3 -> 8.9; bf16 11.1 -> 9.5, 12.0 -> 11.0; 212,992 under one lambda row 36.9 -> 33.9, 48.9 -> 46.9, in short
+// runs; with the board at its power limit, behind long encodes, and together with RecipLambda's redux: 46 -> 40, 58 -> 54.)
 constexpr int kFirstRows = kHalf / 16;
 struct FirstRows {
     float4 m[kFirstRows][2];
