@@ -64,17 +64,20 @@ def _build_call(force: bool) -> None:
             built_for = f.read()
     if not force and built_for == torch.__version__ and os.path.getmtime(CALL) >= max(os.path.getmtime(CALL_SRC), os.path.getmtime(os.path.join(INCLUDE, "kvq.h"))):
         return
-    if os.path.exists(CALL):   # out of date: not left behind where the compiler fails
-        os.remove(CALL)
     root = os.path.dirname(torch.__file__)
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = CALL + ".tmp.%d" % os.getpid()
-    subprocess.check_call([
-        "g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
-        '-DKVQ_TORCH="%s"' % torch.__version__,
-        "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
-        "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), CALL_SRC, "-o", tmp,
-        "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    try:
+        subprocess.check_call([
+            "g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+            '-DKVQ_TORCH="%s"' % torch.__version__,
+            "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+            "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), CALL_SRC, "-o", tmp,
+            "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"])
+    except Exception:
+        if os.path.exists(CALL):   # out of date: not left behind
+            os.remove(CALL)
+        raise
     os.replace(tmp, CALL)
     with open(stamp, "w") as f:
         f.write(torch.__version__)
