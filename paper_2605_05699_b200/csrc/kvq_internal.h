@@ -4,7 +4,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <cmath>
 #include <mutex>
 
 #include "../../include/kvq.h"
