@@ -173,18 +173,24 @@ static kvq_status_t check_lambda(int64_t N, const float *lambda, int64_t n_lambd
 static void fill_params(const kvq_plan *p, FftParams &prm, int64_t N, const float *lambda, int64_t n_lambda,
                         int64_t rows_per_lambda)
 {
-    std::memset(&prm, 0, sizeof(prm));
+    std::memset(static_cast<void *>(&prm), 0, offsetof(FftParams, sign_xor));   // the signs: see sign_words
     prm.N = N;
     prm.lambda = lambda;
     prm.n_lambda = n_lambda;
-    prm.rows_per_lambda = rows_per_lambda < 1 ? 1 : rows_per_lambda;
+    prm.rows_per_lambda = FastDiv(rows_per_lambda);
     prm.out_map = RowMap{1, 1, 0};
     prm.in_map = RowMap{1, 1, 0};
     prm.status = p->d_status;
     prm.first_wait_polls = p->first_wait_polls;
     prm.bits = p->bits;
     prm.operands = p->table_max >= kOperandMin && p->table_max < kOperandMax ? p->d_operands : nullptr;
+}
+
+// the register-FFT kernels alone read the signs from their arguments; every other table has them folded in
+static const FftParams &sign_words(const kvq_plan *p, FftParams &prm)
+{
     std::memcpy(prm.sign_xor, p->sign_xor, sizeof(prm.sign_xor));
+    return prm;
 }
 
 extern "C" {
@@ -437,7 +443,7 @@ static kvq_status_t encode_common(kvq_plan_t *plan, const void *x, kvq_dtype_t d
         e = matvec_flush(plan->D, plan->group, plan->bits, bf16, N, prm, plan->d_b0, plan->d_e0, stream, pos);
         *fused = e == cudaSuccess;
     } else if (impl == KVQ_IMPL_MATVEC) e = matvec_encode(plan->D, plan->group, plan->bits, bf16, N, prm, plan->d_b0, stream, pos);
-    else e = fft_encode(plan->D, plan->group, plan->bits, bf16, N, prm, stream);
+    else e = fft_encode(plan->D, plan->group, plan->bits, bf16, N, sign_words(plan, prm), stream);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return KVQ_ERR_CUDA;
@@ -509,7 +515,7 @@ kvq_status_t kvq_decode(kvq_plan_t *plan, const uint8_t *packed, const void *sca
     prm.scales = const_cast<void *>(scales);
     prm.out = out;
     const cudaError_t e = impl == KVQ_IMPL_MATVEC ? matvec_decode(plan->D, plan->group, plan->bits, bf16, N, prm, plan->d_e0, stream)
-                                                  : fft_decode(plan->D, plan->group, plan->bits, bf16, N, prm, stream);
+                                                  : fft_decode(plan->D, plan->group, plan->bits, bf16, N, sign_words(plan, prm), stream);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return KVQ_ERR_CUDA;
@@ -611,7 +617,7 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
         return KVQ_OK;
     }
     const cudaError_t e = mv ? matvec_decode(plan->D, plan->group, plan->bits, bf16, N, prm, plan->d_e0, stream)
-                             : fft_decode(plan->D, plan->group, plan->bits, bf16, N, prm, stream);
+                             : fft_decode(plan->D, plan->group, plan->bits, bf16, N, sign_words(plan, prm), stream);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return KVQ_ERR_CUDA;

@@ -253,30 +253,41 @@ __device__ __forceinline__ float4 load_input(const float4 *p)
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
-// Tiles of the tensor-core kernels.  Rows are cut into lambda segments of `rpl` rows, a segment into
-// tiles of 128 rows (the last one of a segment may be short), tiles are numbered segment by segment.
-// The cursor walks a CTA's tiles without a 64-bit division per step.
+// Division by a number that the host knows.  The chip divides 64-bit integers in a chain of some hundred instructions, and every role of a
+// persistent kernel began with several such chains, one behind the other: 1.0 us of an encode's 6.7 per launch at one tile per CTA
+// (globaltimer marks in the kernel) stood between a CTA's start and its set-up barrier, 0.3 more in front of each role's first tile.
+// With m = ceil(2^(31 + s) / d), s = ceil(log2 d): floor(n m / 2^(31 + s)) = floor(n / d) for n < 2^31, because m d - 2^(31 + s) < d <= 2^s
+// (Granlund and Montgomery's multiplication by an invariant reciprocal).
 // ---------------------------------------------------------------------------
-struct TileCursor {
-    int64_t seg;   // lambda segment of the current tile
-    int64_t tin;   // index of the tile within its segment
-    int64_t tps;   // tiles per segment
-    __device__ __forceinline__ TileCursor(int64_t tile, int64_t tiles_per_segment)
-        : seg(tile / tiles_per_segment), tin(tile - (tile / tiles_per_segment) * tiles_per_segment), tps(tiles_per_segment)
+struct FastDiv {
+    int64_t d;
+    uint32_t mul, shift;
+    FastDiv() = default;
+    __host__ FastDiv(int64_t divisor) : d(divisor < 1 ? 1 : divisor), mul(0x80000000u), shift(0)
     {
-    }
-    __device__ __forceinline__ void advance(int step)
-    {
-        tin += step;
-        while (tin >= tps) {
-            tin -= tps;
-            ++seg;
+        if (d == 1) return;
+        if (d >> 31) {   // 2^31 and more: 0 for every n < 2^31
+            mul = 0;
+            return;
         }
+        shift = 32u - (uint32_t)__builtin_clz((uint32_t)(d - 1));
+        mul = (uint32_t)((((uint64_t)1 << (31 + shift)) + (uint64_t)d - 1) / (uint64_t)d);
     }
-    __device__ __forceinline__ bool first_of_segment() const { return tin == 0; }
-    __device__ __forceinline__ int64_t row_in_segment() const { return tin * 128; }
+    __host__ __device__ __forceinline__ uint32_t small(uint32_t n) const   // n < 2^31
+    {
+#ifdef __CUDA_ARCH__
+        return __umulhi(2u * n, mul) >> shift;
+#else
+        return (uint32_t)(((uint64_t)n * mul) >> 31 >> shift);
+#endif
+    }
+    __host__ __device__ __forceinline__ int64_t operator()(int64_t n) const { return n >> 31 ? n / d : (int64_t)small((uint32_t)n); }   // n >= 0
 };
 
+// ---------------------------------------------------------------------------
+// Tiles of the tensor-core kernels.  Rows are cut into lambda segments of `rpl` rows, a segment into
+// tiles of 128 rows (the last one of a segment may be short), tiles are numbered segment by segment.
+//
 // The contiguous share of a call's tiles that one CTA (or one CTA pair) of a persistent kernel takes: lambda segments of rpl
 // rows are cut into tiles of 128 rows (256 where a CTA pair works on one tile) (a segment's last tile may be short), n_seg * tps tiles in all, `parts` shares.
 // Contiguous, so that the B operand of a lambda row is rebuilt as rarely as possible.  `segs` consecutive segments have one
@@ -288,41 +299,91 @@ struct TileCursor {
 //   * else, with at least eight tiles per share, the shares are equal in COST, a lambda row counting one unit, the price's lower end,
 //     more than its tiles (a share that would begin inside that unit begins at the row's first tile);
 //   * else they are equal in tiles.
+// TilePlan is the call's half of that, worked out by the host (fewer than 2^31 tiles); TileShare is a CTA's.
+// ---------------------------------------------------------------------------
+struct TilePlan {
+    uint32_t tps;         // tiles per segment
+    uint32_t n_tiles;
+    uint32_t row_tiles;   // tiles per lambda row
+    uint32_t n_rows;      // lambda rows
+    uint32_t inside;      // shares stay inside lambda rows: per_row of them each
+    uint32_t per;         // tiles (inside) or cost units per share
+    uint32_t rebuild;     // cost units of a rebuild
+    FastDiv by_tps, by_per_row, by_cost;   // by_cost: units per lambda row
+    TilePlan() = default;
+    __host__ TilePlan(int64_t n_seg, int64_t rpl, unsigned parts, int tile_rows = 128, int64_t segs = 1)
+    {
+        const int64_t t = (rpl + tile_rows - 1) / tile_rows, tiles = n_seg * t;
+        if (segs > n_seg) segs = n_seg;
+        const int64_t rt = segs * t, rows = (n_seg + segs - 1) / segs, even = (tiles + parts - 1) / parts;
+        tps = (uint32_t)t, n_tiles = (uint32_t)tiles, row_tiles = (uint32_t)rt, n_rows = (uint32_t)rows;
+        inside = rebuild = 0;
+        by_tps = FastDiv(t), by_per_row = by_cost = FastDiv(1);
+        if (rows <= (int64_t)parts) {
+            const int64_t k = parts / rows, p = (rt + k - 1) / k;   // shares per lambda row, tiles per share
+            if (p <= even + 2 || rows == 1) {
+                inside = 1, per = (uint32_t)p, by_per_row = FastDiv(k);
+                return;
+            }
+        }
+        rebuild = tiles >= 8 * (int64_t)parts ? 1 : 0;
+        by_cost = FastDiv(rt + rebuild);
+        per = (uint32_t)((tiles + rows * rebuild + parts - 1) / parts);
+    }
+};
+
 struct TileShare {
     int64_t tps;     // tiles per segment
     int64_t begin;   // first tile of this share
     int n;           // tiles in this share
-    __host__ __device__ __forceinline__ TileShare(int64_t n_seg, int64_t rpl, unsigned part, unsigned parts, int tile_rows = 128, int64_t segs = 1)
+    uint32_t seg, tin;   // segment of the first tile, and its place there
+    __host__ __device__ __forceinline__ TileShare(const TilePlan &p, uint32_t part) : tps(p.tps)
     {
-        tps = (rpl + tile_rows - 1) / tile_rows;
-        const int64_t n_tiles = n_seg * tps;
-        if (segs > n_seg) segs = n_seg;
-        const int64_t row_tiles = segs * tps, n_rows = (n_seg + segs - 1) / segs;
-        const int64_t even = (n_tiles + parts - 1) / parts;
-        if (n_rows <= (int64_t)parts) {
-            const int64_t k = parts / n_rows, per = (row_tiles + k - 1) / k;   // shares per lambda row, tiles per share
-            if (per <= even + 2 || n_rows == 1) {
-                const int64_t row = part / k, from = (part - row * k) * per;
-                int64_t end = from + per < row_tiles ? from + per : row_tiles;
-                begin = row * row_tiles + from;
-                end += row * row_tiles;
-                if (end > n_tiles) end = n_tiles;
-                n = row < n_rows && end > begin ? (int)(end - begin) : 0;
-                return;
-            }
+        uint32_t from, to;
+        if (p.inside) {
+            const uint32_t row = p.by_per_row.small(part), r0 = row * p.row_tiles, at = (part - row * (uint32_t)p.by_per_row.d) * p.per;
+            from = r0 + at, to = r0 + (p.row_tiles - at > p.per && at < p.row_tiles ? at + p.per : p.row_tiles);
+            if (to > p.n_tiles) to = p.n_tiles;
+            if (row >= p.n_rows) to = from;
+        } else {
+            const int64_t total = (int64_t)p.n_tiles + (int64_t)p.n_rows * p.rebuild, u = (int64_t)part * p.per;
+            auto tile_of = [&](int64_t v) -> uint32_t {
+                if (v >= total) return p.n_tiles;
+                const int64_t row = p.by_cost(v);
+                const uint32_t w = (uint32_t)(v - row * p.by_cost.d);
+                return (uint32_t)row * p.row_tiles + (w > p.rebuild ? w - p.rebuild : 0u);
+            };
+            from = tile_of(u), to = tile_of(u + p.per);
         }
-        const int64_t R = n_tiles >= 8 * (int64_t)parts ? 1 : 0;   // cost units of a rebuild
-        const int64_t C = row_tiles + R, total = n_tiles + n_rows * R;
-        const int64_t per = (total + parts - 1) / parts;
-        auto tile_of = [&](int64_t u) -> int64_t {
-            if (u >= total) return n_tiles;
-            const int64_t row = u / C, w = u - row * C;
-            return row * row_tiles + (w > R ? w - R : 0);
-        };
-        begin = tile_of((int64_t)part * per);
-        const int64_t end = tile_of(((int64_t)part + 1) * per);
-        n = end > begin ? (int)(end - begin) : 0;
+        n = to > from ? (int)(to - from) : 0;
+        begin = from;
+        if (n == 0) from = 0;
+        seg = p.by_tps.small(from);
+        tin = from - seg * p.tps;
     }
+    __host__ TileShare(int64_t n_seg, int64_t rpl, unsigned part, unsigned parts, int tile_rows = 128, int64_t segs = 1)
+        : TileShare(TilePlan(n_seg, rpl, parts, tile_rows, segs), part)
+    {
+    }
+};
+
+// Walks a CTA's tiles, from its first one on.
+struct TileCursor {
+    int seg;   // lambda segment of the current tile
+    int tin;   // index of the tile within its segment
+    int tps;   // tiles per segment
+    __device__ __forceinline__ TileCursor(const TileShare &s) : seg((int)s.seg), tin((int)s.tin), tps((int)s.tps) {}
+    __device__ __forceinline__ TileCursor(const TileShare &s, int step) : TileCursor(s) { advance(step); }
+    __device__ __forceinline__ void advance(int step)
+    {
+        tin += step;
+        while (tin >= tps) {
+            tin -= tps;
+            ++seg;
+        }
+    }
+    __device__ __forceinline__ bool first_of_segment() const { return tin == 0; }
+    __device__ __forceinline__ int64_t row_in_segment() const { return (int64_t)tin * 128; }
 };
 
 // ---------------------------------------------------------------------------

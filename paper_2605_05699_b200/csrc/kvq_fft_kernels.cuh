@@ -309,9 +309,9 @@ __device__ __forceinline__ void decode_row(const uint4 *__restrict__ row, const 
 // ------------------------------------------------------------------------------------------
 // kernels
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ int64_t lambda_row_of(int64_t r, int64_t n_lambda, int64_t rows_per_lambda)
+__device__ __forceinline__ int64_t lambda_row_of(int64_t r, int64_t n_lambda, const FastDiv &rows_per_lambda)
 {
-    return n_lambda == 1 ? 0 : r / rows_per_lambda;
+    return n_lambda == 1 ? 0 : rows_per_lambda(r);
 }
 
 // Fills the warp's lambda cache with row `lr` of the table: the values themselves (RECIP ==

@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "../../include/kvq.h"
+#include "kvq_device.cuh"
 
 namespace kvq {
 
@@ -14,10 +15,13 @@ namespace kvq {
 // the block belong to one stream and go to rows base .. base + rps - 1 of it; `stride` = rows per stream of the cache.
 // The identity is {1, 1, 0}; kvq_append is {1, T_max, pos}.
 struct RowMap {
-    int64_t rps, stride, base;
+    FastDiv rps;
+    int64_t stride, base;
     __host__ __device__ __forceinline__ int64_t operator()(int64_t r) const
     {
-        return rps == 1 ? r * stride + base : (r / rps) * stride + base + (r % rps);
+        if (rps.d == 1) return r * stride + base;
+        const int64_t s = rps(r);
+        return s * stride + base + (r - s * rps.d);
     }
 };
 
@@ -30,7 +34,8 @@ struct FftParams {
     void *scales;          // [*, D/group] fp16 (encode: out, decode: in)
     void *out;             // decode: x^ [N, D] half precision
     int64_t N;
-    int64_t n_lambda, rows_per_lambda;
+    int64_t n_lambda;
+    FastDiv rows_per_lambda;
     int per_vector;        // one scale per vector (group = D) instead of one per 32 channels
     RowMap out_map;             // row of packed / scales (encode) or of out (decode) that row r goes to
     RowMap in_map;              // decode: row of packed / scales that row r comes from
@@ -55,7 +60,8 @@ cudaError_t build_encode_operands(int D, const float *e0, unsigned char *out);  
 // [base, base + rows) of each of S streams, `stride` cache rows apart, in packed, scales and out alike; the lambda row of
 // stream s is s / streams_per_lambda.  rows == 0: the flat layout, row r at row r.
 struct CacheView {
-    int64_t rows, stride, base, streams_per_lambda;
+    int64_t rows, stride, base;
+    FastDiv streams_per_lambda;
 };
 
 // Arguments of the tcgen05 DFT-as-GEMM decode kernel (kvq_umma_decode.cu).
@@ -77,7 +83,7 @@ struct GemmParams {
     }
     __host__ __device__ __forceinline__ int64_t lambda_index(int64_t seg) const
     {
-        return n_lambda == 1 ? 0 : view.rows ? seg / view.streams_per_lambda : seg;
+        return n_lambda == 1 ? 0 : view.rows ? view.streams_per_lambda(seg) : seg;
     }
 };
 

@@ -35,10 +35,11 @@ struct MatvecParams {
     void *out;             // decode: [*, D] half precision
     const float *table;    // encode: b0[n][c] (column c of the forward transform along a row); decode: e0[c][n]
     const float *table2;   // fused window flush: e0[c][n], for the way back
-    int64_t N, n_lambda, rows_per_lambda;
-    RowMap out_map, in_map;
+    int64_t N, n_lambda;
+    FastDiv rows_per_lambda;
+    RowMap map;            // where row r lives: encode of its output, decode of both sides (a cache view or the flat layout)
     int group, bits;
-    // Position on the device: when pos_dev is set, the base row of out_map is *pos_dev, read when the kernel runs, and must
+    // Position on the device: when pos_dev is set, the base row of map is *pos_dev, read when the kernel runs, and must
     // lie in [0, pos_limit]; otherwise the launch writes nothing and raises KVQ_DEV_POSITION in *status.
     const int64_t *pos_dev;
     int64_t pos_limit;
@@ -49,7 +50,7 @@ struct MatvecParams {
 // whole grid alike) when that position is outside the cache.
 __device__ __forceinline__ bool resolve_out_map(const MatvecParams &prm, RowMap &map)
 {
-    map = prm.out_map;
+    map = prm.map;
     if (prm.pos_dev) {
         const int64_t p = load_input(prm.pos_dev);
         if (p < 0 || p > prm.pos_limit) {
@@ -72,9 +73,9 @@ struct Geo {
     static constexpr int kSmemBytes = (kV * D + kWarps * kV * D) * (int)sizeof(float);
 };
 
-__device__ __forceinline__ int64_t lambda_row(int64_t r, int64_t n_lambda, int64_t rows_per_lambda)
+__device__ __forceinline__ int64_t lambda_row(int64_t r, int64_t n_lambda, const FastDiv &rows_per_lambda)
 {
-    return n_lambda == 1 ? 0 : r / rows_per_lambda;
+    return n_lambda == 1 ? 0 : rows_per_lambda(r);
 }
 
 // Rows k0 .. k0 + CH - 1 of this warp's slice of the table into registers (coalesced float4 per row).
@@ -322,7 +323,7 @@ __device__ __forceinline__ void dequantise_batch(const MatvecParams &prm, float 
         const int64_t r = v0 + v;
         float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (r < prm.N) {
-            const int64_t irow = prm.in_map(r);
+            const int64_t irow = prm.map(r);
             int q[4];
             if (prm.bits == 4) {
                 const uint32_t w = load_input(reinterpret_cast<const uint16_t *>(pk + irow * (D / 2) + 2 * i));
@@ -361,7 +362,7 @@ __device__ __forceinline__ void decode_batch(const MatvecParams &prm, float4 (&t
 
     const int64_t r = v0 + warp;
     if (r >= prm.N) return;
-    unsigned char *out = static_cast<unsigned char *>(prm.out) + prm.out_map(r) * (2 * D);
+    unsigned char *out = static_cast<unsigned char *>(prm.out) + prm.map(r) * (2 * D);
 #pragma unroll
     for (int p = 0; p < P; ++p) {
         const int i = lane + 32 * p;
@@ -558,7 +559,7 @@ __global__ void __launch_bounds__(kWarps * 32, D == 256 ? 1 : 2) kvq_decode_matv
     const float4 y = slice_matvec<D>(t, zs, red, warp, lane);
     const int64_t r = batch * kV + warp;
     if (r < prm.N && lane < S::Q)
-        *reinterpret_cast<uint2 *>(static_cast<unsigned char *>(prm.out) + prm.out_map(r) * (2 * D) + 2 * (slice * S::W + 4 * lane)) =
+        *reinterpret_cast<uint2 *>(static_cast<unsigned char *>(prm.out) + prm.map(r) * (2 * D) + 2 * (slice * S::W + 4 * lane)) =
             make_uint2(narrow2<BF16>(y.x, y.y), narrow2<BF16>(y.z, y.w));
 }
 
@@ -639,7 +640,7 @@ MatvecParams from_fft(const FftParams &f, const float *table, int group, int bit
     p.table = table;
     p.table2 = nullptr;
     p.N = f.N, p.n_lambda = f.n_lambda, p.rows_per_lambda = f.rows_per_lambda;
-    p.out_map = f.out_map, p.in_map = f.in_map;
+    p.map = f.out_map;
     p.group = group, p.bits = bits;
     p.pos_dev = nullptr, p.pos_limit = 0, p.status = f.status;
     return p;

@@ -92,7 +92,7 @@ struct UmmaAppendParams {
     unsigned char *packed; // [*, D bits / 8] bytes out
     uint16_t *scales;      // [*, D/32] (one scale per vector: [*, 1]) fp16 out
     uint32_t N;            // below 2^31
-    uint32_t rpl;          // rows per lambda row
+    FastDiv rpl;           // rows per lambda row
     int64_t n_lambda;
     RowMap out_map;        // output row of input row r
     float unlift;          // 1 / kOperandLift (as an immediate, or read from device memory: 5120 vectors at D = 128, calls one after another, 4.36 -> 4.41 us)
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float unlift = prm.unlift, Q = prm.bits == 4 ? 7.0f : 127.0f, inv_q = prm.bits == 4 ? 1.0f / 7.0f : 1.0f / 127.0f;
         // lambda of this thread's row and CTA's channels (the same for the whole warp where lambda rows are long: a broadcast out of L1)
         auto lambda_of = [&](uint32_t row) -> const float4 * {
-            const uint32_t at = prm.n_lambda > 1 ? (row < N ? row : N - 1u) / prm.rpl : 0u;
+            const uint32_t at = prm.n_lambda > 1 ? prm.rpl.small(row < N ? row : N - 1u) : 0u;
             return reinterpret_cast<const float4 *>(prm.lambda + (size_t)at * D + half * C::kCh);
         };
         const float4 *lam = lambda_of(first_row(0) + (uint32_t)r);
@@ -377,7 +377,7 @@ cudaError_t launch(int64_t N, const FftParams &f, cudaStream_t stream)
     prm.packed = static_cast<unsigned char *>(f.packed);
     prm.scales = static_cast<uint16_t *>(f.scales);
     prm.N = (uint32_t)N;
-    prm.rpl = (uint32_t)(f.rows_per_lambda < N ? f.rows_per_lambda : N);
+    prm.rpl = f.rows_per_lambda;
     prm.n_lambda = f.n_lambda;
     prm.out_map = f.out_map;
     prm.unlift = 1.0f / kOperandLift;
@@ -430,7 +430,7 @@ bool umma_append_pays(int D, bool bf16, bool per_vector, int64_t N, const FftPar
     }
     const int half_tiles = per_vector ? (D == 64 ? 3 : D == 128 ? 10 : 5) : D == 64 ? 5 : D == 96 ? 16 : D == 128 ? 20 : D == 160 ? 8 : 14;
     const int per_row = (D == 64 ? 2 : D == 96 ? 4 : D == 128 ? 5 : 8) / (per_vector ? 2 : 1);
-    const int64_t rows = f.n_lambda == 1 ? 1 : (N + f.rows_per_lambda - 1) / f.rows_per_lambda;
+    const int64_t rows = f.n_lambda == 1 ? 1 : (N + f.rows_per_lambda.d - 1) / f.rows_per_lambda.d;
     return 2 * ((N + kTile - 1) / kTile) <= (int64_t)half_tiles * slots.sms[dev] + 2 * (int64_t)per_row * (rows - 1);
 }
 

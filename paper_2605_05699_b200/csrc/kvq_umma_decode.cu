@@ -275,8 +275,7 @@ __device__ __forceinline__ void load_row_scales(const uint16_t *__restrict__ sp,
 struct UmmaDecodeParams {
     GemmParams g;
     int64_t rpl;        // rows per lambda segment (N when there is one lambda row)
-    int64_t n_seg;      // segments
-    int64_t segs;       // consecutive segments with one lambda row: 1, or what a cache view's streams share
+    TilePlan plan;      // the call's tiles, cut into shares
     int64_t n_full;     // segments of exactly rpl rows, covered by the main output maps; a shorter last one uses the tail maps
     int64_t phys_rows;  // rows of the packed / scales arrays (N, or the whole cache for a cache view)
     uint32_t flip2[40]; // radix-2 form: sign-bit masks of s_n s_{n + D/2} for the output pairs (n, n + 1), n = 0, 2, .. D/2 - 2
@@ -354,11 +353,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range of tiles
     // ---- per CTA, so that the B operand is rebuilt as rarely as possible
-    const int64_t N = prm.g.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x, kTile, prm.segs);
-    const int64_t tps = share.tps, tile_begin = share.begin;
+    const int64_t rpl = prm.rpl;
+    const TileShare share(prm.plan, blockIdx.x);
     const int n_my = share.n;
-    const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
+    const int64_t seg_first = share.seg;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * D; };
 
     // ---- B for the first tile's lambda row: the sixteen dequant and epilogue warps build it while the
@@ -375,7 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         rows.load(prm.g.b0, 0, warp - 2, lane);
         grid_wait();
         if (warp < 10 && ((warp - 2) >> 2) < n_my) {   // dequant group g's first tile is tile_begin + g
-            const TileCursor first(tile_begin + ((warp - 2) >> 2), tps);
+            const TileCursor first(share, (warp - 2) >> 2);
             const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
             const uint16_t *scales = static_cast<const uint16_t *>(prm.g.scales);
             if (row < prm.phys_rows) {
@@ -417,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             int issued = 0;
             bool ok = true;
-            TileCursor cur(tile_begin, tps);
+            TileCursor cur(share);
             for (int j = 0; j < n_my; ++j, cur.advance(1)) {
                 const int s = j % kInStages;
                 const uint32_t use = (uint32_t)(j / kInStages);
@@ -502,7 +500,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         int64_t cached_row = n_my > 0 ? prm.g.lambda_index(seg_first) : -1;   // the lambda row that B holds (built above)
         float rho = rho_first;
 
-        TileCursor cur(tile_begin + grp, tps), ahead(tile_begin + grp, tps);   // this tile; the tile whose scales are fetched
+        TileCursor cur(share, grp), ahead = cur;   // this tile; the tile whose scales are fetched
         uint32_t sc_next[(G + 1) / 2];
         auto fetch_scales = [&](int j) {
 #pragma unroll
@@ -656,7 +654,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3;
         unsigned char *stg = sOut + (warp - 10) * C::kOutWarpBytes;   // this warp's staging tile
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        TileCursor cur(tile_begin + grp, tps);
+        TileCursor cur(share, grp);
         for (int j = grp; j < n_my; j += 2, cur.advance(2)) {
             const int sc = j % kAccStages;
             if (!wait_or_abort(smem_u32(&ctrl->acc_full[j & 1]), (uint32_t)(j >> 1) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
@@ -770,7 +768,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // ---- tiles of a lambda row too wide for the fp16 B operand: decoded again in fp32, over what the pipeline stored
     if (ctrl->any_wide && !*abort_flag)
-        redo_tiles_fp32<D, BF16OUT, BITS, kTile>(prm.g, tile_begin, n_my, tps, rpl, reinterpret_cast<float *>(smem));
+        redo_tiles_fp32<D, BF16OUT, BITS, kTile>(prm.g, share.begin, n_my, share.tps, rpl, reinterpret_cast<float *>(smem));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -799,11 +797,11 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const ui
 
     UmmaDecodeParams prm;
     prm.g = g;
-    prm.rpl = g.view.rows ? g.view.rows : g.n_lambda == 1 ? N : g.rows_per_lambda;   // a cache view: one segment per stream
-    prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
-    prm.segs = g.n_lambda == 1 ? prm.n_seg : g.view.rows ? g.view.streams_per_lambda : 1;
+    prm.rpl = g.view.rows ? g.view.rows : g.n_lambda == 1 || g.rows_per_lambda > N ? N : g.rows_per_lambda;   // a cache view: one segment per stream
+    const int64_t n_seg = (N + prm.rpl - 1) / prm.rpl;
+    const int64_t segs = g.n_lambda == 1 ? n_seg : g.view.rows ? g.view.streams_per_lambda.d : 1;   // consecutive segments with one lambda row
     prm.n_full = N / prm.rpl;
-    prm.phys_rows = g.view.rows ? prm.n_seg * g.view.stride : N;
+    prm.phys_rows = g.view.rows ? n_seg * g.view.stride : N;
     if (prm.phys_rows >= (int64_t)1 << 31) return cudaErrorInvalidValue;
     const int64_t seg_stride = g.view.rows ? g.view.stride : prm.rpl;   // rows from one segment's first row to the next's
     unsigned char *out0 = static_cast<unsigned char *>(g.out) + (size_t)(g.view.rows ? g.view.base : 0) * (2 * D);
@@ -836,8 +834,9 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const ui
     if (tail_rows == 0) maps.wide_tail = maps.wide, maps.slim_tail = maps.slim;
     if (prm.n_full == 0) maps.wide = maps.wide_tail, maps.slim = maps.slim_tail;
 
-    const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
+    const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
+    prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid, kTile, segs);
     return launch_kernel(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 

@@ -152,8 +152,7 @@ __device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__r
 struct UmmaDecode256Params {
     GemmParams g;
     int64_t rpl;        // rows per lambda segment (N when there is one lambda row)
-    int64_t n_seg;      // segments
-    int64_t segs;       // consecutive segments with one lambda row: 1, or what a cache view's streams share
+    TilePlan plan;      // the call's tiles, cut into shares
     int64_t n_full;     // segments of exactly rpl rows, covered by the main output map; a shorter last one uses the tail map
     int64_t phys_rows;  // rows of the packed / scales arrays (N, or the whole cache for a cache view)
     uint32_t sign_xor[128];   // word m: bit 15 set if s_{2m} = -1, bit 31 set if s_{2m+1} = -1
@@ -204,11 +203,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range of tiles per CTA
-    const int64_t N = prm.g.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x, kTile, prm.segs);
-    const int64_t tps = share.tps, tile_begin = share.begin;
+    const int64_t rpl = prm.rpl;
+    const TileShare share(prm.plan, blockIdx.x);
     const int n_my = share.n;
-    const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
+    const int64_t seg_first = share.seg;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * kD; };
 
     FirstRows rows;
@@ -230,7 +228,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint4 sc_first = make_uint4(0u, 0u, 0u, 0u);
     if (builds_first) {
         if (warp < 10) {
-            const TileCursor first(tile_begin, tps);
+            const TileCursor first(share);
             const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
             if (row < prm.phys_rows) {
                 if (prm.g.per_vector) {
@@ -255,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             int issued = 0;
             bool ok = true;
-            TileCursor cur(tile_begin, tps);
+            TileCursor cur(share);
             for (int j = 0; j < n_my; ++j, cur.advance(1)) {
                 const int s = j % kInStages;
                 ok = wait_or_abort(smem_u32(&ctrl->in_empty[s]), ((uint32_t)(j / kInStages) & 1u) ^ 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT);
@@ -323,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         int64_t cached_row = n_my > 0 ? prm.g.lambda_index(seg_first) : -1;   // the lambda row that B holds (built above)
         float rho = rho_first;
 
-        TileCursor cur(tile_begin, tps), ahead(tile_begin, tps);
+        TileCursor cur(share), ahead(share);
         auto fetch_scales = [&](int j) -> uint4 {
             if (j >= n_my) return make_uint4(0u, 0u, 0u, 0u);
             const int64_t row = prm.g.phys_row(ahead.seg, ahead.row_in_segment(), rpl) + r;
@@ -449,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int ch = (warp - 10) >> 2;                            // this warp's half of the column pairs: n in [64 ch, 64 ch + 64)
         unsigned char *stg_base = sOut + (warp - 10) * kOutWarpBytes;   // per chunk: two [32 rows][64 B] boxes
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        TileCursor cur(tile_begin, tps);
+        TileCursor cur(share);
         for (int j = 0; j < n_my; ++j, cur.advance(1)) {
             if (!wait_or_abort(smem_u32(&ctrl->acc_full), (uint32_t)j & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
             tc_fence_after();
@@ -519,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // ---- tiles of a lambda row too wide for the fp16 B operand: decoded again in fp32, over what the pipeline stored
     if (ctrl->any_wide && !*abort_flag)
-        redo_tiles_fp32<kD, BF16OUT, BITS, kTile>(prm.g, tile_begin, n_my, tps, rpl, reinterpret_cast<float *>(smem));
+        redo_tiles_fp32<kD, BF16OUT, BITS, kTile>(prm.g, share.begin, n_my, share.tps, rpl, reinterpret_cast<float *>(smem));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -548,11 +546,11 @@ cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cud
 
     UmmaDecode256Params prm;
     prm.g = g;
-    prm.rpl = g.view.rows ? g.view.rows : g.n_lambda == 1 ? N : g.rows_per_lambda;   // a cache view: one segment per stream
-    prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
-    prm.segs = g.n_lambda == 1 ? prm.n_seg : g.view.rows ? g.view.streams_per_lambda : 1;
+    prm.rpl = g.view.rows ? g.view.rows : g.n_lambda == 1 || g.rows_per_lambda > N ? N : g.rows_per_lambda;   // a cache view: one segment per stream
+    const int64_t n_seg = (N + prm.rpl - 1) / prm.rpl;
+    const int64_t segs = g.n_lambda == 1 ? n_seg : g.view.rows ? g.view.streams_per_lambda.d : 1;   // consecutive segments with one lambda row
     prm.n_full = N / prm.rpl;
-    prm.phys_rows = g.view.rows ? prm.n_seg * g.view.stride : N;
+    prm.phys_rows = g.view.rows ? n_seg * g.view.stride : N;
     if (prm.phys_rows >= (int64_t)1 << 31) return cudaErrorInvalidValue;
     const int64_t seg_stride = g.view.rows ? g.view.stride : prm.rpl;   // rows from one segment's first row to the next's
     unsigned char *out0 = static_cast<unsigned char *>(g.out) + (size_t)(g.view.rows ? g.view.base : 0) * (2 * kD);
@@ -580,8 +578,9 @@ cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cud
     if (tail_rows == 0) maps.tail = maps.out;
     if (prm.n_full == 0) maps.out = maps.tail;
 
-    const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
+    const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
+    prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid, kTile, segs);
     return launch_kernel(kvq_decode_umma_d256_kernel<BF16OUT, BITS>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 

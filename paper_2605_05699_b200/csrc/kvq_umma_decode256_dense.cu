@@ -103,7 +103,7 @@ __device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__r
 struct UmmaDecode256DenseParams {
     GemmParams g;
     int64_t rpl;        // rows per lambda segment (N when there is one lambda row)
-    int64_t n_seg;      // segments
+    TilePlan plan;      // the call's tiles, cut into shares of the pairs
     int64_t n_full;     // segments of exactly rpl rows, covered by the main output map; a shorter last one uses the tail map
 };
 
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int half = blockIdx.x & 1;            // which 128 output columns this CTA computes
-    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    const int pair = blockIdx.x >> 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kInStages; ++s) {
@@ -152,11 +152,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range of tiles per CTA pair
-    const int64_t N = prm.g.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, (unsigned)pair, (unsigned)n_pairs);
-    const int64_t tps = share.tps, tile_begin = share.begin;
+    const int64_t rpl = prm.rpl;
+    const TileShare share(prm.plan, (uint32_t)pair);
     const int n_my = share.n;
-    const int64_t seg_first = n_my > 0 ? tile_begin / tps : 0;
+    const int64_t seg_first = share.seg;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * kD; };
 
     fence_proxy_async();
@@ -183,7 +182,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             int issued = 0;
             bool ok = true;
-            TileCursor cur(tile_begin, tps);
+            TileCursor cur(share);
             for (int j = 0; j < n_my; ++j, cur.advance(1)) {
                 const int s = j % kInStages;
                 ok = wait_or_abort(smem_u32(&ctrl->in_empty[s]), ((uint32_t)(j / kInStages) & 1u) ^ 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT);
@@ -210,7 +209,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             int n_mma = n_my;
             if (n_my > 0 && !wait_or_abort(smem_u32(&ctrl->b_first), 0u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) n_mma = 0;
             bool ok = true;
-            TileCursor cur(tile_begin, tps);
+            TileCursor cur(share);
             for (int j = 0; j < n_mma && ok; ++j, cur.advance(1)) {
                 const int sc = j % kAccStages;
                 // A new lambda row: a dequant group will overwrite B once every MMA issued so far has read the old one.  This
@@ -265,11 +264,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         int64_t cached_seg = n_my > 0 ? seg_first : -1;   // B holds this row's table (built above)
         float rho = RecipLambda<kD>(lambda_row(seg_first), lane).rho;
 
-        TileCursor cur(tile_begin + grp, tps), ahead(tile_begin + grp, tps);
+        TileCursor cur(share, grp), ahead = cur;
         auto fetch_scales = [&](int j) -> uint4 {
             if (j >= n_my) return make_uint4(0u, 0u, 0u, 0u);
             const int64_t row = ahead.seg * rpl + ahead.row_in_segment() + r;
-            if (row >= N) return make_uint4(0u, 0u, 0u, 0u);
+            if (row >= prm.g.N) return make_uint4(0u, 0u, 0u, 0u);
             if (prm.g.per_vector) {   // one scale per vector: the same value in every group's slot
                 const uint32_t s1 = (uint32_t)load_input(reinterpret_cast<const uint16_t *>(prm.g.scales) + row);
                 const uint32_t s2 = s1 | (s1 << 16);
@@ -384,7 +383,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3;
         unsigned char *stg = sOut + (warp - 10) * kOutWarpBytes;   // one [32 rows][128 B] box
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        TileCursor cur(tile_begin + grp, tps);
+        TileCursor cur(share, grp);
         for (int j = grp; j < n_my; j += 2, cur.advance(2)) {
             const int sc = j % kAccStages;
             if (!wait_or_abort(smem_u32(&ctrl->acc_full[sc]), (uint32_t)(j / kAccStages) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
@@ -436,7 +435,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ---- tiles of a lambda row too wide for the fp16 B operand, or with a scale outside the A operand's range: this CTA's
     // ---- output columns decoded again in fp32
     if (ctrl->any_wide && !*abort_flag)
-        redo_tiles_fp32<kD, BF16OUT, 4, kTile, kHalfN, true>(prm.g, tile_begin, n_my, tps, rpl, reinterpret_cast<float *>(smem), half * kHalfN);
+        redo_tiles_fp32<kD, BF16OUT, 4, kTile, kHalfN, true>(prm.g, share.begin, n_my, share.tps, rpl, reinterpret_cast<float *>(smem), half * kHalfN);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -465,8 +464,8 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream)
 
     UmmaDecode256DenseParams prm;
     prm.g = g;
-    prm.rpl = g.n_lambda == 1 ? N : g.rows_per_lambda;
-    prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
+    prm.rpl = g.n_lambda == 1 || g.rows_per_lambda > N ? N : g.rows_per_lambda;
+    const int64_t n_seg = (N + prm.rpl - 1) / prm.rpl;
     prm.n_full = N / prm.rpl;
 
     UmmaDecode256DenseMaps maps;
@@ -491,8 +490,9 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream)
     if (tail_rows == 0) maps.tail = maps.out;
     if (prm.n_full == 0) maps.out = maps.tail;
 
-    const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
+    const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int64_t pairs = tiles < sms / 2 ? tiles : sms / 2;
+    prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)pairs);
     return launch_kernel(kvq_decode_umma_d256_dense_kernel<BF16OUT>, (unsigned)(2 * pairs), kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 

@@ -235,7 +235,7 @@ struct UmmaEncodeParams {
     int64_t N;
     int64_t n_lambda;
     int64_t rpl;           // rows per lambda segment (N when there is one lambda row)
-    int64_t n_seg;
+    TilePlan plan;         // the call's tiles, cut into shares
     RowMap out_map;        // output row of input row r
     int bits;              // 4: nibble pairs; 8: one two's-complement byte per code, scale = absmax / 127
     uint32_t *status;
@@ -272,8 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range per CTA
     const int64_t N = prm.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, blockIdx.x, gridDim.x);
-    const int64_t tps = share.tps, tile_begin = share.begin;
+    const TileShare share(prm.plan, blockIdx.x);
     const int n_my = share.n;
     // One tile: both sets of epilogue warps share it, four threads to a row.  Back to back, 8000 vectors: D = 96 5.0 -> 4.4 us, 128 5.9 -> 5.3,
     // 160 7.1 -> 6.6 (one scale per vector 7.2 -> 6.8); 18,944: 6.2 -> 5.7, 7.1 -> 6.7, 8.7 -> 8.1.  Not at D = 64, which has two groups, one for
@@ -300,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     grid_wait();
     if (builds_first) {
-        first_seg = tile_begin / tps;
+        first_seg = share.seg;
         const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : first_seg) * D;
         rows.load_lambda(lam, 0, warp - 2, lane);
         first_lift = lift_of<D>(lam, prm.e0, lane);
@@ -319,7 +318,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // =========================== producer ===========================
         if (lane == 0) {
             bool ok = true;
-            TileCursor cur(tile_begin, tps);
+            TileCursor cur(share);
             for (int j = 0; j < n_my; ++j, cur.advance(1)) {
                 const int s = j % kInStages;
                 // The x stage is free once the MMAs of the tile that used it last are complete: that tile's accumulator
@@ -362,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
             const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32);
             uint32_t builds = 0;
-            TileCursor cur(tile_begin, tps);
+            TileCursor cur(share);
             for (int j = 0; j < n_my && first_ok; ++j, cur.advance(1)) {
                 const int s = j % kInStages, sc = j % kAccStages;
                 if (j == 0) {   // all epilogue warps build the first B while the first x tiles are in flight
@@ -422,7 +421,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         };
         float colmax[C::kGroupsPerPart] = {};   // calibration: lane i keeps the running maximum of column i of each of this thread's groups
-        TileCursor cur(tile_begin + set, tps);
+        TileCursor cur(share, set);
         for (int j = set; j < n_my; j += 2, cur.advance(2)) {
             __syncwarp();
             const int64_t seg = cur.seg;
@@ -578,8 +577,8 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     prm.scales = static_cast<uint16_t *>(f.scales);
     prm.N = N;
     prm.n_lambda = f.n_lambda;
-    prm.rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
-    prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
+    prm.rpl = f.n_lambda == 1 || f.rows_per_lambda.d > N ? N : f.rows_per_lambda.d;
+    const int64_t n_seg = (N + prm.rpl - 1) / prm.rpl;
     prm.out_map = f.out_map;
     prm.bits = f.bits;
     prm.status = f.status;
@@ -594,8 +593,9 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
                          CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
 
-    const int64_t tiles = prm.n_seg * ((prm.rpl + kTile - 1) / kTile);
+    const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
+    prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid);
     return launch_kernel(kvq_encode_umma_kernel<D, BF16, CALIB, PERVEC, WIDE>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, tm_x);
 }
 

@@ -167,7 +167,7 @@ struct UmmaEncode256Params {
     int64_t N;
     int64_t n_lambda;
     int64_t rpl;           // rows per lambda segment (N when there is one lambda row)
-    int64_t n_seg;
+    TilePlan plan;         // the call's tiles, cut into shares of the pairs
     RowMap out_map;        // output row of input row r
     uint32_t *status;
     uint32_t *amax_bits;        // calibration only: [D] running column maxima as fp32 bit patterns (start at zero)
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)cluster_rank();       // which ROWS vectors of a tile, and which 128 rows of B, this CTA holds
-    const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+    const int pair = blockIdx.x >> 1;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kRing; ++s) {
@@ -212,14 +212,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 2 ROWS rows; a contiguous range per CTA pair
     const int64_t N = prm.N, rpl = prm.rpl;
-    const TileShare share(prm.n_seg, rpl, (unsigned)pair, (unsigned)n_pairs, 2 * ROWS);
-    const int64_t tps = share.tps, tile_begin = share.begin;
+    const TileShare share(prm.plan, (uint32_t)pair);
+    const int tps = (int)share.tps;
     const int n_my = share.n;
 
     // ---- B for the pair's first lambda row: eight rows per epilogue warp, requested before the set-up barrier
     float first_lift = 1.0f;
     if (n_my > 0 && warp >= 2) {
-        const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : tile_begin / tps) * kD;
+        const float *lam = CALIB ? nullptr : prm.lambda + (prm.n_lambda == 1 ? 0 : (int64_t)share.seg) * kD;
         BuildRows<BF16, CALIB> rows;
         rows.load(prm.e0, rank, (warp - 2) * 8, lane);
         grid_wait();
@@ -247,14 +247,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             bool ok = true;
             int issued = 0;
-            TileCursor cur(tile_begin, tps), ahead(tile_begin, tps);
-            ahead.advance(1);
+            TileCursor cur(share), ahead(share, 1);
             for (int j = 0; j < n_my && ok; ++j, cur.advance(1), ahead.advance(1)) {
-                const int64_t row0 = cur.seg * rpl + cur.tin * (2 * ROWS) + rank * ROWS;   // may lie past the end: zeros
+                const int64_t row0 = cur.seg * rpl + (int64_t)cur.tin * (2 * ROWS) + rank * ROWS;   // may lie past the end: zeros
                 // The next tile's rows are one contiguous run: asked for as such, they come out of DRAM page by page, and the K block
                 // loads, 128 bytes of each row at a time, find them in L2 (1,064,960 bf16 vectors: 278 -> 269 us; two tiles ahead: 273).
                 if (j + 1 < n_my) {
-                    const int64_t next = ahead.seg * rpl + ahead.tin * (2 * ROWS) + rank * ROWS;
+                    const int64_t next = ahead.seg * rpl + (int64_t)ahead.tin * (2 * ROWS) + rank * ROWS;
                     const int64_t n = N - next < ROWS ? N - next : ROWS;
                     if (n > 0) prefetch_l2(prm.x + next * (2 * kD), (uint32_t)n * (2 * kD));
                 }
@@ -282,7 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32);
             uint32_t builds = 0;
             bool ok = true;
-            TileCursor cur(tile_begin, tps);
+            TileCursor cur(share);
             for (int j = 0; j < n_my && ok; ++j, cur.advance(1)) {
                 const int sc = j % kAccStages;
                 if (j == 0) {   // the epilogue warps build the first B while the first x blocks are in flight
@@ -348,11 +347,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         };
         float lift_next = first_lift;
         float colmax[kTG] = {};   // calibration: lane i keeps the running maximum of column i of each of this thread's groups
-        TileCursor cur(tile_begin, tps);
+        TileCursor cur(share);
         for (int j = 0; j < n_my; ++j, cur.advance(1)) {
             __syncwarp();
             const int64_t seg = cur.seg;
-            const int64_t off = cur.tin * (2 * ROWS) + rank * ROWS;
+            const int64_t off = (int64_t)cur.tin * (2 * ROWS) + rank * ROWS;
             const float unlift = 1.0f / lift_next;
 
             // ---- this tile's accumulator.  Where the next tile begins a new lambda row, every MMA that read the old B is complete
@@ -551,8 +550,8 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     prm.scales = static_cast<uint16_t *>(f.scales);
     prm.N = N;
     prm.n_lambda = f.n_lambda;
-    prm.rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
-    prm.n_seg = (N + prm.rpl - 1) / prm.rpl;
+    prm.rpl = f.n_lambda == 1 || f.rows_per_lambda.d > N ? N : f.rows_per_lambda.d;
+    const int64_t n_seg = (N + prm.rpl - 1) / prm.rpl;
     prm.out_map = f.out_map;
     prm.status = f.status;
     prm.amax_bits = amax_bits;
@@ -566,8 +565,9 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
                          CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
 
-    const int64_t tiles = tiles_of(prm.n_seg, prm.rpl, 2 * ROWS);
+    const int64_t tiles = tiles_of(n_seg, prm.rpl, 2 * ROWS);
     const unsigned pairs = (unsigned)(tiles < fit ? tiles : fit);
+    prm.plan = TilePlan(n_seg, prm.rpl, pairs, 2 * ROWS);
     return launch_kernel(kvq_encode_umma_d256_kernel<BF16, CALIB, PERVEC, ROWS>, 2 * pairs, kThreads, C::kSmemBytes, stream, 2, prm, tm_x);
 }
 
@@ -581,7 +581,7 @@ cudaError_t launch_any(int64_t N, const FftParams &f, const float *e0, cudaStrea
             const cudaError_t e = launch<BF16, CALIB, PERVEC, 64>(N, f, e0, stream, amax_bits);
             return e != cudaSuccess ? e : launch<BF16, CALIB, PERVEC, 128>(N, f, e0, stream, amax_bits);
         }
-        const int64_t rpl = f.n_lambda == 1 ? N : f.rows_per_lambda;
+        const int64_t rpl = f.n_lambda == 1 || f.rows_per_lambda.d > N ? N : f.rows_per_lambda.d;
         int fit = 0;
         const cudaError_t e = resident_pairs<BF16, CALIB, PERVEC, 128>(&fit);
         if (e != cudaSuccess) return e;
