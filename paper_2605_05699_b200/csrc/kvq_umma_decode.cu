@@ -47,6 +47,7 @@ namespace {
 
 constexpr int kTile = 128;       // vectors per tile = MMA M
 constexpr int kThreads = 576;    // producer, mma, 2 x 4 dequant, 2 x 4 epilogue warps
+constexpr int kBuilders = 12;    // warps that build the first B: the second dequant group and the epilogue
 constexpr int kMaxInStages = 6;  // packed tiles in flight, at most
 constexpr int kCtrlBytes = 5888;   // barriers and flags, eight tiles' worth of per-row output scales, two rows of reciprocals
 constexpr int kRowScaleSlots = 8;  // a dequant group is never more than seven tiles ahead of the epilogue that reads its slot
@@ -308,12 +309,61 @@ __device__ __noinline__ bool rebuild_b(unsigned char *sB, Ctrl *ctrl, const floa
         return false;
     // The reciprocals go to shared memory only now that nobody reads the ones before them: the MMAs of tile j - 2 were issued after
     // all four warps of this group had arrived for it, done with what they built there, and those of any tile after the first
-    // build, by all sixteen warps, out of recip[0].
+    // build, by its builders, out of recip[0].
     post_reciprocals<D>(ctrl->recip[grp], rl, lane);
     rows.store(sB, ctrl->recip[grp], 0, q, lane);
     rows.rest(sB, b0, ctrl->recip[grp], q, lane);
     fence_proxy_async();   // B is read by the tensor core through the async proxy
     return true;
+}
+
+// What the dequant warps take from the start: rho of the first lambda row and the scales of their first tile's row.
+template <int G>
+struct FirstOperand {
+    float rho = 1.0f;
+    uint32_t sc[(G + 1) / 2] = {};
+};
+
+// The way from the kernel's entry through the set-up barrier for warps 2 to 17, and B for the first tile's lambda row by the last kBuilders of them
+// (w counts from the first builder on): table rows are requested in front of the grid wait, lambda and scales behind it and in front of the
+// barrier.  The group that has the first tile does not build: it dequantises meanwhile, so that the first MMA waits for the longer of the two and not for their sum.
+// Out of line: its registers are then no part of the role loops' allocation.
+// One tile per CTA, back to back, before (all sixteen warps build, then one group dequantises, in line) and now: D = 160 bf16 9.1 -> 8.2 us, fp16 9.1 -> 8.1, D = 96 fp16 5.7 -> 5.4,
+// D = 128 bf16 7.4 -> 7.2; and for the registers 2072 tiles at D = 160 bf16 34.5 -> 32.8, D = 128 bf16 19.4 -> 19.0, fp16 17.3 -> 16.8.  (Without the call the same split
+// made 2072 tiles at D = 128 bf16 20.5.)
+template <int D, bool BF16OUT, int BITS, bool R2>
+__device__ __noinline__ FirstOperand<D / 32> first_operand(unsigned char *sB, Ctrl *ctrl, const float *__restrict__ b0, const float *lam,
+                                                           const uint16_t *row_scales, int per_vector, int w, int lane)
+{
+    constexpr int G = D / 32;
+    FirstOperand<G> r;
+    BuildB<D, BF16OUT, BITS, R2, kBuilders> rows;
+    if (w >= 0) rows.load(b0, 0, w, lane);
+    grid_wait();
+    if (row_scales) {
+        if (per_vector) {
+            const uint32_t s1 = (uint32_t)load_input(row_scales);
+#pragma unroll
+            for (int i = 0; i < (G + 1) / 2; ++i) r.sc[i] = s1 | (s1 << 16);
+        } else {
+            load_row_scales<G>(row_scales, r.sc);
+        }
+    }
+    const RecipLambda<D> rl(lam, lane);
+    r.rho = rl.rho;
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (rl.wide) ctrl->any_wide = 1u;
+    if (w >= 0) {
+        post_reciprocals<D>(ctrl->recip[0], rl, lane);
+        rows.store(sB, ctrl->recip[0], 0, w, lane);
+        rows.rest(sB, b0, ctrl->recip[0], w, lane);
+        fence_proxy_async();   // B is read by the tensor core through the async proxy
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
+    }
+    return r;
 }
 
 template <int D, bool BF16OUT, int BITS, bool R2>
@@ -344,12 +394,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(smem_u32(&ctrl->acc_full[s]), 1);
             mbar_init(smem_u32(&ctrl->acc_empty[s]), 4);
         }
-        mbar_init(smem_u32(&ctrl->b_first), 16);   // first B: the sixteen dequant and epilogue warps build it
+        mbar_init(smem_u32(&ctrl->b_first), kBuilders);
         ctrl->abort = 0u;
         ctrl->any_wide = 0u;
         mbar_init_fence();
+        fence_proxy_async();
     }
-    if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
+    if (warp == 1) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range of tiles
     // ---- per CTA, so that the B operand is rebuilt as rarely as possible
@@ -359,49 +410,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t seg_first = share.seg;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * D; };
 
-    // ---- B for the first tile's lambda row: the sixteen dequant and epilogue warps build it while the
-    // ---- producer's first loads are in flight; the mma warp waits for all of them.  Table rows and lambda are
-    // ---- requested before the set-up barrier, so that their latency runs under it.
-    // ---- The dequant warps also request the scales of their first tile here and keep rho, so that neither costs a round
-    // ---- trip to L2 after the build.
-    float rho_first = 1.0f;
-    uint32_t sc_first[(G + 1) / 2];
-#pragma unroll
-    for (int i = 0; i < (G + 1) / 2; ++i) sc_first[i] = 0u;
+    // ---- B for the first tile's lambda row (first_operand).  The dequant warps also request the scales of their first tile there and
+    // ---- keep rho, so that neither costs a round trip to L2 afterwards.
+    FirstOperand<G> first;
     if (n_my > 0 && warp >= 2) {
-        BuildB<D, BF16OUT, BITS, R2, 16> rows;
-        rows.load(prm.g.b0, 0, warp - 2, lane);
-        grid_wait();
-        if (warp < 10 && ((warp - 2) >> 2) < n_my) {   // dequant group g's first tile is tile_begin + g
-            const TileCursor first(share, (warp - 2) >> 2);
-            const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
-            const uint16_t *scales = static_cast<const uint16_t *>(prm.g.scales);
-            if (row < prm.phys_rows) {
-                if (prm.g.per_vector) {
-                    const uint32_t s1 = (uint32_t)load_input(scales + row);
-#pragma unroll
-                    for (int i = 0; i < (G + 1) / 2; ++i) sc_first[i] = s1 | (s1 << 16);
-                } else {
-                    load_row_scales<G>(scales + row * G, sc_first);
-                }
-            }
+        const uint16_t *row_scales = nullptr;
+        if (warp < 10 && ((warp - 2) >> 2) < n_my) {   // dequant group g's first tile is the share's tile g
+            const TileCursor at(share, (warp - 2) >> 2);
+            const int64_t row = prm.g.phys_row(at.seg, at.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
+            if (row < prm.phys_rows) row_scales = static_cast<const uint16_t *>(prm.g.scales) + row * (prm.g.per_vector ? 1 : G);
         }
-        const RecipLambda<D> rl(lambda_row(seg_first), lane);
-        rho_first = rl.rho;
-        fence_proxy_async();
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (rl.wide) ctrl->any_wide = 1u;
-        post_reciprocals<D>(ctrl->recip[0], rl, lane);
-        rows.store(sB, ctrl->recip[0], 0, warp - 2, lane);
-        rows.rest(sB, prm.g.b0, ctrl->recip[0], warp - 2, lane);
-        fence_proxy_async();   // B is read by the tensor core through the async proxy
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
+        first = first_operand<D, BF16OUT, BITS, R2>(sB, ctrl, prm.g.b0, lambda_row(seg_first), row_scales, prm.g.per_vector, warp - (18 - kBuilders), lane);
     } else {
         grid_wait();
-        fence_proxy_async();
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
@@ -498,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                              : C::kInSwizzleBits == 1 ? (uint32_t)((r >> 2) & 1)
                                                       : 0u;
         int64_t cached_row = n_my > 0 ? prm.g.lambda_index(seg_first) : -1;   // the lambda row that B holds (built above)
-        float rho = rho_first;
+        float rho = first.rho;
 
         TileCursor cur(share, grp), ahead = cur;   // this tile; the tile whose scales are fetched
         uint32_t sc_next[(G + 1) / 2];
@@ -520,7 +541,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         };
 
 #pragma unroll
-        for (int i = 0; i < (G + 1) / 2; ++i) sc_next[i] = sc_first[i];   // requested before the first B build
+        for (int i = 0; i < (G + 1) / 2; ++i) sc_next[i] = first.sc[i];   // requested before the first B build
         for (int j = grp; j < n_my; j += 2, cur.advance(2)) {
             uint32_t sc[(G + 1) / 2];
 #pragma unroll
