@@ -443,6 +443,13 @@ __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b)
     return d;
 }
 
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 __device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b)
 {
     uint64_t d;

@@ -69,12 +69,19 @@ constexpr uint32_t kTmemCols = 512;
 // 134 us (bf16 output: 215 -> 192).  At the other head dimensions, with the
 // quads of the table dealt out evenly and elect.sync, dense form -> this: D = 160 bf16 500,000 vectors 87.9 -> 65.0, 99,993 under three
 // lambda rows 37.9 -> 19.8; fp16 53.9 -> 45.9; D = 96 bf16 41.0 -> 34.9; D = 64 fp16 1M 42.7 -> 39.2; D = 128 bytes, bf16, 303,067: 36.2 -> 29.6.
-template <int D, bool BF16OUT, int BITS = 4, bool R2 = false>
+// PV: one scale per vector (Sec. 3.2 step 3, Sec. 4.1), in the radix-2 form.  sigma rho is the same for all of a row, so it stands behind the
+// contraction: the A operand is the code, exact in one fp16 term, the epilogue multiplies in fp32 (one product and two multiply-adds where it
+// had a sum and a difference), and no row needs operand_rescue.  bf16 output then takes two operand sets instead of three and half the
+// tensor-memory stores; fp16 output loses the rounding of q sigma rho to 11 bits.
+// Against the scaled operand, back to back, 592 and 2072 tiles: byte codes at D = 128 bf16 10.5 -> 8.5 us and 24.2 -> 20.4 (37 x 8191 vectors among others 30.6 -> 25.8), 4-bit codes at D = 160 bf16
+// 14.4 -> 10.6 and 34.4 -> 23.5 (two accumulators where two terms leave room for one), at D = 128 fp16 9.2 -> 8.3 and 19.4 -> 17.6.
+template <int D, bool BF16OUT, int BITS = 4, bool R2 = false, bool PV = false>
 struct Cfg {
     static_assert(D % 32 == 0 && D >= 64 && D <= 160, "head dim not built");
     static_assert(!BF16OUT || BITS == 4 || D <= 128, "two-term operands with byte codes: shared memory holds them for D <= 128 only");
     static_assert(BITS == 4 || BITS == 8, "code width not built");
-    static constexpr int kTerms = BF16OUT ? 2 : 1;         // W_hi (, W_lo); a_hi (, a_lo)
+    static constexpr int kTerms = BF16OUT ? 2 : 1;         // W_hi (, W_lo)
+    static constexpr int kATerms = BF16OUT && !PV ? 2 : 1; // a_hi (, a_lo)
     static constexpr int G = D / 32;                       // groups = 16-byte chunks of a packed row = 32-column accumulator chunks
     static constexpr int kKSteps = D / 16;
     static constexpr int kKBlocks = (D + 63) / 64;         // K blocks of 64 elements (the last one may be half used)
@@ -100,11 +107,11 @@ struct Cfg {
     // behind a_hi).  D = 160: an accumulator and an A term of 80 columns in each half of the 512 columns.  With two-term operands
     // the dense form has a_hi and a_lo of ONE stage there; the radix-2 form, whose MMAs take a third of the time, has two A stages
     // and one accumulator, which the epilogue hands back as soon as it is in registers.
-    static constexpr bool kOneAcc = R2 && D == 160 && BF16OUT;
+    static constexpr bool kOneAcc = R2 && D == 160 && kATerms == 2;
     static constexpr int kAccStages = kOneAcc ? 1 : 2;
     static constexpr uint32_t kAccStride = D <= 128 ? 128 : 256;
     static constexpr uint32_t kOCol = D == 96 ? 64 : D == 160 ? 96 : D / 2;   // R2: the O columns of an accumulator (E at 0)
-    static constexpr int kAStages = kOneAcc ? 2 : BF16OUT ? (D <= 128 ? 2 : 1) : D <= 128 ? 4 : 2;
+    static constexpr int kAStages = kOneAcc ? 2 : kATerms == 2 ? (D <= 128 ? 2 : 1) : D <= 128 ? 4 : 2;
     // The "A full" / "A free" barriers form a ring of at least two, indexed by tile: the two dequant groups take alternate
     // tiles, and a parity wait only tells a phase from its neighbours, so a barrier must not be shared by both groups.
     // Tile j writes A stage j % kAStages once the MMAs of tile j - kAStages have completed (barrier (j - kAStages) % kABars).
@@ -114,7 +121,7 @@ struct Cfg {
     __host__ __device__ static constexpr uint32_t acc_col(int s) { return (uint32_t)s * kAccStride; }
     __host__ __device__ static constexpr uint32_t a_col(int s)
     {
-        return D <= 128 ? 256u + 64u * (uint32_t)kTerms * (uint32_t)s : kOneAcc ? 176u + 160u * (uint32_t)s : (R2 ? 176u : 160u) + 256u * (uint32_t)s;
+        return D <= 128 ? 256u + 64u * (uint32_t)kATerms * (uint32_t)s : kOneAcc ? 176u + 160u * (uint32_t)s : (R2 ? 176u : 160u) + 256u * (uint32_t)s;
     }
     static constexpr int kQuads = D / 4;                   // float4 per table row
     static constexpr uint32_t kIdesc = umma_idesc_m128(R2 ? D / 2 : D, false);
@@ -127,7 +134,7 @@ struct Cfg {
     // caches hold beside the other roles' (a warp waits for an instruction 1.2 to 1.4 times per issue).  D = 160, bf16, 18,944 vectors
     // 10.9 -> 10.1 us, 300,000: 40.6 -> 39.4, 1,000,000: 117 -> 108; encode + decode of 99,993 under three lambda rows 38.0 -> 35.7.
     // (60,000 and 128,000 in a row of decodes alone: the same within 1 %.)  The other forms' loops are short enough: rolled they are 2 to 5 % slower.
-    static constexpr bool kRolled = R2 && BF16OUT && D == 160;
+    static constexpr bool kRolled = R2 && kATerms == 2 && D == 160;
 };
 
 struct Ctrl {
@@ -289,11 +296,11 @@ struct UmmaDecodeMaps {
 };
 
 // The group that meets a lambda row's first tile rebuilds B.  Kept out of line: rare, and the loop around it stays small.
-template <int D, bool BF16OUT, int BITS, bool R2>
+template <int D, bool BF16OUT, int BITS, bool R2, bool PV>
 __device__ __noinline__ bool rebuild_b(unsigned char *sB, Ctrl *ctrl, const float *__restrict__ b0, const RecipLambda<D> &rl, int grp, int q, int lane,
                                        int j, uint32_t *status)
 {
-    using C = Cfg<D, BF16OUT, BITS, R2>;
+    using C = Cfg<D, BF16OUT, BITS, R2, PV>;
     BuildB<D, BF16OUT, BITS, R2, 4> rows;
     rows.load(b0, 0, q, lane);
     // Every MMA issued so far has read B: the commit of the previous tile (the other group's) covers them
@@ -366,11 +373,11 @@ __device__ __noinline__ FirstOperand<D / 32> first_operand(unsigned char *sB, Ct
     return r;
 }
 
-template <int D, bool BF16OUT, int BITS, bool R2>
+template <int D, bool BF16OUT, int BITS, bool R2, bool PV>
 __global__ void __launch_bounds__(kThreads, 1)
     kvq_decode_umma_kernel(const __grid_constant__ UmmaDecodeParams prm, const __grid_constant__ UmmaDecodeMaps maps)
 {
-    using C = Cfg<D, BF16OUT, BITS, R2>;
+    using C = Cfg<D, BF16OUT, BITS, R2, PV>;
     constexpr int G = C::G, kInStages = C::kInStages, kAccStages = C::kAccStages;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -412,15 +419,16 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     // ---- B for the first tile's lambda row (first_operand).  The dequant warps also request the scales of their first tile there and
     // ---- keep rho, so that neither costs a round trip to L2 afterwards.
+    const bool per_vector = PV || (!R2 && prm.g.per_vector);
     FirstOperand<G> first;
     if (n_my > 0 && warp >= 2) {
         const uint16_t *row_scales = nullptr;
         if (warp < 10 && ((warp - 2) >> 2) < n_my) {   // dequant group g's first tile is the share's tile g
             const TileCursor at(share, (warp - 2) >> 2);
             const int64_t row = prm.g.phys_row(at.seg, at.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
-            if (row < prm.phys_rows) row_scales = static_cast<const uint16_t *>(prm.g.scales) + row * (prm.g.per_vector ? 1 : G);
+            if (row < prm.phys_rows) row_scales = static_cast<const uint16_t *>(prm.g.scales) + row * (per_vector ? 1 : G);
         }
-        first = first_operand<D, BF16OUT, BITS, R2>(sB, ctrl, prm.g.b0, lambda_row(seg_first), row_scales, prm.g.per_vector, warp - (18 - kBuilders), lane);
+        first = first_operand<D, BF16OUT, BITS, R2>(sB, ctrl, prm.g.b0, lambda_row(seg_first), row_scales, per_vector, warp - (18 - kBuilders), lane);
     } else {
         grid_wait();
         tc_fence_before();
@@ -478,13 +486,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                     for (int p = 0; p < 2; ++p) {
 #pragma unroll
-                        for (int set = 0; set < (BF16OUT ? 3 : 1); ++set) {   // bf16 output: a_hi W_hi + a_lo W_hi + a_hi W_lo
+                        for (int set = 0; set < C::kATerms + C::kTerms - 1; ++set) {   // bf16 output: a_hi W_hi + a_lo W_hi + a_hi W_lo, or a W_hi + a W_lo
 #pragma unroll
                             for (int ks = 0; ks < D / 32; ++ks) {
-                                const uint32_t b_set = b_lo + (set == 2 ? (uint32_t)((2 * C::kBPart) >> 4) : 0u) + (uint32_t)p * (C::kBPart >> 4);
+                                const uint32_t b_set = b_lo + (set == C::kATerms ? (uint32_t)((2 * C::kBPart) >> 4) : 0u) + (uint32_t)p * (C::kBPart >> 4);
                                 const uint64_t bd = ((uint64_t)b_hi << 32) | (uint64_t)(b_set + (uint32_t)(ks >> 2) * (C::kBPartBlock >> 4) + (uint32_t)(ks & 3) * 2u);
                                 const uint32_t dp = d_tmem + (uint32_t)p * C::kOCol;
-                                const uint32_t ap = a_tmem + (set == 1 ? C::kALo : 0u) + (uint32_t)p * (D / 4) + (uint32_t)ks * 8u;
+                                const uint32_t ap = a_tmem + (C::kATerms == 2 && set == 1 ? C::kALo : 0u) + (uint32_t)p * (D / 4) + (uint32_t)ks * 8u;
                                 if (set > 0 || ks > 0) umma_f16_ts<true>(dp, ap, bd, C::kIdesc);
                                 else umma_f16_ts<false>(dp, ap, bd, C::kIdesc);
                             }
@@ -529,7 +537,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (j < n_my) {
                 const int64_t row = prm.g.phys_row(ahead.seg, ahead.row_in_segment(), rpl) + r;
                 if (row < prm.phys_rows) {
-                    if (prm.g.per_vector) {   // one scale per vector: the same value in every group's slot
+                    if (per_vector) {   // one scale per vector: the same value in every group's slot
                         const uint32_t s1 = (uint32_t)load_input(scales + row);
 #pragma unroll
                         for (int i = 0; i < (G + 1) / 2; ++i) sc_next[i] = s1 | (s1 << 16);
@@ -557,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 rho = rl.rho;
                 if (rl.wide) ctrl->any_wide = 1u;
                 if (cur.first_of_segment() && prm.g.lambda_index(seg - 1) != row_of_seg) {
-                    if (!rebuild_b<D, BF16OUT, BITS, R2>(sB, ctrl, prm.g.b0, rl, grp, q, lane, j, status)) break;
+                    if (!rebuild_b<D, BF16OUT, BITS, R2, PV>(sB, ctrl, prm.g.b0, rl, grp, q, lane, j, status)) break;
                 }
                 cached_row = row_of_seg;
             }
@@ -585,8 +593,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- the A operand q sigma rho is fp16.  A row whose scales would take it out of fp16's normal range (a very
             // ---- small or very large vector) is carried times a power of two instead, which the epilogue takes out again
             // ---- in fp32; every other row has the factor 1 and costs the epilogue nothing.
-            float inv;
-            const float pw = operand_rescue<G>(sc, rho, BITS == 4 ? 9000.0f : 500.0f, inv);   // 7 (127) times this stays inside fp16
+            // ---- One scale per vector (PV): the operand is the code itself, and the epilogue multiplies by sigma rho.
+            float inv, pw = 1.0f;
+            if constexpr (PV) inv = __half2float(__ushort_as_half((unsigned short)(sc[0] & 0xFFFFu))) * rho;
+            else pw = operand_rescue<G>(sc, rho, BITS == 4 ? 9000.0f : 500.0f, inv);   // 7 (127) times this stays inside fp16
             ctrl->row_scale[j & (kRowScaleSlots - 1)][r] = inv;
             // ---- nibbles -> fp16 codes -> times sigma * rho, two codes per instruction
             const uint32_t a_row = tmem_base + ((uint32_t)(q * 32) << 16) + C::a_col(sa);
@@ -602,11 +612,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 const float sig = __half2float(__ushort_as_half((unsigned short)(sc16 & 0xFFFFu)));
                 const __half2 s2 = __float2half2_rn(sig * rho * pw);
-                uint32_t a[16], al[BF16OUT ? 16 : 1];
+                uint32_t a[16], al[C::kATerms == 2 ? 16 : 1];
                 auto put = [&](int k, __half2 q2) {   // K-pair k of the group: one rounding, and what it left behind
-                    const __half2 h = __hmul2(q2, s2);
+                    const __half2 h = PV ? q2 : __hmul2(q2, s2);
                     a[k] = *reinterpret_cast<const uint32_t *>(&h);
-                    if constexpr (BF16OUT) {   // q s2 - h, exact in fp16
+                    if constexpr (C::kATerms == 2) {   // q s2 - h, exact in fp16
                         const __half2 l = __hfma2(q2, s2, __hneg2(h));
                         al[k] = *reinterpret_cast<const uint32_t *>(&l);
                     }
@@ -648,7 +658,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint32_t ao[8] = {a[8], a[9], a[10], a[11], a[12], a[13], a[14], a[15]};
                     tmem_st8(a_row + 8u * (uint32_t)c, ae);
                     tmem_st8(a_row + (uint32_t)(D / 4) + 8u * (uint32_t)c, ao);
-                    if constexpr (BF16OUT) {
+                    if constexpr (C::kATerms == 2) {
                         const uint32_t le[8] = {al[0], al[1], al[2], al[3], al[4], al[5], al[6], al[7]};
                         const uint32_t lo[8] = {al[8], al[9], al[10], al[11], al[12], al[13], al[14], al[15]};
                         tmem_st8(a_row + C::kALo + 8u * (uint32_t)c, le);
@@ -656,7 +666,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 } else {
                     tmem_st16(a_row + 16u * (uint32_t)c, a);
-                    if constexpr (BF16OUT) tmem_st16(a_row + C::kALo + 16u * (uint32_t)c, al);
+                    if constexpr (C::kATerms == 2) tmem_st16(a_row + C::kALo + 16u * (uint32_t)c, al);
                 }
             }
             if constexpr (!kAllCodes) {   // the packed rows were read group by group: only now is their stage free
@@ -683,7 +693,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == 0) bulk_wait_read_all();   // this warp's previous stores have read the staging tile
             __syncwarp();
             const float row_inv = ctrl->row_scale[j & (kRowScaleSlots - 1)][q * 32 + lane];
-            const bool rescale = __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
+            const bool rescale = !PV && __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
+            const uint64_t rs2 = pack_f32x2(row_inv, row_inv), neg2 = pack_f32x2(-row_inv, -row_inv);   // PV: sigma rho
             if constexpr (R2) {
 #pragma unroll(C::kRolled ? 1 : D / 32)
                 for (int h = 0; h < D / 32; ++h) {   // E and O columns 16 h .. 16 h + 15 -> outputs 16 h .. and D / 2 + 16 h ..
@@ -712,7 +723,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                             const float2 e = make_float2(__uint_as_float(ev[i]), __uint_as_float(ev[i + 1]));
                             const float2 o = make_float2(__uint_as_float(ov[i]), __uint_as_float(ov[i + 1]));
                             float2 sum, diff;
-                            if constexpr (C::kPairs) {
+                            if constexpr (PV) {   // (E + O) sigma rho, (E - O) sigma rho
+                                const uint64_t ep = mul_f32x2(pack_f32x2(e.x, e.y), rs2), op = pack_f32x2(o.x, o.y);
+                                sum = unpack_f32x2(fma_f32x2(op, rs2, ep)), diff = unpack_f32x2(fma_f32x2(op, neg2, ep));
+                            } else if constexpr (C::kPairs) {
                                 const uint64_t ep = pack_f32x2(e.x, e.y), op = pack_f32x2(o.x, o.y);
                                 sum = unpack_f32x2(add_f32x2(ep, op)), diff = unpack_f32x2(sub_f32x2(ep, op));
                             } else {
@@ -797,10 +811,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ------------------------------------------------------------------------------------------------
 namespace {
 
-template <int D, bool BF16OUT, int BITS = 4, bool R2 = false>
-cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const uint32_t *sign_xor = nullptr)
+template <int D, bool BF16OUT, int BITS, bool R2, bool PV>
+cudaError_t launch_form(int64_t N, const GemmParams &g, cudaStream_t stream, const uint32_t *sign_xor)
 {
-    using C = Cfg<D, BF16OUT, BITS, R2>;
+    using C = Cfg<D, BF16OUT, BITS, R2, PV>;
     static DeviceSlots slots;
     int dev = 0;
     cudaError_t e = current_device_slot(&dev);
@@ -808,7 +822,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const ui
     int &sms = slots.sms[dev];
     if (sms == 0) {
         int n = 0;
-        if ((e = cudaFuncSetAttribute(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2, PV>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms = n;
     }
@@ -858,7 +872,15 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const ui
     const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
     prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid, kTile, segs);
-    return launch_kernel(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
+    return launch_kernel(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2, PV>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
+}
+
+template <int D, bool BF16OUT, int BITS = 4, bool R2 = false>
+cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream, const uint32_t *sign_xor = nullptr)
+{
+    if constexpr (R2)
+        if (g.per_vector) return launch_form<D, BF16OUT, BITS, R2, true>(N, g, stream, sign_xor);
+    return launch_form<D, BF16OUT, BITS, R2, false>(N, g, stream, sign_xor);
 }
 
 }  // namespace

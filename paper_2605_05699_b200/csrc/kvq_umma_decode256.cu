@@ -56,18 +56,24 @@ constexpr uint32_t kACol0 = 256;                       // accumulator E at 0, O 
 constexpr uint32_t kIdesc = umma_idesc_m128(kHalf, false);
 
 // BITS = 8: byte codes (Sec. 3.2 step 4's int8 output).  A packed row is then 256 B, loaded as two boxes of 128 B.
-template <bool BF16OUT, int BITS = 4>
+// PV: one scale per vector.  The A operand is the code itself, one exact fp16 term, and sigma rho stands in the epilogue: two operand sets for
+// bf16 output instead of three, and two A stages where two terms leave room for one.  Back to back, 592 and 2072 tiles: bf16 22.7 -> 19.5 us and 52.8 -> 42.4, byte codes 23.6 -> 18.7
+// and 58.5 -> 49.7; fp16 16.1 -> 14.8 and 40.6 -> 37.9.
+template <bool BF16OUT, int BITS = 4, bool PV = false>
 struct Cfg {
     static constexpr int kInRow = kD * BITS / 8;       // bytes of a packed row
     static constexpr int kInBytes = kTile * kInRow;    // 16 KB (32 KB for byte codes)
-    static constexpr int kTerms = BF16OUT ? 2 : 1;     // fp16 terms per operand
-    static constexpr int kAStages = BF16OUT ? 1 : 2;   // per parity: 128 columns hold a_hi | a_lo, or two stages of a_hi
+    static constexpr int kTerms = BF16OUT ? 2 : 1;     // fp16 terms of B
+    static constexpr int kATerms = BF16OUT && !PV ? 2 : 1;
+    static constexpr int kAStages = kATerms == 2 ? 1 : 2;   // per parity: 128 columns hold a_hi | a_lo, or two stages of a_hi
     static constexpr int kBBytes = kTerms * 2 * kBPart;
     // packed tiles in flight: what the split B and the 64 KB of output staging leave room for (byte codes with bf16 output:
     // one 32 KB tile, reloaded while the MMAs and the epilogue of the tile before run)
     static constexpr int kInStages = BITS == 8 ? (BF16OUT ? 1 : 2) : BF16OUT ? 2 : 4;
     // per-row output scales of the tiles between a dequant group and the epilogue: as many slots as a group can run ahead
-    static constexpr int kScaleSlots = 2 * kAStages;
+    // (kAStages + 1 are enough, and all that fits beside two terms of B: tile j writes its slot when the MMAs of tile j - kAStages are complete, and these
+    // began when the epilogue of the tile before them had read its own)
+    static constexpr int kScaleSlots = BF16OUT && PV ? 3 : 2 * kAStages;
     static constexpr int kScaleBytes = kScaleSlots * kTile * (int)sizeof(float);
     static constexpr int kSmemBytes = kBBytes + kInStages * kInBytes + 8 * kOutWarpBytes + kCtrlBytes + kScaleBytes + 1024;
     static_assert(kSmemBytes <= 232448, "shared memory over the per-CTA limit");
@@ -163,11 +169,11 @@ struct UmmaDecode256Maps {
     CUtensorMap out, tail;    // output, boxes of 32 columns x 32 rows (64-byte swizzle)
 };
 
-template <bool BF16OUT, int BITS>
+template <bool BF16OUT, int BITS, bool PV>
 __global__ void __launch_bounds__(kThreads, 1)
     kvq_decode_umma_d256_kernel(const __grid_constant__ UmmaDecode256Params prm, const __grid_constant__ UmmaDecode256Maps maps)
 {
-    using C = Cfg<BF16OUT, BITS>;
+    using C = Cfg<BF16OUT, BITS, PV>;
     constexpr int kTerms = C::kTerms, kInStages = C::kInStages, kInBytes = C::kInBytes;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -231,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const TileCursor first(share);
             const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
             if (row < prm.phys_rows) {
-                if (prm.g.per_vector) {
+                if constexpr (PV) {
                     const uint32_t s1 = (uint32_t)load_input(static_cast<const uint16_t *>(prm.g.scales) + row);
                     sc_first = make_uint4(s1 | (s1 << 16), s1 | (s1 << 16), s1 | (s1 << 16), s1 | (s1 << 16));
                 } else {
@@ -294,11 +300,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + (uint32_t)p * kHalf;
                     const uint32_t a_tmem = tmem_base + kACol0 + (uint32_t)p * 128u + (uint32_t)sa * 64u;
-                    // terms: a_hi W_hi (, a_lo W_hi, a_hi W_lo)
+                    // terms: a_hi W_hi (, a_lo W_hi, a_hi W_lo), or a W_hi (, a W_lo)
 #pragma unroll
-                    for (int t = 0; t < (BF16OUT ? 3 : 1); ++t) {
-                        const uint32_t a_base = a_tmem + (t == 1 ? 64u : 0u);
-                        const uint32_t b_part = (uint32_t)((t == 2 ? 2 * kBPart : 0) + p * kBPart) >> 4;
+                    for (int t = 0; t < C::kATerms + kTerms - 1; ++t) {
+                        const uint32_t a_base = a_tmem + (C::kATerms == 2 && t == 1 ? 64u : 0u);
+                        const uint32_t b_part = (uint32_t)((t == C::kATerms ? 2 * kBPart : 0) + p * kBPart) >> 4;
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks) {
                             const uint32_t koff = (uint32_t)(ks >> 2) * (kBBlock >> 4) + (uint32_t)(ks & 3) * 2u;   // (bytes >> 4) of K-step ks
@@ -326,12 +332,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (j >= n_my) return make_uint4(0u, 0u, 0u, 0u);
             const int64_t row = prm.g.phys_row(ahead.seg, ahead.row_in_segment(), rpl) + r;
             if (row >= prm.phys_rows) return make_uint4(0u, 0u, 0u, 0u);
-            if (prm.g.per_vector) {   // one scale per vector: the same value in every group's slot
+            if constexpr (PV) {   // one scale per vector: the same value in every group's slot
                 const uint32_t s1 = (uint32_t)load_input(reinterpret_cast<const uint16_t *>(prm.g.scales) + row);
                 const uint32_t s2 = s1 | (s1 << 16);
                 return make_uint4(s2, s2, s2, s2);
+            } else {
+                return load_input(scales + row);
             }
-            return load_input(scales + row);
         };
         uint4 sc_next = sc_first;   // requested before the first B build
         for (int j = 0; j < n_my; ++j, cur.advance(1)) {
@@ -376,8 +383,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- small or very large vector) is carried times a power of two instead, which the epilogue takes out again
             // ---- in fp32; every other row has the factor 1 and costs the epilogue nothing.  Both parity groups see the
             // ---- same scales and take the same factor; group 0 posts it.
-            float inv;
-            const float pw = operand_rescue<kG>(sc, rho, BITS == 4 ? 9000.0f : 500.0f, inv);   // 7 (127) times this stays inside fp16
+            // ---- One scale per vector: what the epilogue multiplies the row's sums of codes by.
+            float inv, pw = 1.0f;
+            if constexpr (PV) inv = __half2float(__ushort_as_half((unsigned short)(sc[0] & 0xFFFFu))) * rho;
+            else pw = operand_rescue<kG>(sc, rho, BITS == 4 ? 9000.0f : 500.0f, inv);   // 7 (127) times this stays inside fp16
             if (p == 0) row_scale[(j % C::kScaleSlots) * kTile + r] = inv;
             const uint32_t a_row = tmem_base + ((uint32_t)(q * 32) << 16) + kACol0 + (uint32_t)p * 128u + (uint32_t)sa * 64u;
             const __half2 h1032 = __float2half2_rn(1032.0f);
@@ -387,9 +396,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const __half2 s2 = __float2half2_rn(sig * rho * pw);
                 uint32_t a_hi[8], a_lo[8];
                 auto put = [&](int k, __half2 qq) {   // K pair k of the group: one rounding, and what it left behind
-                    const __half2 hi = __hmul2(qq, s2);
+                    const __half2 hi = PV ? qq : __hmul2(qq, s2);
                     a_hi[k] = *reinterpret_cast<const uint32_t *>(&hi);
-                    if constexpr (kTerms == 2) {
+                    if constexpr (C::kATerms == 2) {
                         const __half2 lo = __hfma2(qq, s2, __hneg2(hi));   // q s - hi: exact, the product has 15 (byte codes: 18) bits
                         a_lo[k] = *reinterpret_cast<const uint32_t *>(&lo);
                     }
@@ -429,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 tmem_st8(a_row + 8u * (uint32_t)c, a_hi);
-                if constexpr (kTerms == 2) tmem_st8(a_row + 64u + 8u * (uint32_t)c, a_lo);
+                if constexpr (C::kATerms == 2) tmem_st8(a_row + 64u + 8u * (uint32_t)c, a_lo);
             }
             if constexpr (BITS == 8) {   // the packed rows were read group by group: only now is their stage free
                 __syncwarp();
@@ -457,7 +466,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const CUtensorMap *tm = tail ? &maps.tail : &maps.out;
             const int segc = tail ? 0 : (int)seg;
             const float row_inv = row_scale[(j % C::kScaleSlots) * kTile + q * 32 + lane];
-            const bool rescale = __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
+            const bool rescale = !PV && __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
 #pragma unroll
             for (int cc = 0; cc < 2; ++cc) {   // 32 column pairs at a time: outputs n0 .. n0 + 31 and 128 + n0 ..
                 const int n0 = 64 * ch + 32 * cc;
@@ -490,8 +499,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const int i = 8 * k + 2 * v;
                         const float e0 = __uint_as_float(e[i]), e1 = __uint_as_float(e[i + 1]);
                         const float o0 = __uint_as_float(o[i]), o1 = __uint_as_float(o[i + 1]);
-                        lo[v] = narrow2<BF16OUT>(e0 + o0, e1 + o1);          // s_n is already in E and O
-                        hi[v] = narrow2<BF16OUT>(e0 - o0, e1 - o1) ^ f[v];   // times s_n s_{n+128}
+                        if constexpr (PV) {   // row_inv: sigma rho
+                            const uint64_t ep = mul_f32x2(pack_f32x2(e0, e1), pack_f32x2(row_inv, row_inv)), op = pack_f32x2(o0, o1);
+                            const float2 sum = unpack_f32x2(fma_f32x2(op, pack_f32x2(row_inv, row_inv), ep));
+                            const float2 diff = unpack_f32x2(fma_f32x2(op, pack_f32x2(-row_inv, -row_inv), ep));
+                            lo[v] = narrow2<BF16OUT>(sum.x, sum.y);
+                            hi[v] = narrow2<BF16OUT>(diff.x, diff.y) ^ f[v];
+                        } else {
+                            lo[v] = narrow2<BF16OUT>(e0 + o0, e1 + o1);          // s_n is already in E and O
+                            hi[v] = narrow2<BF16OUT>(e0 - o0, e1 - o1) ^ f[v];   // times s_n s_{n+128}
+                        }
                     }
                     const uint32_t off = (uint32_t)(lane * 64 + ((k ^ ((lane >> 1) & 3)) << 4));   // 64-byte swizzle
                     *reinterpret_cast<uint4 *>(stg + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
@@ -525,10 +542,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ------------------------------------------------------------------------------------------------
 namespace {
 
-template <bool BF16OUT, int BITS>
+template <bool BF16OUT, int BITS, bool PV>
 cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cudaStream_t stream)
 {
-    using C = Cfg<BF16OUT, BITS>;
+    using C = Cfg<BF16OUT, BITS, PV>;
     static DeviceSlots slots;
     int dev = 0;
     cudaError_t e = current_device_slot(&dev);
@@ -536,7 +553,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cud
     int &sms = slots.sms[dev];
     if (sms == 0) {
         int n = 0;
-        if ((e = cudaFuncSetAttribute(kvq_decode_umma_d256_kernel<BF16OUT, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(kvq_decode_umma_d256_kernel<BF16OUT, BITS, PV>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms = n;
     }
@@ -581,15 +598,19 @@ cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cud
     const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
     prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid, kTile, segs);
-    return launch_kernel(kvq_decode_umma_d256_kernel<BF16OUT, BITS>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
+    return launch_kernel(kvq_decode_umma_d256_kernel<BF16OUT, BITS, PV>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 }  // namespace
 
 cudaError_t umma_decode_d256(bool bf16, int bits, int64_t N, const GemmParams &g, const uint32_t *sign_xor, cudaStream_t stream)
 {
-    if (bits == 8) return bf16 ? launch<true, 8>(N, g, sign_xor, stream) : launch<false, 8>(N, g, sign_xor, stream);
-    return bf16 ? launch<true, 4>(N, g, sign_xor, stream) : launch<false, 4>(N, g, sign_xor, stream);
+    if (g.per_vector) {
+        if (bits == 8) return bf16 ? launch<true, 8, true>(N, g, sign_xor, stream) : launch<false, 8, true>(N, g, sign_xor, stream);
+        return bf16 ? launch<true, 4, true>(N, g, sign_xor, stream) : launch<false, 4, true>(N, g, sign_xor, stream);
+    }
+    if (bits == 8) return bf16 ? launch<true, 8, false>(N, g, sign_xor, stream) : launch<false, 8, false>(N, g, sign_xor, stream);
+    return bf16 ? launch<true, 4, false>(N, g, sign_xor, stream) : launch<false, 4, false>(N, g, sign_xor, stream);
 }
 
 }  // namespace kvq

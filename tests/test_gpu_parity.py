@@ -1100,6 +1100,34 @@ def test_one_scale_per_vector_on_the_tensor_cores(D, dtype, N, n_lambda, rpl):
     plan.close()
 
 
+@pytest.mark.parametrize("D,dtype,nbits", [(64, "f16", 8), (64, "bf16", 4), (96, "f16", 4), (96, "bf16", 8), (128, "f16", 8), (128, "bf16", 8), (128, "bf16", 4),
+                                           (160, "f16", 4), (160, "bf16", 4), (256, "f16", 8), (256, "bf16", 4), (256, "bf16", 8)])
+@pytest.mark.parametrize("N,n_lambda,rpl", [(129, 1, 0), (148 * 128 + 1, 1, 0), (20011, 7, 2900), (21000, 300, 70)])
+def test_decode_of_codes_as_operands(D, dtype, nbits, N, n_lambda, rpl):
+    """One scale per vector: the tensor-core decode takes the codes themselves as its operand and the scale in its epilogue.  Every code value, scales
+    over the whole range that the output type can show and zeros among them, the edges of tiles and shares, and lambda rows that change
+    at every tile (B is rebuilt between tiles in flight)."""
+    gen = torch.Generator().manual_seed(1000 * D + N + nbits)
+    odt = DT[dtype]
+    plan = kb.Plan(D, D, 77, bits=nbits)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_AUTO, kb.KVQ_IMPL_GEMM)
+    lam = wl.make_lambda(n_lambda, D, 78)
+    packed = torch.randint(0, 256, (N, D * nbits // 8), generator=gen, dtype=torch.int32).to(torch.uint8)
+    lo, hi = (-6.0, 6.0) if dtype == "f16" else (-14.0, 15.0)   # powers of two; fp16 output: no row overflows or goes subnormal
+    scales = torch.exp2(torch.rand(N, 1, generator=gen) * (hi - lo) + lo).to(torch.float16)
+    scales[::97] = 0.0
+    out = gpu_decode_raw(plan, packed.cuda(), scales.cuda(), lam.cuda(), dtype, rpl)
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    ob, o64 = ko.decode(packed.numpy(), bits(scales), plan.signs(), lam.numpy(), D, odt, rpl, want_f64=True, bits=nbits)
+    parity.check_decode(bits(out), ob, o64, odt, "codes as operands")
+    if dtype == "f16":   # and no further from 64 bits than fp16 output alone makes it: 2^-11 / sqrt(3) of every entry, and W's one rounding to fp16, as much
+        got = out.cpu().double().numpy()
+        live = np.abs(o64).max(1) > 0
+        rel = np.linalg.norm(got - o64, axis=1)[live] / np.linalg.norm(o64, axis=1)[live]
+        assert rel.max() < 2.0 ** -11
+    plan.close()
+
+
 def test_base_variants_append_and_flush_and_refusals():
     D, S, T = 256, 24, 40
     plan = kb.Plan(D, D, 7, bits=8)
