@@ -189,6 +189,10 @@ __device__ __forceinline__ void encode_batch(const MatvecParams &prm, const RowM
     __syncthreads();
     if (last) grid_trigger();   // nothing but the tables is read from here on
 
+    // The way back's table rows where registers hold both slices: requested here, their round trip to L2 runs under the product and the quantizer.
+    constexpr bool kEarly = FLUSH && Gm::kLoops;
+    float4 t2[kEarly ? Gm::CH : 1][P];
+    if constexpr (kEarly) load_rows<D>(prm.table2, warp, lane, 0, t2);
     float z[P][4];
     matvec<D>(prm.table, t, xs, red, warp, lane, z);
 
@@ -263,11 +267,16 @@ __device__ __forceinline__ void encode_batch(const MatvecParams &prm, const RowM
         }
     }
     if constexpr (FLUSH) {
-        float4 t2[Gm::CH][P];
-        load_rows<D>(prm.table2, warp, lane, 0, t2);   // in flight across the barrier
-        __syncthreads();                               // every warp's vector is back in shared memory; red is free again
         float y[P][4];
-        matvec<D>(prm.table2, t2, xs, red, warp, lane, y);
+        if constexpr (kEarly) {
+            __syncthreads();                               // every warp's vector is back in shared memory; red is free again
+            matvec<D>(prm.table2, t2, xs, red, warp, lane, y);
+        } else {
+            float4 t2[Gm::CH][P];
+            load_rows<D>(prm.table2, warp, lane, 0, t2);   // in flight across the barrier
+            __syncthreads();
+            matvec<D>(prm.table2, t2, xs, red, warp, lane, y);
+        }
         if (!live) return;
         unsigned char *out = static_cast<unsigned char *>(prm.out) + orow * (2 * D);
 #pragma unroll
