@@ -117,17 +117,13 @@ __device__ __forceinline__ void put_b_row(unsigned char *sB, const float4 m0, co
     }
 }
 
-// The first B: eight rows of both parities per builder warp, requested in front of the grid wait and all together.  (Before, a warp took
-// sixteen rows of one parity in two round trips behind lambda, and every row crossed L2 for each parity.  Back to back, 1500 fp16
-// vectors 9.7 -> 7.6 us, 10,000: 10.3 -> 8.9; bf16 11.1 -> 9.5, 12.0 -> 11.0; 212,992 under one lambda row 36.9 -> 33.9, 48.9 -> 46.9, in short
-// runs; with the board at its power limit, behind long encodes, and together with RecipLambda's redux: 46 -> 40, 58 -> 54.)
-constexpr int kFirstRows = kHalf / 16;
+// Four rows of both parities of the first B.
 struct FirstRows {
-    float4 m[kFirstRows][2];
+    float4 m[4][2];
     __device__ __forceinline__ void load(const float *__restrict__ b0, int n0, int lane)
     {
 #pragma unroll
-        for (int k = 0; k < kFirstRows; ++k)
+        for (int k = 0; k < 4; ++k)
 #pragma unroll
             for (int h = 0; h < 2; ++h) m[k][h] = __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)(n0 + k) * kD) + 2 * lane + h);
     }
@@ -135,7 +131,7 @@ struct FirstRows {
     __device__ __forceinline__ void store(unsigned char *sB, const Recip &rl, int n0, int lane) const
     {
 #pragma unroll
-        for (int k = 0; k < kFirstRows; ++k)
+        for (int k = 0; k < 4; ++k)
 #pragma unroll
             for (int p = 0; p < 2; ++p) put_b_row<TERMS>(sB, m[k][0], m[k][1], rl, p, n0 + k, lane);
     }
@@ -151,6 +147,52 @@ __device__ __forceinline__ void build_b_rows(unsigned char *sB, const float *__r
         const float4 m1 = __ldg(reinterpret_cast<const float4 *>(b0 + (size_t)n * kD) + 2 * lane + 1);
         put_b_row<TERMS>(sB, m0, m1, rl, p, n, lane);
     }
+}
+
+// What the dequant warps take from the start: rho of the first lambda row and the scales of their first tile's row.
+struct FirstOperand {
+    float rho;
+    uint4 sc;
+};
+
+// The way from the kernel's entry to the first B for warps 2 to 17 (w from 0 on).  Table rows are requested in front of the grid wait, every row once
+// for both parities.  The dequant warps, which have the first tile to dequantise before the first MMA can begin, build four rows each, the epilogue
+// warps twelve.  Out of line: its registers are no part of the role loops' allocation.  Back to back, eight rows each in line -> this: one tile per CTA fp16 9.35 -> 8.7 us,
+// bf16 11.8 -> 11.0; four 14.8 -> 14.2, 21.6 -> 20.7.
+template <int TERMS, bool PV>
+__device__ __noinline__ FirstOperand first_operand(unsigned char *sB, Ctrl *ctrl, const float *__restrict__ b0, const float *lam, const uint16_t *row_scales, int w, int lane)
+{
+    const int n0 = w < 8 ? 96 + 4 * w : 12 * (w - 8);
+    FirstRows r0, r1;
+    r0.load(b0, n0, lane);
+    if (w >= 8) r1.load(b0, n0 + 4, lane);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    grid_wait();
+    FirstOperand first;
+    first.sc = make_uint4(0u, 0u, 0u, 0u);
+    if (row_scales) {
+        if constexpr (PV) {
+            const uint32_t s1 = (uint32_t)load_input(row_scales), s2 = s1 | (s1 << 16);
+            first.sc = make_uint4(s2, s2, s2, s2);
+        } else {
+            first.sc = load_input(reinterpret_cast<const uint4 *>(row_scales));
+        }
+    }
+    const Recip rl(lam, lane);
+    first.rho = rl.rho;
+    if (rl.wide) ctrl->any_wide = 1u;
+    r0.store<TERMS>(sB, rl, n0, lane);
+    if (w >= 8) {
+        r0.load(b0, n0 + 8, lane);
+        r1.store<TERMS>(sB, rl, n0 + 4, lane);
+        r0.store<TERMS>(sB, rl, n0 + 8, lane);
+    }
+    fence_proxy_async();   // B is read by the tensor core through the async proxy
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
+    return first;
 }
 
 }  // namespace
@@ -201,12 +243,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         ctrl->abort = 0u;
         ctrl->any_wide = 0u;
         mbar_init_fence();
+        fence_proxy_async();
     }
     if (threadIdx.x >= 32 && threadIdx.x < 96) {   // sign of s_n s_{n+128}: the xor of the two sign bits
         const int m = threadIdx.x - 32;
         reinterpret_cast<uint32_t *>(ctrl->flip)[m] = prm.sign_xor[m] ^ prm.sign_xor[m + 64];
     }
-    if (warp == 0) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
+    if (warp == 1) tmem_alloc(smem_u32(&ctrl->tmem_base), kTmemCols);
 
     // ---- tiles: lambda segments of rpl rows, cut into tiles of 128 rows; a contiguous range of tiles per CTA
     const int64_t rpl = prm.rpl;
@@ -215,44 +258,26 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int64_t seg_first = share.seg;
     auto lambda_row = [&](int64_t seg) -> const float * { return prm.g.lambda + prm.g.lambda_index(seg) * kD; };
 
-    FirstRows rows;
-    const bool builds_first = n_my > 0 && warp >= 2;
-    if (builds_first) rows.load(prm.g.b0, (warp - 2) * kFirstRows, lane);
-    fence_proxy_async();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    grid_wait();
+    // ---- B for the first tile's lambda row.  The dequant warps also request their first tile's scales there and keep rho, so that neither
+    // ---- costs a round trip to L2 after it.
+    FirstOperand first = {1.0f, {0u, 0u, 0u, 0u}};
+    if (n_my > 0 && warp >= 2) {
+        const uint16_t *row_scales = nullptr;
+        if (warp < 10) {
+            const TileCursor at(share);
+            const int64_t row = prm.g.phys_row(at.seg, at.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
+            if (row < prm.phys_rows) row_scales = static_cast<const uint16_t *>(prm.g.scales) + row * (PV ? 1 : kG);
+        }
+        first = first_operand<kTerms, PV>(sB, ctrl, prm.g.b0, lambda_row(seg_first), row_scales, warp - 2, lane);
+    } else {
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        grid_wait();
+    }
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile uint32_t *abort_flag = &ctrl->abort;
     uint32_t *status = prm.g.status;
-
-    // ---- B for the first tile's lambda row, by the sixteen dequant and epilogue warps
-    // ---- (the dequant warps request their first tile's scales before the build and keep rho from it, so that neither
-    // ---- costs a round trip to L2 after it)
-    float rho_first = 1.0f;
-    uint4 sc_first = make_uint4(0u, 0u, 0u, 0u);
-    if (builds_first) {
-        if (warp < 10) {
-            const TileCursor first(share);
-            const int64_t row = prm.g.phys_row(first.seg, first.row_in_segment(), rpl) + (warp & 3) * 32 + lane;
-            if (row < prm.phys_rows) {
-                if constexpr (PV) {
-                    const uint32_t s1 = (uint32_t)load_input(static_cast<const uint16_t *>(prm.g.scales) + row);
-                    sc_first = make_uint4(s1 | (s1 << 16), s1 | (s1 << 16), s1 | (s1 << 16), s1 | (s1 << 16));
-                } else {
-                    sc_first = load_input(static_cast<const uint4 *>(prm.g.scales) + row);
-                }
-            }
-        }
-        const Recip rl(lambda_row(seg_first), lane);
-        rho_first = rl.rho;
-        if (rl.wide) ctrl->any_wide = 1u;
-        rows.store<kTerms>(sB, rl, (warp - 2) * kFirstRows, lane);
-        fence_proxy_async();   // B is read by the tensor core through the async proxy
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&ctrl->b_first));
-    }
 
     if (warp == 0) {
         // =========================== producer ===========================
@@ -325,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int r = q * 32 + lane;            // tile row and tensor-memory lane of this thread
         const uint4 *scales = static_cast<const uint4 *>(prm.g.scales);   // 8 fp16 scales per row
         int64_t cached_row = n_my > 0 ? prm.g.lambda_index(seg_first) : -1;   // the lambda row that B holds (built above)
-        float rho = rho_first;
+        float rho = first.rho;
 
         TileCursor cur(share), ahead(share);
         auto fetch_scales = [&](int j) -> uint4 {
@@ -340,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 return load_input(scales + row);
             }
         };
-        uint4 sc_next = sc_first;   // requested before the first B build
+        uint4 sc_next = first.sc;   // requested before the first B build
         for (int j = 0; j < n_my; ++j, cur.advance(1)) {
             const uint4 sc4 = sc_next;
             const uint32_t sc[4] = {sc4.x, sc4.y, sc4.z, sc4.w};
@@ -466,7 +491,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             const CUtensorMap *tm = tail ? &maps.tail : &maps.out;
             const int segc = tail ? 0 : (int)seg;
             const float row_inv = row_scale[(j % C::kScaleSlots) * kTile + q * 32 + lane];
+            // The accumulator has one stage: what stands between the first request and its release is on every tile's critical path, so both
+            // chunks are read and staged before either is stored.  2072 tiles fp16 37.2 -> 36.5 us, bf16 53.7 -> 51.1; 1008 under 56 lambda rows 24.3 -> 23.5, 36.2 -> 33 to 36.
+            if (lane == 0) bulk_wait_read_all();   // this warp's stores of the tile before have read the staging boxes
             const bool rescale = !PV && __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
+            __syncwarp();
 #pragma unroll
             for (int cc = 0; cc < 2; ++cc) {   // 32 column pairs at a time: outputs n0 .. n0 + 31 and 128 + n0 ..
                 const int n0 = 64 * ch + 32 * cc;
@@ -487,8 +516,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty));
                 }
-                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // the stores of this chunk's boxes one tile ago have read them
-                __syncwarp();
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {   // 16-byte chunk k of each box row: 8 outputs
                     const uint4 fl = ctrl->flip[(n0 >> 3) + k];   // warp-uniform address: a broadcast
@@ -514,13 +541,18 @@ __global__ void __launch_bounds__(kThreads, 1)
                     *reinterpret_cast<uint4 *>(stg + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                     *reinterpret_cast<uint4 *>(stg + 32 * 64 + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
                 }
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_3d(tm, n0, row_in_seg, segc, smem_u32(stg));
-                    tma_store_3d(tm, kHalf + n0, row_in_seg, segc, smem_u32(stg + 32 * 64));
-                    bulk_commit();
+            }
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+#pragma unroll
+                for (int cc = 0; cc < 2; ++cc) {
+                    const int n0 = 64 * ch + 32 * cc;
+                    const uint32_t stg = smem_u32(stg_base + cc * (2 * 32 * 64));
+                    tma_store_3d(tm, n0, row_in_seg, segc, stg);
+                    tma_store_3d(tm, kHalf + n0, row_in_seg, segc, stg + 32 * 64);
                 }
+                bulk_commit();
             }
         }
         if (lane == 0) bulk_wait_all();
