@@ -345,6 +345,7 @@ kvq_status_t kvq_plan_prepare(kvq_plan_t *plan, kvq_dtype_t dtype)
                                          : umma_decode(plan->D, bf16, plan->bits, 0, g, plan->sign_xor, nullptr, !plan->rot));
     if (gemm_decode_ok(plan, bf16) && !plan->rot && plan->D != 256)   // the form that a rotation set later takes
         also(umma_decode(plan->D, bf16, plan->bits, 0, g, plan->sign_xor, nullptr, false));
+    if (plan->bits == 4 && !per_vector && umma_flush_supported(plan->D)) also(umma_flush(plan->D, bf16, nullptr, 0, g, plan->d_e0, plan->sign_xor, nullptr));
     if (umma_calibrate_supported(plan->D, bf16)) also(umma_calibrate(plan->D, bf16, 0, prm, plan->d_e0, nullptr, nullptr));
     also(matvec_encode(plan->D, plan->group, plan->bits, bf16, 0, prm, plan->d_b0, nullptr));
     also(matvec_decode(plan->D, plan->group, plan->bits, bf16, 0, prm, plan->d_e0, nullptr));
@@ -574,6 +575,48 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
     const int64_t rpl = (streams_per_lambda < 1 ? 1 : streams_per_lambda) * rows;
     const RowMap map{rows, T_max, pos0};
     if (!at && plan->rot && plan->dec_impl == KVQ_IMPL_FFT) return KVQ_ERR_UNSUPPORTED_DIM;
+    const bool mv = flush_decode_is_matvec(plan, N);
+    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    const bool bf16 = dtype == KVQ_BF16;
+    // A large block of a plan without a rotation: the tensor-core decode, reading and writing the window [pos0, pos0 + rows)
+    // of every stream's cache in place through a cache view (tiles of 128 rows per stream, so blocks of 64 rows and more; the whole
+    // cache must fit 32-bit tensor-map coordinates).  Shorter blocks stay in fp32: the tensor cores take 64 x 17 rows at D = 256 in
+    // 21.0 us instead of 28.1, but with operands of 16 bits (fp16 output: relative error 3.4e-4 instead of the output rounding's
+    // 2.1e-4; bf16: two to four times as many outputs off their correct rounding, 1.0e-3 of them at D = 128 instead of 3.8e-4).
+    const bool view = !at && !mv && plan->dec_impl != KVQ_IMPL_FFT && gemm_decode_ok(plan, bf16) && (rows >= 64 || plan->dec_impl == KVQ_IMPL_GEMM) &&
+                      S <= (((int64_t)1 << 31) - 1) / T_max;
+    auto view_params = [&] {
+        GemmParams g;
+        g.packed = packed_cache;
+        g.scales = scales_cache;
+        g.lambda = lambda;
+        g.out = dq_cache;
+        g.b0 = plan->d_b0;
+        g.N = N;
+        g.n_lambda = n_lambda;
+        g.rows_per_lambda = rpl;
+        g.per_vector = plan->group == plan->D;
+        g.status = plan->d_status;
+        g.view = CacheView{rows, T_max, pos0, streams_per_lambda < 1 ? 1 : streams_per_lambda};
+        return g;
+    };
+    // Both directions on the tensor cores: one launch where it is built and pays.  (A shortened first wait is the encode kernel's; and a block that lies in the
+    // dequantized cache itself is read to its end before the first row is written.)
+    const uintptr_t x0 = reinterpret_cast<uintptr_t>(x_block), d0 = reinterpret_cast<uintptr_t>(dq_cache);
+    const bool apart = x0 + (uintptr_t)N * plan->D * 2 <= d0 || d0 + (uintptr_t)S * T_max * plan->D * 2 <= x0;
+    if (view && apart && N < ((int64_t)1 << 31) && plan->group != plan->D && plan->bits == 4 && !plan->rot && umma_flush_pays(plan->D, bf16, S, rows) &&
+        (plan->enc_impl == KVQ_IMPL_GEMM || (plan->enc_impl == KVQ_IMPL_AUTO && N > matvec_max_rows(plan->D))) && plan->first_wait_polls == 0) {
+        if (!x_block || !packed_cache || !scales_cache) return KVQ_ERR_INVALID_ARG;
+        kvq_status_t st = check_lambda(N, lambda, n_lambda, rpl);
+        if (st != KVQ_OK) return st;
+        if (misaligned16(x_block) || misaligned16(packed_cache) || misaligned16(scales_cache)) return KVQ_ERR_ALIGNMENT;
+        if ((st = ensure_device(plan)) != KVQ_OK) return st;
+        if (umma_flush(plan->D, bf16, x_block, N, view_params(), plan->d_e0, plan->sign_xor, stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return KVQ_ERR_CUDA;
+        }
+        return KVQ_OK;
+    }
     bool fused = false;
     const DevicePos pos{pos0_device, T_max - rows};
     kvq_status_t st = encode_common(plan, x_block, dtype, N, lambda, n_lambda, rpl, packed_cache, scales_cache, map, cuda_stream,
@@ -588,29 +631,8 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
     prm.out = dq_cache;
     prm.in_map = map;
     prm.out_map = map;
-    const bool mv = flush_decode_is_matvec(plan, N);
-    cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const bool bf16 = dtype == KVQ_BF16;
-    // A large block of a plan without a rotation: the tensor-core decode, reading and writing the window [pos0, pos0 + rows)
-    // of every stream's cache in place through a cache view (tiles of 128 rows per stream, so blocks of 64 rows and more; the whole
-    // cache must fit 32-bit tensor-map coordinates).  Shorter blocks stay in fp32: the tensor cores take 64 x 17 rows at D = 256 in
-    // 21.0 us instead of 28.1, but with operands of 16 bits (fp16 output: relative error 3.4e-4 instead of the output rounding's
-    // 2.1e-4; bf16: two to four times as many outputs off their correct rounding, 1.0e-3 of them at D = 128 instead of 3.8e-4).
-    if (!mv && plan->dec_impl != KVQ_IMPL_FFT && gemm_decode_ok(plan, bf16) && (rows >= 64 || plan->dec_impl == KVQ_IMPL_GEMM) &&
-        S <= (((int64_t)1 << 31) - 1) / T_max) {
-        GemmParams g;
-        g.packed = packed_cache;
-        g.scales = scales_cache;
-        g.lambda = lambda;
-        g.out = dq_cache;
-        g.b0 = plan->d_b0;
-        g.N = N;
-        g.n_lambda = n_lambda;
-        g.rows_per_lambda = rpl;
-        g.per_vector = plan->group == plan->D;
-        g.status = plan->d_status;
-        g.view = CacheView{rows, T_max, pos0, streams_per_lambda < 1 ? 1 : streams_per_lambda};
-        if (umma_decode(plan->D, bf16, plan->bits, N, g, plan->sign_xor, stream, true) != cudaSuccess) {
+    if (view) {
+        if (umma_decode(plan->D, bf16, plan->bits, N, view_params(), plan->sign_xor, stream, true) != cudaSuccess) {
             (void)cudaGetLastError();
             return KVQ_ERR_CUDA;
         }

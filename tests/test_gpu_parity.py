@@ -694,6 +694,51 @@ def test_flush_of_short_blocks_dequantizes_in_fp32(D, dtype):
         assert torch.equal(got[0], got[1]), S
 
 
+@pytest.mark.parametrize("D", [64, 96, 128])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("S,rows,T_max,pos0,spl", [
+    (3, 700, 701, 1, 3),        # few tiles, a ragged last one per stream
+    (40, 64, 80, 5, 40),        # the shortest block: half tiles
+    (37, 129, 200, 70, 5),      # a tile of one row behind every full one, eight lambda rows, the last with fewer streams
+    (449, 64, 64, 0, 1),        # a lambda row per stream: both operands rebuilt between any two tiles
+    (2, 9500, 9503, 3, 1),      # a tile or two per CTA
+    (32, 3000, 3100, 100, 16),  # five tiles per CTA
+])
+def test_block_flush_in_one_launch_equals_encode_and_decode(D, dtype, S, rows, T_max, pos0, spl):
+    """A large block goes through both contractions in one launch: codes and scales are those of kvq_encode, the dequantized rows those of kvq_decode on them, bit for
+    bit, and nothing beside the block is touched.  One row in 17 is scaled out of the operands' comfort zone; the second lambda row, where there is one, is too
+    wide for the fp16 operand and its tiles are redone in fp32."""
+    tdt = wl.torch_dtype(dtype)
+    plan = kb.Plan(D, G, 77)
+    n_lambda = (S + spl - 1) // spl
+    lam = wl.make_lambda(n_lambda, D, 78)
+    if n_lambda > 1:
+        lam[1, ::3] *= 1e-4
+    lam = lam.cuda()
+    x = wl.make_vectors(S * rows, D, dtype, "k_outlier", 79).view(S, rows, D).cuda()
+    x[:, ::17] *= 2.0 ** -14
+    packed = torch.full((S, T_max, D // 2), 0xAB, dtype=torch.uint8, device="cuda")
+    scales = torch.full((S, T_max, D // G), 1.25, dtype=torch.float16, device="cuda")
+    dq = torch.full((S, T_max, D), 3.0, dtype=tdt, device="cuda")
+    n0 = kb.kvq_launch_count()
+    kb.kvq_flush_block(plan.handle, x, lam, packed, scales, dq, pos0, spl)
+    torch.cuda.synchronize()
+    assert kb.kvq_launch_count() - n0 == 1 and kb.kvq_plan_device_status(plan.handle) == 0
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_GEMM)
+    p2, s2 = plan.empty_packed(S * rows), plan.empty_scales(S * rows)
+    kb.kvq_encode(plan.handle, x.view(S * rows, D), lam, p2, s2, spl * rows)
+    out = torch.empty(S * rows, D, dtype=tdt, device="cuda")
+    kb.kvq_decode(plan.handle, p2, s2, lam, out, spl * rows)
+    torch.cuda.synchronize()
+    block = slice(pos0, pos0 + rows)
+    assert torch.equal(packed[:, block].reshape(S * rows, -1), p2) and torch.equal(scales[:, block].reshape(S * rows, -1), s2)
+    assert torch.equal(dq[:, block].reshape(S * rows, D).view(torch.int16), out.view(torch.int16))
+    mask = torch.ones(T_max, dtype=torch.bool, device="cuda")
+    mask[block] = False
+    assert bool((dq[:, mask] == 3.0).all()) and bool((packed[:, mask] == 0xAB).all()) and bool((scales[:, mask] == 1.25).all())
+    plan.close()
+
+
 @pytest.mark.parametrize("D", [64, 96, 128, 160, 256])
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("group,nbits", [(G, 4), (0, 4), (G, 8)])
