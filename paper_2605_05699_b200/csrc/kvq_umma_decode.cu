@@ -747,7 +747,7 @@ cudaError_t launch_form(int64_t N, const GemmParams &g, cudaStream_t stream, con
     const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
     prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid, kTile, segs);
-    return launch_kernel(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2, PV>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
+    return launch_kernel(kvq_decode_umma_kernel<D, BF16OUT, BITS, R2, PV>, prm.plan.shares, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 template <int D, bool BF16OUT, int BITS = 4, bool R2 = false>

@@ -630,7 +630,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, const uint32_t *sign_xor, cud
     const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
     prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid, kTile, segs);
-    return launch_kernel(kvq_decode_umma_d256_kernel<BF16OUT, BITS, PV>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, maps);
+    return launch_kernel(kvq_decode_umma_d256_kernel<BF16OUT, BITS, PV>, prm.plan.shares, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 }  // namespace

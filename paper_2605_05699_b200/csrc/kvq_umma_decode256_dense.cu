@@ -493,7 +493,7 @@ cudaError_t launch(int64_t N, const GemmParams &g, cudaStream_t stream)
     const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int64_t pairs = tiles < sms / 2 ? tiles : sms / 2;
     prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)pairs);
-    return launch_kernel(kvq_decode_umma_d256_dense_kernel<BF16OUT>, (unsigned)(2 * pairs), kThreads, C::kSmemBytes, stream, 1, prm, maps);
+    return launch_kernel(kvq_decode_umma_d256_dense_kernel<BF16OUT>, 2 * prm.plan.shares, kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 }  // namespace

@@ -505,7 +505,7 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     const int64_t tiles = n_seg * ((prm.rpl + kTile - 1) / kTile);
     const int grid = (int)(tiles < sms ? tiles : sms);
     prm.plan = TilePlan(n_seg, prm.rpl, (unsigned)grid);
-    return launch_kernel(kvq_encode_umma_kernel<D, BF16, CALIB, PERVEC, WIDE>, (unsigned)grid, kThreads, C::kSmemBytes, stream, 1, prm, tm_x);
+    return launch_kernel(kvq_encode_umma_kernel<D, BF16, CALIB, PERVEC, WIDE>, prm.plan.shares, kThreads, C::kSmemBytes, stream, 1, prm, tm_x);
 }
 
 }  // namespace

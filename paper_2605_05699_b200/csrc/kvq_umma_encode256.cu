@@ -579,7 +579,7 @@ cudaError_t launch(int64_t N, const FftParams &f, const float *e0, cudaStream_t 
     const int64_t tiles = tiles_of(n_seg, prm.rpl, 2 * ROWS);
     const unsigned pairs = (unsigned)(tiles < fit ? tiles : fit);
     prm.plan = TilePlan(n_seg, prm.rpl, pairs, 2 * ROWS);
-    return launch_kernel(kvq_encode_umma_d256_kernel<BF16, CALIB, PERVEC, ROWS>, 2 * pairs, kThreads, C::kSmemBytes, stream, 2, prm, tm_x);
+    return launch_kernel(kvq_encode_umma_d256_kernel<BF16, CALIB, PERVEC, ROWS>, 2 * prm.plan.shares, kThreads, C::kSmemBytes, stream, 2, prm, tm_x);
 }
 
 template <bool BF16, bool CALIB, bool PERVEC>

@@ -548,7 +548,7 @@ cudaError_t launch(const void *x, int64_t N, const GemmParams &g, const float *e
     const int64_t tiles = S * ((prm.rows + kTile - 1) / kTile);
     const unsigned grid = (unsigned)(tiles < sms ? tiles : sms);
     prm.plan = TilePlan(S, prm.rows, grid, kTile, g.n_lambda == 1 ? S : g.view.streams_per_lambda.d);
-    return launch_kernel(kvq_flush_umma_kernel<D, BF16>, grid, C::kThreads, C::kSmemBytes, stream, 1, prm, maps);
+    return launch_kernel(kvq_flush_umma_kernel<D, BF16>, prm.plan.shares, C::kThreads, C::kSmemBytes, stream, 1, prm, maps);
 }
 
 }  // namespace
