@@ -145,6 +145,7 @@ struct Ctrl {
     uint64_t a_full[4], a_empty[4];
     uint64_t acc_full[2], acc_empty[2];
     uint64_t b_first;
+    uint64_t meet[4];   // one accumulator: the two epilogue warps of 32 rows
     uint32_t tmem_base;
     volatile uint32_t abort;
     volatile uint32_t any_wide;   // some lambda row of this CTA's tiles is too wide for the fp16 B operand: redone in fp32 at the end
@@ -274,8 +275,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&ctrl->acc_full[s]), 1);
-            mbar_init(smem_u32(&ctrl->acc_empty[s]), 4);
+            mbar_init(smem_u32(&ctrl->acc_empty[s]), C::kOneAcc ? 8 : 4);
         }
+        if constexpr (C::kOneAcc)
+            for (int s = 0; s < 4; ++s) mbar_init(smem_u32(&ctrl->meet[s]), 2);
         mbar_init(smem_u32(&ctrl->b_first), kBuilders);
         ctrl->abort = 0u;
         ctrl->any_wide = 0u;
@@ -558,26 +561,32 @@ __global__ void __launch_bounds__(kThreads, 1)
         // =========================== epilogue: accumulator -> fp16 -> TMA store ===========================
         const int grp = (warp - 10) >> 2;
         const int q = warp & 3;
-        unsigned char *stg = sOut + (warp - 10) * C::kOutWarpBytes;   // this warp's staging tile
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        TileCursor cur(share, grp);
-        for (int j = grp; j < n_my; j += 2, cur.advance(2)) {
+        // One accumulator: both groups take every tile, the first three fifths of its columns and the rest, so that it goes back sooner; the two warps that share 32
+        // rows fill one staging tile of two and meet before the first of them stores it.
+        // bf16, 296, 1036 and 2072 tiles 9.74 -> 9.64 us, 18.5 -> 17.8 and 32.7 -> 31.0.  (148, a tile per CTA, 8.1 -> 8.2: chosen at run time the loop costs more, 8.5.)
+        constexpr bool both = C::kOneAcc;
+        constexpr int step = both ? 1 : 2;
+        const int h0 = both && grp == 1 ? 3 : 0, h1 = both && grp == 0 ? 3 : D / 32;   // 16-column steps of each parity
+        TileCursor cur(share, both ? 0 : grp);
+        for (int j = both ? 0 : grp; j < n_my; j += step, cur.advance(step)) {
             const int sc = j % kAccStages;
+            unsigned char *stg = sOut + (both ? (j & 1) * 4 + (warp - 10) % 4 : warp - 10) * C::kOutWarpBytes;   // this warp's staging tile
             if (!wait_or_abort(smem_u32(&ctrl->acc_full[j & 1]), (uint32_t)(j >> 1) & 1u, abort_flag, status, KVQ_DEV_MMA_TIMEOUT)) break;
             tc_fence_after();
-            if (lane == 0) bulk_wait_read_all();   // this warp's previous stores have read the staging tile
+            if (!both && lane == 0) bulk_wait_read_all();   // this warp's previous stores have read the staging tile
             __syncwarp();
             const float row_inv = ctrl->row_scale[j & (kRowScaleSlots - 1)][q * 32 + lane];
             const bool rescale = !PV && __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
             const uint64_t rs2 = pack_f32x2(row_inv, row_inv), neg2 = pack_f32x2(-row_inv, -row_inv);   // PV: sigma rho
             if constexpr (R2) {
 #pragma unroll(C::kRolled ? 1 : D / 32)
-                for (int h = 0; h < D / 32; ++h) {   // E and O columns 16 h .. 16 h + 15 -> outputs 16 h .. and D / 2 + 16 h ..
+                for (int h = C::kOneAcc ? h0 : 0; h < (C::kOneAcc ? h1 : D / 32); ++h) {   // E and O columns 16 h .. 16 h + 15 -> outputs 16 h .. and D / 2 + 16 h ..
                     uint32_t ev[16], ov[16];
                     tmem_ld16(lane_addr + C::acc_col(sc) + (uint32_t)h * 16u, ev);
                     tmem_ld16(lane_addr + C::acc_col(sc) + C::kOCol + (uint32_t)h * 16u, ov);
                     tmem_ld_wait();
-                    if (h == D / 32 - 1) {   // the last values are in registers: hand the accumulator back
+                    if (h == (C::kOneAcc ? h1 : D / 32) - 1) {   // the last values are in registers: hand the accumulator back
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty[j & 1]));
@@ -651,7 +660,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_before();
             fence_proxy_async();
             __syncwarp();
-            if (lane == 0) {
+            if (both) {
+                if (lane == 0) {
+                    if (grp == 0) bulk_wait_read_all();   // the tile before has left the other staging tile: its partner may fill that next
+                    mbar_arrive(smem_u32(&ctrl->meet[q]));
+                }
+                if (!wait_or_abort(smem_u32(&ctrl->meet[q]), (uint32_t)j & 1u, abort_flag, status, KVQ_DEV_SLOT_TIMEOUT)) break;
+            }
+            if (lane == 0 && (!both || grp == 0)) {
                 if constexpr (!R2) mbar_arrive(smem_u32(&ctrl->acc_empty[j & 1]));
                 const int64_t seg = cur.seg;
                 const int row_in_seg = (int)cur.row_in_segment() + q * 32;
