@@ -310,7 +310,7 @@ struct RecipLambda {
         mn = __uint_as_float(__reduce_min_sync(0xFFFFFFFFu, __float_as_uint(mn)));
         rho = __uint_as_float(__float_as_uint(mx) & 0x7F800000u);   // 2^floor(log2 max): exact to divide by
         wide = mn < rho * 0.00390625f;
-        const float inv = 1.0f / rho;
+        const float inv = rho > 0.0f ? 1.0f / rho : 0.0f;   // every entry infinite, or as good as: nothing comes out of such a row
 #pragma unroll
         for (int p = 0; p < kPasses; ++p) r[p].x *= inv, r[p].y *= inv, r[p].z *= inv, r[p].w *= inv;
     }

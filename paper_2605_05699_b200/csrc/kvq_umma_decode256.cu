@@ -101,9 +101,9 @@ typedef RecipLambda<kD, true> Recip;
 template <int TERMS>
 __device__ __forceinline__ void put_b_row(unsigned char *sB, const float4 m0, const float4 m1, const Recip &rl, int p, int n, int lane)
 {
-    auto sat = [](float v) { return fminf(fmaxf(v, -65504.0f), 65504.0f); };
     const float4 r0 = rl.r[0], r1 = rl.r[1];
-    float w[4] = {sat(p ? m0.y * r0.y : m0.x * r0.x), sat(p ? m1.y * r1.y : m1.x * r1.x), sat(p ? m0.w * r0.w : m0.z * r0.z), sat(p ? m1.w * r1.w : m1.z * r1.z)};
+    // entries of the plain transform are at most sqrt(2 / D), the reciprocals below 2: inside fp16's range
+    float w[4] = {p ? m0.y * r0.y : m0.x * r0.x, p ? m1.y * r1.y : m1.x * r1.x, p ? m0.w * r0.w : m0.z * r0.z, p ? m1.w * r1.w : m1.z * r1.z};
     const int ch = lane >> 1;   // 16-byte chunk of the K-major row: K block ch / 8, chunk ch % 8
     unsigned char *dst = sB + p * kBPart + (ch >> 3) * kBBlock + n * 128 + (((ch & 7) ^ (n & 7)) << 4) + (lane & 1) * 8;
 #pragma unroll

@@ -16,7 +16,8 @@
 //   tensor memory   accumulator 1 [128, 2 D] (two stacked terms) | A2, 64 columns per term | accumulator 2: E, O: all 512 columns at D = 128 with bf16
 //   shared memory   B1 (two terms) | B2 | x tiles | output staging
 //
-// B1 and B2 carry lambda and are rebuilt at a new lambda row, B1 by the quantizing warps, B2 by the output warps, when the last MMA that reads the old one is complete.  Tiles do not cross streams: the output is clipped by its tensor map.  Waits, time-outs and wide lambda rows as in the kernels above.
+// B1 and B2 carry lambda and are rebuilt at a new lambda row, B1 by the quantizing warps, B2 by the output warps, when the last MMA that reads the old one is
+// complete.  Tiles do not cross streams: the output is clipped by its tensor map.  Waits, time-outs and wide lambda rows as in the two kernels that this one joins.
 #include "kvq_decode_fp32.cuh"
 #include "kvq_internal.h"
 #include "kvq_quantize.cuh"

@@ -1145,6 +1145,26 @@ def test_one_scale_per_vector_on_the_tensor_cores(D, dtype, N, n_lambda, rpl):
     plan.close()
 
 
+@pytest.mark.parametrize("D,dtype,per_vector", [(64, "f16", False), (128, "f16", True), (128, "bf16", False), (160, "bf16", False), (256, "f16", False), (256, "bf16", True)])
+def test_decode_under_a_lambda_row_without_finite_entries(D, dtype, per_vector):
+    """1 / max(lambda, 1e-6) is zero on every channel: the rows decode to zeros, and the rows under the lambda rows beside it to what they were."""
+    plan = kb.Plan(D, D if per_vector else G, 79)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_AUTO, kb.KVQ_IMPL_GEMM)
+    rpl, n_lambda = 3000, 3
+    gen = torch.Generator().manual_seed(80 + D)
+    packed = torch.randint(0, 256, (rpl * n_lambda, D // 2), generator=gen, dtype=torch.int32).to(torch.uint8)
+    scales = (torch.rand(rpl * n_lambda, D // plan.group, generator=gen) + 0.1).to(torch.float16)
+    lam = wl.make_lambda(n_lambda, D, 81)
+    lam[1] = float("inf")
+    out = gpu_decode_raw(plan, packed.cuda(), scales.cuda(), lam.cuda(), dtype, rpl).float()
+    assert bool((out[rpl:2 * rpl] == 0).all())
+    for i in (0, 2):
+        rows = slice(i * rpl, (i + 1) * rpl)
+        alone = gpu_decode_raw(plan, packed[rows].contiguous().cuda(), scales[rows].contiguous().cuda(), lam[i:i + 1].contiguous().cuda(), dtype)
+        assert torch.equal(out[rows], alone.float())
+    plan.close()
+
+
 @pytest.mark.parametrize("D,dtype,nbits", [(64, "f16", 8), (64, "bf16", 4), (96, "f16", 4), (96, "bf16", 8), (128, "f16", 8), (128, "bf16", 8), (128, "bf16", 4),
                                            (160, "f16", 4), (160, "bf16", 4), (256, "f16", 8), (256, "bf16", 4), (256, "bf16", 8)])
 @pytest.mark.parametrize("N,n_lambda,rpl", [(129, 1, 0), (148 * 128 + 1, 1, 0), (20011, 7, 2900), (21000, 300, 70)])
