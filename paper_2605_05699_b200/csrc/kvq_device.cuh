@@ -325,8 +325,8 @@ struct TilePlan {
         if (rows <= (int64_t)parts) {
             const int64_t k = parts / rows, p = (rt + k - 1) / k;   // shares per lambda row, tiles per share
             if (p <= even + 2 || rows == 1) {
-                const int64_t used = (rt + p - 1) / p;
-                inside = 1, per = (uint32_t)p, shares = (uint32_t)(rows * used), by_per_row = FastDiv(used);
+                const int64_t used = (rt + p - 1) / p, last = tiles - (rows - 1) * rt;   // the last row may have fewer streams
+                inside = 1, per = (uint32_t)p, shares = (uint32_t)((rows - 1) * used + (last + p - 1) / p), by_per_row = FastDiv(used);
                 return;
             }
         }
@@ -365,10 +365,6 @@ struct TileShare {
         if (n == 0) from = 0;
         seg = p.by_tps.small(from);
         tin = from - seg * p.tps;
-    }
-    __host__ TileShare(int64_t n_seg, int64_t rpl, unsigned part, unsigned parts, int tile_rows = 128, int64_t segs = 1)
-        : TileShare(TilePlan(n_seg, rpl, parts, tile_rows, segs), part)
-    {
     }
 };
 

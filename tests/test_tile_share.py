@@ -1,6 +1,6 @@
-"""The split of a call's tiles over the CTAs of a persistent kernel (TileShare), run on the host: every tile belongs to exactly one
-share, shares follow one another, no share is more than two tiles longer than an even split's, and none holds tiles of two lambda rows
-where the rows can have shares of their own within that length."""
+"""The split of a call's tiles over the CTAs of a persistent kernel (TilePlan, TileShare), run on the host: the shares that are launched hold
+every tile once, in order, none is empty, none is more than two tiles longer than an even split's, and none holds tiles of two lambda
+rows where the rows can have shares of their own within that length; shares beyond those launched would hold nothing."""
 import os
 import shutil
 import subprocess
@@ -22,11 +22,16 @@ int main()
         const long tps = (rpl + rows - 1) / rows, tiles = n_seg * tps, even = (tiles + parts - 1) / parts;
         const long row_tiles = (segs < n_seg ? segs : n_seg) * tps, n_rows = (tiles + row_tiles - 1) / row_tiles;
         const bool apart = n_rows <= (long)parts && (n_rows == 1 || (row_tiles + (long)parts / n_rows - 1) / ((long)parts / n_rows) <= even + 2);
+        const kvq::TilePlan plan(n_seg, rpl, parts, rows, segs);
         long at = 0;
-        for (unsigned p = 0; p < parts; ++p) {
-            const kvq::TileShare s(n_seg, rpl, p, parts, rows, segs);
+        for (unsigned p = 0; p < parts || p < plan.shares; ++p) {
+            const kvq::TileShare s(plan, p);
+            if ((s.n > 0) != (p < plan.shares) || plan.shares > parts) {
+                printf("n_seg %ld rpl %ld segs %ld parts %u: %u shares, share %u has %d tiles\n", n_seg, rpl, segs, parts, plan.shares, p, s.n);
+                return 1;
+            }
             if (s.n == 0) continue;
-            if (s.tps != tps || s.begin != at || s.n < 0 || s.n > even + 2) {
+            if (s.tps != tps || s.seg != (unsigned)(at / tps) || s.tin != (unsigned)(at % tps) || s.begin != at || s.n < 0 || s.n > even + 2) {
                 printf("n_seg %ld rpl %ld segs %ld parts %u: share %u begins at %ld (%ld), %d tiles of %ld\n", n_seg, rpl, segs, parts, p,
                        (long)s.begin, at, s.n, even);
                 return 1;
