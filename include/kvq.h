@@ -156,11 +156,11 @@ kvq_status_t kvq_plan_set_impl(kvq_plan_t *plan, kvq_impl_t encode_impl, kvq_imp
 kvq_status_t kvq_plan_prepare(kvq_plan_t *plan, kvq_dtype_t dtype);
 
 /*
- * kvq_plan_set_wait_limit -- how long the tensor-core encode kernel of D <= 160 and the tensor-core append kernel (fp16
- * appends of many streams, every D) let their first wait run.
+ * kvq_plan_set_wait_limit -- how long the tensor-core encode kernel of D <= 160, the tensor-core append kernel (fp16
+ * appends of many streams, every D) and the one-launch block flush (D <= 128) let their first wait run.
  * Every device-side wait in the library is bounded (about 2^22 polls, seconds of wall time) and ends in
  * a status bit instead of a hang.  This knob shortens ONE of them, the wait of the role that issues the
- * tensor-core instructions for the kernel's first operands (built by the encode kernel, copied by the append kernel), a
+ * tensor-core instructions for the kernel's first operands (built by the encode and flush kernels, copied by the append kernel), a
  * point at which that role has nothing in flight: with a limit of a few polls the launch gives up at once, writes nothing,
  * frees what it holds and raises bit 2 of the status word, so that an integration can see KVQ_ERR_TIMEOUT
  * reported and cleared without a fault.

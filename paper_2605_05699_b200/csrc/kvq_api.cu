@@ -345,7 +345,9 @@ kvq_status_t kvq_plan_prepare(kvq_plan_t *plan, kvq_dtype_t dtype)
                                          : umma_decode(plan->D, bf16, plan->bits, 0, g, plan->sign_xor, nullptr, !plan->rot));
     if (gemm_decode_ok(plan, bf16) && !plan->rot && plan->D != 256)   // the form that a rotation set later takes
         also(umma_decode(plan->D, bf16, plan->bits, 0, g, plan->sign_xor, nullptr, false));
-    if (plan->bits == 4 && !per_vector && umma_flush_supported(plan->D)) also(umma_flush(plan->D, bf16, nullptr, 0, g, plan->d_e0, plan->sign_xor, nullptr));
+    if (plan->bits == 4 && !per_vector && umma_flush_supported(plan->D))
+        for (const uint32_t polls : {0u, plan->first_wait_polls})   // a shortened first wait has a form of its own
+            also(umma_flush(plan->D, bf16, nullptr, 0, g, plan->d_e0, plan->sign_xor, polls, nullptr));
     if (umma_calibrate_supported(plan->D, bf16)) also(umma_calibrate(plan->D, bf16, 0, prm, plan->d_e0, nullptr, nullptr));
     also(matvec_encode(plan->D, plan->group, plan->bits, bf16, 0, prm, plan->d_b0, nullptr));
     also(matvec_decode(plan->D, plan->group, plan->bits, bf16, 0, prm, plan->d_e0, nullptr));
@@ -600,18 +602,18 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
         g.view = CacheView{rows, T_max, pos0, streams_per_lambda < 1 ? 1 : streams_per_lambda};
         return g;
     };
-    // Both directions on the tensor cores: one launch where it is built and pays.  (A shortened first wait is the encode kernel's; and a block that lies in the
-    // dequantized cache itself is read to its end before the first row is written.)
+    // Both directions on the tensor cores: one launch where it is built and pays.  (Not for a block that lies in the dequantized cache itself: it
+    // has to be read to its end before the first row is written.)
     const uintptr_t x0 = reinterpret_cast<uintptr_t>(x_block), d0 = reinterpret_cast<uintptr_t>(dq_cache);
     const bool apart = x0 + (uintptr_t)N * plan->D * 2 <= d0 || d0 + (uintptr_t)S * T_max * plan->D * 2 <= x0;
     if (view && apart && N < ((int64_t)1 << 31) && plan->group != plan->D && plan->bits == 4 && !plan->rot && umma_flush_pays(plan->D, bf16, S, rows) &&
-        (plan->enc_impl == KVQ_IMPL_GEMM || (plan->enc_impl == KVQ_IMPL_AUTO && N > matvec_max_rows(plan->D))) && plan->first_wait_polls == 0) {
+        (plan->enc_impl == KVQ_IMPL_GEMM || (plan->enc_impl == KVQ_IMPL_AUTO && N > matvec_max_rows(plan->D)))) {
         if (!x_block || !packed_cache || !scales_cache) return KVQ_ERR_INVALID_ARG;
         kvq_status_t st = check_lambda(N, lambda, n_lambda, rpl);
         if (st != KVQ_OK) return st;
         if (misaligned16(x_block) || misaligned16(packed_cache) || misaligned16(scales_cache)) return KVQ_ERR_ALIGNMENT;
         if ((st = ensure_device(plan)) != KVQ_OK) return st;
-        if (umma_flush(plan->D, bf16, x_block, N, view_params(), plan->d_e0, plan->sign_xor, stream) != cudaSuccess) {
+        if (umma_flush(plan->D, bf16, x_block, N, view_params(), plan->d_e0, plan->sign_xor, plan->first_wait_polls, stream) != cudaSuccess) {
             (void)cudaGetLastError();
             return KVQ_ERR_CUDA;
         }

@@ -40,7 +40,7 @@ struct FftParams {
     RowMap out_map;             // row of packed / scales (encode) or of out (decode) that row r goes to
     RowMap in_map;              // decode: row of packed / scales that row r comes from
     uint32_t *status;           // per-plan device status word
-    uint32_t first_wait_polls;  // tensor-core encode of D <= 160 and append: polls the mma role gives its first operands (0: the default)
+    uint32_t first_wait_polls;  // tensor-core encode of D <= 160, append and block flush: polls the mma role gives its first operands (0: the default)
     int bits;                   // tensor-core encode: 4 or 8 (the register-FFT launchers take it as an argument)
     const unsigned char *operands;   // tensor-core append: the plan's split operands (build_encode_operands), or null: a table outside [kOperandMin, kOperandMax)
     int append;                 // the call is an append: one new row per stream
@@ -99,7 +99,8 @@ cudaError_t umma_decode(int D, bool bf16, int bits, int64_t N, const GemmParams 
 // a block of a cache view (g.view) through both directions in one launch (kvq_umma_flush.cu): groups of 32, 4-bit codes, no rotation
 bool umma_flush_supported(int D);
 bool umma_flush_pays(int D, bool bf16, int64_t S, int64_t rows);
-cudaError_t umma_flush(int D, bool bf16, const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor, cudaStream_t stream);
+cudaError_t umma_flush(int D, bool bf16, const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor,
+                       uint32_t first_wait_polls /* as in FftParams */, cudaStream_t stream);
 cudaError_t umma_calibrate(int D, bool bf16, int64_t N, const FftParams &prm, const float *e0, uint32_t *amax_bits, cudaStream_t stream);
 cudaError_t umma_calibrate_d256(bool bf16, int64_t N, const FftParams &prm, const float *e0, uint32_t *amax_bits, cudaStream_t stream);
 cudaError_t umma_encode_d256(bool bf16, bool per_vector, int64_t N, const FftParams &prm, const float *e0, cudaStream_t stream);   // kvq_umma_encode256.cu

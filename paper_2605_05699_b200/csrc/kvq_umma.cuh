@@ -335,6 +335,18 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
     return false;
 }
 
+// The mma role's wait for a CTA's first B operand where the host has shortened its limit (kvq_plan_set_wait_limit): the one wait that can be
+// shortened, because the waiting thread has issued nothing yet and can leave at once.  The looks at the barrier do not block, so that "one
+// poll" is over before the operand can possibly be there.
+__device__ __forceinline__ bool wait_first_operand(uint32_t bar, volatile uint32_t *abort_flag, uint32_t *status, uint32_t limit)
+{
+    for (uint32_t it = 0; it < limit; ++it)
+        if (mbar_test_wait(bar, 0u)) return true;
+    *abort_flag = 1u;
+    atomicOr(status, (uint32_t)KVQ_DEV_SLOT_TIMEOUT);
+    return false;
+}
+
 // wait_or_abort with cluster-scope acquire: what the partner CTA wrote before its arrival is visible afterwards
 __device__ __forceinline__ bool wait_cluster_or_abort(uint32_t bar, uint32_t parity, volatile uint32_t *abort_flag, uint32_t *status,
                                                       uint32_t reason)

@@ -106,18 +106,6 @@ struct Ctrl {
 };
 static_assert(sizeof(Ctrl) <= kCtrlBytes, "control block too large");
 
-// The mma role's wait for the CTA's first B operand: the one wait whose limit the host may shorten
-// (kvq_plan_set_wait_limit), because the waiting thread has issued nothing yet and can leave at once.  A shortened limit
-// counts looks at the barrier that do not block, so that "one poll" is over before the operand can possibly be there.
-__device__ __forceinline__ bool wait_first_operand(uint32_t bar, volatile uint32_t *abort_flag, uint32_t *status, uint32_t limit)
-{
-    for (uint32_t it = 0; it < limit; ++it)
-        if (mbar_test_wait(bar, 0u)) return true;
-    *abort_flag = 1u;
-    atomicOr(status, (uint32_t)KVQ_DEV_SLOT_TIMEOUT);
-    return false;
-}
-
 // A set's rebuild of B, once the MMAs that read the old one are complete (phase `parity` of barrier `full_bar`).  Kept out of line:
 // rare, and the loop around it stays small.
 template <int D, bool BF16, bool THREE>

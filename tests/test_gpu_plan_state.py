@@ -209,6 +209,45 @@ def test_the_append_kernels_first_wait_is_reported_and_service_returns(D):
     plan.close()
 
 
+@pytest.mark.parametrize("D", [64, 96, 128])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+def test_the_block_flush_kernels_first_wait_is_reported_and_service_returns(D, dtype):
+    """The same limit governs the one-launch block flush's wait for its first operand.  Five tiles per CTA: the loading role has tiles in flight and waits
+    for a free stage, the quantizing and output roles wait for their first accumulators when the issuing role gives up; all of them leave, nothing is
+    written, and the next call gives what the two-launch form gives."""
+    S, rows, T = 5 * 148, 70, 75
+    plan, two = kb.Plan(D, G, 520), kb.Plan(D, G, 520)
+    kb.kvq_plan_set_impl(two.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_GEMM)
+    dt = wl.torch_dtype(dtype)
+    x, lam = wl.make_vectors(S * rows, D, dtype, "gaussian", 521).view(S, rows, D).cuda(), wl.make_lambda(1, D, 522).cuda()
+
+    def caches():
+        return [torch.full((S, T, D // 2), 0xAB, dtype=torch.uint8, device="cuda"), torch.full((S, T, D // G), 1.25, dtype=torch.float16, device="cuda"),
+                torch.full((S, T, D), 3.0, dtype=dt, device="cuda")]
+
+    got = caches()
+    kb.kvq_plan_set_wait_limit(plan.handle, 1)
+    n0 = kb.kvq_launch_count()
+    kb.kvq_flush_block(plan.handle, x, lam, *got, 5)
+    torch.cuda.synchronize()
+    word = kb.kvq_plan_device_status(plan.handle)
+    assert kb.kvq_launch_count() - n0 == 1 and word & 7 == 4, "status word %d" % word
+    assert all(torch.equal(a, b) for a, b in zip(got, caches()))
+    kb.kvq_plan_clear_device_status(plan.handle)
+    kb.kvq_plan_set_wait_limit(plan.handle, 0)
+    kb.kvq_flush_block(plan.handle, x, lam, *got, 5)
+    packed, scales = two.empty_packed(S * rows), two.empty_scales(S * rows)
+    kb.kvq_encode(two.handle, x.view(S * rows, D), lam, packed, scales)
+    out = torch.empty(S * rows, D, dtype=dt, device="cuda")
+    kb.kvq_decode(two.handle, packed, scales, lam, out)
+    torch.cuda.synchronize()
+    assert kb.kvq_plan_device_status(plan.handle) == 0
+    for a, b, untouched in zip(got, (packed, scales, out), caches()):
+        assert torch.equal(a[:, 5:].reshape(S * rows, -1).view(torch.uint8), b.view(torch.uint8)) and torch.equal(a[:, :5], untouched[:, :5])
+    plan.close()
+    two.close()
+
+
 @pytest.mark.parametrize("D,dtype,group,nbits", [(64, "bf16", 32, 4), (96, "f16", 32, 4), (128, "f16", 32, 4), (128, "bf16", 128, 8),
                                                  (160, "bf16", 32, 4), (256, "bf16", 32, 4), (256, "f16", 256, 4), (256, "bf16", 32, 8)])
 def test_a_call_queued_behind_another_sees_all_that_it_wrote(D, dtype, group, nbits):
