@@ -24,7 +24,7 @@ def body(text, head):
 
 def test_decode_rebuild_writes_its_reciprocals_after_both_waits():
     """A dequant group's reciprocals in shared memory are read by its four warps until the tile they built for is handed over, and
-    row 0 of them by the first build's sixteen warps: both waits (the group's own last tile, the tile before this one) stand
+    row 0 of them by the first build's warps: both waits (the group's own last tile, the tile before this one) stand
     before the write, the readers of the new row behind it."""
     b = body(source("kvq_umma_decode.cu"), "bool rebuild_b(")
     waits = [m.start() for m in re.finditer(r"wait_or_abort\(", b)]
@@ -32,19 +32,45 @@ def test_decode_rebuild_writes_its_reciprocals_after_both_waits():
     assert len(waits) == 2 and max(waits) < post < b.index("rows.store") < b.index("rows.rest")
 
 
+def definitions():
+    """(file, name, head, body) of every function of the kernels' sources."""
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"__launch_bounds__\((?:[^()]|\([^()]*\))*\)", "", source(name))
+        for m in re.finditer(r"(__global__|__device__)[^;{}=]*?\b(\w+)\s*\([^;{}]*\)\s*(?:const\s*)?(?::[^;{}]*)?(?=\{)", text):
+            yield name, m.group(2), m.group(0), body(text[m.end():], "")
+
+
 def test_non_coherent_loads_read_the_plans_tables_only():
     """The grid ahead on the stream may still be writing x, lambda, codes, scales and positions when a kernel comes up: they are read
-    by load_input, behind grid_wait, and never by __ldg."""
+    by load_input and never by __ldg."""
     tables = r"(b0|e0|table|brow)\b"
     for name in sorted(os.listdir(CSRC)):
         text = source(name)
         for m in re.finditer(r"__ldg\(", text):
             line = text[m.end():text.index("\n", m.end())]
             assert re.match(r"(reinterpret_cast<const float4 \*>\()?\(?" + tables, line), "%s: __ldg(%s" % (name, line)
-        for kernel in re.finditer(r"__global__ void [^;{]*?(kvq_\w+_kernel)\(", text, re.S):
-            b = body(text, kernel.group(1) + "(")
-            if "load_input" in b:
-                assert 0 <= b.find("grid_wait()") < b.index("load_input"), "%s: %s reads an input before grid_wait" % (name, kernel.group(1))
+
+
+def test_inputs_are_read_behind_the_grid_wait():
+    """In a kernel, and in every function that waits for the grid ahead on a kernel's behalf, nothing that reads an input, itself or through what it calls,
+    stands in front of grid_wait(); but for a call of a function that waits itself."""
+    found = list(definitions())
+    kernels = {n for _, n, head, _ in found if "__global__" in head}
+    waits = {n for _, n, _, b in found if "grid_wait()" in b}
+    readers, grown = {"load_input"}, 0
+    while len(readers) > grown:   # the functions (and the types, by their constructors) that read an input at any depth
+        grown = len(readers)
+        readers |= {n for _, n, _, b in found if re.search(r"\b(%s)\b" % "|".join(readers), b)}
+        for name in sorted(os.listdir(CSRC)):
+            readers |= {m.group(2) for m in re.finditer(r"typedef (\w+)<[^;]*> (\w+);", source(name)) if m.group(1) in readers}
+    assert {"RecipLambda", "Recip", "lift_of", "load_lambda", "load_row_scales", "rebuild_b", "redo_tiles_fp32"} <= readers
+    assert {"first_operand", "build_forward", "build_inverse"} <= waits & readers and len(waits & kernels) >= 10
+    early = readers - waits
+    for name, n, _, b in found:
+        if n in waits or n in kernels & readers:
+            at, first = b.find("grid_wait()"), re.search(r"\b(%s)\b" % "|".join(early), b)
+            assert at >= 0, "%s: %s reads inputs and never waits" % (name, n)
+            assert first is None or first.start() > at, "%s: %s reads an input (%s) before grid_wait" % (name, n, first.group(0))
 
 
 def test_a_warp_is_together_at_the_instructions_that_want_it_so():
