@@ -694,6 +694,12 @@ def test_flush_of_short_blocks_dequantizes_in_fp32(D, dtype):
         assert torch.equal(got[0], got[1]), S
 
 
+def block_flush_launches(D, dtype, S, rows):
+    """One for blocks of so many tiles of 128 rows per SM, two beyond."""
+    limit = {64: 20, 96: 1 << 30, 128: 6 if dtype == "bf16" else 8}[D]
+    return 1 if S * -(-rows // 128) <= limit * torch.cuda.get_device_properties(0).multi_processor_count else 2
+
+
 @pytest.mark.parametrize("D", [64, 96, 128])
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("S,rows,T_max,pos0,spl", [
@@ -703,11 +709,15 @@ def test_flush_of_short_blocks_dequantizes_in_fp32(D, dtype):
     (449, 64, 64, 0, 1),        # a lambda row per stream: both operands rebuilt between any two tiles
     (2, 9500, 9503, 3, 1),      # a tile or two per CTA
     (32, 3000, 3100, 100, 16),  # five tiles per CTA
+    (148, 2400, 2401, 1, 10),   # nineteen tiles per CTA, where another lambda row may begin at any of them; D = 128: two launches
+    (148, 2500, 2500, 0, 148),  # twenty, one lambda row
+    (370, 1000, 1003, 2, 23),   # twenty, of two or three streams, some with the end of one lambda row and the beginning of the next
+    (148, 2561, 2564, 3, 74),   # twenty-one: D = 64 takes two launches too
 ])
-def test_block_flush_in_one_launch_equals_encode_and_decode(D, dtype, S, rows, T_max, pos0, spl):
-    """A large block goes through both contractions in one launch: codes and scales are those of kvq_encode, the dequantized rows those of kvq_decode on them, bit for
-    bit, and nothing beside the block is touched.  One row in 17 is scaled out of the operands' comfort zone; the second lambda row, where there is one, is too
-    wide for the fp16 operand and its tiles are redone in fp32."""
+def test_block_flush_equals_encode_and_decode(D, dtype, S, rows, T_max, pos0, spl):
+    """A block goes through both contractions in one launch, or through an encode and a decode that finds the rows in the caches: codes and scales are those of
+    kvq_encode, the dequantized rows those of kvq_decode on them, bit for bit, and nothing beside the block is touched.  One row in 17 is scaled out of the
+    operands' comfort zone; the second lambda row, where there is one, is too wide for the fp16 operand and its tiles are redone in fp32."""
     tdt = wl.torch_dtype(dtype)
     plan = kb.Plan(D, G, 77)
     n_lambda = (S + spl - 1) // spl
@@ -723,19 +733,64 @@ def test_block_flush_in_one_launch_equals_encode_and_decode(D, dtype, S, rows, T
     n0 = kb.kvq_launch_count()
     kb.kvq_flush_block(plan.handle, x, lam, packed, scales, dq, pos0, spl)
     torch.cuda.synchronize()
-    assert kb.kvq_launch_count() - n0 == 1 and kb.kvq_plan_device_status(plan.handle) == 0
+    assert kb.kvq_launch_count() - n0 == block_flush_launches(D, dtype, S, rows) and kb.kvq_plan_device_status(plan.handle) == 0
+    check_flushed_block(plan, x, lam, packed, scales, dq, pos0, spl)
+    mask = torch.ones(T_max, dtype=torch.bool, device="cuda")
+    mask[pos0:pos0 + rows] = False
+    assert bool((dq[:, mask] == 3.0).all()) and bool((packed[:, mask] == 0xAB).all()) and bool((scales[:, mask] == 1.25).all())
+    plan.close()
+
+
+def check_flushed_block(plan, x, lam, packed, scales, dq, pos0, spl):
+    S, rows, D = x.shape
     kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_GEMM)
     p2, s2 = plan.empty_packed(S * rows), plan.empty_scales(S * rows)
     kb.kvq_encode(plan.handle, x.view(S * rows, D), lam, p2, s2, spl * rows)
-    out = torch.empty(S * rows, D, dtype=tdt, device="cuda")
+    out = torch.empty(S * rows, D, dtype=x.dtype, device="cuda")
     kb.kvq_decode(plan.handle, p2, s2, lam, out, spl * rows)
     torch.cuda.synchronize()
     block = slice(pos0, pos0 + rows)
     assert torch.equal(packed[:, block].reshape(S * rows, -1), p2) and torch.equal(scales[:, block].reshape(S * rows, -1), s2)
     assert torch.equal(dq[:, block].reshape(S * rows, D).view(torch.int16), out.view(torch.int16))
-    mask = torch.ones(T_max, dtype=torch.bool, device="cuda")
-    mask[block] = False
-    assert bool((dq[:, mask] == 3.0).all()) and bool((packed[:, mask] == 0xAB).all()) and bool((scales[:, mask] == 1.25).all())
+
+
+@pytest.mark.parametrize("D,dtype,tiles", [(64, "f16", 20), (64, "bf16", 20), (128, "f16", 8), (128, "bf16", 6)])
+def test_block_flush_on_both_sides_of_the_one_launch_limit(D, dtype, tiles):
+    S = torch.cuda.get_device_properties(0).multi_processor_count
+    for rows, launches in ((128 * tiles, 1), (128 * tiles + 1, 2)):
+        plan = kb.Plan(D, G, 81)
+        lam = wl.make_lambda(3, D, 82).cuda()
+        x = wl.make_vectors(S * rows, D, dtype, "gaussian", 83).view(S, rows, D).cuda()
+        caches = [torch.empty(S, rows + 2, D // 2, dtype=torch.uint8, device="cuda"), torch.empty(S, rows + 2, D // G, dtype=torch.float16, device="cuda"),
+                  torch.empty(S, rows + 2, D, dtype=x.dtype, device="cuda")]
+        n0 = kb.kvq_launch_count()
+        kb.kvq_flush_block(plan.handle, x, lam, *caches, 1, 50)
+        assert kb.kvq_launch_count() - n0 == launches
+        check_flushed_block(plan, x, lam, *caches, 1, 50)
+        assert kb.kvq_plan_device_status(plan.handle) == 0
+        plan.close()
+
+
+@pytest.mark.parametrize("D", [64, 96, 128])
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("at", ["before", "across_the_front", "ahead_of_the_rows", "behind_the_rows", "the_rows", "across_the_end", "after"])
+def test_block_flush_of_rows_that_lie_in_the_dequantized_cache(D, dtype, at):
+    """Vectors that share memory with the cache they are dequantized into are read to their end before a row is written: the call takes two launches, with the result
+    that vectors elsewhere give.  Vectors that end where the cache begins, or begin where it ends, share nothing and take one."""
+    rows, T, pos0 = 2500, 4000, 600
+    offset = {"before": 0, "across_the_front": 1, "ahead_of_the_rows": rows, "behind_the_rows": rows + pos0 + 400, "the_rows": rows + pos0, "across_the_end": rows + T - 1,
+              "after": rows + T}[at]   # of the vectors, in rows of one buffer that holds the cache from row `rows` on
+    plan = kb.Plan(D, G, 85)
+    lam = wl.make_lambda(1, D, 86).cuda()
+    buf = wl.make_vectors(2 * rows + T, D, dtype, "gaussian", 87).cuda()
+    x, dq = buf[offset:offset + rows].unsqueeze(0), buf[rows:rows + T].unsqueeze(0)
+    apart = x.clone()
+    packed, scales = (torch.empty(1, T, n, dtype=t, device="cuda") for n, t in ((D // 2, torch.uint8), (D // G, torch.float16)))
+    n0 = kb.kvq_launch_count()
+    kb.kvq_flush_block(plan.handle, x, lam, packed, scales, dq, pos0, 1)
+    assert kb.kvq_launch_count() - n0 == (1 if at in ("before", "after") else 2)
+    check_flushed_block(plan, apart, lam, packed, scales, dq, pos0, 1)
+    assert kb.kvq_plan_device_status(plan.handle) == 0
     plan.close()
 
 
@@ -1142,6 +1197,32 @@ def test_one_scale_per_vector_on_the_tensor_cores(D, dtype, N, n_lambda, rpl):
     out = gpu_decode(plan, packed, scales, lam.cuda(), dtype, rpl)
     ob, o64 = ko.decode(pk, sb, sg, lam.numpy(), D, odt, rpl, want_f64=True)
     parity.check_decode(bits(out), ob, o64, odt, "per-vector decode")
+    plan.close()
+
+
+@pytest.mark.parametrize("D,dtype,nbits", [(64, "f16", 4), (64, "bf16", 8), (96, "f16", 8), (96, "bf16", 4), (128, "f16", 4), (128, "bf16", 4), (128, "bf16", 8), (160, "f16", 4),
+                                           (160, "bf16", 4), (256, "f16", 4), (256, "bf16", 4), (256, "f16", 8), (256, "bf16", 8)])
+@pytest.mark.parametrize("rpl,n_lambda", [(200, 900), (504, 460), (148 * 1300, 1)])
+def test_decode_of_codes_as_operands_over_many_tiles_equals_small_calls(D, dtype, nbits, rpl, n_lambda):
+    """One scale per vector, eleven tiles and more per CTA: every ring of the pipeline comes round several times, under one lambda row and with rows of two and four tiles,
+    whose operand is built again between tiles in flight.  The same kernel on pieces of one tile per CTA gives the same bits."""
+    N = rpl * n_lambda - 37
+    plan = kb.Plan(D, D, 26, nbits)
+    kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_AUTO, kb.KVQ_IMPL_GEMM)
+    lam = wl.make_lambda(n_lambda, D, 27).cuda()
+    packed, scales = plan.empty_packed(N), plan.empty_scales(N)
+    kb.kvq_encode(plan.handle, wl.make_vectors(N, D, dtype, "lognormal", 28).cuda(), lam, packed, scales, rpl)
+    want = torch.empty(N, D, dtype=wl.torch_dtype(dtype), device="cuda")
+    piece = min(rpl, 128 * 64)
+    for a in range(0, N, piece):
+        b = min(N, a + piece)
+        kb.kvq_decode(plan.handle, packed[a:b], scales[a:b], lam[a // rpl], want[a:b])
+    out = torch.empty_like(want)
+    for _ in range(20):
+        out.zero_()
+        kb.kvq_decode(plan.handle, packed, scales, lam, out, rpl)
+        assert torch.equal(out, want)
+    assert kb.kvq_plan_device_status(plan.handle) == 0
     plan.close()
 
 
