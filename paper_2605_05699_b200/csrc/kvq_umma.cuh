@@ -278,6 +278,14 @@ __device__ __forceinline__ float operand_rescue(const uint32_t (&sc)[(G + 1) / 2
     return __uint_as_float((uint32_t)(127 + 7 - e) << 23);
 }
 
+// sigma rho of a row with one scale per vector, sigma in the low half of `sc`: what its sums of codes are multiplied by.  An infinite sigma gives NaN, the
+// sum that infinite products of both signs and 0 times infinity would have.
+__device__ __forceinline__ float vector_factor(uint32_t sc, float rho)
+{
+    const float sigma = __half2float(__ushort_as_half((unsigned short)(sc & 0xFFFFu)));
+    return fmaf(sigma, rho, sigma - sigma);
+}
+
 // 1 / max(lambda, 1e-6) for the channels this lane covers (4 i .. 4 i + 3, i = lane and, for D > 128, lane + 32; NEIGHBOURS: i = 2 lane and
 // 2 lane + 1), divided by rho, the power of two that brings the row's largest reciprocal into [1, 2).  Every lane gets rho.
 template <int D, bool NEIGHBOURS = false>

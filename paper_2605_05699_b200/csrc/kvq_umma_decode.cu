@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- in fp32; every other row has the factor 1 and costs the epilogue nothing.
             // ---- One scale per vector (PV): the operand is the code itself, and the epilogue multiplies by sigma rho.
             float inv, pw = 1.0f;
-            if constexpr (PV) inv = __half2float(__ushort_as_half((unsigned short)(sc[0] & 0xFFFFu))) * rho;
+            if constexpr (PV) inv = vector_factor(sc[0], rho);
             else pw = operand_rescue<G>(sc, rho, BITS == 4 ? 9000.0f : 500.0f, inv);   // 7 (127) times this stays inside fp16
             ctrl->row_scale[j & (kRowScaleSlots - 1)][r] = inv;
             // ---- nibbles -> fp16 codes -> times sigma * rho, two codes per instruction

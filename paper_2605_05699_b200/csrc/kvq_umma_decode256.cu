@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             // ---- same scales and take the same factor; group 0 posts it.
             // ---- One scale per vector: what the epilogue multiplies the row's sums of codes by.
             float inv, pw = 1.0f;
-            if constexpr (PV) inv = __half2float(__ushort_as_half((unsigned short)(sc[0] & 0xFFFFu))) * rho;
+            if constexpr (PV) inv = vector_factor(sc[0], rho);
             else pw = operand_rescue<kG>(sc, rho, BITS == 4 ? 9000.0f : 500.0f, inv);   // 7 (127) times this stays inside fp16
             if (p == 0) row_scale[(j % C::kScaleSlots) * kTile + r] = inv;
             const uint32_t a_row = tmem_base + ((uint32_t)(q * 32) << 16) + kACol0 + (uint32_t)p * 128u + (uint32_t)sa * 64u;

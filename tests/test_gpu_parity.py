@@ -1200,6 +1200,28 @@ def test_one_scale_per_vector_on_the_tensor_cores(D, dtype, N, n_lambda, rpl):
     plan.close()
 
 
+@pytest.mark.parametrize("D,dtype,nbits", [(64, "bf16", 4), (96, "f16", 4), (128, "f16", 4), (128, "bf16", 8), (160, "bf16", 4), (256, "f16", 8), (256, "bf16", 4)])
+def test_decode_of_a_vector_whose_one_scale_is_not_finite(D, dtype, nbits):
+    """No encode stores such a scale.  A code times infinity and a sum of infinities of both signs are NaN: so is every entry of the row, on the tensor cores
+    (where the scale stands behind the sums of codes) as in the register FFT; the rows around it are what they are without it."""
+    N = 148 * 128 + 300
+    gen = torch.Generator().manual_seed(29)
+    packed = torch.randint(0, 256, (N, D * nbits // 8), generator=gen, dtype=torch.int32).to(torch.uint8).cuda()
+    scales = (torch.rand(N, 1, generator=gen) + 0.1).to(torch.float16).cuda()
+    lam = wl.make_lambda(1, D, 30).cuda()
+    odd = scales.clone()
+    bad = torch.zeros(N, dtype=torch.bool, device="cuda")
+    for start, value in ((5, "inf"), (6, "-inf"), (7, "nan")):
+        odd[start::41] = float(value)
+        bad[start::41] = True
+    for impl in (kb.KVQ_IMPL_GEMM, kb.KVQ_IMPL_FFT):
+        plan = kb.Plan(D, D, 31, bits=nbits)
+        kb.kvq_plan_set_impl(plan.handle, kb.KVQ_IMPL_AUTO, impl)
+        want, out = gpu_decode_raw(plan, packed, scales, lam, dtype), gpu_decode_raw(plan, packed, odd, lam, dtype)
+        assert bool(torch.isnan(out[bad]).all()) and torch.equal(out[~bad], want[~bad]), impl
+        plan.close()
+
+
 @pytest.mark.parametrize("D,dtype,nbits", [(64, "f16", 4), (64, "bf16", 8), (96, "f16", 8), (96, "bf16", 4), (128, "f16", 4), (128, "bf16", 4), (128, "bf16", 8), (160, "f16", 4),
                                            (160, "bf16", 4), (256, "f16", 4), (256, "bf16", 4), (256, "f16", 8), (256, "bf16", 8)])
 @pytest.mark.parametrize("rpl,n_lambda", [(200, 900), (504, 460), (148 * 1300, 1)])
