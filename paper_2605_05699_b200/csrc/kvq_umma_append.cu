@@ -406,15 +406,21 @@ cudaError_t build_encode_operands(int D, const float *e0, unsigned char *out)
     return e != cudaSuccess ? e : cudaStreamSynchronize(nullptr);
 }
 
-// Where it pays: all but the largest calls.  Both kernels' time per call, back to back, 148 CTAs, this one and (those above):
-//   D = 64    one lambda row: 1 tile per CTA 3.5 us (4.7), 3: 5.5 (5.7), 4: 6.4 (6.0); 300 rows: 6: 8.7 (9.9), 10: 13.3 (11.9)
-//   D = 96    one: 1: 3.8 (6.1), 8: 11.4 (11.8), 14: 18.0 (17.8); 52 rows: 10: 15.3 (15.3); 300: 14: 20.4 (22.6), 20: 29.2 (27.6)
-//   D = 128   one: 1: 4.4 (7.1), 4: 8.4 (10.0), 10: 16.5 (18.2), 30: 43.7 (44.0); three: 10: 17.2 (17.3); 300: 20: 35.4 (36.2)
-//   D = 160   one: 1: 6.1 (8.6), 4: 12.4 (12.4), 6: 17.4 (16.5); 52: 10: 26.0 (28.8); 300: 20: 53.5 (53.7)
-//   D = 256   one: 1: 7.4 (11.9), 6: 28.1 (29.9), 8: 37.3 (37.0); 52: 10: 45.8 (49.0); 300: 20: 87.9 (97.9)
-//   one scale per vector: D = 64: 1: 4.0 (5.0), 3: 6.9 (6.2); 96: 3: 7.9 (8.1); 128: 3: 8.3 (9.4), 6: 13.2 (13.3); 160: 3: 11.5 (11.8)
-// So: as many tiles per CTA as make even with one lambda row (beyond, the multiplies cost more than the builds), and for every further
-// lambda row, whose build and short tile the other kernels pay for, some tiles more.  N == 0 (kvq_plan_prepare): whether it is built.
+// Where it pays: up to some tiles of 128 vectors per CTA under one lambda row (beyond, the multiplies by lambda cost more than the encode's one build), a few more
+// under several, and for every further lambda row, whose build and short tile the encode kernels pay for, some tiles more.  Graphs of 20 calls, 148 CTAs, us, this
+// kernel and (the encode); a stream of calls and calls alone change over at the same sizes:
+//                 one lambda row, tiles per CTA                        three                         52                     300 (stream)
+//   D = 64        1: 3.6 (3.75), 2: 4.5 (4.1)                          1: 3.6 (3.7), 2: 4.65 (4.5)   2: 4.6 (4.5)           7: 9.5 (10.3), 8: 10.6 (10.4)
+//   D = 96        7: 10.0 (10.4), 8: 11.0 (11.0), 10: 13.0 (12.8)      8: 11.4 (11.7)                9: 13.4 (13.6)         14: 18.7 (21.3), 20: 29 (27.5)
+//   D = 128       5: 10.0 (10.2), 6: 11.4 (11.2), 10: 16.7 (15.1)      7: 12.8 (12.9), 8: 14.2 (13.8)  10: 16.9 (17.9)      20: 35.4 (35.1)
+//   D = 160       2: 8.0 (8.9), 2.5: 9.9 (9.7), 4: 12.4 (11.5)         4: 12.5 (12.6), 5: 14.4 (14.2)  10: 25.2 (28.5)        14: 40.5 (43.9), 20: 58.8 (57.9)
+//   D = 256       5: 22.0 (23.3), 6: 26.2 (26.2), 7: 31.7 (30.3)       6: 26.1 (27.7)                10: 47.6 (49.2)        20: 101 (107)
+//   one scale per vector:
+//   D = 64        1: 4.3 (4.3), 2: 5.7 (4.9)                           1: 4.15 (4.1)                 2: 5.8 (5.15)          5: 10.2 (10.2)
+//   D = 96        1: 4.7 (5.2), 2: 6.35 (5.9)                          2: 6.5 (7.0), 2.5: 7.9 (7.1)  3: 8.0 (8.8)           9: 17.8 (18.4)
+//   D = 128       4: 9.8 (10.0), 5: 11.4 (11.3)                        6: 13.0 (13.2)                9: 18.4 (18.8)         14: 28.0 (31.2), 20: 40.7 (39.4)
+//   D = 160       2: 8.7 (9.2), 2.5: 10.7 (10.0)                       2: 8.8 (9.7), 2.5: 11.0 (10.0)  5: 15.8 (16.1)       12: 36.7 (37.1)
+// N == 0 (kvq_plan_prepare): whether it is built.
 bool umma_append_pays(int D, bool bf16, bool per_vector, int64_t N, const FftParams &f)
 {
     if (bf16 || (D == 256 && per_vector)) return false;
@@ -428,10 +434,11 @@ bool umma_append_pays(int D, bool bf16, bool per_vector, int64_t N, const FftPar
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
         slots.sms[dev] = n;
     }
-    const int half_tiles = per_vector ? (D == 64 ? 3 : D == 128 ? 10 : 5) : D == 64 ? 5 : D == 96 ? 16 : D == 128 ? 20 : D == 160 ? 8 : 14;
-    const int per_row = (D == 64 ? 2 : D == 96 ? 4 : D == 128 ? 5 : 8) / (per_vector ? 2 : 1);
+    struct Line { int one, several, more; };   // half tiles per CTA under one lambda row, under several; tiles for every further row
+    const Line at = per_vector ? (D == 64 ? Line{2, 2, 1} : D == 96 ? Line{2, 4, 3} : D == 128 ? Line{8, 12, 5} : Line{4, 4, 5})
+                               : (D == 64 ? Line{2, 2, 3} : D == 96 ? Line{14, 16, 4} : D == 128 ? Line{10, 14, 6} : D == 160 ? Line{4, 8, 8} : Line{12, 12, 8});
     const int64_t rows = f.n_lambda == 1 ? 1 : (N + f.rows_per_lambda.d - 1) / f.rows_per_lambda.d;
-    return 2 * ((N + kTile - 1) / kTile) <= (int64_t)half_tiles * slots.sms[dev] + 2 * (int64_t)per_row * (rows - 1);
+    return 2 * ((N + kTile - 1) / kTile) <= (int64_t)(rows == 1 ? at.one : at.several) * slots.sms[dev] + 2 * (int64_t)at.more * (rows - 1);
 }
 
 cudaError_t umma_append(int D, bool per_vector, int64_t N, const FftParams &f, cudaStream_t stream)

@@ -272,12 +272,13 @@ def test_append_at_the_edges_of_its_tiles(D, S, n_lambda, spl):
     run_append(D, S, n_lambda, spl)
 
 
-@pytest.mark.parametrize("D,per_vector,nbits,tiles", [(64, False, 4, 370), (64, True, 4, 222), (96, True, 8, 370), (160, False, 8, 592), (160, True, 4, 370),
-                                                      (256, True, 4, 100)])
-def test_append_on_both_sides_of_its_limit(D, per_vector, nbits, tiles):
-    """The longest call of the append kernel and one vector more, and a layout that it is not built for."""
+@pytest.mark.parametrize("D,per_vector,nbits,n_lambda,tiles", [(64, False, 4, 1, 148), (64, True, 4, 1, 148), (96, True, 8, 1, 148), (160, False, 8, 1, 296), (160, True, 4, 1, 296),
+                                                               (256, True, 4, 1, 100), (64, False, 4, 300, 148 + 3 * 299), (64, True, 8, 300, 148 + 299),
+                                                               (96, True, 4, 300, 296 + 3 * 299), (128, True, 4, 1, 592), (160, True, 4, 100, 296 + 5 * 99)])
+def test_append_on_both_sides_of_its_limit(D, per_vector, nbits, n_lambda, tiles):
+    """The longest call of the append kernel and one vector more, with one lambda row and with many, and a layout that it is not built for."""
     for S in (tiles * 128, tiles * 128 + 1):
-        run_append(D, S, 1, 0, per_vector, nbits)
+        run_append(D, S, n_lambda, -(-S // n_lambda) if n_lambda > 1 else 0, per_vector, nbits)
 
 
 @pytest.mark.parametrize("D,per_vector,nbits", [(64, False, 4), (64, True, 8), (96, True, 4), (128, False, 8), (128, True, 4), (160, False, 4), (256, False, 4), (256, False, 8)])
@@ -343,16 +344,16 @@ def test_append_of_degenerate_rows(D):
         plan.close()
 
 
-@pytest.mark.parametrize("D,per_vector,half_tiles,per_row", [(64, False, 5, 2), (64, True, 3, 1), (96, False, 16, 4), (128, False, 20, 5), (128, True, 10, 2),
-                                                             (160, False, 8, 8), (160, True, 5, 4), (256, False, 14, 8)])
-def test_which_kernel_serves_an_append(D, per_vector, half_tiles, per_row):
+@pytest.mark.parametrize("D,per_vector,one,several,more", [(64, False, 2, 2, 3), (64, True, 2, 2, 1), (96, False, 14, 16, 4), (96, True, 2, 4, 3), (128, False, 10, 14, 6),
+                                                           (128, True, 8, 12, 5), (160, False, 4, 8, 8), (160, True, 4, 4, 5), (256, False, 12, 12, 8)])
+def test_which_kernel_serves_an_append(D, per_vector, one, several, more):
     """On both sides of the append kernel's limit, with one lambda row and with three, whatever the device's number of SMs."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     plan = kb.Plan(D, D if per_vector else G, 6)
     kb.kvq_plan_prepare(plan.handle, torch.float16)
     encode = "kvq_encode_umma_d256_kernel" if D == 256 else "kvq_encode_umma_kernel"
     for rows in (1, 3):
-        most = 128 * ((half_tiles * sms + 2 * per_row * (rows - 1)) // 2)
+        most = 128 * (((one if rows == 1 else several) * sms + 2 * more * (rows - 1)) // 2)
         x, lam = torch.zeros(most + 1, D, dtype=torch.float16, device="cuda"), torch.ones(rows, D, device="cuda")
         packed, scales = plan.empty_packed(most + 1).view(most + 1, 1, -1), plan.empty_scales(most + 1).view(most + 1, 1, -1)
         for S, kernel in ((most, "kvq_append_umma_kernel"), (most + 1, encode)):
