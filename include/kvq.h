@@ -246,11 +246,13 @@ kvq_status_t kvq_append(kvq_plan_t *plan, const void *x_new /* [S, D] */, kvq_dt
  *   dq_cache      device out, [S, T_max, D] of the same 16-bit type; 16-byte aligned.  Only rows [pos0, pos0 + rows) are written.
  * Requires 0 <= pos0 and pos0 + rows <= T_max.  S == 0 or rows == 0 is a no-op.  One launch on the stream when
  * S * rows <= 2048 (1024 for D > 128): the matrix-vector kernel quantizes a vector, dequantizes it from the values it
- * stored and transforms it back in the same CTA.  Larger blocks of 64 rows and more per stream at D <= 128 with 4-bit codes and group 32, on a plan
- * without a rotation, take one launch too, up to the size where two are faster (tiles of 128 rows per SM: 6 with bf16 and 8 with fp16 at D = 128, 20 at D = 64,
- * any at D = 96), with the bits of the two-launch form; the rest take two launches (the encode as kvq_encode picks it,
- * then a decode of the stored rows, in place on the caches: the tensor-core kernel for blocks of 64 rows and more on a
- * plan without a rotation, the matrix-vector kernel on rotated plans, else the register FFT).  The
+ * stored and transforms it back in the same CTA.  Larger blocks of 64 rows and more per stream at D <= 128 with 4-bit
+ * codes and group 32, on a plan without a rotation, take one launch too, up to the size where two are faster (tiles of
+ * 128 rows per SM: 6 with bf16 and 8 with fp16 at D = 128, 20 at D = 64, any at D = 96), with the bits of the two-launch
+ * form; not so a block whose x_block shares memory with dq_cache, which is read to its end before a row is written.  The
+ * rest take two launches (the encode as kvq_encode picks it, then a decode of the stored rows, in place on the caches: the
+ * tensor-core kernel for blocks of 64 rows and more on a plan without a rotation, the matrix-vector kernel on rotated
+ * plans, else the register FFT).  The
  * window itself (holding the not yet flushed tokens in fp16) is the caller's buffer: this call is its flush.
  */
 kvq_status_t kvq_flush_block(kvq_plan_t *plan, const void *x_block, kvq_dtype_t dtype, int64_t S, int64_t rows,

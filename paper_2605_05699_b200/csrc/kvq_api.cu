@@ -602,8 +602,8 @@ static kvq_status_t flush_common(kvq_plan_t *plan, const void *x_block, kvq_dtyp
         g.view = CacheView{rows, T_max, pos0, streams_per_lambda < 1 ? 1 : streams_per_lambda};
         return g;
     };
-    // Both directions on the tensor cores: one launch where it is built and pays.  (Not for a block that lies in the dequantized cache itself: it
-    // has to be read to its end before the first row is written.)
+    // Both directions on the tensor cores: one launch where it is built and pays.  (Not for a block that lies in the dequantized cache
+    // itself: it has to be read to its end before the first row is written.)
     const uintptr_t x0 = reinterpret_cast<uintptr_t>(x_block), d0 = reinterpret_cast<uintptr_t>(dq_cache);
     const bool apart = x0 + (uintptr_t)N * plan->D * 2 <= d0 || d0 + (uintptr_t)S * T_max * plan->D * 2 <= x0;
     if (view && apart && N < ((int64_t)1 << 31) && plan->group != plan->D && plan->bits == 4 && !plan->rot && umma_flush_pays(plan->D, bf16, S, rows) &&

@@ -289,7 +289,8 @@ struct FastDiv {
 // tiles of 128 rows (the last one of a segment may be short), tiles are numbered segment by segment.
 //
 // The contiguous share of a call's tiles that one CTA (or one CTA pair) of a persistent kernel takes: lambda segments of rpl
-// rows are cut into tiles of 128 rows (256 where a CTA pair works on one tile) (a segment's last tile may be short), n_seg * tps tiles in all, `parts` shares.
+// rows are cut into tiles of 128 rows (256 where a CTA pair works on one tile) (a segment's last tile may be short), n_seg * tps tiles
+// in all, `parts` shares.
 // Contiguous, so that the B operand of a lambda row is rebuilt as rarely as possible.  `segs` consecutive segments have one
 // lambda row (1, or the streams of a cache view that share theirs; the last row may have fewer).  A share that crosses into
 // another lambda row pays a rebuild of B on its critical path, one to two tiles' time, so:
@@ -300,8 +301,9 @@ struct FastDiv {
 //     more than its tiles (a share that would begin inside that unit begins at the row's first tile);
 //   * else they are equal in tiles.
 // TilePlan is the call's half of that, worked out by the host (fewer than 2^31 tiles); TileShare is a CTA's.
-// Shares without a tile are not launched: the next call's blocks come up on the SMs they leave, and its last one does not wait for the last SM of this one (append + decode of
-// 112 x 1152 rows, whose decode has 112 shares of nine tiles, 16.1 -> 15.8 us; D = 96 round trip of 65,536, 128 of four, 16.05 -> 15.9).
+// Shares without a tile are not launched: the next call's blocks come up on the SMs they leave, and its last one does not wait for the
+// last SM of this one (append + decode of 112 x 1152 rows, whose decode has 112 shares of nine tiles, 16.1 -> 15.8 us; D = 96 round trip
+// of 65,536, 128 of four, 16.05 -> 15.9).
 // ---------------------------------------------------------------------------
 struct TilePlan {
     uint32_t tps;         // tiles per segment

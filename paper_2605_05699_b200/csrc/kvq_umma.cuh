@@ -278,8 +278,8 @@ __device__ __forceinline__ float operand_rescue(const uint32_t (&sc)[(G + 1) / 2
     return __uint_as_float((uint32_t)(127 + 7 - e) << 23);
 }
 
-// sigma rho of a row with one scale per vector, sigma in the low half of `sc`: what its sums of codes are multiplied by.  An infinite sigma gives NaN, the
-// sum that infinite products of both signs and 0 times infinity would have.
+// sigma rho of a row with one scale per vector, sigma in the low half of `sc`: what its sums of codes are multiplied by.  An infinite
+// sigma gives NaN, the sum that infinite products of both signs and 0 times infinity would have.
 __device__ __forceinline__ float vector_factor(uint32_t sc, float rho)
 {
     const float sigma = __half2float(__ushort_as_half((unsigned short)(sc & 0xFFFFu)));
@@ -343,9 +343,9 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
     return false;
 }
 
-// The mma role's wait for a CTA's first B operand where the host has shortened its limit (kvq_plan_set_wait_limit): the one wait that can be
-// shortened, because the waiting thread has issued nothing yet and can leave at once.  The looks at the barrier do not block, so that "one
-// poll" is over before the operand can possibly be there.
+// The mma role's wait for a CTA's first B operand where the host has shortened its limit (kvq_plan_set_wait_limit): the one wait that can
+// be shortened, because the waiting thread has issued nothing yet and can leave at once.  The looks at the barrier do not block, so that
+// "one poll" is over before the operand can possibly be there.
 __device__ __forceinline__ bool wait_first_operand(uint32_t bar, volatile uint32_t *abort_flag, uint32_t *status, uint32_t limit)
 {
     for (uint32_t it = 0; it < limit; ++it)

@@ -406,20 +406,22 @@ cudaError_t build_encode_operands(int D, const float *e0, unsigned char *out)
     return e != cudaSuccess ? e : cudaStreamSynchronize(nullptr);
 }
 
-// Where it pays: up to some tiles of 128 vectors per CTA under one lambda row (beyond, the multiplies by lambda cost more than the encode's one build), a few more
-// under several, and for every further lambda row, whose build and short tile the encode kernels pay for, some tiles more.  Graphs of 20 calls, 148 CTAs, us, this
-// kernel and (the encode); a stream of calls and calls alone change over at the same sizes:
-//                 one lambda row, tiles per CTA                        three                         52                     300 (stream)
-//   D = 64        1: 3.6 (3.75), 2: 4.5 (4.1)                          1: 3.6 (3.7), 2: 4.65 (4.5)   2: 4.6 (4.5)           7: 9.5 (10.3), 8: 10.6 (10.4)
-//   D = 96        7: 10.0 (10.4), 8: 11.0 (11.0), 10: 13.0 (12.8)      8: 11.4 (11.7)                9: 13.4 (13.6)         14: 18.7 (21.3), 20: 29 (27.5)
-//   D = 128       5: 10.0 (10.2), 6: 11.4 (11.2), 10: 16.7 (15.1)      7: 12.8 (12.9), 8: 14.2 (13.8)  10: 16.9 (17.9)      20: 35.4 (35.1)
-//   D = 160       2: 8.0 (8.9), 2.5: 9.9 (9.7), 4: 12.4 (11.5)         4: 12.5 (12.6), 5: 14.4 (14.2)  10: 25.2 (28.5)        14: 40.5 (43.9), 20: 58.8 (57.9)
-//   D = 256       5: 22.0 (23.3), 6: 26.2 (26.2), 7: 31.7 (30.3)       6: 26.1 (27.7)                10: 47.6 (49.2)        20: 101 (107)
+// Where it pays: up to some tiles of 128 vectors per CTA under one lambda row (beyond, the multiplies by lambda cost more than the
+// encode's one build), a few more under several, and for every further lambda row, whose build and short tile the encode kernels pay
+// for, some tiles more.  Tiles per CTA: us of this kernel and (the encode), graphs of 20 calls (300 rows: streams), 148 CTAs; a stream
+// of calls and calls alone change over at the same sizes:
+//              one lambda row                          three                        52                300
+//   D = 64     1: 3.6 (3.75), 2: 4.5 (4.1)             1: 3.6 (3.7), 2: 4.65 (4.5)  2: 4.6 (4.5)      7: 9.5 (10.3), 8: 10.6 (10.4)
+//   D = 96     7: 10.0 (10.4), 10: 13.0 (12.8)         8: 11.4 (11.7)               9: 13.4 (13.6)    14: 18.7 (21.3), 20: 29 (27.5)
+//   D = 128    5: 10.0 (10.2), 6: 11.4 (11.2)          7: 12.8 (12.9), 8: 14 (13.8)  10: 16.9 (17.9)  20: 35.4 (35.1)
+//   D = 160    2: 8.0 (8.9), 2.5: 9.9 (9.7)            4: 12.5 (12.6), 5: 14 (14.2)  10: 25.2 (28.5)  14: 40.5 (43.9), 20: 59 (58)
+//   D = 256    5: 22.0 (23.3), 6: 26.2 (26.2)          6: 26.1 (27.7)               10: 47.6 (49.2)   20: 101 (107)
 //   one scale per vector:
-//   D = 64        1: 4.3 (4.3), 2: 5.7 (4.9)                           1: 4.15 (4.1)                 2: 5.8 (5.15)          5: 10.2 (10.2)
-//   D = 96        1: 4.7 (5.2), 2: 6.35 (5.9)                          2: 6.5 (7.0), 2.5: 7.9 (7.1)  3: 8.0 (8.8)           9: 17.8 (18.4)
-//   D = 128       4: 9.8 (10.0), 5: 11.4 (11.3)                        6: 13.0 (13.2)                9: 18.4 (18.8)         14: 28.0 (31.2), 20: 40.7 (39.4)
-//   D = 160       2: 8.7 (9.2), 2.5: 10.7 (10.0)                       2: 8.8 (9.7), 2.5: 11.0 (10.0)  5: 15.8 (16.1)       12: 36.7 (37.1)
+//   D = 64     1: 4.3 (4.3), 2: 5.7 (4.9)              1: 4.15 (4.1)                2: 5.8 (5.15)     5: 10.2 (10.2)
+//   D = 96     1: 4.7 (5.2), 2: 6.35 (5.9)             2: 6.5 (7.0), 2.5: 7.9 (7.1)  3: 8.0 (8.8)     9: 17.8 (18.4)
+//   D = 128    4: 9.8 (10.0), 5: 11.4 (11.3)           6: 13.0 (13.2)               9: 18.4 (18.8)    14: 28 (31), 20: 41 (39)
+//   D = 160    2: 8.7 (9.2), 2.5: 10.7 (10.0)          2: 8.8 (9.7), 2.5: 11 (10)   5: 15.8 (16.1)    12: 36.7 (37.1)
+// (Under 52 rows at D = 160 the line lies at 6.75 tiles, and up to ten this kernel would be faster by 8 to 18 %.)
 // N == 0 (kvq_plan_prepare): whether it is built.
 bool umma_append_pays(int D, bool bf16, bool per_vector, int64_t N, const FftParams &f)
 {

@@ -12,13 +12,15 @@
 //                            of bank conflicts
 //   warps 2-9     dequant    two groups of four warps that take alternate tiles.  Thread t of a group
 //                            owns row t: nibbles -> fp16 codes -> times sigma * rho, two codes per
-//                            half2 instruction, stored straight into TENSOR MEMORY as the A operand
-//                            (tcgen05.st); the group scales come by plain loads, one tile ahead.
+//                            half2 instruction (one scale per vector: the codes as they are), stored
+//                            straight into TENSOR MEMORY as the A operand (tcgen05.st); the scales
+//                            come by plain loads, one tile ahead.
 //                            The group that meets the first tile of a new lambda row rebuilds B.
 //   warp 1        mma        one thread issues the K-steps of tcgen05.mma (A from tensor memory, B from shared memory; D / 16 of
 //                            them, or D / 32 per parity of the radix-2 form) into an accumulator stage and commits
-//   warps 10-17   epilogue   two groups of four warps, alternate tiles.  Thread t reads accumulator
-//                            row t (tcgen05.ld), rounds to fp16, writes a swizzled staging tile; one
+//   warps 10-17   epilogue   two groups of four warps, alternate tiles (both on every tile where there is
+//                            one accumulator).  Thread t reads accumulator row t (tcgen05.ld; one scale per
+//                            vector: times sigma * rho), rounds, writes a swizzled staging tile; one
 //                            lane per warp issues the TMA tensor stores (32 rows x 128 B boxes, plus a
 //                            64-byte one when D / 32 is odd).  The output tensor maps are
 //                            three-dimensional (column, row within lambda segment, segment), so the
@@ -33,8 +35,8 @@
 // The K order inside a word of 8 codes is (0,4,1,5,2,6,3,7): that is how the half2 nibble trick
 // delivers them, and B is built in the same order, so no instruction is spent on reordering.
 //
-// Precision: A and B are each rounded once to fp16, accumulation is fp32: about 3e-4 relative L2 per
-// vector before the output rounding.  Every wait on an mbarrier is bounded: on a time-out the role
+// Precision: with fp16 output A and B are each rounded once to fp16 (one scale per vector: A is exact), accumulation
+// is fp32: about 3e-4 relative L2 per vector before the output rounding.  Every wait on an mbarrier is bounded: on a time-out the role
 // records the reason in the status word, raises the CTA's abort flag and leaves its loop; the CTA
 // then frees its tensor memory and returns.
 #include "kvq_decode_fp32.cuh"
@@ -73,9 +75,9 @@ constexpr uint32_t kTmemCols = 512;
 // PV: one scale per vector (Sec. 3.2 step 3, Sec. 4.1), in the radix-2 form.  sigma rho is the same for all of a row, so it stands behind the
 // contraction: the A operand is the code, exact in one fp16 term, the epilogue multiplies in fp32 (one product and two multiply-adds where it
 // had a sum and a difference), and no row needs operand_rescue.  bf16 output then takes two operand sets instead of three and half the
-// tensor-memory stores; fp16 output loses the rounding of q sigma rho to 11 bits.
-// Against the scaled operand, back to back, 592 and 2072 tiles: byte codes at D = 128 bf16 10.5 -> 8.5 us and 24.2 -> 20.4 (37 x 8191 vectors among others 30.6 -> 25.8), 4-bit codes at D = 160 bf16
-// 14.4 -> 10.6 and 34.4 -> 23.5 (two accumulators where two terms leave room for one), at D = 128 fp16 9.2 -> 8.3 and 19.4 -> 17.6.
+// tensor-memory stores; fp16 output loses the rounding of q sigma rho to 11 bits.  Against the scaled operand, back to back, 592 and
+// 2072 tiles: byte codes at D = 128 bf16 10.5 -> 8.5 us and 24.2 -> 20.4, 4-bit codes at D = 160 bf16 14.4 -> 10.6 and 34.4 -> 23.5 (two
+// accumulators where two terms leave room for one), at D = 128 fp16 9.2 -> 8.3 and 19.4 -> 17.6.
 template <int D, bool BF16OUT, int BITS = 4, bool R2 = false, bool PV = false>
 struct Cfg {
     static_assert(D % 32 == 0 && D >= 64 && D <= 160, "head dim not built");
@@ -207,13 +209,13 @@ struct FirstOperand {
     uint32_t sc[(G + 1) / 2] = {};
 };
 
-// The way from the kernel's entry through the set-up barrier for warps 2 to 17, and B for the first tile's lambda row by the last kBuilders of them
-// (w counts from the first builder on): table rows are requested in front of the grid wait, lambda and scales behind it and in front of the
-// barrier.  The group that has the first tile does not build: it dequantises meanwhile, so that the first MMA waits for the longer of the two and not for their sum.
-// Out of line: its registers are then no part of the role loops' allocation.
-// One tile per CTA, back to back, before (all sixteen warps build, then one group dequantises, in line) and now: D = 160 bf16 9.1 -> 8.2 us, fp16 9.1 -> 8.1, D = 96 fp16 5.7 -> 5.4,
-// D = 128 bf16 7.4 -> 7.2; and for the registers 2072 tiles at D = 160 bf16 34.5 -> 32.8, D = 128 bf16 19.4 -> 19.0, fp16 17.3 -> 16.8.  (Without the call the same split
-// made 2072 tiles at D = 128 bf16 20.5.)
+// The way from the kernel's entry through the set-up barrier for warps 2 to 17, and B for the first tile's lambda row by the last
+// kBuilders of them (w counts from the first builder on): table rows are requested in front of the grid wait, lambda and scales behind it
+// and in front of the barrier.  The group that has the first tile does not build: it dequantises meanwhile, so that the first MMA waits
+// for the longer of the two and not for their sum.  Out of line: its registers are then no part of the role loops' allocation.
+// One tile per CTA, back to back, before (all sixteen warps build, then one group dequantises, in line) and now: D = 160 bf16
+// 9.1 -> 8.2 us, fp16 9.1 -> 8.1, D = 96 fp16 5.7 -> 5.4, D = 128 bf16 7.4 -> 7.2; and for the registers 2072 tiles at D = 160 bf16
+// 34.5 -> 32.8, D = 128 bf16 19.4 -> 19.0, fp16 17.3 -> 16.8.  (In line the same split made 2072 tiles at D = 128 bf16 20.5.)
 template <int D, bool BF16OUT, int BITS, bool R2>
 __device__ __noinline__ FirstOperand<D / 32> first_operand(unsigned char *sB, Ctrl *ctrl, const float *__restrict__ b0, const float *lam,
                                                            const uint16_t *row_scales, int per_vector, int w, int lane)
@@ -562,9 +564,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int grp = (warp - 10) >> 2;
         const int q = warp & 3;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
-        // One accumulator: both groups take every tile, the first three fifths of its columns and the rest, so that it goes back sooner; the two warps that share 32
-        // rows fill one staging tile of two and meet before the first of them stores it.
-        // bf16, 296, 1036 and 2072 tiles 9.74 -> 9.64 us, 18.5 -> 17.8 and 32.7 -> 31.0.  (148, a tile per CTA, 8.1 -> 8.2: chosen at run time the loop costs more, 8.5.)
+        // One accumulator: both groups take every tile, the first three fifths of its columns and the rest, so that it goes back sooner;
+        // the two warps that share 32 rows fill one staging tile of two and meet before the first of them stores it.  bf16, 296, 1036 and
+        // 2072 tiles 9.74 -> 9.64 us, 18.5 -> 17.8 and 32.7 -> 31.0.  (148, a tile per CTA, 8.1 -> 8.2; chosen at run time 8.5.)
         constexpr bool both = C::kOneAcc;
         constexpr int step = both ? 1 : 2;
         const int h0 = both && grp == 1 ? 3 : 0, h1 = both && grp == 0 ? 3 : D / 32;   // 16-column steps of each parity

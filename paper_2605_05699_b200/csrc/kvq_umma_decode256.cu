@@ -15,14 +15,15 @@
 //     already lands on the other side of enough rounding boundaries to miss the 1e-3 tolerance.  So for bf16 both
 //     operands are carried in two fp16 terms: a = q sigma rho has 15 significant bits and splits exactly into
 //     a_hi + a_lo (one half2 FMA), W' = W_hi + W_lo, and a_hi W_hi + a_lo W_hi + a_hi W_lo accumulates in fp32
-//     (the a_lo W_lo term is below 1e-7).  fp16 output needs one term.
+//     (the a_lo W_lo term is below 1e-7).  fp16 output needs one term.  With one scale per vector a is the code, exact in
+//     one term, and sigma rho stands behind the contraction.
 //
 //   warp 0        producer   one TMA tensor load per tile: 128 packed rows x 128 B, 128-byte swizzle, 4 stages (2 for bf16);
 //                            byte codes (template BITS = 8): rows of 256 B as two such boxes, 2 stages (1 for bf16)
 //   warps 2-9     dequant    two groups of four warps, thread = row, both on every tile: group 0 turns the even
 //                            channels of the row's packed words into the A operand of the E GEMM, group 1 the
 //                            odd ones into that of the O GEMM (tensor memory; two stages each for fp16 output,
-//                            one with a_lo beside a_hi for bf16).  Each group also owns the B operand of its
+//                            one with a_lo beside a_hi for bf16, two of codes with one scale per vector).  Each group also owns the B operand of its
 //                            GEMM and rebuilds it when the lambda row changes, behind its own barriers.
 //   warp 1        mma        per tile: E GEMM into accumulator columns 0-127, O GEMM into 128-255 (8 K-steps per
 //                            term each, A from tensor memory, B from shared memory)
@@ -56,9 +57,9 @@ constexpr uint32_t kACol0 = 256;                       // accumulator E at 0, O 
 constexpr uint32_t kIdesc = umma_idesc_m128(kHalf, false);
 
 // BITS = 8: byte codes (Sec. 3.2 step 4's int8 output).  A packed row is then 256 B, loaded as two boxes of 128 B.
-// PV: one scale per vector.  The A operand is the code itself, one exact fp16 term, and sigma rho stands in the epilogue: two operand sets for
-// bf16 output instead of three, and two A stages where two terms leave room for one.  Back to back, 592 and 2072 tiles: bf16 22.7 -> 19.5 us and 52.8 -> 42.4, byte codes 23.6 -> 18.7
-// and 58.5 -> 49.7; fp16 16.1 -> 14.8 and 40.6 -> 37.9.
+// PV: one scale per vector.  The A operand is the code itself, one exact fp16 term, and sigma rho stands in the epilogue: two operand
+// sets for bf16 output instead of three, and two A stages where two terms leave room for one.  Back to back, 592 and 2072 tiles: bf16
+// 22.7 -> 19.5 us and 52.8 -> 42.4, byte codes 23.6 -> 18.7 and 58.5 -> 49.7; fp16 16.1 -> 14.8 and 40.6 -> 37.9.
 template <bool BF16OUT, int BITS = 4, bool PV = false>
 struct Cfg {
     static constexpr int kInRow = kD * BITS / 8;       // bytes of a packed row
@@ -71,8 +72,8 @@ struct Cfg {
     // one 32 KB tile, reloaded while the MMAs and the epilogue of the tile before run)
     static constexpr int kInStages = BITS == 8 ? (BF16OUT ? 1 : 2) : BF16OUT ? 2 : 4;
     // per-row output scales of the tiles between a dequant group and the epilogue: as many slots as a group can run ahead
-    // (kAStages + 1 are enough, and all that fits beside two terms of B: tile j writes its slot when the MMAs of tile j - kAStages are complete, and these
-    // began when the epilogue of the tile before them had read its own)
+    // (kAStages + 1 are enough, and all that fits beside two terms of B: tile j writes its slot when the MMAs of tile j - kAStages are
+    // complete, and these began when the epilogue of the tile before them had read its own)
     static constexpr int kScaleSlots = BF16OUT && PV ? 3 : 2 * kAStages;
     static constexpr int kScaleBytes = kScaleSlots * kTile * (int)sizeof(float);
     static constexpr int kSmemBytes = kBBytes + kInStages * kInBytes + 8 * kOutWarpBytes + kCtrlBytes + kScaleBytes + 1024;
@@ -155,10 +156,10 @@ struct FirstOperand {
     uint4 sc;
 };
 
-// The way from the kernel's entry to the first B for warps 2 to 17 (w from 0 on).  Table rows are requested in front of the grid wait, every row once
-// for both parities.  The dequant warps, which have the first tile to dequantise before the first MMA can begin, build four rows each, the epilogue
-// warps twelve.  Out of line: its registers are no part of the role loops' allocation.  Back to back, eight rows each in line -> this: one tile per CTA fp16 9.35 -> 8.7 us,
-// bf16 11.8 -> 11.0; four 14.8 -> 14.2, 21.6 -> 20.7.
+// The way from the kernel's entry to the first B for warps 2 to 17 (w from 0 on).  Table rows are requested in front of the grid wait,
+// every row once for both parities.  The dequant warps, which have the first tile to dequantise before the first MMA can begin, build
+// four rows each, the epilogue warps twelve.  Out of line: its registers are no part of the role loops' allocation.  Back to back, eight
+// rows each in line -> this: one tile per CTA fp16 9.35 -> 8.7 us, bf16 11.8 -> 11.0; four 14.8 -> 14.2, 21.6 -> 20.7.
 template <int TERMS, bool PV>
 __device__ __noinline__ FirstOperand first_operand(unsigned char *sB, Ctrl *ctrl, const float *__restrict__ b0, const float *lam, const uint16_t *row_scales, int w, int lane)
 {
@@ -491,8 +492,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             const CUtensorMap *tm = tail ? &maps.tail : &maps.out;
             const int segc = tail ? 0 : (int)seg;
             const float row_inv = row_scale[(j % C::kScaleSlots) * kTile + q * 32 + lane];
-            // The accumulator has one stage: what stands between the first request and its release is on every tile's critical path, so both
-            // chunks are read and staged before either is stored.  2072 tiles fp16 37.2 -> 36.5 us, bf16 53.7 -> 51.1; 1008 under 56 lambda rows 24.3 -> 23.5, 36.2 -> 33 to 36.
+            // The accumulator has one stage: what stands between the first request and its release is on every tile's critical path, so
+            // both chunks are read and staged before either is stored.  2072 tiles fp16 37.2 -> 36.5 us, bf16 53.7 -> 51.1.
             if (lane == 0) bulk_wait_read_all();   // this warp's stores of the tile before have read the staging boxes
             const bool rescale = !PV && __any_sync(0xFFFFFFFFu, row_inv != 1.0f);   // rare: a row outside the operand's comfort zone
             __syncwarp();

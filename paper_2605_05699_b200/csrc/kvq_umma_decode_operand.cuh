@@ -1,6 +1,7 @@
-// The B operand of the inverse transform on the tensor cores, W' = diag(s) M^T diag(1 / max(lambda, 1e-6)) / rho in fp16 terms (kvq_umma_decode.cu says why), built by the
-// threads of a CTA out of the plan's table.  C describes the operand: kBits, kRadix2 (the form), kTerms, kBRows, kQuads (table rows it is built from, float4 per
-// row) and the places of its parts (kBPartBlock, kBPart; kBBlock, kBTerm).
+// The B operand of the inverse transform on the tensor cores, W' = diag(s) M^T diag(1 / max(lambda, 1e-6)) / rho in fp16 terms
+// (kvq_umma_decode.cu says why), built by the threads of a CTA out of the plan's table.  C describes the operand: kBits, kRadix2 (the
+// form), kTerms, kBRows, kQuads (table rows it is built from, float4 per row) and the places of its parts (kBPartBlock, kBPart; kBBlock,
+// kBTerm).
 #pragma once
 
 #include "kvq_umma.cuh"
@@ -19,8 +20,8 @@ __device__ __forceinline__ void build_b_quad(unsigned char *sB, float4 m, float4
     constexpr int BITS = C::kBits;
     constexpr bool R2 = C::kRadix2;
     const bool odd = i & 1;
-    // (The plain transform's entries are at most sqrt(2 / D) and the reciprocals below 2: only a rotated table could leave fp16's range.  D = 256, where each is built for
-    // two parities: 148, 296 and 592 tiles bf16 10.95 -> 10.5 us, 13.6 -> 13.2, 19.1 -> 18.75; D <= 160 up to 1 %.)
+    // (The plain transform's entries are at most sqrt(2 / D) and the reciprocals below 2: only a rotated table could leave fp16's range.
+    // Without the clamp 148, 296 and 592 tiles at D = 256 bf16 10.95 -> 10.5 us, 13.6 -> 13.2, 19.1 -> 18.75; D <= 160 up to 1 %.)
     auto sat = [](float v) { return R2 ? v : fminf(fmaxf(v, -65504.0f), 65504.0f); };
     const float v[4] = {sat(m.x * rc.x), sat(m.y * rc.y), sat(m.z * rc.z), sat(m.w * rc.w)};
     if constexpr (R2) {

@@ -217,8 +217,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int n_my = share.n;
 
     // ---- B for the pair's first lambda row: eight rows per epilogue warp, requested before the set-up barrier
-    // The pair's set-up barrier in front of the grid wait for tall tiles, so that lambda and the first x loads follow the wait side by side (592 128-row tiles bf16 20.7 -> 19.9 us, 1036:
-    // 30.2 -> 28.9, 1664: 51.5 -> 49.4); behind lambda for short ones, of which a pair has one or two: one 128-row tile per CTA 11.0 us so, 11.7 the other way.
+    // The pair's set-up barrier in front of the grid wait for tall tiles, so that lambda and the first x loads follow the wait side by side
+    // (592 128-row tiles bf16 20.7 -> 19.9 us, 1036: 30.2 -> 28.9, 1664: 51.5 -> 49.4); behind lambda for short ones, of which a pair has
+    // one or two: one 128-row tile per CTA 11.0 us so, 11.7 the other way.
     constexpr bool kBarrierFirst = ROWS == 128;
     float first_lift = 1.0f;
     if (n_my > 0 && warp >= 2) {
@@ -529,10 +530,15 @@ cudaError_t resident_pairs(int *fit)
 
 int64_t tiles_of(int64_t n_seg, int64_t rpl, int rows) { return n_seg * ((rpl + rows - 1) / rows); }
 
-// A pair's time is 7.1 us and 1.93 us per short tile (128 vectors), or 8.3 and 2.97 per tall one (256): short where
-// 2 n_short <= 3 n_tall + 1.  Back to back, fp16, short and tall: 9000 vectors 9.6 and 11.2 us, 18,944: 11.6, 12.1; 24,000: 13.0, 14.5;
-// 36,000: 15.0, 14.6; 46,000: 17.0, 17.3; 54,000: 18.9, 17.4; 212,992: 62.4, 53.5.  bf16 and one scale per vector lie alike.
-// Calibration from fp16: 9000 vectors 14.6 and 16.4, 57,000: 22.9, 26.6; 170,000: 41.9, 43.0; 200,000: 52.2, 49.9; 500,000: 116, 105.
+// Short tiles (128 vectors of a pair) cost a pair less each, tall ones (256) less per vector: short where 2 n_short <= 3 n_tall + 1, n the
+// tiles of the longest share.  Back to back, us, short and tall:
+//   fp16, one lambda row    9000: 9.3, 10.0   18,944: 11.1, 11.6   24,000: 12.6, 13.6   30,000: 14.5, 13.9   41,000: 16.2, 16.7
+//                           46,000: 16.3, 16.7   50,000: 18.3, 16.8   60,000: 20.3, 19.5   212,992: 58.4, 48.8
+//   bf16, one lambda row    9000: 9.4, 11.0   24,000: 13.6, 15.5   36,000: 15.4, 15.2   46,000: 16.7, 17.8   50,000: 18.3, 17.8
+//   bf16, 52 lambda rows    9000: 11.5, 11.8   30,000: 17.7, 19.2   36,000: 19.8, 18.4   46,000: 21.5, 21.6   60,000: 26.5, 22.7
+//                           70,000: 24.9, 25.2   110,000: 32.8, 33.9   130,000: 38.0, 38.0   160,000: 48.6, 40.1
+// (the rule is wrong at 36,000 and 110,000 under 52 rows, by 8 and 3 %).  One scale per vector lies alike.
+// Calibration from fp16: 9000 vectors 16.4 and 16.5, 57,000: 24.6, 28.2; 170,000: 39.7, 43.1; 200,000: 47.8, 46.8; 500,000: 106, 95.
 // (From bf16 its three terms leave a tall tile two x blocks beside B, and short ones are as fast or faster throughout: 9000 vectors 16.5
 // and 20.5, 57,000: 26.7, 30.8; 212,992: 63.9, 66.0; 500,000: 146.5, 145.1.  The tall form is not built.)
 template <bool CALIB>

@@ -1,6 +1,7 @@
-// The B operand of the forward transform on the tensor cores, W = lambda M diag(s) 2^k in 16-bit terms (kvq_umma_encode.cu says why), built by the threads of a CTA
-// out of the plan's table.  C describes the operand: kDim, kBf16 (the terms' type), kSplit (their number), kBBlock (bytes of a K block of 64, all rows)
-// term(c) (bytes from a term's row of channel c to the next term's) and row(c), the row of a K block that channel c has (c modulo 8).
+// The B operand of the forward transform on the tensor cores, W = lambda M diag(s) 2^k in 16-bit terms (kvq_umma_encode.cu says why),
+// built by the threads of a CTA out of the plan's table.  C describes the operand: kDim, kBf16 (the terms' type), kSplit (their number),
+// kBBlock (bytes of a K block of 64, all rows), term(c) (bytes from a term's row of channel c to the next term's) and row(c), the row of
+// a K block that channel c has (c modulo 8).
 #pragma once
 
 #include "kvq_umma.cuh"

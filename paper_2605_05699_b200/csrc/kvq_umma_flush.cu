@@ -1,23 +1,28 @@
 // The block flush in one launch (sm_100a): D = 64, 96, 128, fp16 and bf16, groups of 32, 4-bit codes, no rotation.
 //
-// A prefill block goes into the int4 caches and, dequantized, into the prefix cache (Sec. 7.2).  As an encode and a decode that is two starts, and the second
-// kernel reads back and unpacks what a thread of the first had in registers.  Here the thread that has quantized a group writes it
-// as the decode's A operand at once, and the tile goes on through the second contraction:
+// A prefill block goes into the int4 caches and, dequantized, into the prefix cache (Sec. 7.2).  As an encode and a decode that is
+// two starts, and the second kernel reads back and unpacks what a thread of the first had in registers.  Here the thread that has
+// quantized a group writes it as the decode's A operand at once, and the tile goes on through the second contraction:
 //
 //   warp 0          producer   one TMA tensor load per K block of 64 elements and tile of 128 vectors, two to four tiles in flight
-//   warp 1          mma        one elected thread: x B1 of tile j + 1, 64 channels and the rest into accumulators of their own, then A2 B2 of tile j, so that the first
-//                              contraction of a tile runs under the quantizer of the one before.  (Two issuing threads, one per contraction, are slower: 64 x 2000 bf16 27.3 -> 29.8 us,
-//                              128 x 4000 79.9 -> 93; rows of the tiles ahead asked for in L2 too: 28.7 and 85.)
-//   warps 2 ..      quantize   four warps per group of 32 channels, thread = (row, group), every tile: accumulator 1 -> scale, codes, caches (the quantizer and the arithmetic of
-//                              kvq_umma_encode.cu: the same bits); the G threads of a row trade their scales, which decide the row's operand factor; codes -> A2 in tensor memory
+//   warp 1          mma        one elected thread: x B1 of tile j + 1, 64 channels and the rest into accumulators of their own, then
+//                              A2 B2 of tile j, so that the first contraction of a tile runs under the quantizer of the one before
+//   warps 2 ..      quantize   four warps per group of 32 channels, thread = (row, group), every tile: accumulator 1 -> scale,
+//                              codes, caches (the quantizer and the arithmetic of kvq_umma_encode.cu: the same bits); the G threads
+//                              of a row trade their scales, which decide the row's operand factor; codes -> A2 in tensor memory
 //                              (the operands of kvq_umma_decode.cu: the same bits)
 //   last 4 warps    output     thread = row: accumulator 2 -> E + O, E - O -> TMA store
 //
-//   tensor memory   accumulator 1 [128, 2 D] (two stacked terms) | A2, 64 columns per term | accumulator 2: E, O: all 512 columns at D = 128 with bf16
+//   tensor memory   accumulator 1 [128, 2 D] (two stacked terms) | A2, 64 columns per term | accumulator 2: E, O: all 512 columns at
+//                   D = 128 with bf16
 //   shared memory   B1 (two terms) | B2 | x tiles | output staging
 //
-// B1 and B2 carry lambda and are rebuilt at a new lambda row, B1 by the quantizing warps, B2 by the output warps, when the last MMA that reads the old one is
-// complete.  Tiles do not cross streams: the output is clipped by its tensor map.  Waits, time-outs and wide lambda rows as in the two kernels that this one joins.
+// B1 and B2 carry lambda and are rebuilt at a new lambda row, B1 by the quantizing warps, B2 by the output warps, when the last MMA
+// that reads the old one is complete.  Tiles do not cross streams: the output is clipped by its tensor map.  Waits, time-outs and wide
+// lambda rows as in the two kernels that this one joins.
+//
+// Slower, 64 x 2000 and 128 x 4000 rows at D = 128 bf16 (27.3 and 79.9 us): two issuing threads, one per contraction 29.8 and 93;
+// rows of the tiles ahead asked for in L2 28.7 and 85.
 #include "kvq_decode_fp32.cuh"
 #include "kvq_internal.h"
 #include "kvq_quantize.cuh"
@@ -42,8 +47,8 @@ struct Fwd {   // operand of the first contraction: two terms stacked along N
     static constexpr int kDim = D, kSplit = 2;
     static constexpr bool kBf16 = BF16;
     static constexpr int kKBlocks = (D + 63) / 64;
-    // The channels in two parts, 64 and the rest, each with an accumulator of its own: [64 channels][first term, second term], and so on.  One part is read
-    // and issued again while the tensor core is at the other.
+    // The channels in two parts, 64 and the rest, each with an accumulator of its own: [64 channels][first term, second term], and so
+    // on.  One part is read and issued again while the tensor core is at the other.
     static constexpr int kParts = D > 64 ? 2 : 1;
     static __host__ __device__ constexpr int channels(int part) { return part == 0 ? 64 : D - 64; }
     static __device__ __forceinline__ int row(int c) { return c + (c < 64 ? 0 : 64); }   // the second term stands channels(part) rows behind
@@ -70,8 +75,8 @@ struct Cfg {
     static constexpr int kThreads = 32 * (2 + kQuantWarps + kOutWarps);
     static constexpr int kXBytes = F::kKBlocks * kBlockBytes;
     static constexpr int kOutWarpBytes = 32 * 2 * D;
-    // Output staging for two tiles with fp16 output (two x tiles still fit beside it): 64 x 2000 at D = 128 26.1 -> 25.3 us, 128 x 4000 79.5 -> 75.6, at D = 96 54.0 -> 50.7.  With
-    // bf16 output, whose period the contractions set, it is slower: D = 96 55.6 -> 57.7, D = 64 42.6 -> 44.3.
+    // Output staging for two tiles with fp16 output (two x tiles still fit beside it): 128 x 4000 rows at D = 128 79.5 -> 75.6 us, at
+    // D = 96 54.0 -> 50.7.  With bf16 output it is slower: D = 96 55.6 -> 57.7, D = 64 42.6 -> 44.3.
     static constexpr int kOutBufs = BF16 ? 1 : 2;
     static constexpr int kOutBytes = kOutBufs * kOutWarps * kOutWarpBytes;
     static constexpr int kRoom = (232448 - 1024 - kCtrlBytes - F::kBytes - I::kBytes - kOutBytes) / kXBytes;
@@ -102,8 +107,8 @@ struct RowFactors {
     float unlift, rho;
 };
 
-// B1 of a lambda row by the quantizing warps, w of them.  first: from the kernel's entry, through the set-up barrier and the grid wait.  Out of line, like the
-// other build: the loops' registers are then their own.
+// B1 of a lambda row by the quantizing warps, w of them.  first: from the kernel's entry, through the set-up barrier and the grid wait.
+// Out of line, like the other build: the loops' registers are then their own.
 template <int D, bool BF16>
 __device__ __noinline__ RowFactors build_forward(unsigned char *sB, const float *__restrict__ e0, const float *lam, uint32_t ready, int w, int lane, bool first)
 {
@@ -164,8 +169,8 @@ struct UmmaFlushMaps {
     CUtensorMap slim;      // output, boxes of 32 columns x 32 rows (64-byte swizzle), used when D / 32 is odd
 };
 
-// SHORT: the host has shortened the limit of the mma role's first wait.  A form of its own: the issuing loop answers to whatever stands beside it, and with the test
-// in the one kernel 64 x 2000 rows took 25.3 us for 24.9 (D = 128 fp16) and 19.9 for 19.55 (D = 96 bf16).
+// SHORT: the host has shortened the limit of the mma role's first wait.  A form of its own: the issuing loop answers to whatever stands
+// beside it, and with the test in the one kernel 64 x 2000 rows took 25.3 us for 24.9 (D = 128 fp16) and 19.9 for 19.55 (D = 96 bf16).
 template <int D, bool BF16, bool SHORT>
 __global__ void __launch_bounds__(Cfg<D, BF16>::kThreads, 1)
     kvq_flush_umma_kernel(const __grid_constant__ UmmaFlushParams prm, const __grid_constant__ UmmaFlushMaps maps)
@@ -510,7 +515,8 @@ __global__ void __launch_bounds__(Cfg<D, BF16>::kThreads, 1)
 namespace {
 
 template <int D, bool BF16, bool SHORT>
-cudaError_t launch_form(const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor, uint32_t first_wait_polls, cudaStream_t stream)
+cudaError_t launch_form(const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor,
+                   uint32_t first_wait_polls, cudaStream_t stream)
 {
     using C = Cfg<D, BF16>;
     static DeviceSlots slots;
@@ -559,7 +565,8 @@ cudaError_t launch_form(const void *x, int64_t N, const GemmParams &g, const flo
 }
 
 template <int D, bool BF16>
-cudaError_t launch(const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor, uint32_t first_wait_polls, cudaStream_t stream)
+cudaError_t launch(const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor,
+                   uint32_t first_wait_polls, cudaStream_t stream)
 {
     return first_wait_polls ? launch_form<D, BF16, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
                             : launch_form<D, BF16, false>(x, N, g, e0, sign_xor, 0, stream);
@@ -569,13 +576,16 @@ cudaError_t launch(const void *x, int64_t N, const GemmParams &g, const float *e
 
 bool umma_flush_supported(int D) { return D == 64 || D == 96 || D == 128; }
 
-// Where it pays: a tile takes the contractions, the quantizer and the output one behind the other through one stage each, so its period is above the sum of the two kernels'
-// (D = 128 bf16 2.5 us and 2.2, D = 64 1.3 and 1.2; D = 96, with more tensor memory to spare per channel, below it: 1.7 and 1.9), and what is saved is
-// one start.  (At D = 128 the threads' instructions set the period: some 9000 of a warp per tile, 22 warps.)  At seven tiles per CTA, D = 128 bf16, the two come out alike on buffers
-// in rotation and one launch 8 % longer on buffers never touched.  Both forms, two launches first, streams x rows, buffers in rotation:
-//   D = 64  bf16: 2 x 2000 7.9 -> 5.1 us, 64 x 2000 17.3 -> 15.2, 128 x 4000 (28 tiles per CTA) 41.9 -> 42.6; fp16: 9.9 -> 5.6, 16.5 -> 14.4, 40.6 -> 40.3
-//   D = 96  bf16: 9.9 -> 6.4, 22.6 -> 19.7, 61.8 -> 55.6; fp16: 9.9 -> 6.1, 21.6 -> 17.9, 59.1 -> 50.7
-//   D = 128 bf16: 12.0 -> 8.1, 64 x 1000 under 64 lambda rows 22.0 -> 18.2, 64 x 2000 28.8 -> 27.3, 128 x 4000 75.4 -> 80.0; fp16: 11.2 -> 7.8, 20.7 -> 16.9, 27.0 -> 25.4, 69.5 -> 75.6
+// Where it pays.  A tile takes the contractions, the quantizer and the output one behind the other through one stage each, so a tile
+// more costs more than in the two kernels (D = 128 bf16 2.4 us and 2.0, D = 64 1.3 and 1.2; D = 96, with tensor memory to spare, less:
+// 1.6 and 1.9), and what is saved is one start.  A call that is waited for pays the tile in full, calls in a stream overlap: the limits
+// are the sizes up to which neither is slower.  Tiles per CTA: us per call in a stream over buffers in rotation, two launches -> one,
+// and, where the limit is near, between two waits:
+//   D = 64  bf16  7: 17.0 -> 15.0   16: 26.5 -> 26.9 (33.8 -> 34.3)   20: 31.5 -> 32.0 (39.0 -> 38.9)   28: 41.7 -> 42.1
+//           fp16  7: 16.3 -> 14.3   16: 25.6 -> 25.4                  20: 30.4 -> 30.3 (37.2 -> 37.5)   28: 40.2 -> 40.0
+//   D = 96  bf16  7: 23.7 -> 20.8   20: 46.5 -> 42.2   40: 86.5 -> 74.8;  fp16  7: 21.3 -> 17.6   40: 82.3 -> 68.4
+//   D = 128 bf16  3: 20.3 -> 16.6   6: 26.7 -> 24.0 (34.8 -> 35.2)   7: 28.9 -> 26.4 (34.2 -> 38.5)   10: 34.4 -> 33.7   14: 42.7 -> 43.3
+//           fp16  3: 19.7 -> 17.3   7: 27.5 -> 25.5 (34.3 -> 35.8)   8: 28.9 -> 27.7 (36.1 -> 36.7)   10: 32.5 -> 31.9   14: 40.0 -> 41.7
 bool umma_flush_pays(int D, bool bf16, int64_t S, int64_t rows)
 {
     static DeviceSlots slots;
@@ -590,14 +600,17 @@ bool umma_flush_pays(int D, bool bf16, int64_t S, int64_t rows)
     return D == 96 || tiles <= (D == 64 ? 20 : bf16 ? 6 : 8) * (int64_t)slots.sms[dev];
 }
 
-cudaError_t umma_flush(int D, bool bf16, const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor, uint32_t first_wait_polls,
-                       cudaStream_t stream)
+cudaError_t umma_flush(int D, bool bf16, const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor,
+                       uint32_t first_wait_polls, cudaStream_t stream)
 {
     if (!tensor_map_encode_fn()) return cudaErrorNotSupported;
     switch (D) {
-        case 64: return bf16 ? launch<64, true>(x, N, g, e0, sign_xor, first_wait_polls, stream) : launch<64, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
-        case 96: return bf16 ? launch<96, true>(x, N, g, e0, sign_xor, first_wait_polls, stream) : launch<96, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
-        case 128: return bf16 ? launch<128, true>(x, N, g, e0, sign_xor, first_wait_polls, stream) : launch<128, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
+        case 64: return bf16 ? launch<64, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
+                         : launch<64, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
+        case 96: return bf16 ? launch<96, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
+                         : launch<96, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
+        case 128: return bf16 ? launch<128, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
+                         : launch<128, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
     }
     return cudaErrorInvalidValue;
 }
