@@ -516,7 +516,7 @@ namespace {
 
 template <int D, bool BF16, bool SHORT>
 cudaError_t launch_form(const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor,
-                   uint32_t first_wait_polls, cudaStream_t stream)
+                        uint32_t first_wait_polls, cudaStream_t stream)
 {
     using C = Cfg<D, BF16>;
     static DeviceSlots slots;
@@ -568,8 +568,9 @@ template <int D, bool BF16>
 cudaError_t launch(const void *x, int64_t N, const GemmParams &g, const float *e0, const uint32_t *sign_xor,
                    uint32_t first_wait_polls, cudaStream_t stream)
 {
-    return first_wait_polls ? launch_form<D, BF16, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
-                            : launch_form<D, BF16, false>(x, N, g, e0, sign_xor, 0, stream);
+    // 0, and limits that are no shorter than the default: the default
+    return first_wait_polls && first_wait_polls < kWaitPolls ? launch_form<D, BF16, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
+                                                             : launch_form<D, BF16, false>(x, N, g, e0, sign_xor, 0, stream);
 }
 
 }  // namespace
@@ -606,11 +607,11 @@ cudaError_t umma_flush(int D, bool bf16, const void *x, int64_t N, const GemmPar
     if (!tensor_map_encode_fn()) return cudaErrorNotSupported;
     switch (D) {
         case 64: return bf16 ? launch<64, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
-                         : launch<64, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
+                             : launch<64, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
         case 96: return bf16 ? launch<96, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
-                         : launch<96, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
+                             : launch<96, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
         case 128: return bf16 ? launch<128, true>(x, N, g, e0, sign_xor, first_wait_polls, stream)
-                         : launch<128, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
+                              : launch<128, false>(x, N, g, e0, sign_xor, first_wait_polls, stream);
     }
     return cudaErrorInvalidValue;
 }

@@ -234,8 +234,13 @@ def test_the_block_flush_kernels_first_wait_is_reported_and_service_returns(D, d
     assert kb.kvq_launch_count() - n0 == 1 and word & 7 == 4, "status word %d" % word
     assert all(torch.equal(a, b) for a, b in zip(got, caches()))
     kb.kvq_plan_clear_device_status(plan.handle)
-    kb.kvq_plan_set_wait_limit(plan.handle, 0)
-    kb.kvq_flush_block(plan.handle, x, lam, *got, 5)
+    for polls in (0xFFFFFFFF, 1 << 21, 0):   # longer than the default, long enough, the default again
+        kb.kvq_plan_set_wait_limit(plan.handle, polls)
+        for a in got:
+            a[:, 5:].zero_()
+        kb.kvq_flush_block(plan.handle, x, lam, *got, 5)
+        torch.cuda.synchronize()
+        assert bool(got[2][:, 5:].any(dim=-1).all()) and kb.kvq_plan_device_status(plan.handle) == 0
     packed, scales = two.empty_packed(S * rows), two.empty_scales(S * rows)
     kb.kvq_encode(two.handle, x.view(S * rows, D), lam, packed, scales)
     out = torch.empty(S * rows, D, dtype=dt, device="cuda")
